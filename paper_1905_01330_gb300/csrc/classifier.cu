@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "classifier_f32.h"
 #include "classifier_tc.h"
 #include "tn_internal.h"
 
@@ -29,179 +30,6 @@ namespace {
 
 constexpr int CLS_MAXN = 1024;  // sites passed by value to the sweep kernel
 constexpr int CLS_MAXCHI = 128;
-constexpr int BT = 32;          // samples per CTA of the float32 sweep
-
-struct SweepParams {
-  int32_t n, batch, half, mode;  // half: 0 left (sites 0..ls-1), 1 right (n-1..ls+1); mode 0 fwd, 1 adjoint
-  int32_t t_begin, t_end;        // steps [t_begin, t_end) in sweep order (adjoint runs them backwards)
-  int32_t store_every;           // forward: keep the vector entering step t if (t - store_base) % store_every == 0
-  int32_t store_base;
-  int32_t bond[CLS_MAXN + 1];
-  const float* core[CLS_MAXN];
-  const float* pixels;  // [batch, n]
-  float* state;         // [batch, chi]: vector in, vector out
-  double* lam;          // [batch] forward log-scale, in/out
-  float* store;         // forward: [slot][batch][chi]
-  float* sc;            // [t][batch] per-step scale (forward writes, adjoint reads)
-  float* xout;          // adjoint: [t - t_begin][batch][2 chi] operands of the core gradients
-};
-
-// One CTA sweeps BT samples of one half-chain over [t_begin, t_end).
-template <int CHI>
-__global__ void __launch_bounds__(2 * CHI)
-cls_sweep_simt(const __grid_constant__ SweepParams p) {
-  constexpr int NT = 2 * CHI;
-  constexpr int GQ = CHI / 4;  // threads sharing one group of 4 samples
-  extern __shared__ float smem[];
-  float* Ls = smem;                       // [CHI][2][CHI]
-  float* S = Ls + 2 * CHI * CHI;          // [BT][CHI + 1]
-  float* phi = S + BT * (CHI + 1);        // [2][BT]
-  float* scl = phi + 2 * BT;              // [BT]
-  double* lam = reinterpret_cast<double*>(scl + BT + (BT & 1));  // [BT]
-  const int tid = threadIdx.x;
-  const int b0 = blockIdx.x * BT;
-  const int B = p.batch;
-  const int bq = tid / GQ, jq = tid % GQ;
-  constexpr int SR = CHI + 1;
-
-  for (int i = tid; i < BT * CHI; i += NT) {
-    const int b = i / CHI, k = i % CHI;
-    S[b * SR + k] = (b0 + b < B) ? p.state[(int64_t)(b0 + b) * CHI + k] : 0.0f;
-  }
-  if (tid < BT) lam[tid] = (p.mode == 0 && b0 + tid < B) ? p.lam[b0 + tid] : 0.0;
-  __syncthreads();
-
-  const int nsteps = p.t_end - p.t_begin;
-  for (int q = 0; q < nsteps; ++q) {
-    const int t = p.mode == 0 ? p.t_begin + q : p.t_end - 1 - q;
-    const int site = p.half == 0 ? t : p.n - 1 - t;
-    // forward on the left and adjoint on the right read the core as
-    // L[k=a, s, j=c]; the other two read it transposed, L[k=c, s, j=a]
-    const bool natural = (p.half == 0) == (p.mode == 0);
-    const int Da = p.bond[site], Dc = p.bond[site + 1];
-    const int Din = natural ? Da : Dc, Dout = natural ? Dc : Da;
-    const float* __restrict__ A = p.core[site];
-    for (int i = tid; i < CHI * 2 * CHI; i += NT) {
-      const int j = i % CHI, s = (i / CHI) & 1, k = i / (2 * CHI);
-      float v = 0.0f;
-      if (k < Din && j < Dout) v = natural ? __ldg(A + ((int64_t)k * 2 + s) * Dc + j) : __ldg(A + ((int64_t)j * 2 + s) * Dc + k);
-      Ls[i] = v;
-    }
-    if (tid < BT) {
-      const float x = (b0 + tid < B) ? __ldg(p.pixels + (int64_t)(b0 + tid) * p.n + site) : 0.0f;
-      phi[tid] = cospif(0.5f * x);
-      phi[BT + tid] = sinpif(0.5f * x);
-      if (p.mode == 1) scl[tid] = (b0 + tid < B) ? p.sc[(int64_t)t * B + b0 + tid] : 1.0f;
-    }
-    if (p.mode == 0 && p.store && ((t - p.store_base) % p.store_every) == 0) {
-      float* dst = p.store + (int64_t)((t - p.store_base) / p.store_every) * B * CHI;
-      for (int i = tid; i < BT * CHI; i += NT) {
-        const int b = i / CHI, k = i % CHI;
-        if (b0 + b < B) dst[(int64_t)(b0 + b) * CHI + k] = S[b * SR + k];
-      }
-    }
-    __syncthreads();
-    if (p.mode == 1) {
-      // operands of dL for this step: Phi_s(x_b) g'_b[k] / scale_b; the left
-      // half stores them as [b][s][k], the right half as [b][k][s]
-      float* dst = p.xout + (int64_t)(t - p.t_begin) * B * 2 * CHI;
-      for (int i = tid; i < BT * 2 * CHI; i += NT) {
-        const int b = i / (2 * CHI), r = i % (2 * CHI);
-        if (b0 + b >= B) continue;
-        int s, k;
-        if (p.half == 0) { s = r / CHI; k = r % CHI; }
-        else { k = r >> 1; s = r & 1; }
-        dst[(int64_t)(b0 + b) * 2 * CHI + r] = phi[s * BT + b] * S[b * SR + k] / scl[b];
-      }
-    }
-
-    float acc0[4][4], acc1[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) { acc0[i][j] = 0.0f; acc1[i][j] = 0.0f; }
-    for (int k = 0; k < Din; ++k) {
-      float sv[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) sv[i] = S[(bq * 4 + i) * SR + k];
-      const float4 l0 = *reinterpret_cast<const float4*>(Ls + (k * 2 + 0) * CHI + jq * 4);
-      const float4 l1 = *reinterpret_cast<const float4*>(Ls + (k * 2 + 1) * CHI + jq * 4);
-      const float a0[4] = {l0.x, l0.y, l0.z, l0.w}, a1[4] = {l1.x, l1.y, l1.z, l1.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          acc0[i][j] = fmaf(sv[i], a0[j], acc0[i][j]);
-          acc1[i][j] = fmaf(sv[i], a1[j], acc1[i][j]);
-        }
-    }
-    float out[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int b = bq * 4 + i;
-      const float f0 = phi[b], f1 = phi[BT + b];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) out[i][j] = f0 * acc0[i][j] + f1 * acc1[i][j];
-    }
-    if (p.mode == 0) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        float m = 0.0f;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) m = fmaxf(m, fabsf(out[i][j]));
-#pragma unroll
-        for (int o = GQ / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        const float sc = m > 0.0f ? m : 1.0f;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) out[i][j] = out[i][j] / sc;
-        const int b = bq * 4 + i;
-        if (jq == 0) {
-          lam[b] += (double)logf(sc);  // float32 log, float64 running sum
-          if (b0 + b < B) p.sc[(int64_t)t * B + b0 + b] = sc;
-        }
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float sc = scl[bq * 4 + i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) out[i][j] = out[i][j] / sc;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) S[(bq * 4 + i) * SR + jq * 4 + j] = out[i][j];
-    __syncthreads();
-  }
-  for (int i = tid; i < BT * CHI; i += NT) {
-    const int b = i / CHI, k = i % CHI;
-    if (b0 + b < B) p.state[(int64_t)(b0 + b) * CHI + k] = S[b * SR + k];
-  }
-  if (p.mode == 0 && tid < BT && b0 + tid < B) p.lam[b0 + tid] = lam[tid];
-}
-
-template <int CHI>
-size_t sweep_smem() {
-  return sizeof(float) * (2 * CHI * CHI + BT * (CHI + 1) + 3 * BT + 2) + sizeof(double) * BT;
-}
-
-template <int CHI>
-int launch_sweep_chi(const SweepParams& p, cudaStream_t s) {
-  const size_t smem = sweep_smem<CHI>();
-  static std::atomic<uint64_t> attr{0};
-  if (!smem_limit_once((const void*)cls_sweep_simt<CHI>, smem, &attr)) return TN_ERR_CUDA;
-  cls_sweep_simt<CHI><<<(p.batch + BT - 1) / BT, 2 * CHI, smem, s>>>(p);
-  return cudaGetLastError() == cudaSuccess ? TN_OK : TN_ERR_CUDA;
-}
-
-int launch_sweep(int chi, const SweepParams& p, cudaStream_t s) {
-  if (p.t_end <= p.t_begin) return TN_OK;
-  if (chi == 32) return launch_sweep_chi<32>(p, s);
-  if (chi == 64) return launch_sweep_chi<64>(p, s);
-  return launch_sweep_chi<128>(p, s);
-}
 
 // ------------------------------------------------------------- label core
 // The label core C[a, s, l, c] meets the two half-chain vectors vL, vR:
@@ -360,12 +188,10 @@ struct ClsLayout {
   float* replay[2];     // running vector of a segment's recomputation [batch][chi]
   double* replay_lam[2];
   // float32 path
-  float* seg;      // recomputed vectors of one segment [seg_len][batch][chi]
-  float* X;        // [seg_len][batch][2 chi]
-  uint8_t* plan_ws;  // every segment's grouped plan, one region each
-  size_t plan_bytes;
-  int plan_count;
-  // tensor-core path
+  float* seg[2];   // recomputed vectors of one segment [seg_len][batch][chi]
+  float* H[2];     // the adjoint's g / scale of one segment, likewise
+  float2* phi[2];  // its feature pairs [seg_len][cls_f32_phi_row]
+  // tensor-core path (the images are the float32 path's too)
   uint8_t* fimg[2];  // forward core images per half
   uint8_t* aimg[2];  // adjoint core images per half
   uint8_t* vseg[2];  // bf16 vector tiles of one segment per half
@@ -415,19 +241,16 @@ ClsLayout cls_layout(uint8_t* base, const tn_mps* W, int ls, int L, int batch, i
     w.replay[h] = reinterpret_cast<float*>(take(bwd ? vec : 0));
     w.replay_lam[h] = reinterpret_cast<double*>(take(bwd ? sizeof(double) * (size_t)batch : 0));
   }
-  // float32 backward: recomputed vectors and gradient operands of a segment,
-  // and one grouped plan per segment (descriptors, split results to zero and
-  // the unit map: each spec at most 2 x 1 output tiles of 128 (2 chi <= 256)
-  // times ceil(batch / 2048) k ranges)
-  w.seg = reinterpret_cast<float*>(take(bwd && ck > 1 ? vec * (size_t)w.seg_len : 0));
-  w.X = reinterpret_cast<float*>(take(bwd ? 2 * vec * (size_t)w.seg_len : 0));
-  const size_t units_per_spec = 2 * (size_t)((batch + 64 * MAX_SLABS_PER_UNIT - 1) / (64 * MAX_SLABS_PER_UNIT));
-  w.plan_bytes = bwd ? align256(sizeof(ContractDesc) * (size_t)w.seg_len) + align256(sizeof(ZeroRange) * (size_t)w.seg_len) +
-                           align256(sizeof(int32_t) * (size_t)w.seg_len * units_per_spec)
-                     : 0;
-  w.plan_count = bwd ? (w.T[0] + w.seg_len - 1) / w.seg_len + (w.T[1] + w.seg_len - 1) / w.seg_len : 0;
-  w.plan_ws = take(w.plan_bytes * (size_t)w.plan_count);
-  // tensor-core path (sized for the split BF16x3 images, the larger)
+  // float32 backward: recomputed vectors, adjoint vectors and features of
+  // both halves' segments
+  for (int h = 0; h < 2; ++h) {
+    const size_t steps = (size_t)std::min(w.seg_len, std::max(w.T[h], 1));
+    w.seg[h] = reinterpret_cast<float*>(take(bwd && ck > 1 ? vec * steps : 0));
+    w.H[h] = reinterpret_cast<float*>(take(bwd ? vec * steps : 0));
+    w.phi[h] = reinterpret_cast<float2*>(take(bwd ? sizeof(float2) * cls_f32_phi_row(batch) * steps : 0));
+  }
+  // core images (sized for the split BF16x3 ones, as large as the float32
+  // ones or larger) and the tensor-core path's vector tiles
   for (int h = 0; h < 2; ++h) {
     w.fimg[h] = take(cls_fwd_image_bytes(chi, 1) * (size_t)w.T[h]);
     w.aimg[h] = take(bwd ? cls_adj_image_bytes(chi, 1) * (size_t)w.T[h] : 0);
@@ -455,20 +278,38 @@ int check_classifier(const tn_mps* W, int ls, int L, const float* pixels, int ba
   return TN_OK;
 }
 
-SweepParams sweep_params(const tn_mps* W, const ClsLayout& w, const float* pixels, int half, int mode) {
-  SweepParams p;
+// Both halves' cores packed into the float32 images of one kind.
+int pack_images_f32(const tn_mps* W, const ClsLayout& w, int adjoint, cudaStream_t s) {
+  ClsF32PackParams pp;
+  memset(&pp, 0, sizeof(pp));
+  pp.n = W->n;
+  pp.chi = w.chi;
+  pp.adjoint = adjoint;
+  for (int i = 0; i <= W->n; ++i) pp.bond[i] = (int32_t)W->bond[i];
+  for (int i = 0; i < W->n; ++i) pp.core[i] = W->cores[i];
+  for (int h = 0; h < 2; ++h) {
+    pp.T[h] = w.T[h];
+    pp.images[h] = reinterpret_cast<float*>(adjoint ? w.aimg[h] : w.fimg[h]);
+  }
+  return cls_f32_pack(pp, s);
+}
+
+ClsF32Params f32_params(const tn_mps* W, const ClsLayout& w, const float* pixels, int adjoint) {
+  ClsF32Params p;
   memset(&p, 0, sizeof(p));
   p.n = W->n;
   p.batch = w.batch;
-  p.half = half;
-  p.mode = mode;
-  for (int i = 0; i <= W->n; ++i) p.bond[i] = (int32_t)W->bond[i];
-  for (int i = 0; i < W->n; ++i) p.core[i] = W->cores[i];
-  p.pixels = pixels;
-  p.state = w.state[half];
-  p.lam = w.lam[half];
-  p.sc = w.sc[half];
+  int64_t kmax = 1;
+  for (int i = 0; i <= W->n; ++i) kmax = std::max(kmax, W->bond[i]);
+  p.kmax = (int32_t)((kmax + 3) / 4 * 4);
   p.store_every = 1;
+  p.pixels = pixels;
+  for (int h = 0; h < 2; ++h) {
+    p.t_end[h] = w.T[h];
+    p.images[h] = reinterpret_cast<const float*>(adjoint ? w.aimg[h] : w.fimg[h]);
+    p.sc[h] = w.sc[h];
+  }
+  p.status = status_word();
   return p;
 }
 
@@ -546,6 +387,21 @@ LabelParams label_params(const tn_mps* W, const ClsLayout& w, const float* pixel
 // the float32 kernel's time).
 int label_prec(int prec) { return prec == TN_PREC_FP32 ? TN_PREC_FP32 : TN_PREC_BF16X3; }
 
+// The accumulated per-step gradients of both halves into the cores' shapes.
+int scatter_gradients(const tn_mps* W, const ClsLayout& w, float* const* dcores, cudaStream_t s) {
+  ClsScatterParams sp;
+  memset(&sp, 0, sizeof(sp));
+  sp.n = W->n;
+  sp.chi = w.chi;
+  sp.T[0] = w.T[0];
+  sp.T[1] = w.T[1];
+  for (int i = 0; i <= W->n; ++i) sp.bond[i] = (int32_t)W->bond[i];
+  for (int i = 0; i < W->n; ++i) sp.dcore[i] = dcores[i];
+  sp.grad[0] = w.grad[0];
+  sp.grad[1] = w.grad[1];
+  return cls_scatter_grad(sp, s);
+}
+
 // G[b, a, s, l] = sum_c vR[b, c] C[a, s, l, c].
 int label_G(const tn_mps* W, const ClsLayout& w, int prec, cudaStream_t s) {
   const int64_t DL = W->bond[w.ls], DR = W->bond[w.ls + 1], B = w.batch, L = w.L;
@@ -596,17 +452,15 @@ int tn_mps_classify(const tn_mps* W, int label_site, int n_labels, const float* 
     if (cudaGetLastError() != cudaSuccess) return TN_ERR_CUDA;
   }
   if (prec == TN_PREC_FP32) {
+    if ((rc = pack_images_f32(W, w, 0, s)) != TN_OK) return rc;
+    ClsF32Params p = f32_params(W, w, pixels, 0);
     for (int h = 0; h < 2; ++h) {
-      SweepParams p = sweep_params(W, w, pixels, h, 0);
-      p.t_begin = 0;
-      p.t_end = w.T[h];
-      if (ckpt_every > 0) {
-        p.store = w.ckpt[h];
-        p.store_every = ckpt_every;
-        p.store_base = 0;
-      }
-      if ((rc = launch_sweep(w.chi, p, s)) != TN_OK) return rc;
+      p.state[h] = w.state[h];
+      p.lam[h] = w.lam[h];
+      if (ckpt_every > 0) p.store[h] = w.ckpt[h];
     }
+    p.store_every = ckpt_every > 0 ? ckpt_every : 1;
+    if ((rc = cls_f32_sweep(w.chi, 0, p, s)) != TN_OK) return rc;
   } else {
     // both half-chains in one tcgen05 launch
     const int split = prec == TN_PREC_BF16X3;
@@ -644,6 +498,7 @@ int tn_mps_classify_backward(const tn_mps* W, int label_site, int n_labels, cons
   const int chi = w.chi, n = W->n, ls = label_site, L = n_labels;
   const int split = prec == TN_PREC_BF16X3;
   if (prec != TN_PREC_FP32 && !cls_adj_tc_supported(chi, split)) return TN_ERR_UNSUPPORTED;
+  if (prec == TN_PREC_FP32 && batch > 0 && stream_capturing(s)) return TN_ERR_UNSUPPORTED;  // as documented
   if (batch == 0) {
     for (int i = 0; i < n; ++i) {
       const int64_t e = W->bond[i] * 2 * W->bond[i + 1] * (i == ls ? L : 1);
@@ -730,106 +585,53 @@ int tn_mps_classify_backward(const tn_mps* W, int label_site, int n_labels, cons
       if ((rc = cls_fwd_tc_launch(chi, split, f, s)) != TN_OK) return rc;
       if ((rc = cls_adj_tc_launch(chi, split, a, s)) != TN_OK) return rc;
     }
-    ClsScatterParams sp;
-    memset(&sp, 0, sizeof(sp));
-    sp.n = n;
-    sp.chi = chi;
-    sp.T[0] = w.T[0];
-    sp.T[1] = w.T[1];
-    for (int i = 0; i <= n; ++i) sp.bond[i] = (int32_t)W->bond[i];
-    for (int i = 0; i < n; ++i) sp.dcore[i] = dcores[i];
-    sp.grad[0] = w.grad[0];
-    sp.grad[1] = w.grad[1];
-    return cls_scatter_grad(sp, s);
+    return scatter_gradients(W, w, dcores, s);
   }
 
-  // float32: per half and segment (from the label core outwards) the
-  // recomputed vectors, the adjoint sweep writing the gradient operands, and
-  // one grouped tensordot over the batch for the segment's cores. The
-  // segments' plans are built and uploaded before the first sweep.
-  struct SegPlan {
-    int h, t0, t1;
-    const float* vecs;
-    tn_group_plan* plan;
-    uint8_t* ws;
-  };
-  std::vector<SegPlan> plans;
-  auto destroy_all = [&]() {
-    for (auto& sp : plans)
-      if (sp.plan) tn_group_plan_destroy(sp.plan);
-  };
+  // float32: per round one launch recomputes both halves' segments from
+  // their kept vectors (the replay rewrites the same per-step scales), one
+  // runs both adjoint segments keeping g / scale and the features of every
+  // step, and one sums the segment's core gradients over the batch
+  if ((rc = pack_images_f32(W, w, 0, s)) != TN_OK) return rc;
+  if ((rc = pack_images_f32(W, w, 1, s)) != TN_OK) return rc;
   for (int h = 0; h < 2; ++h)
-    for (int k = 0; k < nseg[h]; ++k) {
+    if (w.T[h] > 0 &&
+        cudaMemsetAsync(w.grad[h], 0, sizeof(float) * (size_t)w.T[h] * chi * 2 * chi, s) != cudaSuccess)
+      return TN_ERR_CUDA;
+  for (int k = 0; k < rounds; ++k) {
+    ClsF32Params f = f32_params(W, w, pixels, 0);
+    ClsF32Params a = f32_params(W, w, pixels, 1);
+    ClsF32GradParams g;
+    memset(&g, 0, sizeof(g));
+    g.batch = batch;
+    g.status = f.status;
+    for (int h = 0; h < 2; ++h) {
       int t0, t1;
       seg_range(h, k, &t0, &t1);
-      const float* vecs = ckpt_every <= 1 ? w.ckpt[h] + (int64_t)t0 * batch * chi : w.seg;
-      std::vector<tn_contract_spec> specs((size_t)(t1 - t0));
-      for (int t = t0; t < t1; ++t) {
-        const int site = h == 0 ? t : n - 1 - t;
-        const int64_t Da = W->bond[site], Dc = W->bond[site + 1];
-        tn_contract_spec& sp = specs[(size_t)(t - t0)];
-        memset(&sp, 0, sizeof(sp));
-        float* v = const_cast<float*>(vecs) + (int64_t)(t - t0) * batch * chi;
-        float* x = w.X + (int64_t)(t - t0) * batch * 2 * chi;
-        const int64_t shd[3] = {Da, 2, Dc}, std0[3] = {0, 0, 0};
-        sp.C = strided(dcores[site], 3, shd, std0);
-        sp.nshared = 1;
-        if (h == 0) {
-          // dW[a, s, c] = sum_b v_b[a] X_b[s, c]
-          const int64_t shv[2] = {batch, Da}, stv[2] = {chi, 1};
-          const int64_t shx[3] = {batch, 2, Dc}, stx[3] = {2 * chi, chi, 1};
-          sp.A = strided(v, 2, shv, stv);
-          sp.B = strided(x, 3, shx, stx);
-        } else {
-          // dW[a, s, c] = sum_b X_b[a, s] v_b[c]
-          const int64_t shx[3] = {batch, Da, 2}, stx[3] = {2 * chi, 2, 1};
-          const int64_t shv[2] = {batch, Dc}, stv[2] = {chi, 1};
-          sp.A = strided(x, 3, shx, stx);
-          sp.B = strided(v, 2, shv, stv);
-        }
+      f.t_begin[h] = a.t_begin[h] = g.t_begin[h] = t0;
+      f.t_end[h] = a.t_end[h] = g.t_end[h] = t1;
+      if (ckpt_every > 1) {
+        if (t1 > t0 && cudaMemcpyAsync(w.replay[h], w.ckpt[h] + (int64_t)(t0 / ckpt_every) * batch * chi, vbytes,
+                                       cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+          return TN_ERR_CUDA;
+        f.state[h] = w.replay[h];
+        f.lam[h] = w.replay_lam[h];
+        f.store[h] = w.seg[h];
+        f.store_base[h] = t0;
       }
-      SegPlan sp{h, t0, t1, vecs, nullptr, w.plan_ws + (size_t)plans.size() * w.plan_bytes};
-      if ((rc = group_plan_create_ex(specs.data(), (int)specs.size(), TN_PREC_FP32, false, &sp.plan)) != TN_OK) {
-        destroy_all();
-        return rc;
-      }
-      plans.push_back(sp);
-      if ((rc = tn_group_plan_upload(sp.plan, sp.ws, w.plan_bytes, s)) != TN_OK) {
-        destroy_all();
-        return rc;
-      }
+      a.state[h] = w.g[h];
+      a.h[h] = w.H[h];
+      a.phi[h] = w.phi[h];
+      g.v[h] = ckpt_every > 1 ? w.seg[h] : w.ckpt[h] + (int64_t)t0 * batch * chi;
+      g.h[h] = w.H[h];
+      g.phi[h] = w.phi[h];
+      g.grad[h] = w.grad[h];
     }
-  for (const SegPlan& sp : plans) {
-    const int h = sp.h, t0 = sp.t0, t1 = sp.t1;
-    if (ckpt_every > 1) {
-      // recompute the segment from its kept vector, keeping the vector
-      // entering every step; the replay rewrites the same per-step scales
-      if (cudaMemcpyAsync(w.replay[h], w.ckpt[h] + (int64_t)(t0 / ckpt_every) * batch * chi, vbytes,
-                          cudaMemcpyDeviceToDevice, s) != cudaSuccess) {
-        destroy_all();
-        return TN_ERR_CUDA;
-      }
-      SweepParams p = sweep_params(W, w, pixels, h, 0);
-      p.state = w.replay[h];
-      p.lam = w.replay_lam[h];
-      p.t_begin = t0;
-      p.t_end = t1;
-      p.store = w.seg;
-      p.store_every = 1;
-      p.store_base = t0;
-      if ((rc = launch_sweep(chi, p, s)) != TN_OK) break;
-    }
-    // adjoint steps t1-1 .. t0: g <- adjoint step, X[t - t0] <- gradient operands
-    SweepParams p = sweep_params(W, w, pixels, h, 1);
-    p.state = w.g[h];
-    p.t_begin = t0;
-    p.t_end = t1;
-    p.xout = w.X;
-    if ((rc = launch_sweep(chi, p, s)) != TN_OK) break;
-    if ((rc = tn_group_plan_run(sp.plan, sp.ws, w.plan_bytes, s)) != TN_OK) break;
+    if (ckpt_every > 1 && (rc = cls_f32_sweep(chi, 0, f, s)) != TN_OK) return rc;
+    if ((rc = cls_f32_sweep(chi, 1, a, s)) != TN_OK) return rc;
+    if ((rc = cls_f32_grad(chi, g, s)) != TN_OK) return rc;
   }
-  destroy_all();
-  return rc;
+  return scatter_gradients(W, w, dcores, s);
 }
 
 }  // extern "C"

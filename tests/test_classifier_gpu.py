@@ -314,3 +314,37 @@ def test_backward_under_graph_capture(tn):
     grads = tn.mps_classify_backward(dc, ls, px, dft, ws, prec="fp32", ckpt_every=4)
     torch.cuda.synchronize()
     assert tn.sync_status() == 0 and all(bool(torch.isfinite(g).all()) for g in grads)
+
+
+@pytest.mark.parametrize("chi,B,ls,ck", [(8, 1, 3, 2), (32, 129, 4, 1), (32, 2433, 4, 3), (33, 15, 6, 4), (40, 1217, 3, 2),
+                                         (64, 2433, 4, 3), (64, 17, 0, 2), (100, 65, 7, 3), (128, 1217, 5, 4),
+                                         (128, 2433, 4, 3)])
+def test_fp32_sweep_tiles(tn, chi, B, ls, ck):
+    # the float32 sweep's sample tiles (16, 32 and 64 samples; 32, 64 and 128
+    # at chi <= 32: chosen by the batch) with ragged last tiles, bonds padded
+    # to 32, 64 and 128 and uneven along the chain, a chain with an empty half,
+    # odd batches (the gradient's feature rows are padded to an even count).
+    # Tolerances as above: 1e-5 sqrt(sites) scores, 1e-4 gradients.
+    n, L = 8, 3
+    bonds = [1] + [max(1, chi - 3 * (i % 3)) for i in range(n - 1)] + [1]
+    cores = []
+    for i in range(n):
+        a, b = bonds[i], bonds[i + 1]
+        shape = (a, 2, L, b) if i == ls else (a, 2, b)
+        eps = synth.normal_f32(synth.substream(700 + chi, i), shape, 0.1)
+        eye = np.eye(a, b, dtype=np.float32)
+        cores.append(eps + (eye[:, None, None, :] if i == ls else eye[:, None, :]))
+    px = synth.pixels(B, n, seed=72)
+    y = synth.labels(B, L, seed=73)
+    ft_ref, lam_ref = oracle.classify(cores, ls, px)
+    loss_ref, g_ref = oracle.classify_grad(cores, ls, px, y)
+    dc = [dev(c) for c in cores]
+    ft, lam, ws = tn.mps_classify(dc, ls, dev(px), prec="fp32", ckpt_every=ck)
+    loss, dft = tn.mps_classify_loss(ft, torch.from_numpy(y).cuda())
+    grads = tn.mps_classify_backward(dc, ls, dev(px), dft, ws, prec="fp32", ckpt_every=ck)
+    assert tn.sync_status() == 0
+    assert score_err(ft, lam, ft_ref, lam_ref).max() <= 1e-5 * math.sqrt(n)
+    assert abs(loss.item() - loss_ref) <= 1e-5 * abs(loss_ref)
+    for i, (g, r) in enumerate(zip(grads, g_ref)):
+        err = np.linalg.norm(g.double().cpu().numpy() - r) / np.linalg.norm(r)
+        assert err <= 1e-4, (i, err)
