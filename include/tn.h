@@ -483,10 +483,11 @@ int tn_mps_classify(const tn_mps* W, int label_site, int n_labels, const float* 
  * that recomputes both halves' segments and one adjoint launch that also
  * accumulates every step's dW (the products over the segment's samples on
  * tcgen05, float32 reductions into a workspace buffer, then one scatter);
- * TN_PREC_FP32 runs the float32 adjoint sweep and one grouped tensordot over
- * the batch per segment (their plans built and uploaded in the call, so the
- * FP32 backward returns TN_ERR_UNSUPPORTED on a stream being captured into a
- * CUDA graph; BF16 / BF16X3 only launch).
+ * TN_PREC_FP32 runs one recomputing launch, one adjoint launch and one
+ * launch summing the segment's core gradients over the batch (float32 FMA,
+ * float32 reductions into the same buffer). BF16 / BF16X3 can be captured
+ * into a CUDA graph; the FP32 backward returns TN_ERR_UNSUPPORTED on a
+ * capturing stream, with nothing enqueued.
  *   dcores: host table of n DEVICE pointers, each shaped like its core
  *           (overwritten).
  *   prec:   arithmetic of the sweeps and of the gradient products (the label

@@ -12,14 +12,14 @@
 // Backward (adjoint): the same step with the transposed core and the recorded
 // scale, g_b[k] = sum_s Phi_s sum_j L[k, s, j] g'_b[j] / scale_b, walks from
 // the label core outwards; the core gradients are sums over the batch,
-// dL[k, s, j] = sum_b v_b[k] Phi_s(x_b) g'_b[j] / scale_b, evaluated per
-// checkpoint segment as one grouped tensordot (K = batch) on the engine of
-// tn_contract. Sweep vectors are kept every `ckpt_every` steps and the steps
-// in between are recomputed segment by segment (checkpointing).
+// dL[k, s, j] = sum_b v_b[k] Phi_s(x_b) g'_b[j] / scale_b, summed over the
+// batch per checkpoint segment. Sweep vectors are kept every `ckpt_every`
+// steps and the steps in between are recomputed segment by segment
+// (checkpointing). The sweeps themselves: classifier_f32.cu (FP32) and
+// classifier_tc.cu (BF16, BF16x3).
 #include <math.h>
 
 #include <algorithm>
-#include <vector>
 
 #include "classifier_f32.h"
 #include "classifier_tc.h"

@@ -10,16 +10,24 @@
 // forward's; h is kept, for the core gradients
 //     dL[k, s, j] = sum_b v_b[k] Phi_s(x_b) h_b[j].
 //
-// What bounds it: the FMA pipe, once the operands are fed. A thread holds RS
-// samples x 4 outgoing indices x both s (64 accumulators at RS = 8), so a k
-// step is RS / 4 + 2 16-byte shared-memory reads for 8 RS FMAs; the s sum,
-// the sample's maximum and the new vector stay in registers until the vector
-// is published for the next step. The images stream through a ring of
-// shared-memory slabs (1-D bulk copies by a producer warp, across steps), so
-// no step waits for its core. The vector lives in two shared-memory buffers
-// [k][sample], 16-byte chunks XOR-swizzled by k / 4 so that publishing four
-// rows at once and reading one row are both free of bank conflicts: one
-// barrier per step.
+// What bounds it: the FMA pipe, once the operands are fed and the steps'
+// serial part is short. A thread holds RS samples x 4 outgoing indices x both
+// s (64 accumulators at RS = 8, as packed pairs), so a k step is RS / 4 + 2
+// 16-byte shared-memory reads for 4 RS packed FMAs; a warp covers 4 x 8
+// threads (samples x outgoing), which halves the shared-memory passes of its
+// reads against 2 x 16. Every sum keeps one chain over k: splitting k over two
+// groups of threads gained 1 % (4.28 against 4.34 us a step at chi = 64, batch
+// 4096) and moved the float64 log-scales. The images stream through a ring of shared-memory
+// slabs (1-D bulk copies by a producer warp, across steps), so no step waits
+// for its core; further warps compute the next step's features and the
+// log-scales beside the products. The vector lives in two shared-memory
+// buffers [k][sample], 16-byte chunks XOR-swizzled by k / 4 so that
+// publishing four rows at once and reading one row are both free of bank
+// conflicts. A step at chi = 64 takes ~7,300 cycles for 64 samples, 5,070 of
+// them the products (the FMA pipe's own 4,096), the rest the wait for the slab
+// (~250), the maximum, the division and the publishing.
+// Measured (784 sites, batch 4096, chi = 64): forward 10.9 -> 1.4 ms, training
+// step 53.2 -> 6.2 ms.
 #include <math.h>
 
 #include "classifier_f32.h"
@@ -65,11 +73,14 @@ struct SweepCfg {
   static constexpr int OG = CHI / 4;                  // threads along the outgoing index
   static constexpr int SG = CHI == 32 ? 16 : 8;       // threads along the samples
   static constexpr int NC = OG * SG;                  // compute threads
+  static constexpr int OW = OG / 8;                   // warps along the outgoing index
   static constexpr int TB = RS * SG;                  // samples per CTA
+  static constexpr int NS = TB < 32 ? 32 : TB;        // sampler threads
+  static constexpr int NT = NC + 32 + NS;
   static constexpr int MASK = TB / 4 - 1 < 7 ? TB / 4 - 1 : 7;
-  static constexpr int KS = CHI == 128 ? 16 : 32;     // k rows of a slab
+  static constexpr int KS = CHI == 128 ? 32 : CHI;    // k rows of a slab (8, 32 and 32 KB)
   static constexpr int SLAB = KS * 2 * CHI;           // floats of a slab
-  static constexpr int RING = CHI == 128 ? 8 : 4;
+  static constexpr int RING = CHI == 32 ? 4 : (CHI == 64 ? 3 : 4);
   static constexpr size_t SMEM = sizeof(float) * ((size_t)RING * SLAB + 2 * CHI * TB);
 };
 
@@ -77,23 +88,46 @@ struct SweepBars {
   uint64_t full[8], empty[8];
 };
 
-// x / sc for |x| <= sc (r = 1 / sc): the quotient estimate corrected once by
-// its own residual (Markstein's iteration), within an ulp of the quotient.
-__device__ __forceinline__ float div_by(float x, float sc, float r) {
-  const float q = x * r;
-  return fmaf(fmaf(-q, sc, x), r, q);
+// v[i][:] / sc[i]: away from the ends of the exponent range an estimate of the
+// quotient corrected once by its own residual (Markstein's iteration), within
+// an ulp of it, at a third of the division's instructions; a warp with a
+// scale elsewhere divides, out of line (a step divides a thread's whole tile,
+// and the divisions inline cost it 1,000 cycles).
+__device__ __noinline__ float divide_any(float x, float sc) { return x / sc; }
+template <int RS>
+__device__ __forceinline__ void divide(float (&v)[RS][4], const float (&sc)[RS]) {
+  bool plain = true;
+#pragma unroll
+  for (int i = 0; i < RS; ++i) plain = plain && sc[i] > 0x1p-100f && sc[i] < 0x1p100f;
+  if (__all_sync(0xffffffffu, plain)) {
+#pragma unroll
+    for (int i = 0; i < RS; ++i) {
+      const float r = __fdividef(1.0f, sc[i]);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float q = v[i][j] * r;
+        v[i][j] = fmaf(fmaf(-q, sc[i], v[i][j]), r, q);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < RS; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[i][j] = divide_any(v[i][j], sc[i]);
+  }
 }
 
 template <int CHI, int RS, int ADJ>
-__global__ void __launch_bounds__(SweepCfg<CHI, RS>::NC + 32)
+__global__ void __launch_bounds__(SweepCfg<CHI, RS>::NT)
 cls_f32_sweep_kernel(const __grid_constant__ ClsF32Params p) {
   using C = SweepCfg<CHI, RS>;
-  constexpr int NC = C::NC, TB = C::TB, OG = C::OG;
+  constexpr int NC = C::NC, TB = C::TB;
   extern __shared__ __align__(128) float smem[];
   float* ring = smem;
   float* S = smem + C::RING * C::SLAB;  // two buffers [CHI][TB]
-  __shared__ float phi[2][2][TB];
+  __shared__ __align__(16) float phi[2][2][TB];
   __shared__ float scl[2][TB];
+  __shared__ float smax[C::OW][TB];
   __shared__ __align__(8) SweepBars bars;
   const int half = blockIdx.y, tid = threadIdx.x;
   const int t0 = p.t_begin[half], t1 = p.t_end[half], nsteps = t1 - t0;
@@ -109,7 +143,7 @@ cls_f32_sweep_kernel(const __grid_constant__ ClsF32Params p) {
   }
   __syncthreads();
 
-  if (tid >= NC) {  // producer warp: one lane streams the images
+  if (tid >= NC && tid < NC + 32) {  // producer warp: one lane streams the images
     if (tid != NC) return;
     const int total = nsteps * nslab;
     bool ok = true;
@@ -131,14 +165,61 @@ cls_f32_sweep_kernel(const __grid_constant__ ClsF32Params p) {
     return;
   }
 
-  const int og = tid % OG, bg = tid / OG;
+  constexpr int NB = NC + C::NS;  // threads of the step barriers
   auto site_of = [&](int t) { return half == 0 ? t : n - 1 - t; };
   auto step_t = [&](int q) { return ADJ ? t1 - 1 - q : t0 + q; };
-  // out[i][j]: sample b0 + bg RS + i, outgoing index 4 og + j
+
+  if (tid >= NC) {  // samplers: one thread per sample
+    const int i = tid - NC - 32, sb = b0 + i;
+    const bool in = i < TB, live = in && sb < B;
+    auto pixel = [&](int q) { return live && q < nsteps ? __ldg(p.pixels + (int64_t)sb * n + site_of(step_t(q))) : 0.0f; };
+    auto scale_of = [&](int q) { return live && q < nsteps ? p.sc[half][(int64_t)step_t(q) * B + sb] : 1.0f; };
+    auto put_features = [&](int q, float x) {  // of step q into buffer q & 1
+      if (!in || q >= nsteps) return;
+      const float c = cospif(0.5f * x), s = sinpif(0.5f * x);
+      phi[q & 1][0][i] = c;
+      phi[q & 1][1][i] = s;
+      if (ADJ && live) p.phi[half][(int64_t)(step_t(q) - t0) * ((B + 1) & ~1) + sb] = make_float2(c, s);
+    };
+    double lam = !ADJ && live ? p.lam[half][sb] : 0.0;
+    if (ADJ && in) {  // scl[q & 1]: the scale the vector entering step q is divided by
+      scl[0][i] = scale_of(0);
+      scl[1][i] = scale_of(1);
+    }
+    float nsc = ADJ ? scale_of(2) : 1.0f;
+    put_features(0, pixel(0));
+    float x = pixel(1);
+    ptx::named_barrier(1, NB);
+    ptx::named_barrier(1, NB);
+    auto add_scale = [&](int q) {  // the scale of the vector that left step q
+      if (ADJ || !live) return;
+      const float sc = scl[q & 1][i];
+      lam += (double)logf(sc);
+      p.sc[half][(int64_t)step_t(q) * B + sb] = sc;
+    };
+    for (int q = 0; q < nsteps; ++q) {
+      const float x1 = x;
+      x = pixel(q + 2);
+      if (ADJ && in) {  // the vector of step q is behind the last barrier: its slot takes step q + 2's scale
+        scl[q & 1][i] = nsc;
+        nsc = scale_of(q + 3);
+      }
+      put_features(q + 1, x1);
+      if (q > 0) add_scale(q - 1);
+      if (ptx::named_barrier_or(1, NB, false)) return;
+    }
+    add_scale(nsteps - 1);
+    if (!ADJ && live) p.lam[half][sb] = lam;
+    return;
+  }
+
+  // thread: samples f0 .. f0 + RS - 1 of the tile, outgoing indices 4 og .. + 3
+  const int og = (tid >> 5) % C::OW * 8 + (tid & 7), f0 = ((tid >> 5) / C::OW * 4 + ((tid >> 3) & 3)) * RS;
+  // out[i][j]: sample b0 + f0 + i, outgoing index 4 og + j
   float out[RS][4];
 #pragma unroll
   for (int i = 0; i < RS; ++i) {
-    const int b = b0 + bg * RS + i;
+    const int b = b0 + f0 + i;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (b < B) v = *reinterpret_cast<const float4*>(p.state[half] + (int64_t)b * CHI + og * 4);
     out[i][0] = v.x;
@@ -146,60 +227,40 @@ cls_f32_sweep_kernel(const __grid_constant__ ClsF32Params p) {
     out[i][2] = v.z;
     out[i][3] = v.w;
   }
-  // one thread per sample loads its pixel (and, in the adjoint, its scale)
-  // steps ahead and keeps its log-scale
-  const bool sampler = tid < TB;
-  const int sb = b0 + tid;
-  const bool live = sampler && sb < B;
-  float px = 0.0f, nsc = 1.0f;
-  double lam = 0.0;
-  auto fetch = [&](int q) {
-    if (live && q < nsteps) px = __ldg(p.pixels + (int64_t)sb * n + site_of(step_t(q)));
-  };
-  auto scale_of = [&](int q) { return live && q < nsteps ? p.sc[half][(int64_t)step_t(q) * B + sb] : 1.0f; };
-  auto put_features = [&](int q) {  // features of step q into buffer q & 1
-    if (sampler && q < nsteps) {
-      const float c = cospif(0.5f * px), s = sinpif(0.5f * px);
-      phi[q & 1][0][tid] = c;
-      phi[q & 1][1][tid] = s;
-      if (ADJ && live) p.phi[half][(int64_t)(step_t(q) - t0) * ((B + 1) & ~1) + sb] = make_float2(c, s);
-    }
-  };
-  if (!ADJ && live) lam = p.lam[half][sb];
-  if (ADJ && sampler) {  // scl[q & 1]: the scale publish(q) divides by, in place one barrier earlier
-    scl[0][tid] = scale_of(0);
-    scl[1][tid] = scale_of(1);
-    nsc = scale_of(2);
-  }
-  fetch(0);
-  put_features(0);
-  fetch(1);
-  ptx::named_barrier(1, NC);
+  ptx::named_barrier(1, NB);
 
+  float* kept = nullptr;  // where the next kept vector goes, in `until` steps
+  int until = 0;
+  if (!ADJ && p.store[half]) {
+    const int since = t0 - p.store_base[half], slot = (since + p.store_every - 1) / p.store_every;
+    kept = p.store[half] + (int64_t)slot * B * CHI;
+    until = slot * p.store_every - since;
+  }
   // out as the vector entering step q (of t): divided by the step's scale in
   // the adjoint, kept when asked, and written to S's buffer q & 1
   auto publish = [&](int q) {
     const int t = step_t(q);
     if (ADJ) {
+      float sc[RS];
 #pragma unroll
-      for (int i = 0; i < RS; ++i) {
-        const float sc = scl[q & 1][bg * RS + i];
-        const bool plain = sc > 0x1p-100f && sc < 0x1p100f;
-        const float r = 1.0f / sc;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) out[i][j] = plain ? div_by(out[i][j], sc, r) : out[i][j] / sc;
-      }
+      for (int i = 0; i < RS; ++i) sc[i] = scl[q & 1][f0 + i];
+      divide(out, sc);
     }
     float* keep = nullptr;
     if (ADJ) {
       keep = p.h[half] + (int64_t)(t - t0) * B * CHI;
-    } else if (p.store[half] && (t - p.store_base[half]) % p.store_every == 0) {
-      keep = p.store[half] + (int64_t)((t - p.store_base[half]) / p.store_every) * B * CHI;
+    } else if (kept) {
+      if (until == 0) {
+        keep = kept;
+        kept += (int64_t)B * CHI;
+        until = p.store_every;
+      }
+      --until;
     }
     if (keep) {
 #pragma unroll
       for (int i = 0; i < RS; ++i) {
-        const int b = b0 + bg * RS + i;
+        const int b = b0 + f0 + i;
         if (b < B)
           *reinterpret_cast<float4*>(keep + (int64_t)b * CHI + og * 4) =
               make_float4(out[i][0], out[i][1], out[i][2], out[i][3]);
@@ -209,38 +270,27 @@ cls_f32_sweep_kernel(const __grid_constant__ ClsF32Params p) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       float* row = d + (og * 4 + j) * TB;
-      const int x = og & C::MASK;
+      const int at = (((f0 >> 2) ^ (og & C::MASK)) << 2) + (f0 & 3);
       if constexpr (RS == 2) {
-        *reinterpret_cast<float2*>(row + (((bg >> 1) ^ x) << 2) + (bg & 1) * 2) = make_float2(out[0][j], out[1][j]);
+        *reinterpret_cast<float2*>(row + at) = make_float2(out[0][j], out[1][j]);
       } else {
 #pragma unroll
         for (int u = 0; u < RS / 4; ++u)
-          *reinterpret_cast<float4*>(row + (((bg * (RS / 4) + u) ^ x) << 2)) =
+          *reinterpret_cast<float4*>(row + ((((f0 >> 2) + u) ^ (og & C::MASK)) << 2)) =
               make_float4(out[u * 4][j], out[u * 4 + 1][j], out[u * 4 + 2][j], out[u * 4 + 3][j]);
       }
     }
   };
   publish(0);
-  ptx::named_barrier(1, NC);
+  ptx::named_barrier(1, NB);
 
   int it = 0;  // slabs consumed
   for (int q = 0; q < nsteps; ++q) {
-    put_features(q + 1);
-    fetch(q + 2);
-    if (ADJ && sampler) {  // publish(q) is behind the last barrier: its slot takes step q + 2's scale
-      scl[q & 1][tid] = nsc;
-      nsc = scale_of(q + 3);
-    }
-    if (!ADJ && q > 0 && live) {  // the previous step's scale, off the critical path
-      const float sc = scl[(q - 1) & 1][tid];
-      lam += (double)logf(sc);
-      p.sc[half][(int64_t)step_t(q - 1) * B + sb] = sc;
-    }
-    float acc0[RS][4], acc1[RS][4];
+    float2 acc0[RS][2], acc1[RS][2];
 #pragma unroll
     for (int i = 0; i < RS; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc0[i][j] = acc1[i][j] = 0.0f;
+      for (int j = 0; j < 2; ++j) acc0[i][j] = acc1[i][j] = make_float2(0.f, 0.f);
     const float* Sq = S + (q & 1) * CHI * TB;
     bool ok = true;
     for (int sl = 0; sl < nslab; ++sl, ++it) {
@@ -248,7 +298,7 @@ cls_f32_sweep_kernel(const __grid_constant__ ClsF32Params p) {
       ok = ok && ptx::mbar_wait(ptx::smem_addr(&bars.full[st]), (it / C::RING) & 1, p.status);
       const int k0 = sl * C::KS, rows = min(C::KS, kmax - k0);
       const float* L = ring + st * C::SLAB + og * 4;
-#pragma unroll 2
+#pragma unroll 1
       for (int kq = 0; kq < rows; kq += 4) {
         const int x = ((k0 + kq) >> 2) & C::MASK;
 #pragma unroll
@@ -256,13 +306,13 @@ cls_f32_sweep_kernel(const __grid_constant__ ClsF32Params p) {
           const float* row = Sq + (k0 + kq + kk) * TB;
           float v[RS];
           if constexpr (RS == 2) {
-            const float2 a = *reinterpret_cast<const float2*>(row + (((bg >> 1) ^ x) << 2) + (bg & 1) * 2);
+            const float2 a = *reinterpret_cast<const float2*>(row + (((f0 >> 2) ^ x) << 2) + (f0 & 3));
             v[0] = a.x;
             v[1] = a.y;
           } else {
 #pragma unroll
             for (int u = 0; u < RS / 4; ++u) {
-              const float4 a = *reinterpret_cast<const float4*>(row + (((bg * (RS / 4) + u) ^ x) << 2));
+              const float4 a = *reinterpret_cast<const float4*>(row + ((((f0 >> 2) + u) ^ x) << 2));
               v[u * 4] = a.x;
               v[u * 4 + 1] = a.y;
               v[u * 4 + 2] = a.z;
@@ -271,55 +321,75 @@ cls_f32_sweep_kernel(const __grid_constant__ ClsF32Params p) {
           }
           const float4 l0 = *reinterpret_cast<const float4*>(L + (kq + kk) * 2 * CHI);
           const float4 l1 = *reinterpret_cast<const float4*>(L + (kq + kk) * 2 * CHI + CHI);
-          const float a0[4] = {l0.x, l0.y, l0.z, l0.w}, a1[4] = {l1.x, l1.y, l1.z, l1.w};
+          const float2 a0[2] = {make_float2(l0.x, l0.y), make_float2(l0.z, l0.w)};
+          const float2 a1[2] = {make_float2(l1.x, l1.y), make_float2(l1.z, l1.w)};
 #pragma unroll
-          for (int i = 0; i < RS; ++i)
+          for (int i = 0; i < RS; ++i) {
+            const float2 vv = make_float2(v[i], v[i]);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              acc0[i][j] = fmaf(v[i], a0[j], acc0[i][j]);
-              acc1[i][j] = fmaf(v[i], a1[j], acc1[i][j]);
+            for (int j = 0; j < 2; ++j) {
+              acc0[i][j] = __ffma2_rn(vv, a0[j], acc0[i][j]);
+              acc1[i][j] = __ffma2_rn(vv, a1[j], acc1[i][j]);
             }
+          }
         }
       }
       __syncwarp();
       if ((tid & 31) == 0) ptx::mbar_arrive(ptx::smem_addr(&bars.empty[st]));
     }
 #pragma unroll
-    for (int i = 0; i < RS; ++i) {
-      const float f0 = phi[q & 1][0][bg * RS + i], f1 = phi[q & 1][1][bg * RS + i];
+    for (int i = 0; i < RS; i += 2) {
+      const float2 p0 = *reinterpret_cast<const float2*>(&phi[q & 1][0][f0 + i]);
+      const float2 p1 = *reinterpret_cast<const float2*>(&phi[q & 1][1][f0 + i]);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) out[i][j] = f0 * acc0[i][j] + f1 * acc1[i][j];
+      for (int j = 0; j < 2; ++j) {
+        out[i][2 * j] = p0.x * acc0[i][j].x + p1.x * acc1[i][j].x;
+        out[i][2 * j + 1] = p0.x * acc0[i][j].y + p1.x * acc1[i][j].y;
+        out[i + 1][2 * j] = p0.y * acc0[i + 1][j].x + p1.y * acc1[i + 1][j].x;
+        out[i + 1][2 * j + 1] = p0.y * acc0[i + 1][j].y + p1.y * acc1[i + 1][j].y;
+      }
     }
     if (!ADJ) {
+      // the sample's largest magnitude: over the thread's four, the warp's
+      // eight threads of the sample, then the warps along the outgoing index
+      float m[RS];
 #pragma unroll
       for (int i = 0; i < RS; ++i) {
-        float m = fmaxf(fmaxf(fabsf(out[i][0]), fabsf(out[i][1])), fmaxf(fabsf(out[i][2]), fabsf(out[i][3])));
+        m[i] = fmaxf(fmaxf(fabsf(out[i][0]), fabsf(out[i][1])), fmaxf(fabsf(out[i][2]), fabsf(out[i][3])));
 #pragma unroll
-        for (int o = OG / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        const float sc = m > 0.0f ? m : 1.0f;
-        const bool plain = sc > 0x1p-100f && sc < 0x1p100f;
-        const float r = 1.0f / sc;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) out[i][j] = plain ? div_by(out[i][j], sc, r) : out[i][j] / sc;
-        if (og == 0) scl[q & 1][bg * RS + i] = sc;
+        for (int o = 4; o > 0; o >>= 1) m[i] = fmaxf(m[i], __shfl_xor_sync(0xffffffffu, m[i], o));
       }
+      if constexpr (C::OW > 1) {
+        if ((tid & 7) == 0) {
+#pragma unroll
+          for (int i = 0; i < RS; ++i) smax[og >> 3][f0 + i] = m[i];
+        }
+        ptx::named_barrier(2, NC);
+#pragma unroll
+        for (int i = 0; i < RS; ++i) {
+          m[i] = smax[0][f0 + i];
+#pragma unroll
+          for (int u = 1; u < C::OW; ++u) m[i] = fmaxf(m[i], smax[u][f0 + i]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < RS; ++i) {
+        if (!(m[i] > 0.0f)) m[i] = 1.0f;
+        if (og == 0) scl[q & 1][f0 + i] = m[i];
+      }
+      divide(out, m);
     }
     if (q + 1 < nsteps) publish(q + 1);
     // the next vector, features and scales are in place for every warp; a
     // warp whose copy never came takes all of them out together
-    if (ptx::named_barrier_or(1, NC, !ok)) return;
+    if (ptx::named_barrier_or(1, NB, !ok)) return;
   }
 #pragma unroll
   for (int i = 0; i < RS; ++i) {
-    const int b = b0 + bg * RS + i;
+    const int b = b0 + f0 + i;
     if (b < B)
       *reinterpret_cast<float4*>(p.state[half] + (int64_t)b * CHI + og * 4) =
           make_float4(out[i][0], out[i][1], out[i][2], out[i][3]);
-  }
-  if (!ADJ && live) {
-    const float sc = scl[(nsteps - 1) & 1][tid];
-    p.lam[half][sb] = lam + (double)logf(sc);
-    p.sc[half][(int64_t)step_t(nsteps - 1) * B + sb] = sc;
   }
 }
 
@@ -329,7 +399,7 @@ int launch_sweep(const ClsF32Params& p, cudaStream_t s) {
   static std::atomic<uint64_t> attr{0};
   if (!smem_limit_once((const void*)cls_f32_sweep_kernel<CHI, RS, ADJ>, C::SMEM, &attr)) return TN_ERR_CUDA;
   const dim3 grid((unsigned)((p.batch + C::TB - 1) / C::TB), 2);
-  cls_f32_sweep_kernel<CHI, RS, ADJ><<<grid, C::NC + 32, C::SMEM, s>>>(p);
+  cls_f32_sweep_kernel<CHI, RS, ADJ><<<grid, C::NT, C::SMEM, s>>>(p);
   return cudaGetLastError() == cudaSuccess ? TN_OK : TN_ERR_CUDA;
 }
 
