@@ -196,6 +196,7 @@ int tn::contract_internal(const tn_tensor* A, const int* legsA, const tn_tensor*
   if (prec == TN_PREC_FP32 && d.M <= SKINNY_MAX && d.K <= SKINNY_MAX && d.N >= 4096)
     return launch_contract_skinny(d, s);
   plan_units(&d, min_units_single());
+  if (prec == TN_PREC_FP32) plan_simt(&d, SimtPlan::alone);
   if (prec != TN_PREC_FP32 && scratch && packed_single_bytes(d, prec) <= scratch_bytes)
     return contract_packed_single(d, prec, scratch, scratch_bytes, s);
   if (d.splits > 1 &&
@@ -380,8 +381,35 @@ int tn::group_plan_create_ex(const tn_contract_spec* specs, int nspecs, int prec
     *plan = p;
     return TN_OK;
   }
-  auto unit_work = [](const ContractDesc& d) {
-    return (double)std::min<int64_t>(d.M, TC_BM) * (double)std::min<int64_t>(d.N, TC_BN) *
+  // FP32 plans whose contractions all have a small first operand (the MPO
+  // step of a batch of environment sweeps) run one thread per result column
+  if (prec == TN_PREC_FP32 && !p->descs.empty()) {
+    p->skinny = true;
+    for (const auto& d : p->descs) {
+      if (d.M > SKINNY_MAX || d.K > SKINNY_MAX) p->skinny = false;
+      p->max_n = std::max(p->max_n, d.N);
+    }
+  }
+  if (prec == TN_PREC_FP32 && !p->skinny) {
+    // a large group keeps a tile's k ranges (2048 shared indices each) in one
+    // unit, up to four of them, where a contraction has 16 tiles or more: no
+    // zeroing pass and no atomics, and the units still outnumber the CTAs
+    // that run at once eight times over
+    int64_t units = 0;
+    for (const auto& d : p->descs) units += (int64_t)d.tiles_m * d.tiles_n * d.splits;
+    for (auto& d : p->descs) {
+      if (units >= 8 * min_units_single() && (int64_t)d.tiles_m * d.tiles_n >= 16) {
+        const int64_t range = 4 * 64 * MAX_SLABS_PER_UNIT;
+        d.splits = (int32_t)((d.K + range - 1) / range);
+        d.k_per_split = range;
+      }
+      plan_simt(&d, SimtPlan::group);
+    }
+  }
+  auto unit_work = [&](const ContractDesc& d) {
+    const bool simt = prec == TN_PREC_FP32 && !p->skinny;
+    return (double)std::min<int64_t>(d.M, simt ? simt_tile_m(d.tile) : TC_BM) *
+           (double)std::min<int64_t>(d.N, simt ? simt_tile_n(d.tile) : TC_BN) *
            (double)std::min<int64_t>(d.K, d.k_per_split);
   };
   std::stable_sort(p->descs.begin(), p->descs.end(), [&](const ContractDesc& a, const ContractDesc& b) {
@@ -400,15 +428,6 @@ int tn::group_plan_create_ex(const tn_contract_spec* specs, int nspecs, int prec
     const ContractDesc& d = p->descs[i];
     const int64_t n = (int64_t)d.tiles_m * d.tiles_n * d.splits;
     std::fill(p->unit_desc.begin() + d.tile_begin, p->unit_desc.begin() + d.tile_begin + n, (int32_t)i);
-  }
-  // FP32 plans whose contractions all have a small first operand (the MPO
-  // step of a batch of environment sweeps) run one thread per result column
-  if (prec == TN_PREC_FP32 && !p->descs.empty()) {
-    p->skinny = true;
-    for (const auto& d : p->descs) {
-      if (d.M > SKINNY_MAX || d.K > SKINNY_MAX) p->skinny = false;
-      p->max_n = std::max(p->max_n, d.N);
-    }
   }
   *plan = p;
   return TN_OK;

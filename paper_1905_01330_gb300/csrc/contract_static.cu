@@ -88,6 +88,7 @@ extern "C" int tn_contract_grouped_static(const tn_contract_spec* specs, int nsp
       continue;
     }
     plan_units(&d, 1);
+    if (prec == TN_PREC_FP32) plan_simt(&d, SimtPlan::pairs);  // 128 x 128 tiles: the documented unit count
     h_descs[nd++] = d;
   }
   // largest work units first, as the allocating entry point does

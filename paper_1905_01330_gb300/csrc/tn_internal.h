@@ -27,10 +27,12 @@ struct ContractDesc {
   int32_t tiles_m, tiles_n;
   int32_t splits;      // k ranges the shared index is cut into (split-K); results are summed
                        // into C with float32 atomic adds when > 1, so C is zeroed first
-  int32_t pad0;
+  int32_t tile;        // FP32: tile shape of the CUDA-core kernel (plan_simt)
   int64_t k_per_split; // shared indices per k range (a multiple of 64)
   int64_t tile_begin;  // first global work unit of this spec in a grouped launch
-  int64_t pad1;        // size a multiple of 16 bytes (bulk async copies)
+  int32_t swapped;     // FP32: A and B exchanged (m over B's free legs), C stored as C[n][m]
+  int16_t vec;         // FP32: bit 0 / 1: A / B gathered in 16-byte loads
+  int16_t chunk;       // FP32: shared indices summed in one chain, in 64s
   int32_t mdim[TN_MAX_RANK];
   int32_t ndim[TN_MAX_RANK];
   int32_t kdim[TN_MAX_RANK];
@@ -63,8 +65,12 @@ int launch_contract_skinny(const ContractDesc& d, cudaStream_t stream);
 int launch_contract_skinny_grouped(const ContractDesc* descs, int count, int64_t max_n, cudaStream_t stream);
 
 // Tile shapes of the kernels (used by the planner to count tiles).
-constexpr int SIMT_BM = 128, SIMT_BN = 128;
 constexpr int TC_BM = 128, TC_BN = 128;
+// CUDA-core kernel: 64 x 128, 32 x 128, 16 x 256, and a 128 x 128 unit run as
+// two 64 x 128 tiles (callers that count units in 128 x 128 tiles).
+constexpr int SIMT_TILES = 3, SIMT_TILE_PAIR = 3;
+__host__ __device__ constexpr int simt_tile_m(int tile) { return tile == SIMT_TILE_PAIR ? 128 : (64 >> tile); }
+__host__ __device__ constexpr int simt_tile_n(int tile) { return tile == 2 ? 256 : 128; }
 // Longest k range of one work unit, in 64-wide slabs: a spec whose shared
 // index is longer is split so no single CTA serialises a huge K.
 constexpr int MAX_SLABS_PER_UNIT = 32;
@@ -72,6 +78,12 @@ constexpr int MAX_SLABS_PER_UNIT = 32;
 // Sets tiles_m/n, splits and k_per_split; `min_units` asks for at least that
 // many work units when K is long enough to split (keeping >= 4 slabs per unit).
 void plan_units(ContractDesc* d, int64_t min_units);
+// Tile shape, orientation, load widths and k ranges of an FP32 contraction
+// planned by plan_units, whose k ranges become the chains a result is summed
+// in: alone (a unit may run several of them, so that the tiles fill the SMs),
+// in a group (the k ranges as given) or as 128 x 128 units (as given).
+enum class SimtPlan { alone, group, pairs };
+void plan_simt(ContractDesc* d, SimtPlan how);
 // Work units a lone contraction asks plan_units for (two per SM).
 int64_t min_units_single();
 // The same for the packed GEMM (longer k ranges when a spec has many tiles).

@@ -324,3 +324,45 @@ def test_grouped_plan_on_pinned_host_operands(tn):
             ref = Cd.cpu()
             assert torch.isfinite(Ch).all()
             assert (Ch - ref).abs().max().item() <= 1e-5 * max(1.0, ref.abs().max().item()), prec
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (63, 129, 15), (64, 128, 16), (65, 257, 17), (130, 31, 2100), (17, 260, 64),
+                                   (260, 5, 300), (1030, 1024, 2)])
+def test_fp32_tiles_and_gathers(tn, M, N, K):
+    # the float32 kernel's tile shapes and both orientations at their edges,
+    # k ranges past one chain (2048), and every way an operand is gathered:
+    # unit stride along the rows or along k, in 16-byte or single loads (a
+    # view that starts one element in, rows padded to an odd length)
+    for ta in (0, 1):
+        for tb in (0, 1):
+            for off in (0, 1):
+                sa, sb = ((K, M) if ta else (M, K)), ((K, N) if tb else (N, K))
+                A, B = rand(31 + ta, sa), rand(41 + tb, sb)
+                At = torch.zeros(sa[0], sa[1] + 3 * off, device="cuda")[:, off:off + sa[1]]
+                Bt = torch.zeros(sb[0], sb[1] + 3 * off, device="cuda")[:, off:off + sb[1]]
+                At.copy_(torch.from_numpy(A))
+                Bt.copy_(torch.from_numpy(B))
+                la, lb = [0 if ta else 1], [0 if tb else 1]
+                check(tn.contract(At, la, Bt, lb, prec="fp32"), A, la, B, lb, "fp32")
+
+
+def test_fp32_group_with_long_k_ranges(tn):
+    # a group large enough that a contraction of 20 or more tiles keeps its k
+    # ranges in one unit (chains of 2048 added up in shared memory), beside
+    # thin ones in both orientations whose k ranges are added atomically
+    fill = torch.ones(2048, 64, device="cuda")
+    specs = [(fill, [1], fill, [1], torch.empty(2048, 2048, device="cuda")) for _ in range(10)]
+    host = []
+    for i, (M, N, K) in enumerate([(600, 400, 4200), (9, 300, 4200), (500, 7, 2200)]):
+        A, B = rand(51 + i, (M, K)), rand(61 + i, (K, N))
+        C = torch.empty(M, N, device="cuda")
+        specs.append((torch.from_numpy(A).cuda(), [1], torch.from_numpy(B).cuda(), [0], C))
+        host.append((A, B, C))
+    plan = tn.GroupPlan(specs, prec="fp32")
+    plan.run()
+    torch.cuda.synchronize()
+    assert tn.sync_status() == 0
+    for A, B, C in host:
+        check(C, A, [1], B, [0], "fp32")
+    for sp in specs[:10]:
+        assert torch.equal(sp[4], torch.full_like(sp[4], 64.0))
