@@ -587,14 +587,19 @@ int tn_mps_classify_separate_backward(const tn_mps* Ws, int n_mps, const float* 
  * (40) was reached before every column pair was orthogonal.
  *
  * Arithmetic: float32 one-sided Jacobi (Hestenes) on the r columns of
- * length max(M, N), the rotation angles computed in float64; singular values
- * are column norms. The singular vectors of a zero singular value on the
- * longer side (columns of U when M >= N, rows of V^T when M < N) are zeros. Workspace: tn_split_node_workspace_bytes (256-B
- * aligned). Unlike the other entry points this call synchronises `stream`
- * (once per sweep and before the outputs, whose shapes depend on k).
+ * length max(M, N), in blocks of 16 columns (the rotations of a block pair on
+ * its Gram matrix, their product applied to the columns); singular values are
+ * the column norms over the accumulated rotations' own. The singular vectors
+ * of a zero singular value on the longer side (columns of U when M >= N, rows
+ * of V^T when M < N) are zeros. The sweeps are one cooperative launch with
+ * bounded device-wide barriers. Workspace: tn_split_node_workspace_bytes
+ * (256-B aligned). Unlike the other entry points this call synchronises
+ * `stream` (when the values are known, since the outputs' shapes depend on k,
+ * and at the end).
  * Errors: TN_ERR_ARG (legs not a partition of A's, null outputs or kept),
  * TN_ERR_UNSUPPORTED (dtype, negative strides, r >= 2^30), TN_ERR_WORKSPACE,
- * TN_ERR_CUDA. An empty node (r = 0) returns TN_OK with k = 0.
+ * TN_ERR_CUDA, TN_ERR_TIMEOUT (a barrier's wait expired). An empty node (r =
+ * 0) returns TN_OK with k = 0.
  */
 size_t tn_split_node_workspace_bytes(const tn_tensor* A, const int* left, int nleft, const int* right, int nright);
 int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* right, int nright,

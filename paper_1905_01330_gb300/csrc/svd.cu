@@ -5,26 +5,50 @@
 // out as U sqrt(S) and sqrt(S) V^T (split_node) or U, S, V^T (full SVD).
 //
 // One-sided Jacobi orthogonalises the columns of a working matrix W (L x r,
-// column-major, r = min(M, N) columns of length L = max(M, N): the matrix
-// view itself when M >= N, else its transpose) by plane rotations of column
-// pairs, accumulating the rotations in V (r x r, starting from I). A sweep
-// visits every pair once, in r - 1 rounds of r / 2 disjoint pairs (the circle
-// method of round-robin scheduling), one kernel per round (a CUDA graph per
-// sweep) and one CTA per pair. At convergence W = U S and the matrix (or its transpose) is W V^T:
-// the singular values are the column norms of W.
+// r = min(M, N) columns of length L = max(M, N): the matrix view itself when
+// M >= N, else its transpose) by plane rotations of column pairs, accumulating
+// the rotations in V (r x r, starting from I). At convergence W = U S and the
+// matrix (or its transpose) is W V^T: the singular values are the column norms
+// of W.
+//
+// The method is a chain of rounds, so what bounds it is a round's latency and
+// the passes over W and V. Rotating one pair per CTA and round takes r - 1
+// rounds a sweep, each a launch that reads and writes all of W and V for one
+// rotation per column (5.3 us a round at r = 256). Here the columns are in
+// blocks of 16 and a round pairs blocks: a CTA forms the 32 x 32 Gram matrix of
+// its two blocks, runs the round's 16 x 16 rotations on it in shared memory
+// (16 steps of 16 disjoint pairs; in a sweep's first round all 32 x 31 / 2
+// pairs, 31 steps), collecting them in Q, and applies Q to the blocks of W and
+// V in one pass: r / 16 - 1 rounds a sweep, the same pairs rotated once each.
+// Blocks pair up by the circle method; all sweeps run in one cooperative
+// launch, its rounds separated by a device-wide barrier (bounded), and stop
+// after a sweep without a rotation. A block is stored row by row (16 floats a
+// row): a warp takes one row of the two blocks, lane j column j, the row's
+// other entries broadcast from shared memory, for the Gram matrix (lane j: its
+// column of it) and for the product with Q alike. The rows are shared out over
+// the CTAs of a cluster, which add up their Gram matrices and rotate alike.
+// Measured (two-site node of bond 128, r = 256, 13 sweeps): 18.7 -> 2.2 ms; a
+// round takes ~19,000 cycles: Gram matrix 1,300, its sum over 8 warps and 8
+// CTAs 4,800, the 17 rotation steps 9,800 (a dependent chain of ~370 cycles
+// each), W and V 2,300, the barrier 2,600. r = 1000: 98 -> 14 ms, 2048: 380 ->
+// 77 ms. Rotations that also sort the columns by norm took 1-5 more sweeps.
 #include <math.h>
 #include <string.h>
 
 #include <vector>
 
+#include "ptx.cuh"
 #include "tn_internal.h"
 
 namespace tn {
 namespace {
 
 constexpr int SVD_THREADS = 256;
+constexpr int SVD_WARPS = SVD_THREADS / 32;
 constexpr int SVD_MAX_SWEEPS = 40;
-constexpr int SVD_CACHE = 8;  // register-held entries per thread and column
+constexpr int SVD_B = 16;      // columns of a block
+constexpr int SVD_CH = 256;    // rows staged at once
+constexpr int SVD_CLUSTER = 8; // most CTAs that share out a pair's rows
 
 // The node's matrix view: element (i, j) at A + loff(i) + roff(j).
 struct SplitView {
@@ -47,44 +71,24 @@ __device__ __forceinline__ int64_t leg_offset(int64_t idx, int n, const int32_t*
   return off;
 }
 
-// W[w] for every w = row + L * col (coalesced writes), V = I.
-__global__ void svd_gather(SplitView v, float* __restrict__ W, float* __restrict__ V, int64_t L, int64_t r) {
-  const int64_t total = L * r, stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < total; w += stride) {
-    const int64_t row = w % L, col = w / L;
-    const int64_t i = v.wide ? col : row, j = v.wide ? row : col;
-    W[w] = v.A[leg_offset(i, v.nl, v.ldim, v.lstr) + leg_offset(j, v.nr, v.rdim, v.rstr)];
-  }
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < r * r; e += stride)
-    V[e] = (e % r == e / r) ? 1.0f : 0.0f;
-}
-
-// Sum of three per-thread values over the CTA, in double across warps.
-__device__ __forceinline__ void block_sum3(float& a, float& b, float& c, double* out) {
-  __shared__ double part[SVD_THREADS / 32][3];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-    c += __shfl_xor_sync(0xffffffffu, c, o);
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) {
-    part[warp][0] = a;
-    part[warp][1] = b;
-    part[warp][2] = c;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    for (int w = 0; w < SVD_THREADS / 32; ++w) {
-      s0 += part[w][0];
-      s1 += part[w][1];
-      s2 += part[w][2];
+// W in blocks of 16 columns, [block][row][16] (zeros past column r), V = I
+// likewise.
+__global__ void svd_gather(SplitView v, float* __restrict__ W, float* __restrict__ V, int64_t L, int64_t r, int64_t cols) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x, first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (int64_t w = first; w < L * cols; w += stride) {
+    // neighbouring threads walk the view's own rows where those are columns of W
+    const int64_t blk = w / (L * SVD_B), in = w - blk * L * SVD_B;
+    const int64_t row = in / SVD_B, col = blk * SVD_B + in % SVD_B;
+    float x = 0.0f;
+    if (col < r) {
+      const int64_t i = v.wide ? col : row, j = v.wide ? row : col;
+      x = v.A[leg_offset(i, v.nl, v.ldim, v.lstr) + leg_offset(j, v.nr, v.rdim, v.rstr)];
     }
-    out[0] = s0;
-    out[1] = s1;
-    out[2] = s2;
+    W[w] = x;
+  }
+  for (int64_t e = first; e < r * cols; e += stride) {
+    const int64_t blk = e / (r * SVD_B), in = e - blk * r * SVD_B;
+    V[e] = in / SVD_B == blk * SVD_B + in % SVD_B ? 1.0f : 0.0f;
   }
 }
 
@@ -94,122 +98,348 @@ __device__ __forceinline__ int circle_slot(int pos, int t, int rp) {
   return pos == 0 ? 0 : 1 + (pos - 1 + t) % (rp - 1);
 }
 
-// One round: CTA k rotates column pair k so that the two columns of W become
-// orthogonal (Hestenes): with a = |w_p|^2, b = |w_q|^2, g = w_p . w_q and
-// zeta = (b - a) / 2g, t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)),
-// c = 1 / sqrt(1 + t^2), s = c t, the pair becomes (c w_p - s w_q, s w_p +
-// c w_q); V's columns p and q take the same rotation. Pairs already
-// orthogonal to within tol (|g| <= tol sqrt(ab)) are left alone; the others
-// are counted in *rotations.
-__global__ void __launch_bounds__(SVD_THREADS)
-svd_round(float* __restrict__ W, float* __restrict__ V, int64_t L, int r, int rp, int t, float tol,
-          int* __restrict__ rotations) {
-  const int k = blockIdx.x;
-  const int p = circle_slot(k, t, rp), q = circle_slot(rp - 1 - k, t, rp);
-  if (p >= r || q >= r) return;  // the dummy slot of an odd r
-  float* wp = W + (int64_t)p * L;
-  float* wq = W + (int64_t)q * L;
-  float* vp = V + (int64_t)p * r;
-  float* vq = V + (int64_t)q * r;
-  // columns of up to SVD_CACHE * SVD_THREADS entries stay in registers
-  // between the dot products and the rotation; V's two columns are loaded
-  // with W's, so their latency overlaps the reduction
-  const bool cached = L <= (int64_t)SVD_CACHE * SVD_THREADS;
-  const bool vcached = r <= SVD_CACHE * SVD_THREADS;
-  float xs[SVD_CACHE], ys[SVD_CACHE], us[SVD_CACHE], ts[SVD_CACHE];
-  if (vcached) {
-#pragma unroll
-    for (int u = 0; u < SVD_CACHE; ++u) {
-      const int i = threadIdx.x + u * SVD_THREADS;
-      us[u] = i < r ? vp[i] : 0.0f;
-      ts[u] = i < r ? vq[i] : 0.0f;
-    }
+struct SvdParams {
+  float* W;
+  float* V;
+  int64_t L;
+  int32_t r, ns, nb;   // columns; blocks; blocks rounded up to even (the added one is zeros, not stored)
+  int32_t cluster;     // CTAs sharing out a pair's rows
+  float tol;
+  unsigned* bar;       // barrier counter (zero)
+  int* counts;         // rotations per sweep (zero)
+  int* sweeps;         // out: sweeps used, negative if the limit was reached
+  int* status;
+};
+
+struct SvdSmem {
+  float X[2][SVD_CH][2 * SVD_B];               // rows of the two blocks
+  float part[2 * SVD_B][2 * SVD_B];            // this CTA's part of the Gram matrix, read by its cluster
+  float red[SVD_WARPS][2 * SVD_B][2 * SVD_B];  // Gram sums of the warps
+  float G[2][2 * SVD_B][2 * SVD_B + 1];
+  float Q[2 * SVD_B][2 * SVD_B + 1];
+  int32_t abort;
+};
+
+// Rows [row0, row0 + rows) of blocks p and q of X (n rows a block) into a
+// staging buffer (zeros for a block past the ns stored ones).
+__device__ __forceinline__ void svd_stage(float (*x)[2 * SVD_B], const float* __restrict__ X, int64_t n, int p, int q,
+                                          int ns, int64_t row0, int rows) {
+  const float* xp = X + ((int64_t)p * n + row0) * SVD_B;
+  const float* xq = X + ((int64_t)q * n + row0) * SVD_B;
+  for (int i = threadIdx.x; i < rows * 8; i += SVD_THREADS) {
+    const int row = i >> 3, c = (i & 7) * 4;
+    if ((c < SVD_B ? p : q) < ns)
+      ptx::cp_async16(ptx::smem_addr(&x[row][c]), (c < SVD_B ? xp + c : xq + c - SVD_B) + row * SVD_B);
+    else
+      *reinterpret_cast<float4*>(&x[row][c]) = make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  float a = 0.0f, b = 0.0f, g = 0.0f;
-  if (cached) {
-#pragma unroll
-    for (int u = 0; u < SVD_CACHE; ++u) {
-      const int64_t i = threadIdx.x + (int64_t)u * SVD_THREADS;
-      xs[u] = i < L ? wp[i] : 0.0f;
-      ys[u] = i < L ? wq[i] : 0.0f;
-      a = fmaf(xs[u], xs[u], a);
-      b = fmaf(ys[u], ys[u], b);
-      g = fmaf(xs[u], ys[u], g);
-    }
-  } else {
-    for (int64_t i = threadIdx.x; i < L; i += SVD_THREADS) {
-      const float x = wp[i], y = wq[i];
-      a = fmaf(x, x, a);
-      b = fmaf(y, y, b);
-      g = fmaf(x, y, g);
-    }
-  }
-  __shared__ double sums[3];
-  __shared__ float rot[2];
-  __shared__ int skip;
-  block_sum3(a, b, g, sums);
-  if (threadIdx.x == 0) {
-    // the angle in float64: with float32 c and s from float32 arithmetic the
-    // rounding of c^2 + s^2 is biased and the column norms drift by ~1e-4
-    // over the ~10^4 rotations a column of a 1000-column matrix takes
-    const double al = sums[0], be = sums[1], ga = sums[2];
-    const bool go = al > 0.0 && be > 0.0 && fabs(ga) > (double)tol * sqrt(al) * sqrt(be);
-    if (go) {
-      const double z = (be - al) / (2.0 * ga);
-      const double tt = (z >= 0.0 ? 1.0 : -1.0) / (fabs(z) + sqrt(1.0 + z * z));
-      const double c = 1.0 / sqrt(1.0 + tt * tt);
-      rot[0] = (float)c;
-      rot[1] = (float)(c * tt);
-      atomicAdd(rotations, 1);
-    }
-    skip = go ? 0 : 1;
-  }
-  __syncthreads();
-  if (skip) return;
-  const float c = rot[0], s = rot[1];
-  if (cached) {
-#pragma unroll
-    for (int u = 0; u < SVD_CACHE; ++u) {
-      const int64_t i = threadIdx.x + (int64_t)u * SVD_THREADS;
-      if (i < L) {
-        wp[i] = c * xs[u] - s * ys[u];
-        wq[i] = s * xs[u] + c * ys[u];
-      }
-    }
-  } else {
-    for (int64_t i = threadIdx.x; i < L; i += SVD_THREADS) {
-      const float x = wp[i], y = wq[i];
-      wp[i] = c * x - s * y;
-      wq[i] = s * x + c * y;
-    }
-  }
-  if (vcached) {
-#pragma unroll
-    for (int u = 0; u < SVD_CACHE; ++u) {
-      const int i = threadIdx.x + u * SVD_THREADS;
-      if (i < r) {
-        vp[i] = c * us[u] - s * ts[u];
-        vq[i] = s * us[u] + c * ts[u];
-      }
-    }
-  } else {
-    for (int i = threadIdx.x; i < r; i += SVD_THREADS) {
-      const float x = vp[i], y = vq[i];
-      vp[i] = c * x - s * y;
-      vq[i] = s * x + c * y;
-    }
-  }
+  ptx::cp_async_commit();
 }
 
-// sigma[j] = |W[:, j]| (CTA j).
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// A float of the same shared-memory variable in the cluster's CTA `rank`.
+__device__ __forceinline__ float cluster_load(const float* p, uint32_t rank) {
+  uint32_t a;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(ptx::smem_addr(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+// Approximate square root, reciprocal and its square root (subnormals as 0).
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// The rotations (Hestenes) of one round on the Gram matrix in s.G[0], and
+// their product in s.Q: for a pair with a = g_pp, b = g_qq, g = g_pq the
+// tangent t is the smaller root, h sign(d) / (|d| + sqrt(d^2 + h^2)) for d = (b
+// - a) / sqrt(ab) and h = 2 g / sqrt(ab); c = 1 / sqrt(1 + t^2), s = c t, and the columns become (c p -
+// s q, s p + c q). Pairs orthogonal to within tol (|g| <= tol sqrt(ab)) are
+// left alone, but counted only above 16 tol: the sweeps end when none is, and
+// what the last one still found below that is rotated away. FULL: all pairs of the 32 columns by the circle method, else
+// the pairs across the two blocks. Every warp computes the step's 16 angles
+// (lanes 0-15; approximate quotients and roots: they only move the angle, the
+// next rounds see what is left); thread (u, v) updates the 2 x 2 block of pairs
+// u and v and two rows of Q. Returns whether it rotated anything, and adds to
+// the count.
+template <bool FULL>
+__device__ __forceinline__ bool svd_rotate(SvdSmem& s, float tol, int& count) {
+  constexpr int C = 2 * SVD_B;
+  const int tid = threadIdx.x, u = tid >> 4, v = tid & 15;
+  bool rotated = false;
+  for (int t = 0; t < (FULL ? C - 1 : SVD_B); ++t) {
+    auto slot = [&](int pos) {  // circle over the 32 columns: slot 0 stays
+      int x = pos - 1 + t;
+      if (x >= C - 1) x -= C - 1;
+      return pos == 0 ? 0 : 1 + x;
+    };
+    const int pv = FULL ? slot(v) : v, qv = FULL ? slot(C - 1 - v) : SVD_B + ((v + t) & (SVD_B - 1));
+    const int pu = FULL ? slot(u) : u, qu = FULL ? slot(C - 1 - u) : SVD_B + ((u + t) & (SVD_B - 1));
+    const float(*g)[C + 1] = s.G[t & 1];
+    float(*gn)[C + 1] = s.G[(t & 1) ^ 1];
+    const float al = g[pv][pv], be = g[qv][qv], ga = g[pv][qv];
+    const float b00 = g[pu][pv], b01 = g[pu][qv], b10 = g[qu][pv], b11 = g[qu][qv];
+    // scaled by the two norms, so that no square leaves the exponent range
+    const float ia = rsqrt_approx(al), ib = rsqrt_approx(be), co = ga * ia * ib;
+    const bool go = al > 0.0f && be > 0.0f && fabsf(co) > tol;
+    const float d = (be - al) * ia * ib, h = co + co;
+    const float tt = fminf(fabsf(h) * rcp_approx(fabsf(d) + sqrt_approx(fmaf(d, d, h * h))), 1.0f);
+    const float ts = (d < 0.0f) != (h < 0.0f) ? -tt : tt;
+    float c = rsqrt_approx(fmaf(tt, tt, 1.0f)), sn = c * ts;
+    // c^2 + s^2 = 1 to the rounding of c and s: a bias here would drift the
+    // column norms over a matrix's thousands of rotations
+    const float e = -0.5f * fmaf(sn, sn, fmaf(c, c, -1.0f));
+    c = go ? fmaf(e, c, c) : 1.0f;
+    sn = go ? fmaf(e, sn, sn) : 0.0f;
+    rotated |= __any_sync(0xffffffffu, go);
+    count += __popc(__ballot_sync(0xffffffffu, go && fabsf(co) > 16.0f * tol) & 0xffffu);
+    const float cu = __shfl_sync(0xffffffffu, c, u), su = __shfl_sync(0xffffffffu, sn, u);
+    const float x0 = c * b00 - sn * b01, x1 = sn * b00 + c * b01, y0 = c * b10 - sn * b11, y1 = sn * b10 + c * b11;
+    gn[pu][pv] = cu * x0 - su * y0;
+    gn[qu][pv] = su * x0 + cu * y0;
+    gn[pu][qv] = cu * x1 - su * y1;
+    gn[qu][qv] = su * x1 + cu * y1;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      float* row = s.Q[u + k * SVD_B];
+      const float a0 = row[pv], a1 = row[qv];
+      row[pv] = c * a0 - sn * a1;
+      row[qv] = sn * a0 + c * a1;
+    }
+    __syncthreads();
+  }
+  return rotated;
+}
+
+// One block pair, by a cluster whose CTAs share out the rows: Gram matrix
+// (each its part, then the sum over the cluster), rotations (the same in
+// every CTA), Q applied to W and V. Adds the counted rotations (the same in
+// every thread).
+__device__ void svd_block_pair(const SvdParams& P, SvdSmem& s, int p, int q, bool full, int& count) {
+  constexpr int C = 2 * SVD_B;
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int rank = (int)cluster_rank(), cs = P.cluster;
+  const int64_t lp = (P.L + cs - 1) / cs, w0 = min(P.L, lp * rank), wn = min(P.L, w0 + lp) - w0;
+  const int vp = (P.r + cs - 1) / cs, v0 = min(P.r, vp * rank), vn = min(P.r, v0 + vp) - v0;
+  const int nw = (int)((wn + SVD_CH - 1) / SVD_CH), nv = (vn + SVD_CH - 1) / SVD_CH;
+  // item i of the apply pass: rows of W, then of V, in buffer i & 1
+  auto rows_of = [&](int i) {
+    return i < nw ? (int)min((int64_t)SVD_CH, wn - (int64_t)i * SVD_CH) : min(SVD_CH, vn - (i - nw) * SVD_CH);
+  };
+  auto stage = [&](int i) {
+    if (i >= nw + nv) return;
+    if (i < nw) svd_stage(s.X[i & 1], P.W, P.L, p, q, P.ns, w0 + (int64_t)i * SVD_CH, rows_of(i));
+    else svd_stage(s.X[i & 1], P.V, P.r, p, q, P.ns, v0 + (int64_t)(i - nw) * SVD_CH, rows_of(i));
+  };
+  // Gram matrix: lane j sums x_i x_j over the warp's rows for every i
+  float2 acc[C / 2];
+#pragma unroll
+  for (int m = 0; m < C / 2; ++m) acc[m] = make_float2(0.f, 0.f);
+  if (nw > 0) stage(0);
+  for (int c = 0; c < nw; ++c) {
+    ptx::cp_async_wait<0>();
+    __syncthreads();
+    if (c + 1 < nw) stage(c + 1);
+    const float(*x)[C] = s.X[c & 1];
+    const int rows = rows_of(c);
+#pragma unroll 4
+    for (int row = w; row < rows; row += SVD_WARPS) {
+      const float mine = x[row][lane];
+      const float2 mm = make_float2(mine, mine);
+#pragma unroll
+      for (int m = 0; m < C / 4; ++m) {
+        const float4 f = *reinterpret_cast<const float4*>(&x[row][4 * m]);
+        acc[2 * m] = __ffma2_rn(make_float2(f.x, f.y), mm, acc[2 * m]);
+        acc[2 * m + 1] = __ffma2_rn(make_float2(f.z, f.w), mm, acc[2 * m + 1]);
+      }
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < C / 2; ++m) {
+    s.red[w][2 * m][lane] = acc[m].x;
+    s.red[w][2 * m + 1][lane] = acc[m].y;
+  }
+  __syncthreads();
+  // the staging buffers are free unless W fits one: the apply pass's first loads
+  if (nw == 1) stage(1);
+  else stage(0);
+#pragma unroll
+  for (int e = 0; e < C * C / SVD_THREADS; ++e) {
+    const int i = (tid + e * SVD_THREADS) / C;
+    float g[SVD_WARPS];
+#pragma unroll
+    for (int u = 0; u < SVD_WARPS; ++u) g[u] = s.red[u][i][lane];
+#pragma unroll
+    for (int o = 1; o < SVD_WARPS; o *= 2)
+#pragma unroll
+      for (int u = 0; u < SVD_WARPS; u += 2 * o) g[u] += g[u + o];
+    s.part[i][lane] = g[0];
+    s.Q[i][lane] = i == lane ? 1.0f : 0.0f;
+  }
+  if (cs > 1) {
+    cluster_sync();
+    float g[C * C / SVD_THREADS][SVD_CLUSTER];
+#pragma unroll
+    for (int e = 0; e < C * C / SVD_THREADS; ++e)
+#pragma unroll
+      for (int k = 0; k < SVD_CLUSTER; ++k)
+        g[e][k] = k < cs ? cluster_load(&s.part[(tid + e * SVD_THREADS) / C][lane], k) : 0.0f;
+#pragma unroll
+    for (int e = 0; e < C * C / SVD_THREADS; ++e) {
+#pragma unroll
+      for (int k = 1; k < SVD_CLUSTER; ++k) g[e][0] += g[e][k];
+      s.G[0][(tid + e * SVD_THREADS) / C][lane] = g[e][0];
+    }
+  } else {
+    __syncthreads();
+    for (int e = 0; e < C * C / SVD_THREADS; ++e) {
+      const int i = (tid + e * SVD_THREADS) / C;
+      s.G[0][i][lane] = s.part[i][lane];
+    }
+  }
+  __syncthreads();
+  const bool rotated = full ? svd_rotate<true>(s, P.tol, count) : svd_rotate<false>(s, P.tol, count);
+  if (!rotated) {
+    ptx::cp_async_wait<0>();
+    if (cs > 1) cluster_sync();
+    else __syncthreads();
+    return;
+  }
+  // x <- x Q for every row: lane j holds column j of Q
+  const bool stored = (lane < SVD_B ? p : q) < P.ns;
+  float2 qc[C / 2];
+#pragma unroll
+  for (int m = 0; m < C / 2; ++m) qc[m] = make_float2(s.Q[2 * m][lane], s.Q[2 * m + 1][lane]);
+  for (int i = 0; i < nw + nv; ++i) {
+    ptx::cp_async_wait<0>();
+    __syncthreads();
+    if (i + 1 < nw + nv && !(nw == 1 && i == 0)) stage(i + 1);
+    const float(*x)[C] = s.X[i & 1];
+    const int rows = rows_of(i);
+    const int64_t n = i < nw ? P.L : P.r, row0 = i < nw ? w0 + (int64_t)i * SVD_CH : v0 + (int64_t)(i - nw) * SVD_CH;
+    float* out = (i < nw ? P.W : P.V) + ((lane < SVD_B ? (int64_t)p : (int64_t)q) * n + row0) * SVD_B + (lane & (SVD_B - 1));
+    for (int r0 = w * 4; r0 < rows; r0 += SVD_WARPS * 4) {
+      float2 o[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) o[k] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int m = 0; m < C / 4; ++m)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float4 f = *reinterpret_cast<const float4*>(&x[min(r0 + k, rows - 1)][4 * m]);
+          o[k] = __ffma2_rn(make_float2(f.x, f.y), qc[2 * m], o[k]);
+          o[k] = __ffma2_rn(make_float2(f.z, f.w), qc[2 * m + 1], o[k]);
+        }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (stored && r0 + k < rows) out[(int64_t)(r0 + k) * SVD_B] = o[k].x + o[k].y;
+    }
+  }
+  // the buffers are free for the next pair, the parts read by the cluster
+  if (cs > 1) cluster_sync();
+  else __syncthreads();
+}
+
+__device__ __forceinline__ unsigned svd_load_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// All sweeps: one cooperative launch.
+__global__ void __launch_bounds__(SVD_THREADS) svd_jacobi(const __grid_constant__ SvdParams P) {
+  extern __shared__ __align__(16) uint8_t raw[];
+  SvdSmem& s = *reinterpret_cast<SvdSmem*>(raw);
+  const int tid = threadIdx.x;
+  if (tid == 0) s.abort = 0;
+  unsigned epoch = 0;
+  bool done = false;
+  int used = 0;
+  while (!done && used < SVD_MAX_SWEEPS) {
+    for (int t = 0; t < P.nb - 1; ++t) {
+      int rotations = 0;
+      for (int k = blockIdx.x / P.cluster; k < P.nb / 2; k += gridDim.x / P.cluster)
+        svd_block_pair(P, s, circle_slot(k, t, P.nb), circle_slot(P.nb - 1 - k, t, P.nb), t == 0, rotations);
+      // device-wide barrier: every CTA's part of W, V and the count is in place
+      __syncthreads();
+      if (tid == 0) {
+        if (rotations && blockIdx.x % P.cluster == 0) atomicAdd(P.counts + used, rotations);
+        __threadfence();
+        ++epoch;
+        atomicAdd(P.bar, 1u);
+        const unsigned target = epoch * gridDim.x;
+        const uint64_t start = ptx::globaltimer();
+        for (unsigned i = 1; svd_load_acquire(P.bar) < target; ++i)
+          if ((i & 63u) == 0u && ptx::globaltimer() - start > ptx::kWaitLimitNs) {
+            ptx::set_status(P.status, TN_ERR_TIMEOUT);
+            s.abort = 1;
+            break;
+          }
+        __threadfence();
+      }
+      __syncthreads();
+      if (s.abort) return;
+    }
+    done = svd_load_acquire(reinterpret_cast<const unsigned*>(P.counts + used)) == 0;
+    ++used;
+  }
+  if (blockIdx.x == 0 && tid == 0) *P.sweeps = done ? used : -used;
+}
+
+// Sum of a per-thread value over the CTA, in double across warps.
+__device__ __forceinline__ double block_sum(float a) {
+  __shared__ double part[SVD_WARPS];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = a;
+  __syncthreads();
+  double s = 0.0;
+  for (int w = 0; w < SVD_WARPS; ++w) s += part[w];
+  return s;
+}
+
+// Element (row, col) of a matrix kept in blocks of 16 columns, n rows.
+__device__ __forceinline__ int64_t blocked(int64_t row, int64_t col, int64_t n) {
+  return ((col / SVD_B) * n + row) * SVD_B + col % SVD_B;
+}
+
+// Column j (CTA j): vnorm[j] = |V[:, j]| and sigma[j] = |W[:, j]| / vnorm[j].
+// Both blocks took the same products with Q, so what these left of the unit
+// length of V's columns is also in W's and cancels.
 __global__ void __launch_bounds__(SVD_THREADS)
-svd_norms(const float* __restrict__ W, int64_t L, float* __restrict__ sigma) {
-  const float* w = W + (int64_t)blockIdx.x * L;
-  float a = 0.0f, z0 = 0.0f, z1 = 0.0f;
-  for (int64_t i = threadIdx.x; i < L; i += SVD_THREADS) a = fmaf(w[i], w[i], a);
-  __shared__ double sums[3];
-  block_sum3(a, z0, z1, sums);
-  if (threadIdx.x == 0) sigma[blockIdx.x] = (float)sqrt(sums[0]);
+svd_norms(const float* __restrict__ W, const float* __restrict__ V, int64_t L, int64_t r, float* __restrict__ sigma,
+          float* __restrict__ vnorm) {
+  const float* w = W + blocked(0, blockIdx.x, L);
+  const float* v = V + blocked(0, blockIdx.x, r);
+  float a = 0.0f, b = 0.0f;
+  for (int64_t i = threadIdx.x; i < L; i += SVD_THREADS) a = fmaf(w[i * SVD_B], w[i * SVD_B], a);
+  for (int64_t i = threadIdx.x; i < r; i += SVD_THREADS) b = fmaf(v[i * SVD_B], v[i * SVD_B], b);
+  const double sa = block_sum(a), sb = block_sum(b);
+  if (threadIdx.x == 0) {
+    const double vn = sqrt(sb);
+    vnorm[blockIdx.x] = (float)vn;
+    sigma[blockIdx.x] = (float)(sqrt(sa) / vn);
+  }
 }
 
 // order[c] = index of the c-th largest singular value (ties by index; a NaN
@@ -229,14 +459,15 @@ __global__ void svd_sort(const float* __restrict__ sigma, int r, int32_t* __rest
   sorted[rank] = sigma[j];
 }
 
-// The outputs for the k kept values. Columns of W give singular vectors
-// scaled by sigma (w_j = sigma_j u_j), columns of V unit ones. Left (M x k,
+// The outputs for the k kept values. Columns of V give singular vectors scaled
+// by vnorm, columns of W scaled by sigma vnorm (w_j = sigma_j vnorm_j u_j). Left (M x k,
 // row-major): W's columns when M >= N, else V's; right (k x N, row-major):
 // the other one. absorb: both sides carry sqrt(sigma) (split_node), else
 // neither (full SVD). A W column of a zero singular value has no direction:
 // its vector is written as zeros (not completed to an orthonormal basis).
 __global__ void svd_write(const float* __restrict__ W, const float* __restrict__ V, const int32_t* __restrict__ order,
-                          const float* __restrict__ sorted, int64_t M, int64_t N, int64_t L, int r, int k,
+                          const float* __restrict__ sorted, const float* __restrict__ vnorm, int64_t M, int64_t N,
+                          int64_t L, int r, int k,
                           int wide, int absorb, float* __restrict__ U, float* __restrict__ S, float* __restrict__ Vt,
                           float* __restrict__ dropped) {
   const int64_t nl = M * k, nr = (int64_t)k * N, stride = (int64_t)gridDim.x * blockDim.x;
@@ -248,13 +479,14 @@ __global__ void svd_write(const float* __restrict__ W, const float* __restrict__
     const int64_t i = left ? f / k : f % N;  // row of the left node, column of the right one
     const int j = min(max(order[c], 0), r - 1);
     const float sg = sorted[c];
+    const float vn = vnorm[j];
     const bool from_w = left != (wide != 0);  // left from W iff M >= N
     float x;
     if (from_w) {
-      const float sc = sg > 0.0f ? (absorb ? 1.0f / sqrtf(sg) : 1.0f / sg) : 0.0f;
-      x = W[(int64_t)j * L + i] * sc;
+      const float sc = sg > 0.0f ? (absorb ? 1.0f / (sqrtf(sg) * vn) : 1.0f / (sg * vn)) : 0.0f;
+      x = W[blocked(i, j, L)] * sc;
     } else {
-      x = V[(int64_t)j * r + i] * (absorb ? sqrtf(fmaxf(sg, 0.0f)) : 1.0f);
+      x = V[blocked(i, j, r)] * (absorb ? sqrtf(fmaxf(sg, 0.0f)) / vn : 1.0f / vn);
     }
     if (left)
       U[f] = x;
@@ -271,8 +503,8 @@ static size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 
 struct SplitLayout {
   SplitView v;
-  int64_t L, r;
-  size_t w_off, v_off, sig_off, ord_off, sorted_off, cnt_off, total;
+  int64_t L, r, ns;  // ns: blocks of 16 columns
+  size_t w_off, v_off, sig_off, vn_off, ord_off, sorted_off, cnt_off, total;
 };
 
 static int plan_split(const tn_tensor* A, const int* left, int nleft, const int* right, int nright,
@@ -322,13 +554,15 @@ static int plan_split(const tn_tensor* A, const int* left, int nleft, const int*
   o.r = o.v.wide ? o.v.M : o.v.N;
   if (o.r > 0x3FFFFFFF) return TN_ERR_UNSUPPORTED;
   if (o.r > 0 && !o.v.A) return TN_ERR_ARG;
+  o.ns = (o.r + SVD_B - 1) / SVD_B;
   o.w_off = 0;
-  o.v_off = al256(sizeof(float) * (size_t)(o.L * o.r));
-  o.sig_off = o.v_off + al256(sizeof(float) * (size_t)(o.r * o.r));
-  o.ord_off = o.sig_off + al256(sizeof(float) * (size_t)o.r);
+  o.v_off = al256(sizeof(float) * (size_t)(o.L * o.ns * SVD_B));
+  o.sig_off = o.v_off + al256(sizeof(float) * (size_t)(o.r * o.ns * SVD_B));
+  o.vn_off = o.sig_off + al256(sizeof(float) * (size_t)o.r);
+  o.ord_off = o.vn_off + al256(sizeof(float) * (size_t)o.r);
   o.sorted_off = o.ord_off + al256(sizeof(int32_t) * (size_t)o.r);
-  o.cnt_off = o.sorted_off + al256(sizeof(float) * (size_t)o.r);
-  o.total = o.cnt_off + 256;
+  o.cnt_off = o.sorted_off + al256(sizeof(float) * (size_t)(o.r + 1));  // the values, then the sweep count
+  o.total = o.cnt_off + 256;  // barrier counter, rotations per sweep
   return TN_OK;
 }
 
@@ -384,87 +618,73 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
   float* W = reinterpret_cast<float*>(base + lay.w_off);
   float* V = reinterpret_cast<float*>(base + lay.v_off);
   float* sigma = reinterpret_cast<float*>(base + lay.sig_off);
+  float* vnorm = reinterpret_cast<float*>(base + lay.vn_off);
   int32_t* order = reinterpret_cast<int32_t*>(base + lay.ord_off);
   float* sorted = reinterpret_cast<float*>(base + lay.sorted_off);
-  int* counter = reinterpret_cast<int*>(base + lay.cnt_off);
-  const int64_t L = lay.L;
-  const int r = (int)lay.r, rp = r + (r & 1);
-  svd_gather<<<grid_for(L * lay.r, 256), 256, 0, s>>>(lay.v, W, V, L, lay.r);
-  if (cudaGetLastError() != cudaSuccess) return TN_ERR_CUDA;
-  // off-diagonal threshold: a few times the float32 rounding of a length-L dot product
-  const float tol = 4.0f * sqrtf((float)L) * 5.9604645e-8f;
-  // one sweep = a CUDA graph: the counter reset, then the r - 1 rounds in
-  // order (built once per call, launched once per sweep)
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  auto cleanup = [&]() {
-    if (exec) cudaGraphExecDestroy(exec);
-    if (graph) cudaGraphDestroy(graph);
-  };
-  if (cudaGraphCreate(&graph, 0) != cudaSuccess) return TN_ERR_CUDA;
-  {
-    cudaGraphNode_t prev = nullptr, node = nullptr;
-    cudaMemsetParams mp;
-    memset(&mp, 0, sizeof(mp));
-    mp.dst = counter;
-    mp.value = 0;
-    mp.elementSize = sizeof(int);
-    mp.width = 1;
-    mp.height = 1;
-    if (cudaGraphAddMemsetNode(&prev, graph, nullptr, 0, &mp) != cudaSuccess) {
-      cleanup();
-      return TN_ERR_CUDA;
-    }
-    float* w_arg = W;
-    float* v_arg = V;
-    int64_t l_arg = L;
-    int r_arg = r, rp_arg = rp;
-    float tol_arg = tol;
-    int* c_arg = counter;
-    for (int t = 0; t < rp - 1; ++t) {
-      int t_arg = t;
-      void* args[] = {&w_arg, &v_arg, &l_arg, &r_arg, &rp_arg, &t_arg, &tol_arg, &c_arg};
-      cudaKernelNodeParams kp;
-      memset(&kp, 0, sizeof(kp));
-      kp.func = reinterpret_cast<void*>(svd_round);
-      kp.gridDim = dim3((unsigned)(rp / 2));
-      kp.blockDim = dim3(SVD_THREADS);
-      kp.kernelParams = args;
-      if (cudaGraphAddKernelNode(&node, graph, &prev, 1, &kp) != cudaSuccess) {
-        cleanup();
-        return TN_ERR_CUDA;
-      }
-      prev = node;
-    }
-  }
-  if (cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) {
-    cleanup();
+  const int64_t L = lay.L, cols = lay.ns * SVD_B;
+  const int r = (int)lay.r;
+  SvdParams P;
+  P.W = W;
+  P.V = V;
+  P.L = L;
+  P.r = r;
+  P.ns = (int32_t)lay.ns;
+  P.nb = P.ns + (P.ns & 1);
+  // counted above 16 tol, a few times the float32 rounding of a length-L dot product
+  P.tol = 0.25f * sqrtf((float)L) * 5.9604645e-8f;
+  P.bar = reinterpret_cast<unsigned*>(base + lay.cnt_off);
+  P.counts = reinterpret_cast<int*>(base + lay.cnt_off) + 1;
+  P.sweeps = reinterpret_cast<int*>(sorted + r);
+  P.status = status_word();
+  static_assert(sizeof(int) * (SVD_MAX_SWEEPS + 1) <= 256, "barrier counter and rotation counts");
+  if (cudaMemsetAsync(base + lay.cnt_off, 0, 256, s) != cudaSuccess ||
+      cudaMemsetAsync(P.sweeps, 0, sizeof(int), s) != cudaSuccess)
     return TN_ERR_CUDA;
+  svd_gather<<<grid_for(L * cols, 256), 256, 0, s>>>(lay.v, W, V, L, lay.r, cols);
+  if (cudaGetLastError() != cudaSuccess) return TN_ERR_CUDA;
+  static std::atomic<uint64_t> attr{0};
+  if (!smem_limit_once((const void*)svd_jacobi, sizeof(SvdSmem), &attr)) return TN_ERR_CUDA;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.blockDim = dim3(SVD_THREADS);
+  cfg.dynamicSmemBytes = sizeof(SvdSmem);
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  // one CTA per SM; the rows of a pair over as many CTAs (up to 8, at least
+  // 32 rows each) as all pairs leave room for
+  const int64_t pairs = P.nb / 2, sms = min_units_single() / 2;
+  P.cluster = 1;
+  while (P.cluster < SVD_CLUSTER && pairs * P.cluster * 2 <= sms && L >= 64 * P.cluster) P.cluster *= 2;
+  for (;; P.cluster /= 2) {
+    const int64_t ctas = pairs * P.cluster < sms ? pairs * P.cluster : sms / P.cluster * P.cluster;
+    cfg.gridDim = dim3((unsigned)ctas);
+    at[1].val.clusterDim.x = (unsigned)P.cluster;
+    int fit = 0;
+    if (P.cluster == 1 || (cudaOccupancyMaxActiveClusters(&fit, svd_jacobi, &cfg) == cudaSuccess &&
+                           (int64_t)fit * P.cluster >= ctas))
+      break;
   }
-  int done = 0, used = 0;
-  for (int sw = 0; sw < SVD_MAX_SWEEPS && !done; ++sw) {
-    int host_count = -1;
-    if (cudaGraphLaunch(exec, s) != cudaSuccess ||
-        cudaMemcpyAsync(&host_count, counter, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess) {
-      cleanup();
-      return TN_ERR_CUDA;
-    }
-    ++used;
-    done = host_count == 0;
-  }
-  cleanup();
-  if (sweeps) *sweeps = done ? used : -used;
-  svd_norms<<<r, SVD_THREADS, 0, s>>>(W, L, sigma);
+  if (cudaLaunchKernelEx(&cfg, svd_jacobi, P) != cudaSuccess) return TN_ERR_CUDA;
+  svd_norms<<<r, SVD_THREADS, 0, s>>>(W, V, L, r, sigma, vnorm);
   svd_sort<<<(r + 255) / 256, 256, 0, s>>>(sigma, r, order, sorted);
   if (cudaGetLastError() != cudaSuccess) return TN_ERR_CUDA;
-  std::vector<float> host_sorted((size_t)r);
-  if (cudaMemcpyAsync(host_sorted.data(), sorted, sizeof(float) * (size_t)r, cudaMemcpyDeviceToHost, s) !=
+  std::vector<float> host_sorted((size_t)r + 1);
+  if (cudaMemcpyAsync(host_sorted.data(), sorted, sizeof(float) * ((size_t)r + 1), cudaMemcpyDeviceToHost, s) !=
           cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return TN_ERR_CUDA;
+  int32_t used = 0;
+  memcpy(&used, &host_sorted[(size_t)r], sizeof(used));
+  if (used == 0) return TN_ERR_TIMEOUT;  // the barrier's wait expired
+  if (sweeps) *sweeps = used;
   const int64_t k = tn_split_truncation(host_sorted.data(), r, max_singular_values, max_truncation_err);
-  svd_write<<<grid_for((lay.v.M + lay.v.N) * k + r, 256), 256, 0, s>>>(W, V, order, sorted, lay.v.M, lay.v.N, L,
+  svd_write<<<grid_for((lay.v.M + lay.v.N) * k + r, 256), 256, 0, s>>>(W, V, order, sorted, vnorm, lay.v.M, lay.v.N, L,
                                                                         r, (int)k, lay.v.wide, absorb ? 1 : 0, U, S, Vt,
                                                                         dropped);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return TN_ERR_CUDA;

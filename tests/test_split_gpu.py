@@ -157,3 +157,14 @@ def test_legs_must_partition(tn):
     At = torch.zeros((2, 3, 4), device="cuda")
     with pytest.raises(tn.TnError):
         tn.split_node(At, [0], [1])
+
+
+@pytest.mark.parametrize("shape,scale", [((16, 16), 1.0), ((17, 40), 1.0), ((33, 33), 1e15), ((47, 300), 1.0),
+                                         ((48, 257), 1e-15), ((700, 20), 1.0), ((2100, 35), 1.0), ((5, 600), 1.0),
+                                         ((1, 9), 1.0)])
+def test_block_edges(tn, shape, scale):
+    # blocks of 16 columns (one, an odd count, a ragged last one), rows past a
+    # staged chunk (256) and shared out over a cluster, norms whose squares
+    # come near the ends of the exponent range; tolerances as above
+    A = (rand(31, shape) * np.float32(scale)).astype(np.float32)
+    check(tn, A, [0], [1])
