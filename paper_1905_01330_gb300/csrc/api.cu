@@ -222,9 +222,16 @@ int spec_class(const ContractDesc& d) {
   return d.K <= 512 ? 1 : 2;
 }
 
-tn::PackedSchedule default_schedule(int cls) {
+// Before any tuning. BF16 contractions with 128 rows or more on both sides take
+// 256-wide tiles (each block of the wider operand then feeds 256 results: the
+// GEMM launch of 2048 random specs 3.87 -> 2.81 ms, of 512 with dimensions off
+// every power of two 1.11 -> 0.95; 64 specs 120 -> 93 us), unless so few units
+// are left (`wide` false) that SMs would idle.
+tn::PackedSchedule default_schedule(int prec, int cls, bool wide) {
   tn::PackedSchedule sc;
-  sc.store16 = cls == 2 ? 1 : 0;  // measured: whole-sector stores help long-k specs only
+  if (prec == TN_PREC_BF16 && cls > 0 && wide) sc.q_tile = 256;
+  // measured: whole-sector stores help long-k specs only (256-wide tiles store whole rows anyway)
+  else sc.store16 = cls == 2 ? 1 : 0;
   return sc;
 }
 
@@ -369,14 +376,19 @@ int tn::group_plan_create_ex(const tn_contract_spec* specs, int nspecs, int prec
       p->reserve_punits = std::max(p->reserve_punits, p->pp.units.size());
       p->reserve_packed = std::max(p->reserve_packed, p->pp.packed_bytes);
     }
-    for (int c = 0; c < 3; ++c) p->sched[c] = default_schedule(c);
+    bool tuned = false;
+    for (int c = 0; c < 3; ++c) p->sched[c] = default_schedule(prec, c, true);
     {
       std::lock_guard<std::mutex> lk(g_tune_lock);
       auto it = g_tune_cache.find(p->signature);
-      if (it != g_tune_cache.end())
-        for (int c = 0; c < 3; ++c) p->sched[c] = it->second.sc[c];
+      tuned = it != g_tune_cache.end();
+      for (int c = 0; tuned && c < 3; ++c) p->sched[c] = it->second.sc[c];
     }
-    const int rc = build_packed(p);
+    int rc = build_packed(p);
+    if (rc == TN_OK && !tuned && p->packed_tiles < min_units_single()) {
+      for (int c = 0; c < 3; ++c) p->sched[c] = default_schedule(prec, c, false);
+      rc = build_packed(p);
+    }
     if (rc != TN_OK) { delete p; return rc; }
     *plan = p;
     return TN_OK;
