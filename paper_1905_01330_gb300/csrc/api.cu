@@ -253,6 +253,7 @@ int build_packed(tn_group_plan* p, bool allow_fuse = true) {
                                &p->pp, ext);
     if (rc != TN_OK) return rc;
   }
+  cut_pack_units(&p->pp);
   // largest units first: tensor time plus memory time of one unit
   auto cost = [](const GemmDesc& g) {
     const double pr = (double)std::min<int64_t>(g.RP, 128), qr = (double)std::min<int64_t>(g.RQ, g.q_tile);
@@ -595,6 +596,14 @@ int tn::group_plan_ext_layout(const tn_group_plan* plan, int i, ExtPLayout* out)
     out->kstrA[q] = d.kstrA[q];
   }
   return TN_OK;
+}
+
+bool tn::group_plan_watch_max(tn_group_plan* plan, int i, unsigned* bits) {
+  if (!plan || !plan->packed || i < 0 || (size_t)i >= plan->descs.size() || plan->ext_p[(size_t)i] ||
+      plan->pp.job_hi_off[2 * (size_t)i] == SIZE_MAX)
+    return false;
+  plan->pp.jobs[2 * (size_t)i].amax = bits;
+  return true;
 }
 
 int tn::group_plan_upload_shared(const tn_group_plan* plan, void* lists, size_t bytes, void* packed,

@@ -6,7 +6,8 @@
 // count per site does not grow with the batch: (i) one grouped contraction,
 // (ii) one grouped float32 kernel that also applies the previous site's
 // deferred power-of-two rescale, (iii) one grouped contraction, then one
-// grouped max-abs pass over the count new environments. BF16 / BF16X3 with
+// grouped max-abs pass over the count new environments (none where the next
+// site's pack reads every environment: it finds the maxima). BF16 / BF16X3 with
 // an extended MPO of (bond) x d <= 8: step (ii) writes each chain's T2
 // straight into the (iii) plan's packed region as its first operand (whole
 // MN-major blocks), so that plan packs only the cores.
@@ -148,6 +149,7 @@ struct GroupedSweep {
   std::vector<StepIIPack> psteps;     // n * count (hi / lo: offsets in the packed region until laid out)
   std::vector<int64_t> max_items;     // per site: the largest step (ii) work of a chain
   std::vector<int64_t> max_cols;      // per site: the largest Da Db of the batch
+  std::vector<uint8_t> packed_max;    // per site: its pack finds the largest |L| entering it
   std::vector<ChainInit> inits;
   std::vector<ChainFinal> finals;
   std::vector<int64_t> woff;          // extended MPO of every site
@@ -269,6 +271,12 @@ int build_sweep(const tn_mps* psis, int count, const tn_mpo* H, int prec, uint8_
                                     j == 1 && g->fused ? ext.data() : nullptr);
       if (rc != TN_OK) return rc;
       g->plans.emplace_back(p);
+      if (j == 0) {
+        bool all = i > 0;
+        for (int k = 0; k < count && all; ++k) all = group_plan_watch_max(p, k, bits + (size_t)count * (i - 1) + k);
+        for (int k = 0; k < count && !all; ++k) group_plan_watch_max(p, k, nullptr);
+        g->packed_max.push_back(all ? 1 : 0);
+      }
       if (j == 1 && g->fused) {
         // step (ii) of every chain writes its T2 where the (iii) plan reads P
         int64_t mi = 1;
@@ -395,7 +403,7 @@ int run_sweep(const tn_expect_plan* pl, double* result, cudaStream_t s) {
     if ((rc = group_plan_run_shared(g.plans[p0 + 1].get(), base + g.plan_off[p0 + 1], g.plan_bytes[p0 + 1], s)) !=
         TN_OK)
       return rc;
-    if (i + 1 < g.n) {
+    if (i + 1 < g.n && !g.packed_max[(size_t)i + 1]) {
       int64_t longest = 1;
       for (int k = 0; k < count; ++k) longest = std::max(longest, g.segs[(size_t)count * i + k].n);
       const dim3 grid((unsigned)std::min<int64_t>((longest + 2047) / 2048, 64), (unsigned)count);

@@ -231,6 +231,14 @@ __device__ __forceinline__ void pack_blocks(const PackJob& J, int first, int cou
   }
 }
 
+// Raises *bits to the bits of the warp's largest m (non-negative floats order
+// as their bit patterns do).
+__device__ __forceinline__ void raise_max(unsigned* bits, float m) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(bits, __float_as_uint(m));
+}
+
 // Grouped form: one CTA per pack unit of the uploaded lists.
 // Copies job J into shared memory (all threads, then a barrier).
 __device__ __forceinline__ void stage_job(const PackJob& J, PackSmem& sm) {
@@ -247,6 +255,12 @@ pack_kernel(const PackJob* __restrict__ jobs, const PackUnit* __restrict__ units
   PackSmem& sm = *reinterpret_cast<PackSmem*>(pack_smem_raw);
   const PackUnit un = units[blockIdx.x];
   stage_job(jobs[un.job], sm);
+  if (sm.job.amax) {
+    float m = 0.0f;
+    pack_blocks<true>(sm.job, un.first, un.count, sm, &m);
+    raise_max(sm.job.amax, m);
+    return;
+  }
   pack_blocks(sm.job, un.first, un.count, sm);
 }
 
@@ -277,9 +291,7 @@ pack_pair_kernel(const __grid_constant__ PackPair pp) {
   if (which == 0 && pp.maxbits) {
     float m = 0.0f;
     pack_blocks<true>(J, first, min(per, nb - first), sm, &m);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(pp.maxbits, __float_as_uint(m));
+    raise_max(pp.maxbits, m);
     return;
   }
   pack_blocks(J, first, min(per, nb - first), sm);
@@ -1873,6 +1885,28 @@ void fused_tables(const ContractDesc& d, std::vector<int32_t>* tab, int64_t* rta
   while ((tab->size() - (size_t)*ktab_off) % PK) tab->push_back(0);
 }
 
+void cut_pack_units(PackedPlan* pp) {
+  // A unit reads about 256 KB, but a small plan is cut finer, down to a block
+  // or the blocks packed at once, so that eight units an SM are there to
+  // share it (a site of a 16-state energy batch, 22 MB: 85 units of 256 KB
+  // took 32 us, single blocks about 20).
+  int64_t total = 0;
+  auto packed = [&](size_t j) { return pp->job_hi_off[j] != SIZE_MAX && !pp->job_ext[j]; };
+  for (size_t j = 0; j < pp->jobs.size(); ++j)
+    if (packed(j)) total += 2 * (int64_t)job_bytes(pp->jobs[j]);
+  const int64_t share = total / (8 * (int64_t)sm_count());
+  pp->units.clear();
+  for (size_t j = 0; j < pp->jobs.size(); ++j) {
+    if (!packed(j)) continue;
+    const PackJob& jb = pp->jobs[j];
+    const int32_t nb = jb.tiles * jb.slabs;
+    int32_t per = blocks_per_unit(jb);
+    const int64_t fair = share / (2 * jb.block_bytes);
+    if (fair < per) per = (int32_t)std::max<int64_t>(1, fair / jb.nbv) * jb.nbv;
+    for (int32_t f = 0; f < nb; f += per) pp->units.push_back(PackUnit{(int32_t)j, f, std::min(per, nb - f), 0});
+  }
+}
+
 int plan_packed(const ContractDesc& d, int prec, const PackedSchedule& sc, bool fuse, int64_t rtab_off,
                 int64_t ktab_off, const TmaBox* box, int64_t map, PackedPlan* pp, bool ext_p) {
   PackJob ja = make_job(d, d.A, d.M, d.nm, d.mdim, d.mstr, d.kstrA);
@@ -1953,14 +1987,6 @@ int plan_packed(const ContractDesc& d, int prec, const PackedSchedule& sc, bool 
   pp->job_lo_off.push_back(split ? off_blo : SIZE_MAX);
   pp->job_ext.push_back(ext_p ? 1 : 0);
   pp->job_ext.push_back(0);
-  for (int w = 0; w < 2; ++w) {
-    if (!(w == 0 ? pack_a : pack_b)) continue;
-    const PackJob& j = pp->jobs[(size_t)ja_idx + w];
-    const int32_t nb = j.tiles * j.slabs;
-    const int32_t per = blocks_per_unit(j);
-    for (int32_t f = 0; f < nb; f += per) pp->units.push_back(PackUnit{ja_idx + w, f, std::min(per, nb - f), 0});
-  }
-
   g.store16 = sc.store16;
   g.P_off = swap ? off_b : off_a;
   g.Q_off = swap ? off_a : off_b;

@@ -38,6 +38,7 @@ struct PackJob {
   const int32_t* ktab;    // and of every shared index, K entries (32-byte aligned, zero-padded
                           // to whole 64-wide slabs)
   int64_t rtab_off, ktab_off;  // host: their element offsets in the plan's table region, -1 none
+  unsigned* amax;         // device (or null): raised to the bits of the operand's largest |value|
   int32_t rdim[TN_MAX_RANK];
   int32_t kdim[TN_MAX_RANK];
   int64_t rstr[TN_MAX_RANK];
@@ -141,6 +142,9 @@ struct PackedPlan {
 // never fused); TN_ERR_UNSUPPORTED if A would be the GEMM's narrower side.
 int plan_packed(const ContractDesc& d, int prec, const PackedSchedule& sc, bool fuse, int64_t rtab_off,
                 int64_t ktab_off, const TmaBox* box, int64_t map, PackedPlan* pp, bool ext_p = false);
+
+// Cuts the plan's pack jobs into units, once all contractions are appended.
+void cut_pack_units(PackedPlan* pp);
 
 // The operand on the MMA's 128-row side of contraction d: B when it has more
 // rows and A fewer than 128, else A.

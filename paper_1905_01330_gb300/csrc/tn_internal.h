@@ -123,6 +123,11 @@ struct ExtPLayout {
 };
 int group_plan_ext_layout(const tn_group_plan* plan, int i, ExtPLayout* out);
 
+// Has the plan's pack raise *bits (device) to the bits of the largest |value|
+// of spec i's first operand whenever it runs; false when that operand is not
+// packed. Before the upload.
+bool group_plan_watch_max(tn_group_plan* plan, int i, unsigned* bits);
+
 // Plans that run one after another on a stream can share one region for
 // their packed bf16 blocks: the lists go to `lists` (group_plan_list_bytes),
 // the blocks to `packed` (group_plan_packed_bytes, 256-byte aligned).
