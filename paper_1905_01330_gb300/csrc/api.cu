@@ -628,13 +628,25 @@ int tn_group_plan_upload(const tn_group_plan* plan, void* workspace, size_t byte
 
 }  // extern "C"
 
-static int run_impl(const tn_group_plan* plan, void* workspace, cudaStream_t s);
+static int run_impl(const tn_group_plan* plan, void* workspace, bool packed, cudaStream_t s);
+static void pack_list(const tn_group_plan* plan, void* workspace, int i, tn::PackLists* pl);
 
-int tn::group_plan_run_shared(const tn_group_plan* plan, void* lists, size_t bytes, cudaStream_t s) {
+int tn::group_plan_run_shared(const tn_group_plan* plan, void* lists, size_t bytes, bool packed, cudaStream_t s) {
   if (!plan) return TN_ERR_ARG;
   int rc = check_ws_need(list_bytes(plan), lists, bytes);
   if (rc != TN_OK) return rc;
-  return run_impl(plan, lists, s);
+  return run_impl(plan, lists, packed, s);
+}
+
+int tn::group_plan_pack_two(const tn_group_plan* a, void* lists_a, const tn_group_plan* b, void* lists_b,
+                            cudaStream_t s) {
+  if (!a || !b || !a->packed || !b->packed) return TN_ERR_ARG;
+  tn::PackLists pl;
+  memset(&pl, 0, sizeof(pl));
+  pack_list(a, lists_a, 0, &pl);
+  pack_list(b, lists_b, 1, &pl);
+  if (pl.n[0] + pl.n[1] == 0) return TN_ERR_ARG;  // nothing would zero the unit counters
+  return launch_pack(pl, s);
 }
 
 extern "C" {
@@ -643,7 +655,7 @@ int tn_group_plan_run(const tn_group_plan* plan, void* workspace, size_t bytes, 
   if (!plan) return TN_ERR_ARG;
   int rc = check_ws(plan, workspace, bytes);
   if (rc != TN_OK) return rc;
-  return run_impl(plan, workspace, static_cast<cudaStream_t>(stream));
+  return run_impl(plan, workspace, false, static_cast<cudaStream_t>(stream));
 }
 
 }  // extern "C"
@@ -674,17 +686,29 @@ static int launch_count(const tn_group_plan* plan) {
   return launch_list(plan, kinds);
 }
 
-static int run_one(const tn_group_plan* plan, void* workspace, LaunchKind k, cudaStream_t s) {
+// The plan's pack as list i of a pack launch.
+static void pack_list(const tn_group_plan* plan, void* workspace, int i, tn::PackLists* pl) {
+  uint8_t* base = static_cast<uint8_t*>(workspace);
+  pl->jobs[i] = reinterpret_cast<const PackJob*>(base + jobs_offset(plan));
+  pl->units[i] = reinterpret_cast<const PackUnit*>(base + punits_offset(plan));
+  pl->n[i] = (int64_t)plan->pp.units.size();
+  pl->ctr[i] = reinterpret_cast<uint32_t*>(base + ctr_offset(plan));
+}
+
+// zero_ctr: the launch zeroes its own unit counter (else the pack before it has).
+static int run_one(const tn_group_plan* plan, void* workspace, LaunchKind k, bool zero_ctr, cudaStream_t s) {
   uint8_t* base = static_cast<uint8_t*>(workspace);
   const int32_t* map = reinterpret_cast<const int32_t*>(base + map_offset(plan));
   switch (k) {
     case L_ZERO:
       return launch_zero(reinterpret_cast<const ZeroRange*>(base + zero_offset(plan)), (int)plan->zero_ranges.size(),
                          s);
-    case L_PACK:
-      return launch_pack(reinterpret_cast<const PackJob*>(base + jobs_offset(plan)),
-                         reinterpret_cast<const PackUnit*>(base + punits_offset(plan)),
-                         (int64_t)plan->pp.units.size(), s);
+    case L_PACK: {
+      tn::PackLists pl;
+      memset(&pl, 0, sizeof(pl));
+      pack_list(plan, workspace, 0, &pl);
+      return launch_pack(pl, s);
+    }
     case L_FUSED:
       return launch_fused_gemm(reinterpret_cast<const GemmDesc*>(base), map + plan->packed_tiles,
                                reinterpret_cast<const PackJob*>(base + jobs_offset(plan)),
@@ -692,13 +716,13 @@ static int run_one(const tn_group_plan* plan, void* workspace, LaunchKind k, cud
     case L_TMA:
       return launch_tma_gemm(reinterpret_cast<const GemmDesc*>(base), map + plan->tma_tiles,
                              plan->total_tiles - plan->tma_tiles,
-                             reinterpret_cast<uint32_t*>(base + ctr_offset(plan)) + 1, s);
+                             reinterpret_cast<uint32_t*>(base + ctr_offset(plan)) + 1, zero_ctr, s);
     default:
       break;
   }
   if (plan->packed)
     return launch_packed_gemm(reinterpret_cast<const GemmDesc*>(base), map, plan->packed_tiles, plan->prec,
-                              reinterpret_cast<uint32_t*>(base + ctr_offset(plan)), s);
+                              reinterpret_cast<uint32_t*>(base + ctr_offset(plan)), zero_ctr, s);
   const ContractDesc* g = reinterpret_cast<const ContractDesc*>(base);
   if (plan->prec == TN_PREC_FP32 && plan->skinny)
     return launch_contract_skinny_grouped(g, (int)plan->descs.size(), plan->max_n, s);
@@ -706,14 +730,17 @@ static int run_one(const tn_group_plan* plan, void* workspace, LaunchKind k, cud
   return launch_contract_tc(plan->descs[0], g, map, plan->total_tiles, plan->prec, s);
 }
 
-static int run_impl(const tn_group_plan* plan, void* workspace, cudaStream_t s) {
+// packed: the plan's pack ran already (group_plan_pack_two).
+static int run_impl(const tn_group_plan* plan, void* workspace, bool packed, cudaStream_t s) {
   for (const auto& z : plan->zeros)
     if (cudaMemsetAsync(z.C, 0, sizeof(float) * (size_t)(z.M * z.N), s) != cudaSuccess) return TN_ERR_CUDA;
   LaunchKind kinds[MAX_LAUNCHES];
   const int n = launch_list(plan, kinds);
   for (int i = 0; i < n; ++i) {
-    const int rc = run_one(plan, workspace, kinds[i], s);
+    if (kinds[i] == L_PACK && packed) continue;
+    const int rc = run_one(plan, workspace, kinds[i], !packed, s);
     if (rc != TN_OK) return rc;
+    if (kinds[i] == L_PACK) packed = true;
   }
   return TN_OK;
 }
@@ -731,7 +758,7 @@ int tn_group_plan_run_launch(const tn_group_plan* plan, void* workspace, size_t 
   if (index == 0)
     for (const auto& z : plan->zeros)
       if (cudaMemsetAsync(z.C, 0, sizeof(float) * (size_t)(z.M * z.N), s) != cudaSuccess) return TN_ERR_CUDA;
-  return run_one(plan, workspace, kinds[index], s);
+  return run_one(plan, workspace, kinds[index], true, s);
 }
 
 const char* tn_group_plan_launch_name(const tn_group_plan* plan, int index) {
@@ -812,9 +839,9 @@ int tn_group_plan_autotune(tn_group_plan* plan, void* workspace, size_t bytes, v
   auto trial = [&](float* ms) -> int {
     int r = build_packed(plan);
     if (r == TN_OK) r = upload_impl(plan, workspace, base + packed_offset(plan), s, false);
-    if (r == TN_OK) r = run_impl(plan, workspace, s);
+    if (r == TN_OK) r = run_impl(plan, workspace, false, s);
     if (r == TN_OK && cudaEventRecord(e0, s) != cudaSuccess) r = TN_ERR_CUDA;
-    for (int k = 0; k < 2 && r == TN_OK; ++k) r = run_impl(plan, workspace, s);
+    for (int k = 0; k < 2 && r == TN_OK; ++k) r = run_impl(plan, workspace, false, s);
     if (r == TN_OK && (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
                        cudaEventElapsedTime(ms, e0, e1) != cudaSuccess))
       r = TN_ERR_CUDA;

@@ -153,10 +153,12 @@ struct GroupedSweep {
   std::vector<ChainInit> inits;
   std::vector<ChainFinal> finals;
   std::vector<int64_t> woff;          // extended MPO of every site
-  size_t off_lg = 0, off_bits = 0, off_segs = 0, off_steps = 0, off_psteps = 0, off_init = 0, off_final = 0,
-         off_packed = 0;
+  size_t off_lg = 0, off_bits = 0, off_segs = 0, off_steps = 0, off_psteps = 0, off_init = 0, off_final = 0;
+  size_t off_packed[2] = {0, 0};
   size_t off_w = 0, total = 0;
-  size_t packed_bytes = 0;  // largest packed-operand region of one plan
+  // largest packed-operand region of a plan: of all plans, or (fused mode) of
+  // the (i) and of the (iii) plans, whose packs run in one launch per site
+  size_t packed_bytes[2] = {0, 0};
   int64_t nbits = 0;
 };
 
@@ -204,7 +206,8 @@ int build_sweep(const tn_mps* psis, int count, const tn_mpo* H, int prec, uint8_
     b.L[0] = take(sizeof(float) * W1 * D * D);
     b.L[1] = take(sizeof(float) * W1 * D * D);
     b.T1 = take(sizeof(float) * W1 * D * d * D);
-    b.T2 = take(sizeof(float) * W1 * D * d * D);
+    // fused: T2 exists in packed form only; the (iii) plan never reads this address
+    b.T2 = g->fused ? b.T1 : take(sizeof(float) * W1 * D * d * D);
   }
   int64_t wtot = 0;
   for (int i = 0; i < n; ++i) {
@@ -311,16 +314,21 @@ int build_sweep(const tn_mps* psis, int count, const tn_mpo* H, int prec, uint8_
       g->plan_off.push_back(off);
       g->plan_bytes.push_back(bytes);
       off += align256(bytes);
-      g->packed_bytes = std::max(g->packed_bytes, group_plan_packed_bytes(p));
+      size_t& region = g->packed_bytes[g->fused ? j : 0];
+      region = std::max(region, group_plan_packed_bytes(p));
     }
   }
-  // one region for the packed operands of whichever plan is running (the
-  // plans run one after another on the stream)
-  g->off_packed = off;
-  off += align256(g->packed_bytes);
+  // regions for the packed operands of whichever site is running (the sites
+  // run one after another on the stream)
+  g->off_packed[0] = g->off_packed[1] = off;
+  off += align256(g->packed_bytes[0]);
+  if (g->fused) {
+    g->off_packed[1] = off;
+    off += align256(g->packed_bytes[1]);
+  }
   for (auto& q : g->psteps) {
-    q.hi = base + g->off_packed + (uintptr_t)q.hi;
-    if (q.lo) q.lo = base + g->off_packed + (uintptr_t)q.lo;
+    q.hi = base + g->off_packed[1] + (uintptr_t)q.hi;
+    if (q.lo) q.lo = base + g->off_packed[1] + (uintptr_t)q.lo;
   }
   g->off_segs = off;
   off += align256(sizeof(Segment) * g->segs.size());
@@ -389,7 +397,14 @@ int run_sweep(const tn_expect_plan* pl, double* result, cudaStream_t s) {
   const StepII* steps = reinterpret_cast<const StepII*>(base + g.off_steps);
   for (int i = 0; i < g.n; ++i) {
     const size_t p0 = (size_t)i * 2;
-    if ((rc = group_plan_run_shared(g.plans[p0].get(), base + g.plan_off[p0], g.plan_bytes[p0], s)) != TN_OK)
+    // fused: L, the core for (i) and the core for (iii) packed in one launch,
+    // which also resets the GEMMs' unit counters: four launches a site, where
+    // separate packs and resets made eight (16 states of up to 512: 158 us a
+    // site -> 145 us)
+    if (g.fused && (rc = group_plan_pack_two(g.plans[p0].get(), base + g.plan_off[p0], g.plans[p0 + 1].get(),
+                                             base + g.plan_off[p0 + 1], s)) != TN_OK)
+      return rc;
+    if ((rc = group_plan_run_shared(g.plans[p0].get(), base + g.plan_off[p0], g.plan_bytes[p0], g.fused, s)) != TN_OK)
       return rc;
     const StepII& q0 = g.steps[(size_t)count * i];
     if (g.fused) {
@@ -400,8 +415,8 @@ int run_sweep(const tn_expect_plan* pl, double* result, cudaStream_t s) {
                                                 (int64_t)q0.wa * q0.d, (int64_t)q0.wb * q0.d, s)) != TN_OK) {
       return rc;
     }
-    if ((rc = group_plan_run_shared(g.plans[p0 + 1].get(), base + g.plan_off[p0 + 1], g.plan_bytes[p0 + 1], s)) !=
-        TN_OK)
+    if ((rc = group_plan_run_shared(g.plans[p0 + 1].get(), base + g.plan_off[p0 + 1], g.plan_bytes[p0 + 1], g.fused,
+                                    s)) != TN_OK)
       return rc;
     if (i + 1 < g.n && !g.packed_max[(size_t)i + 1]) {
       int64_t longest = 1;
@@ -446,7 +461,7 @@ int tn_mps_expect_grouped_plan(const tn_mps* psis, int count, const tn_mpo* H, i
   // and final tables
   for (size_t j = 0; j < g.plans.size(); ++j) {
     if (g.plan_bytes[j] == 0) continue;
-    rc = group_plan_upload_shared(g.plans[j].get(), base + g.plan_off[j], g.plan_bytes[j], base + g.off_packed, s);
+    rc = group_plan_upload_shared(g.plans[j].get(), base + g.plan_off[j], g.plan_bytes[j], base + g.off_packed[j & 1], s);
     if (rc != TN_OK) return rc;
   }
   if (cudaMemcpyAsync(base + g.off_segs, g.segs.data(), sizeof(Segment) * g.segs.size(), cudaMemcpyHostToDevice,

@@ -249,12 +249,17 @@ __device__ __forceinline__ void stage_job(const PackJob& J, PackSmem& sm) {
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(PACK_THREADS)
-pack_kernel(const PackJob* __restrict__ jobs, const PackUnit* __restrict__ units) {
+__global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const __grid_constant__ PackLists pl) {
   extern __shared__ __align__(16) uint8_t pack_smem_raw[];
   PackSmem& sm = *reinterpret_cast<PackSmem*>(pack_smem_raw);
-  const PackUnit un = units[blockIdx.x];
-  stage_job(jobs[un.job], sm);
+  // the GEMMs that follow claim their units from these
+  if (blockIdx.x == 0 && threadIdx.x < 2) {
+    if (pl.ctr[0]) pl.ctr[0][threadIdx.x] = 0u;
+    if (pl.ctr[1]) pl.ctr[1][threadIdx.x] = 0u;
+  }
+  const int l = (int64_t)blockIdx.x < pl.n[0] ? 0 : 1;
+  const PackUnit un = pl.units[l][blockIdx.x - (l ? pl.n[0] : 0)];
+  stage_job(pl.jobs[l][un.job], sm);
   if (sm.job.amax) {
     float m = 0.0f;
     pack_blocks<true>(sm.job, un.first, un.count, sm, &m);
@@ -1544,21 +1549,22 @@ int launch_gemm(const GemmDesc& single, const GemmDesc* descs, const int32_t* ma
 
 }  // namespace
 
-int launch_pack(const PackJob* jobs, const PackUnit* units, int64_t nunits, cudaStream_t s) {
-  if (nunits <= 0) return TN_OK;
-  if (nunits > 0x7FFFFFFF) return TN_ERR_UNSUPPORTED;
+int launch_pack(const PackLists& pl, cudaStream_t s) {
+  const int64_t units = pl.n[0] + pl.n[1];
+  if (units <= 0) return TN_OK;
+  if (units > 0x7FFFFFFF) return TN_ERR_UNSUPPORTED;
   if (!pack_attr()) return TN_ERR_CUDA;
-  pack_kernel<<<(unsigned)nunits, PACK_THREADS, PACK_SMEM, s>>>(jobs, units);
+  pack_kernel<<<(unsigned)units, PACK_THREADS, PACK_SMEM, s>>>(pl);
   return cudaGetLastError() == cudaSuccess ? TN_OK : TN_ERR_CUDA;
 }
 
 int launch_packed_gemm(const GemmDesc* descs, const int32_t* map, int64_t units, int prec, uint32_t* unit_ctr,
-                       cudaStream_t s) {
+                       bool zero_ctr, cudaStream_t s) {
   if (units <= 0) return TN_OK;
   if (units > 0x7FFFFFFF) return TN_ERR_UNSUPPORTED;
   if (prec != TN_PREC_BF16 && prec != TN_PREC_BF16X3) return TN_ERR_ARG;
   // the launch's CTAs claim units from this counter
-  if (unit_ctr && cudaMemsetAsync(unit_ctr, 0, sizeof(uint32_t), s) != cudaSuccess) return TN_ERR_CUDA;
+  if (unit_ctr && zero_ctr && cudaMemsetAsync(unit_ctr, 0, sizeof(uint32_t), s) != cudaSuccess) return TN_ERR_CUDA;
   GemmDesc none;
   memset(&none, 0, sizeof(none));
   if (prec == TN_PREC_BF16) return launch_gemm<0, 0>(none, descs, map, nullptr, units, s, unit_ctr);
@@ -1575,12 +1581,13 @@ int launch_fused_gemm(const GemmDesc* descs, const int32_t* map, const PackJob* 
   return launch_gemm<0, 1>(none, descs, map, jobs, units, s);
 }
 
-int launch_tma_gemm(const GemmDesc* descs, const int32_t* map, int64_t units, uint32_t* unit_ctr, cudaStream_t s) {
+int launch_tma_gemm(const GemmDesc* descs, const int32_t* map, int64_t units, uint32_t* unit_ctr, bool zero_ctr,
+                    cudaStream_t s) {
   if (units <= 0) return TN_OK;
   if (units > 0x7FFFFFFF) return TN_ERR_UNSUPPORTED;
   if (!descs || !map || !unit_ctr) return TN_ERR_ARG;
   // the launch's CTAs claim units from this counter
-  if (cudaMemsetAsync(unit_ctr, 0, sizeof(uint32_t), s) != cudaSuccess) return TN_ERR_CUDA;
+  if (zero_ctr && cudaMemsetAsync(unit_ctr, 0, sizeof(uint32_t), s) != cudaSuccess) return TN_ERR_CUDA;
   GemmDesc none;
   memset(&none, 0, sizeof(none));
   return launch_gemm<0, 2>(none, descs, map, nullptr, units, s, unit_ctr);

@@ -156,7 +156,16 @@ inline bool p_is_b(const ContractDesc& d) { return d.N > d.M && d.M < 128; }
 // lengths); returns the element offsets of the two runs.
 void fused_tables(const ContractDesc& d, std::vector<int32_t>* tab, int64_t* rtab_off, int64_t* ktab_off);
 
-int launch_pack(const PackJob* jobs, const PackUnit* units, int64_t nunits, cudaStream_t s);
+// One pack launch over the units of one plan or (the packs of two plans that
+// run one after another, into separate regions) two; zeroes the plans' unit
+// counters (two words each; null: none) for the GEMM launches that follow.
+struct PackLists {
+  const PackJob* jobs[2];
+  const PackUnit* units[2];
+  int64_t n[2];
+  uint32_t* ctr[2];
+};
+int launch_pack(const PackLists& pl, cudaStream_t s);
 
 // One contraction through pack + GEMM with its lists passed by value
 // (launch-only, capturable): packed blocks go to `scratch` (256-byte
@@ -200,18 +209,18 @@ __host__ __device__ inline uint32_t mn_block_chunk(int mg, int k) {
   return (uint32_t)((mg >> 3) * 8192 + (k >> 3) * 1024 + (k & 7) * 128 + (((mg & 7) ^ (k & 7)) << 4));
 }
 // unit_ctr (or null: units assigned statically): the device counter the
-// launch's CTAs claim units from (zeroed here, before the launch, on the same
-// stream).
+// launch's CTAs claim units from (zero_ctr: zeroed here, before the launch, on
+// the same stream; else zeroed by the pack before it).
 int launch_packed_gemm(const GemmDesc* descs, const int32_t* map, int64_t units, int prec, uint32_t* unit_ctr,
-                       cudaStream_t s);
+                       bool zero_ctr, cudaStream_t s);
 // The fused GEMM (BF16): units whose P is read as float32 through jobs[pjob]
 // and rounded to bf16 in shared memory, Q packed.
 int launch_fused_gemm(const GemmDesc* descs, const int32_t* map, const PackJob* jobs, int64_t units,
                       cudaStream_t s);
 // The fused TMA GEMM (BF16): units whose P tiles are boxes of its tensor map
 // (GemmDesc::tmap), loaded as float32 and rounded to bf16 in shared memory;
-// its CTAs claim units from the device counter unit_ctr (zeroed here, before
-// the launch, on the same stream).
-int launch_tma_gemm(const GemmDesc* descs, const int32_t* map, int64_t units, uint32_t* unit_ctr, cudaStream_t s);
+// its CTAs claim units from the device counter unit_ctr (zero_ctr as above).
+int launch_tma_gemm(const GemmDesc* descs, const int32_t* map, int64_t units, uint32_t* unit_ctr, bool zero_ctr,
+                    cudaStream_t s);
 
 }  // namespace tn

@@ -243,7 +243,7 @@ int tn_staged_plan_run(const tn_staged_plan* plan, void* workspace, size_t bytes
     if (cudaEventRecord(plan->ready[c], h2d) != cudaSuccess || cudaStreamWaitEvent(comp, plan->ready[c], 0) !=
                                                                     cudaSuccess)
       return TN_ERR_CUDA;
-    const int rc = tn::group_plan_run_shared(ch.plan, base + ch.list_off, ch.list_bytes, comp);
+    const int rc = tn::group_plan_run_shared(ch.plan, base + ch.list_off, ch.list_bytes, false, comp);
     if (rc != TN_OK) return rc;
     if (cudaEventRecord(plan->done[c], comp) != cudaSuccess || cudaStreamWaitEvent(d2h, plan->done[c], 0) !=
                                                                    cudaSuccess)

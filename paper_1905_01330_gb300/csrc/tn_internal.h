@@ -134,7 +134,11 @@ bool group_plan_watch_max(tn_group_plan* plan, int i, unsigned* bits);
 size_t group_plan_list_bytes(const tn_group_plan* plan);
 size_t group_plan_packed_bytes(const tn_group_plan* plan);
 int group_plan_upload_shared(const tn_group_plan* plan, void* lists, size_t bytes, void* packed, cudaStream_t s);
-int group_plan_run_shared(const tn_group_plan* plan, void* lists, size_t bytes, cudaStream_t s);
+// packed: without the pack, which group_plan_pack_two has run.
+int group_plan_run_shared(const tn_group_plan* plan, void* lists, size_t bytes, bool packed, cudaStream_t s);
+// The packs of two plans (with packed regions of their own) in one launch.
+int group_plan_pack_two(const tn_group_plan* a, void* lists_a, const tn_group_plan* b, void* lists_b,
+                        cudaStream_t s);
 
 // Step (ii) of an energy sweep with a deferred, exact rescale (mps.cu):
 //   T2[w', s', a', b] = 2^-e sum_{w,s} W'[w, w', s, s'] T1[w, a', s, b],
