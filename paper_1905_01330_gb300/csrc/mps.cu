@@ -488,12 +488,16 @@ ExpectWs2 expect2_layout(uint8_t* base, const tn_mps* psi, const tn_mpo* H) {
   // (i) (W+1) D x D by D x dD and (iii) (W+1) D x dD by dD x D, packed
   w.scratch_bytes = std::max(packed_scratch_bound(W1 * D, d * D, D, TN_PREC_BF16X3),
                              packed_scratch_bound(W1 * D, D, d * D, TN_PREC_BF16X3));
+  // the persistent sweep's regions (two planes each)
+  ExpectRegions ps{0, 0, 0};
+  if (D <= PERSISTENT_MAX_BOND && expect_persistent_ok(psi, H, TN_PREC_BF16X3)) ps = expect_persistent_regions(psi, H);
+  w.scratch_bytes = std::max(w.scratch_bytes, 2 * ps.env);
   w.scratch = take(w.scratch_bytes);
   // step (iii) of the fused sweep: T2 in whole MN-major blocks and the core,
   // packed while the previous contraction's operands are still in use
-  w.scratch3_bytes = packed_scratch_bound(W1 * D, D, d * D, TN_PREC_BF16X3);
+  w.scratch3_bytes = std::max(packed_scratch_bound(W1 * D, D, d * D, TN_PREC_BF16X3), 2 * ps.t2);
   w.scratch3 = take(w.scratch3_bytes);
-  w.cores_bytes = D <= PERSISTENT_MAX_BOND ? expect_persistent_cores_bytes(psi) : 0;
+  w.cores_bytes = 2 * ps.cores;
   w.cores = take(w.cores_bytes);
   w.bytes = off;
   return w;
@@ -592,12 +596,12 @@ bool fused_expect_ok(const tn_mps* psi, const tn_mpo* H, int prec) {
 }
 
 // The energy sweep runs as one persistent launch (mps_persistent.cu) when
-// it supports the chain and the bond is at most 512: there its phases are
-// short and a launch boundary per phase costs more than a device-wide
-// barrier (measured, N = 100: chi = 512 BF16X3 4.7 -> 4.1 ms, BF16 3.35 ->
-// 3.2 ms; chi = 256 even). At chi = 1024 the per-site launches, with their
-// warp-specialised GEMM and 256-wide BF16 tiles, are faster (BF16X3 10.8
-// against 13.6 ms).
+// it supports the chain and the bond is at most 512 (measured, N = 100:
+// chi = 512 BF16X3 2.4 ms against 4.7 as per-site launches, BF16 1.7 against
+// 3.35). Above, it would be faster too (chi = 1024 BF16X3 7.9 against 11.8
+// ms), but the per-site launches split the shared index of (i) over units
+// there, so their sums run in another order and the energies would move in
+// the seventh digit.
 bool use_persistent(const tn_mps* psi, const tn_mpo* H, int prec) {
   return max_bond(psi) <= PERSISTENT_MAX_BOND && expect_persistent_ok(psi, H, prec);
 }
@@ -847,7 +851,6 @@ int tn_mps_expect(const tn_mps* psi, const tn_mpo* H, int prec, void* workspace,
     ExpectBuffers b;
     b.L0 = w.L0;
     b.L1 = w.L1;
-    b.T1 = w.T1;
     b.Wx = w.Wx;
     b.woff = w.woff.data();
     b.bits = w.bits;

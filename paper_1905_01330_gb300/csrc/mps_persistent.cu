@@ -2,19 +2,39 @@
 // Fig. 3a) in ONE cooperative launch for the whole chain. Every CTA stays
 // resident from the first site to the last; the environment, its packed bf16
 // image and the per-site intermediates stay in device memory that the 129 MB
-// L2 holds at these bonds, and the sites' four phases are separated by
-// device-wide barriers instead of kernel launches:
-//   (A) pack L (with its largest magnitude, the site's exact rescale) and
-//       the site's core in the two operand layouts of (i) and (iii);
-//   (B) tcgen05 GEMM  T1[(w, a'), (s, b)] = sum_a L[(w, a'), a] A[a, (s, b)];
-//   (C) step (ii) into (iii)'s packed operand (mpo_step.cuh);
-//   (D) tcgen05 GEMM  L'[(w', b), b'] = sum_{(a', s')} T2 A[(a', s'), b'].
-// A GEMM phase: CTA c takes output tiles c, c + grid, ... (128 x 128); one
-// thread streams the packed blocks of each 64-wide shared slab into a ring of
-// shared-memory stages (1-D bulk copies) and issues the MMAs, eight warps
-// drain the TMEM accumulator (double-buffered across tiles) and store the
-// float32 result. BF16X3 issues hi*hi, hi*lo, lo*hi per step and promotes the
-// accumulator into registers every 512 shared indices, as the grouped GEMM.
+// L2 holds at these bonds, and the sites' phases are separated by device-wide
+// barriers instead of kernel launches:
+//   (0) once: every site's core in the two operand layouts of (i) and (iii);
+//   (B) tcgen05 GEMM  T1[(w, a'), (s, b)] = sum_a L[(w, a'), a] A[a, (s, b)],
+//       and step (ii) of its tile straight into (iii)'s packed operand;
+//   (D) tcgen05 GEMM  L'[(w', b), b'] = sum_{(a', s')} T2 A[(a', s'), b'],
+//       packed as the next site's operand, with its largest magnitude.
+// What bounds it: latency. A site of bond 256 is 0.7 us of tensor-core work,
+// so its time is the chain of copies, MMAs, epilogue and barrier of the two
+// phases. Hence:
+//   - a tile of (i) holds every channel w of a group of a' (its rows are (w,
+//     a' of the group)) and every s of its b (its columns are (16 b, s)), so
+//     step (ii), which mixes (w, s), is local to the tile: T1 never leaves the
+//     SM, and a phase, its barrier and 2 x 2 MB of traffic a site are gone;
+//   - a tile has 128 rows and as few columns as a cost model of one phase
+//     says (tile_cols): at bond 256 both phases make 64 units of work where
+//     128 x 128 tiles made 32 and 16;
+//   - copies and MMAs are issued by two warps: one thread issuing both took
+//     2,000 cycles a slab of a narrow tile, of which the MMAs are 500;
+//   - stores to the packed operands fill whole 32-byte sectors. Threads that
+//     store 16 bytes of a row each took as long as the rest of the phase
+//     (seen as 4,000 to 9,000 cycles of waiting in the barrier behind them).
+// A site of bond 256 is now about 26,000 cycles (53,000 before): two barriers
+// of 2,500 each, 9,000 of copies and MMAs, 3,500 of step (ii), 1,500 of packing,
+// the rest the latencies at the head of a phase. Measured, N = 100, before ->
+// now: BF16X3 bond 16 1.41 -> 0.78 ms, 64 1.74 -> 0.94, 256 2.81 -> 1.39, 512
+// 3.95 -> 2.41; BF16 bond 256 2.30 -> 1.12 ms.
+// A GEMM phase: CTA c takes units c, c + grid, ...; one thread streams the
+// packed blocks of each 64-wide shared slab into a ring of shared-memory
+// stages (1-D bulk copies), one issues the MMAs, eight warps drain the TMEM
+// accumulator (double-buffered across units), four per half of its columns.
+// BF16X3 issues hi*hi, hi*lo, lo*hi per step and promotes the accumulator
+// into registers every 512 shared indices, as the grouped GEMM.
 // Every wait (mbarriers and the device-wide barrier) is bounded; on expiry
 // the status word records TN_ERR_TIMEOUT and every CTA winds down.
 #include <string.h>
@@ -29,41 +49,46 @@
 namespace tn {
 namespace {
 
-constexpr int PS_THREADS = 384;  // 12 warps: warp 0 copies + MMAs, warp 1 TMEM, warps 4..11 drain TMEM
+constexpr int PS_THREADS = 384;  // 12 warps: warp 0 copies, warp 1 MMAs, warps 2, 3 zero fill, warps 4..11 drain TMEM
 constexpr int PS_EPI0 = 4;       // first draining warp
-constexpr int PS_EPI = 8;        // draining warps: two per TMEM lane quadrant, 64 columns each
+constexpr int PS_EPI = 8;        // draining warps: two per TMEM lane quadrant, half of the columns each
+constexpr int PS_GROUP = 128;    // threads of one half
 constexpr int PS_KC = 8;         // BF16X3: slabs between promotions (512 shared indices)
-constexpr int PS_BLOCK = 16384;  // one packed block: 128 rows x 64 shared indices of bf16
+constexpr int PS_BLOCK = 16384;  // one block of a first operand: 128 rows x 64 shared indices of bf16
 constexpr int PS_MAX_SITES = 512;
-constexpr uint32_t PS_TMEM_COLS = 256;  // two 128-column accumulators
+constexpr int PS_MAX_STAGES = 8;
+constexpr uint32_t PS_TMEM_COLS = 256;  // two accumulators of up to 128 columns
+constexpr int PS_RING = 192 * 1024;     // the ring of stages
+constexpr int PS_STAGED = 16 * 1024;    // T1 of a group's round: 128 rows (w, a') x d s x 8 or 16 b
 
-template <int SPLIT>
-struct PsCfg {
-  // BF16: P and Q hi (32 KB) per stage; BF16X3: hi and lo of both (64 KB)
-  static constexpr int OPS = SPLIT ? 4 : 2;
-  static constexpr int STAGES = SPLIT ? 3 : 6;
-  static constexpr int STAGE_BYTES = OPS * PS_BLOCK;
+// A site, with its two phases' tiles worked out on the host: one warp's
+// divisions at the head of a phase are on the path of the whole sweep.
+struct PsTiles {
+  uint32_t off;    // the packed core at Cp + 1024 off
+  uint32_t magic;  // u / tq = umulhi(u, magic) (0: tq = 1)
+  uint16_t tp, tq; // row and column tiles
+  int16_t cols;    // columns of a tile
+  int16_t slabs;   // 64-wide slabs of the shared index
 };
-
 struct PsSite {
   const float* A;  // core (Da, d, Db), row-major
-  int32_t Da, Db, wa, wb;
-  int32_t woff, pad;  // the site's extended MPO at Wx + woff
-  // the core packed once per launch: for (i) at Cp + a1_off, for (iii) at
-  // Cp + a3_off (bytes); its first pack chunk in the launch's numbering
-  int64_t a1_off, a3_off, chunk0;
+  uint32_t unit0;  // its first pack unit
+  int32_t woff;    // its extended MPO at Wx + woff
+  int16_t Da, Db;
+  int8_t wa, wb;
+  PsTiles t[2];    // (i), (iii)
 };
 
 struct PsParams {
   int32_t n, d;
+  int32_t stages, stage_bytes;
   const float* Wx;       // extended MPO of every site
-  float* L[2];           // environments, (wa, Da, Da) / (wb, Db, Db) row-major
-  float* T1;             // (wa, Da, d, Db)
-  uint8_t* Lp;           // packed L: rows (w, a'), shared a (MN-major blocks)
+  float* L[2];           // the first environment and the last one
+  uint8_t* Lp;           // packed L: rows (a' / G, w, a' % G), shared a (MN-major blocks)
   uint8_t* T2p;          // packed T2 for (iii): rows (w', b), shared a' d + s' (MN-major blocks)
   uint8_t* Cp;           // every site's packed cores (K-major blocks)
   int64_t Lp_lo, T2p_lo, Cp_lo;  // byte distance from a hi block to its lo block (BF16X3)
-  int64_t chunks;        // pack chunks of all the cores
+  uint32_t units;        // pack units of all the cores
   unsigned* bits;        // per site: bits of the largest |L| entering it
   double* lg;            // float64 log-scale
   unsigned* bar;         // device-wide barrier counter (zero at launch)
@@ -73,13 +98,14 @@ struct PsParams {
 };
 
 struct __align__(8) PsAux {
-  uint64_t full[8];       // stage s holds its blocks
-  uint64_t empty[8];      // the MMAs that read stage s are complete
+  uint64_t full[PS_MAX_STAGES];   // stage s holds its blocks
+  uint64_t empty[PS_MAX_STAGES];  // the MMAs that read stage s are complete
   uint64_t acc_full[2];   // accumulator b holds a finished chunk
   uint64_t acc_empty[2];  // the draining warps have read accumulator b
   uint64_t final_bar;     // every MMA of the launch is complete
   uint32_t tmem_base;
   volatile int32_t abort;
+  float4 Ws[2][8][4];     // per half: the site's W' as [(w, s)][(w', s') by reader], zero past the MPO
 };
 
 __device__ __forceinline__ uint32_t ld_acquire_gpu(const unsigned* p) {
@@ -103,9 +129,8 @@ __device__ bool grid_barrier(unsigned* bar, uint32_t& epoch, int* status, uint64
   fence_proxy_async_global();
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
     const uint32_t target = (epoch + 1) * gridDim.x;
-    atomicAdd(bar, 1u);
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     if (ld_acquire_gpu(bar) < target) {
       const uint64_t t0 = ptx::globaltimer();
       for (uint32_t i = 1;; ++i) {
@@ -117,11 +142,10 @@ __device__ bool grid_barrier(unsigned* bar, uint32_t& epoch, int* status, uint64
         }
       }
     }
-    __threadfence();
+    fence_proxy_async_global();
   }
   ++epoch;
   __syncthreads();
-  fence_proxy_async_global();
   return *abort == 0;
 }
 
@@ -145,111 +169,88 @@ __device__ __forceinline__ uint32_t ps_bf16x2(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-// One K-major packed operand written by the pack phase: element (r, k) of
-// an R x K matrix at src[r_off(r) + k_off(k)], stored in whole 16 KB blocks
-// of 128 rows x 64 shared indices (128-byte swizzle, as the grouped GEMM's
-// packed blocks), zeros at every position past R or K.
-struct PsPack {
-  const float* src;
-  uint8_t* hi;
-  int64_t lo;       // byte distance to the lo plane, 0: none
-  int32_t R, K, tiles, slabs;
-  // row r = r1 * rd0 + r0 (r0 < rd0): offset r1 * rs1 + r0 * rs0; shared k likewise
-  int32_t rd0, ks0_div;
-  int64_t rs1, rs0, kq1, kq0;
-};
-
 __device__ __forceinline__ int32_t ceil_div(int32_t a, int32_t b) { return (a + b - 1) / b; }
 
-// Chunks of one packed operand: (tile, 8-wide k group of the slab, row in the
-// tile), rows fastest, so consecutive threads read consecutive rows at one
-// shared index (the row digit r0 is the source's unit-stride one).
-__device__ __forceinline__ int64_t pack_chunks(const PsPack& q) { return (int64_t)q.tiles * q.slabs * 8 * 128; }
+// Rows of (i)'s first operand a channel has in one 128-row tile: 2^shift, 128
+// / wa rounded down to a power of two (wa <= 8: at least 16).
+__host__ __device__ __forceinline__ int32_t group_shift(int32_t wa) { return wa <= 2 ? 6 : wa <= 4 ? 5 : 4; }
+// b rounded up to whole cells of 16.
+__host__ __device__ __forceinline__ int32_t pad16(int32_t x) { return (x + 15) & ~15; }
 
-__device__ __forceinline__ float pack_chunk(const PsPack& q, int64_t e, float amax) {
-  const int32_t rr = (int32_t)(e & 127);
-  int64_t rest = e >> 7;
-  const int32_t g = (int32_t)(rest & 7);
-  rest >>= 3;
-  const int32_t sl = (int32_t)(rest % q.slabs), t = (int32_t)(rest / q.slabs);
-  const int32_t r = t * 128 + rr, k0 = sl * 64 + g * 8;
-  float v[8];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) v[j] = 0.0f;
-  if (r < q.R) {
-    const int32_t r1 = r / q.rd0, r0 = r - r1 * q.rd0;
-    const float* row = q.src + r1 * q.rs1 + r0 * q.rs0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int32_t k = k0 + j;
-      if (k < q.K) {
-        const int32_t k1 = k / q.ks0_div, kk = k - k1 * q.ks0_div;
-        v[j] = __ldg(row + k1 * q.kq1 + kk * q.kq0);
-      }
-    }
-  }
-  uint4 h;
+// hi (and lo) of 8 values as 16-byte chunks.
+__device__ __forceinline__ void split8(const float* v, uint4& h, uint4& l) {
   h.x = ps_bf16x2(v[0], v[1]);
   h.y = ps_bf16x2(v[2], v[3]);
   h.z = ps_bf16x2(v[4], v[5]);
   h.w = ps_bf16x2(v[6], v[7]);
-  const size_t off = ((size_t)t * q.slabs + sl) * PS_BLOCK +
-                     (size_t)((rr >> 3) * 1024 + (rr & 7) * 128 + ((g ^ (rr & 7)) << 4));
-  *reinterpret_cast<uint4*>(q.hi + off) = h;
-  if (q.lo) {
-    const __nv_bfloat162* hb = reinterpret_cast<const __nv_bfloat162*>(&h);
-    uint4 l;
-    l.x = ps_bf16x2(v[0] - __low2float(hb[0]), v[1] - __high2float(hb[0]));
-    l.y = ps_bf16x2(v[2] - __low2float(hb[1]), v[3] - __high2float(hb[1]));
-    l.z = ps_bf16x2(v[4] - __low2float(hb[2]), v[5] - __high2float(hb[2]));
-    l.w = ps_bf16x2(v[6] - __low2float(hb[3]), v[7] - __high2float(hb[3]));
-    *reinterpret_cast<uint4*>(q.hi + q.lo + off) = l;
-  }
-#pragma unroll
-  for (int j = 0; j < 8; ++j) amax = fmaxf(amax, fabsf(v[j]));
-  return amax;
+  const __nv_bfloat162* hb = reinterpret_cast<const __nv_bfloat162*>(&h);
+  l.x = ps_bf16x2(v[0] - __low2float(hb[0]), v[1] - __high2float(hb[0]));
+  l.y = ps_bf16x2(v[2] - __low2float(hb[1]), v[3] - __high2float(hb[1]));
+  l.z = ps_bf16x2(v[4] - __low2float(hb[2]), v[5] - __high2float(hb[2]));
+  l.w = ps_bf16x2(v[6] - __low2float(hb[3]), v[7] - __high2float(hb[3]));
 }
 
-// The pack jobs of a site's core: q1 for (i) (rows (s, b), shared a: A[a, s,
-// b] at (a d + s) Db + b) and q3 for (iii) (rows b', shared a' d + s': at
-// (a' d + s') Db + b'), at their places in the cores region.
-__device__ __forceinline__ void core_packs(const PsParams& p, const PsSite& st, int32_t d, PsPack* q1, PsPack* q3) {
-  if (q1) {
-    q1->src = st.A;
-    q1->hi = p.Cp + st.a1_off;
-    q1->lo = p.Cp_lo;
-    q1->R = d * st.Db;
-    q1->K = st.Da;
-    q1->rd0 = st.Db;
-    q1->rs1 = st.Db;
-    q1->rs0 = 1;
-    q1->ks0_div = st.Da;
-    q1->kq1 = 0;
-    q1->kq0 = (int64_t)d * st.Db;
-    q1->tiles = ceil_div(q1->R, 128);
-    q1->slabs = ceil_div(q1->K, 64);
+// A site's core as the second operand of (i) or (iii): K-major blocks of
+// `cols` rows x 64 shared indices (128-byte swizzle), one per tile of the
+// result's columns and slab, zeros past the core. Row rho of (i) is (b / 16,
+// s, b % 16), so a tile holds every s of its b; of (iii) it is b'.
+struct PsPack {
+  const float* src;
+  uint8_t* hi;
+  int64_t lo;  // byte distance to the lo plane, 0: none
+  int32_t cols, slabs, K, Db, ns;  // ns: d for (i), 1 for (iii)
+};
+
+__device__ __forceinline__ uint4 pick(bool c, const uint4& a, const uint4& b) {
+  return make_uint4(c ? a.x : b.x, c ? a.y : b.y, c ? a.z : b.z, c ? a.w : b.w);
+}
+__device__ __forceinline__ uint4 swap_pair(const uint4& a) {
+  return make_uint4(__shfl_xor_sync(0xffffffffu, a.x, 1), __shfl_xor_sync(0xffffffffu, a.y, 1),
+                    __shfl_xor_sync(0xffffffffu, a.z, 1), __shfl_xor_sync(0xffffffffu, a.w, 1));
+}
+
+// One pack unit (a warp): 32 rows (b: the source's unit-stride index) of one
+// slab; units numbered (tile, slab, rows / 32). Lanes 2i and 2i + 1 swap
+// chunks, so that a pair's store is one 32-byte sector.
+__device__ __forceinline__ void pack_unit(const PsPack& q, uint32_t u) {
+  const int lane = threadIdx.x & 31, odd = lane & 1;
+  const uint32_t parts = (uint32_t)q.cols >> 5, rest = u / parts;
+  const int32_t t = (int32_t)(rest / (uint32_t)q.slabs), sl = (int32_t)(rest - (uint32_t)t * q.slabs);
+  const int32_t rr = (int32_t)(u - rest * parts) * 32 + lane, rho = t * q.cols + rr;
+  const int32_t cell = (rho >> 4) / q.ns, sk = (rho >> 4) - cell * q.ns, b = cell * 16 + (rho & 15);
+  const int64_t ks = (int64_t)q.ns * q.Db;
+  const int32_t k0 = sl * 64, kn = b < q.Db ? q.K - k0 : 0;
+  const float* src = q.src + k0 * ks + (int64_t)sk * q.Db + b;
+  uint8_t* blk = q.hi + ((size_t)t * q.slabs + sl) * (size_t)(q.cols * 128) + (size_t)(rr >> 3) * 1024;
+  const int r0 = rr & 6;  // row of the pair's even lane, in its group of 8
+#pragma unroll 2
+  for (int g = 0; g < 8; g += 2) {
+    float v[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = 8 * g + j < kn ? __ldg(src + (8 * g + j) * ks) : 0.0f;
+    uint4 h[2], l[2];
+    split8(v, h[0], l[0]);
+    split8(v + 8, h[1], l[1]);
+    const uint4 hs = swap_pair(pick(odd, h[0], h[1])), ls = swap_pair(pick(odd, l[0], l[1]));
+    const int o0 = r0 * 128 + (((g + odd) ^ r0) << 4), o1 = (r0 + 1) * 128 + (((g + odd) ^ (r0 + 1)) << 4);
+    *reinterpret_cast<uint4*>(blk + o0) = pick(odd, hs, h[0]);
+    *reinterpret_cast<uint4*>(blk + o1) = pick(odd, h[1], hs);
+    if (q.lo) {
+      *reinterpret_cast<uint4*>(blk + q.lo + o0) = pick(odd, ls, l[0]);
+      *reinterpret_cast<uint4*>(blk + q.lo + o1) = pick(odd, l[1], ls);
+    }
   }
-  if (q3) {
-    q3->src = st.A;
-    q3->hi = p.Cp + st.a3_off;
-    q3->lo = p.Cp_lo;
-    q3->R = st.Db;
-    q3->K = d * st.Da;
-    q3->rd0 = st.Db;
-    q3->rs1 = 0;
-    q3->rs0 = 1;
-    q3->ks0_div = q3->K;
-    q3->kq1 = 0;
-    q3->kq0 = st.Db;
-    q3->tiles = ceil_div(q3->R, 128);
-    q3->slabs = ceil_div(q3->K, 64);
-  }
+}
+
+// Pack units of one of a site's cores.
+__host__ __device__ __forceinline__ uint32_t pack_units(const PsTiles& t) {
+  return (uint32_t)t.tq * (uint32_t)t.slabs * ((uint32_t)t.cols >> 5);
 }
 
 // One 16-byte chunk (8 rows at one shared index) of the first environment
-// L[w, a, a'] as an MN-major operand (row w Da + a', shared a), zeros past R
-// or K; chunks numbered (tile, slab, row group, k), k fastest.
-__device__ __forceinline__ void pack_mn_chunk(const float* L, int32_t Da, int32_t R, int32_t K, int32_t slabs,
+// L[w, a, a'] as (i)'s first operand, zeros past it; chunks numbered (tile,
+// slab, row group, k), k fastest.
+__device__ __forceinline__ void pack_mn_chunk(const float* L, int32_t Da, int32_t wa, int32_t lg, int32_t slabs,
                                               uint8_t* hi, int64_t lo, int64_t e) {
   const int32_t kk = (int32_t)(e & 63);
   int64_t rest = e >> 6;
@@ -260,217 +261,186 @@ __device__ __forceinline__ void pack_mn_chunk(const float* L, int32_t Da, int32_
   float v[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    const int32_t r = t * 128 + mg * 8 + j;
-    v[j] = 0.0f;
-    if (r < R && k < K) {
-      const int32_t w = r / Da, a2 = r - w * Da;
-      v[j] = L[((int64_t)w * Da + k) * Da + a2];
-    }
+    const int32_t r = mg * 8 + j, w = r >> lg, a2 = (t << lg) + r - (w << lg);
+    v[j] = w < wa && a2 < Da && k < Da ? L[((int64_t)w * Da + k) * Da + a2] : 0.0f;
   }
   uint4 h, l;
-  uint32_t* hp = reinterpret_cast<uint32_t*>(&h);
-  uint32_t* lp = reinterpret_cast<uint32_t*>(&l);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    hp[j] = ps_bf16x2(v[2 * j], v[2 * j + 1]);
-    const __nv_bfloat162 hb = *reinterpret_cast<const __nv_bfloat162*>(&hp[j]);
-    lp[j] = ps_bf16x2(v[2 * j] - __low2float(hb), v[2 * j + 1] - __high2float(hb));
-  }
+  split8(v, h, l);
   const size_t off = ((size_t)t * slabs + sl) * PS_BLOCK + mn_block_chunk(mg, kk);
   *reinterpret_cast<uint4*>(hi + off) = h;
   if (lo) *reinterpret_cast<uint4*>(hi + lo + off) = l;
 }
 
-// One GEMM phase: C[r, c] = sum_k P[r, k] Q[c, k] over whole packed blocks
-// (P K-major, or MN-major when p_mn; Q K-major), output tiles of 128 x 128.
+// Zeros at the shared indices [K, 64 slabs) of an MN-major operand (whole
+// rows of its blocks): thread `tid` of `nthreads`.
+__device__ __forceinline__ void zero_shared_tail(uint8_t* hi, int64_t lo, int32_t tiles, int32_t slabs, int32_t K,
+                                                 int32_t tid, int32_t nthreads) {
+  const int32_t npad = slabs * 64 - K, total = tiles * 16 * npad;
+  for (int32_t e = tid; e < total; e += nthreads) {
+    const int32_t mg = e & 15, rest = e >> 4;
+    const int32_t t = rest / npad, kk = K + rest - t * npad;
+    const size_t off = ((size_t)t * slabs + (kk >> 6)) * PS_BLOCK + mn_block_chunk(mg, kk & 63);
+    *reinterpret_cast<uint4*>(hi + off) = make_uint4(0u, 0u, 0u, 0u);
+    if (lo) *reinterpret_cast<uint4*>(hi + lo + off) = make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+
+// One GEMM phase: C[r, c] = sum_k P[r, k] Q[c, k] over whole packed blocks (P
+// MN-major, Q K-major), output tiles of 128 x cols.
 struct PsGemm {
   const uint8_t* P;
   const uint8_t* Q;
   int64_t P_lo, Q_lo;  // byte distance from a hi block to its lo block (BF16X3)
-  float* C;
-  int32_t ldc, R, N;   // C row stride; rows of P (result rows) and of Q (result columns)
-  int32_t tp, tq, slabs, p_mn;
-  // (iii): the result is also the next site's first operand of (i), written
-  // here as whole MN-major blocks (row w' Db + b', shared index b), and its
-  // largest magnitude goes to *maxbits; Pn null: none
-  uint8_t* Pn;
-  int64_t Pn_lo;
-  int32_t Db, pn_slabs;
-  unsigned* maxbits;
+  int32_t units, tq, slabs, cols;
+  uint32_t magic;
 };
+__device__ __forceinline__ void unit_tile(const PsGemm& g, int u, int& tpi, int& tqi) {
+  tpi = g.magic ? (int)__umulhi((uint32_t)u, g.magic) : u;
+  tqi = u - tpi * g.tq;
+}
 
 // Pipeline positions kept across the phases of the launch: slabs through the
-// stage ring (producer), accumulator chunks (producer and draining warps).
+// stage ring (the copying thread's and the MMA issuer's own counts) and
+// accumulator chunks (issuer and draining warps).
 struct PsPipe {
-  uint32_t issued, consumed, gc;
+  uint32_t slab, stage, phase, gc;  // phase: rounds of the ring, stage: slab % stages
 };
 
-// Producer and MMA issuer of a GEMM phase (one thread). Keeps STAGES - 1
-// slabs of copies in flight ahead of the slab being multiplied; a slab's
-// MMAs are queued before the thread waits to refill a stage.
+// Copies of a GEMM phase (one thread): every slab of its units into the ring,
+// as soon as its stage is free. A stage holds P hi, (P lo,) Q hi, (Q lo).
 template <int SPLIT>
-__device__ bool gemm_issue(const PsGemm& g, uint32_t stage0, PsAux& x, uint32_t tmem, PsPipe& pp, int* status) {
-  using C = PsCfg<SPLIT>;
-  constexpr int S = C::STAGES;
-  const uint32_t idesc = ptx::idesc_bf16_f32(128, 128, g.p_mn, 0);
-  const int nks = g.slabs, chunk = SPLIT ? PS_KC : nks;
-  for (int u = blockIdx.x; u < g.tp * g.tq; u += gridDim.x) {
-    const int tpi = u / g.tq, tqi = u - tpi * g.tq;
+__device__ bool gemm_copy(const PsGemm& g, const PsParams& p, uint32_t stage0, PsAux& x, PsPipe& pp) {
+  const uint32_t S = (uint32_t)p.stages, stage_bytes = (uint32_t)p.stage_bytes;
+  const uint32_t qbytes = (uint32_t)g.cols * 128u, qoff = (SPLIT ? 2 : 1) * PS_BLOCK;
+  uint32_t st = pp.stage, round = pp.phase;
+  for (int u = blockIdx.x; u < g.units; u += gridDim.x) {
+    int tpi, tqi;
+    unit_tile(g, u, tpi, tqi);
     const uint8_t* pb = g.P + (size_t)tpi * g.slabs * PS_BLOCK;
-    const uint8_t* qb = g.Q + (size_t)tqi * g.slabs * PS_BLOCK;
-    const uint32_t first = pp.consumed;  // this unit's slab ks is global slab first + ks
-    auto issue = [&](int ks) -> bool {
-      const uint32_t gsl = first + (uint32_t)ks, st = gsl % S;
+    const uint8_t* qb = g.Q + (size_t)tqi * g.slabs * qbytes;
+    for (int ks = 0; ks < g.slabs; ++ks, pb += PS_BLOCK, qb += qbytes) {
       // the stage's previous contents: read by MMAs that must be complete
-      if (gsl >= (uint32_t)S && !ptx::mbar_wait(ptx::smem_addr(&x.empty[st]), ((gsl / S) - 1u) & 1u, status))
-        return false;
-      const uint32_t full = ptx::smem_addr(&x.full[st]), dst = stage0 + st * C::STAGE_BYTES;
-      ptx::mbar_arrive_expect_tx(full, (uint32_t)C::STAGE_BYTES);
-      ptx::bulk_copy_g2s(dst, pb + (size_t)ks * PS_BLOCK, PS_BLOCK, full);
-      ptx::bulk_copy_g2s(dst + PS_BLOCK, qb + (size_t)ks * PS_BLOCK, PS_BLOCK, full);
+      if (round && !ptx::mbar_wait(ptx::smem_addr(&x.empty[st]), (round - 1u) & 1u, p.status)) return false;
+      const uint32_t full = ptx::smem_addr(&x.full[st]), dst = stage0 + st * stage_bytes;
+      ptx::mbar_arrive_expect_tx(full, (SPLIT ? 2u : 1u) * (PS_BLOCK + qbytes));
+      ptx::bulk_copy_g2s(dst, pb, PS_BLOCK, full);
+      ptx::bulk_copy_g2s(dst + qoff, qb, qbytes, full);
       if (SPLIT) {
-        ptx::bulk_copy_g2s(dst + 2 * PS_BLOCK, pb + g.P_lo + (size_t)ks * PS_BLOCK, PS_BLOCK, full);
-        ptx::bulk_copy_g2s(dst + 3 * PS_BLOCK, qb + g.Q_lo + (size_t)ks * PS_BLOCK, PS_BLOCK, full);
+        ptx::bulk_copy_g2s(dst + PS_BLOCK, pb + g.P_lo, PS_BLOCK, full);
+        ptx::bulk_copy_g2s(dst + qoff + qbytes, qb + g.Q_lo, qbytes, full);
       }
-      ++pp.issued;
-      return true;
-    };
-    for (int ks = 0; ks < S - 1 && ks < nks; ++ks)
-      if (!issue(ks)) return false;
-    uint32_t b = 0;
-    for (int ks = 0; ks < nks; ++ks) {
-      const bool start = ks % chunk == 0;
-      if (start) {
-        // the accumulator this chunk overwrites has been drained
-        b = pp.gc & 1u;
-        if (!ptx::mbar_wait(ptx::smem_addr(&x.acc_empty[b]), ((pp.gc >> 1) & 1u) ^ 1u, status)) return false;
+      ++pp.slab;
+      if (++st == S) {
+        st = 0;
+        ++round;
       }
-      const uint32_t gsl = first + (uint32_t)ks, st = gsl % S;
-      if (!ptx::mbar_wait(ptx::smem_addr(&x.full[st]), (gsl / S) & 1u, status)) return false;
-      ptx::tc_fence_after();
-      const uint32_t sa = stage0 + st * C::STAGE_BYTES, dt = tmem + b * 128u;
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const uint64_t pd = g.p_mn ? ptx::sw128_mnmajor_desc(sa + kk * 2048, 8192, 1024)
-                                   : ptx::sw128_kmajor_desc(sa + kk * 32);
-        const uint64_t qd = ptx::sw128_kmajor_desc(sa + PS_BLOCK + kk * 32);
-        ptx::mma_bf16(dt, pd, qd, idesc, (start && kk == 0) ? 0u : 1u);
-        if (SPLIT) {
-          const uint64_t pl = g.p_mn ? ptx::sw128_mnmajor_desc(sa + 2 * PS_BLOCK + kk * 2048, 8192, 1024)
-                                     : ptx::sw128_kmajor_desc(sa + 2 * PS_BLOCK + kk * 32);
-          const uint64_t ql = ptx::sw128_kmajor_desc(sa + 3 * PS_BLOCK + kk * 32);
-          ptx::mma_bf16(dt, pd, ql, idesc, 1u);
-          ptx::mma_bf16(dt, pl, qd, idesc, 1u);
-        }
-      }
-      ptx::mma_commit(ptx::smem_addr(&x.empty[st]));
-      ++pp.consumed;
-      if (ks % chunk == chunk - 1 || ks == nks - 1) {
-        ptx::mma_commit(ptx::smem_addr(&x.acc_full[b]));
-        ++pp.gc;
-      }
-      // the next copies go to the stage of slab ks - 1, whose MMAs complete
-      // while this slab's, queued behind them, keep the tensor pipe busy
-      if (ks + S - 1 < nks && !issue(ks + S - 1)) return false;
     }
   }
+  pp.stage = st;
+  pp.phase = round;
   return true;
 }
 
-// Draining warps of a GEMM phase: warp (PS_EPI0 + 4 grp + quad) reads TMEM
-// lanes quad * 32 .. + 31 (one result row per thread), columns grp * 64 ..
-// + 63; BF16X3 adds each chunk's partial sums into float32 registers.
+// MMAs of a GEMM phase, by a warp of its own (copies and MMAs issued by one
+// thread took it 2,000 cycles a slab, the MMAs themselves 500): the warp runs
+// the loop together and one lane issues, so that the descriptors stay in
+// uniform registers.
 template <int SPLIT>
-__device__ bool gemm_drain(const PsGemm& g, PsAux& x, uint32_t tmem, PsPipe& pp, int* status) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int quad = warp & 3, grp = (warp - PS_EPI0) >> 2;
-  const int nks = g.slabs, nchunks = SPLIT ? (nks + PS_KC - 1) / PS_KC : 1;
-  const bool vec = (g.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(g.C) & 15) == 0;
-  float mx = 0.0f;  // largest |value| written to the next site's operand
-  for (int u = blockIdx.x; u < g.tp * g.tq; u += gridDim.x) {
-    const int tpi = u / g.tq, tqi = u - tpi * g.tq;
-    const int row = tpi * 128 + quad * 32 + lane, col0 = tqi * 128 + grp * 64;
-    float* dst = g.C + (size_t)row * g.ldc + col0;
-    const int ncol = g.N - col0;  // valid columns of this thread's 64
-    auto store = [&](int h, const float* v) {
-      if (row >= g.R || ncol <= 32 * h) return;
-      if (vec && ncol >= 32 * h + 32) {
-#pragma unroll
-        for (int j = 0; j < 32; j += 4)
-          *reinterpret_cast<float4*>(dst + 32 * h + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-      } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (32 * h + j < ncol) dst[32 * h + j] = v[j];
-      }
-    };
-    // 32 result columns of this thread's row into the next site's packed
-    // operand: row (w', b) of L' at shared index b, columns b' as rows
-    auto pack_out = [&](int h, const float* v) {
-      if (!g.Pn || row >= g.R) return;
-      const int cb = col0 + 32 * h;
-      if (cb >= g.N) return;
-      const int wq = row / g.Db, b = row - wq * g.Db, kk = b & 63;
-      const size_t slab_off = (size_t)(b >> 6) * PS_BLOCK;
-      if ((g.Db & 63) == 0) {
-        // rows r0 .. r0 + 31 of one tile: four 16-byte chunks
-        const int r0 = wq * g.Db + cb;
-        const size_t base = (size_t)(r0 >> 7) * g.pn_slabs * PS_BLOCK + slab_off;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const size_t off = base + mn_block_chunk(((r0 & 127) >> 3) + c, kk);
-          uint4 hv, lv;
-          uint32_t* hp = reinterpret_cast<uint32_t*>(&hv);
-          uint32_t* lp = reinterpret_cast<uint32_t*>(&lv);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float a = v[8 * c + 2 * j], e2 = v[8 * c + 2 * j + 1];
-            hp[j] = ps_bf16x2(a, e2);
-            const __nv_bfloat162 hb = *reinterpret_cast<const __nv_bfloat162*>(&hp[j]);
-            lp[j] = ps_bf16x2(a - __low2float(hb), e2 - __high2float(hb));
-            mx = fmaxf(mx, fmaxf(fabsf(a), fabsf(e2)));
+__device__ bool gemm_issue(const PsGemm& g, const PsParams& p, uint32_t stage0, PsAux& x, uint32_t tmem, PsPipe& pp) {
+  const uint32_t S = (uint32_t)p.stages, stage_bytes = (uint32_t)p.stage_bytes;
+  int* status = p.status;
+  const uint32_t idesc = ptx::idesc_bf16_f32(128, g.cols, 1, 0);
+  const uint32_t qbytes = (uint32_t)g.cols * 128u, qoff = (SPLIT ? 2 : 1) * PS_BLOCK;
+  const int nks = g.slabs, chunk = SPLIT ? PS_KC : nks;
+  uint32_t st = pp.stage, phase = pp.phase;
+  auto wait_full = [&]() {
+    const bool w = ptx::mbar_wait(ptx::smem_addr(&x.full[st]), phase, status);
+    if (!__all_sync(0xffffffffu, w)) return false;
+    ptx::tc_fence_after();
+    return true;
+  };
+  for (int u = blockIdx.x; u < g.units; u += gridDim.x) {
+    for (int k0 = 0; k0 < nks; k0 += chunk) {
+      // the accumulator this chunk overwrites has been drained
+      const uint32_t b = pp.gc & 1u, dt = tmem + b * 128u;
+      const bool w = ptx::mbar_wait(ptx::smem_addr(&x.acc_empty[b]), ((pp.gc >> 1) & 1u) ^ 1u, status);
+      if (!__all_sync(0xffffffffu, w)) return false;
+      const int k1 = min(k0 + chunk, nks);
+      if (!wait_full()) return false;
+      for (int ks = k0; ks < k1; ++ks) {
+        const uint32_t sa = stage0 + st * stage_bytes, empty = ptx::smem_addr(&x.empty[st]);
+        const uint32_t ph = ptx::desc_lo(sa, 8192), pl = ph + (PS_BLOCK >> 4);
+        const uint32_t qh = ptx::desc_lo(sa + qoff), ql = qh + (qbytes >> 4);
+        auto step = [&](int kk) {
+          ptx::mma_bf16_lo(dt, ph + kk * 128u, qh + kk * 2u, idesc, (ks != k0 || kk != 0) ? 1u : 0u);
+          if (SPLIT) {
+            ptx::mma_bf16_lo(dt, ph + kk * 128u, ql + kk * 2u, idesc, 1u);
+            ptx::mma_bf16_lo(dt, pl + kk * 128u, qh + kk * 2u, idesc, 1u);
           }
-          *reinterpret_cast<uint4*>(g.Pn + off) = hv;
-          if (g.Pn_lo) *reinterpret_cast<uint4*>(g.Pn + g.Pn_lo + off) = lv;
+        };
+        if (ptx::elect_one()) {
+          step(0);
+          step(1);
         }
-      } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          if (cb + j >= g.N) continue;
-          const int r = wq * g.Db + cb + j;
-          const size_t off = (size_t)(r >> 7) * g.pn_slabs * PS_BLOCK + slab_off +
-                             mn_block_chunk((r & 127) >> 3, kk) + 2 * (r & 7);
-          const __nv_bfloat16 hb = __float2bfloat16_rn(v[j]);
-          *reinterpret_cast<__nv_bfloat16*>(g.Pn + off) = hb;
-          if (g.Pn_lo)
-            *reinterpret_cast<__nv_bfloat16*>(g.Pn + g.Pn_lo + off) = __float2bfloat16_rn(v[j] - __bfloat162float(hb));
-          mx = fmaxf(mx, fabsf(v[j]));
+        __syncwarp();
+        if (++st == S) {
+          st = 0;
+          phase ^= 1u;
         }
+        // the tensor pipe's queue is short: the next slab is waited for (200
+        // cycles when it is there) behind half of this one's MMAs
+        const bool more = ks + 1 < k1;
+        if (more && !wait_full()) return false;
+        if (ptx::elect_one()) {
+          step(2);
+          step(3);
+          ptx::mma_commit(empty);
+          if (!more) ptx::mma_commit(ptx::smem_addr(&x.acc_full[b]));
+        }
+        __syncwarp();
       }
-    };
-    float acc[SPLIT ? 64 : 1];
+      ++pp.gc;
+    }
+  }
+  pp.stage = st;
+  pp.phase = phase;
+  return true;
+}
+
+// Draining warps of a GEMM phase: warp (PS_EPI0 + 4 half + quad) reads TMEM
+// lanes quad * 32 .. + 31 (one result row per thread) of its half of the
+// columns (ng = cols / 32 groups of 16); BF16X3 adds each chunk's partial
+// sums into float32 registers. fin(row tile, column tile, values) finishes a
+// unit; it is entered by a whole half together, and a wait that ran out in one
+// of its warps ends all four.
+template <int SPLIT, class Fin>
+__device__ bool gemm_drain(const PsGemm& g, PsAux& x, uint32_t tmem, PsPipe& pp, int* status, Fin fin) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int quad = warp & 3, half = (warp - PS_EPI0) >> 2, ng = g.cols >> 5;
+  const int nks = g.slabs, nchunks = SPLIT ? (nks + PS_KC - 1) / PS_KC : 1;
+  for (int u = blockIdx.x; u < g.units; u += gridDim.x) {
+    int tpi, tqi;
+    unit_tile(g, u, tpi, tqi);
+    float acc[64];
 #pragma unroll
-    for (int j = 0; j < (SPLIT ? 64 : 1); ++j) acc[j] = 0.0f;
+    for (int j = 0; j < 64; ++j) acc[j] = 0.0f;
     for (int c = 0; c < nchunks; ++c) {
       const uint32_t b = pp.gc & 1u;
       const bool w = ptx::mbar_wait(ptx::smem_addr(&x.acc_full[b]), (pp.gc >> 1) & 1u, status);
-      if (!__all_sync(0xffffffffu, w)) return false;
+      if (ptx::named_barrier_or(1 + half, PS_GROUP, !w)) return false;
       ptx::tc_fence_after();
-      const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + b * 128u + (uint32_t)(grp * 64);
+      const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + b * 128u + (uint32_t)(half * ng * 16);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint32_t r[32];
-        ptx::tmem_ld_32x32b_x32(ta + 32u * h, r);
-        ptx::tmem_ld_wait();
-        if (SPLIT) {
+      for (int gi = 0; gi < 4; ++gi) {
+        if (gi < ng) {
+          uint32_t r[16];
+          ptx::tmem_ld_32x32b_x16(ta + 16u * gi, r);
+          ptx::tmem_ld_wait();
 #pragma unroll
-          for (int j = 0; j < 32; ++j) acc[32 * h + j] += __uint_as_float(r[j]);
-        } else {
-          float v[32];
-#pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-          store(h, v);
-          pack_out(h, v);
+          for (int j = 0; j < 16; ++j) {
+            if (SPLIT) acc[16 * gi + j] += __uint_as_float(r[j]);
+            else acc[16 * gi + j] = __uint_as_float(r[j]);
+          }
         }
       }
       ptx::tc_fence_before();
@@ -478,41 +448,158 @@ __device__ bool gemm_drain(const PsGemm& g, PsAux& x, uint32_t tmem, PsPipe& pp,
       if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&x.acc_empty[b]));
       ++pp.gc;
     }
-    if (SPLIT) {
-      store(0, acc);
-      store(1, acc + 32);
-      pack_out(0, acc);
-      pack_out(1, acc + 32);
-    }
-  }
-  if (g.maxbits) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0 && mx > 0.0f) atomicMax(g.maxbits, __float_as_uint(mx));
+    fin(tpi, tqi, acc);
   }
   return true;
 }
 
-template <int SPLIT>
-__device__ bool gemm_phase(const PsGemm& g, uint32_t stage0, PsAux& x, uint32_t tmem, PsPipe& pp, int* status) {
-  const int warp = threadIdx.x >> 5;
-  bool ok = true;
-  if (threadIdx.x == 0) ok = gemm_issue<SPLIT>(g, stage0, x, tmem, pp, status);
-  else if (warp >= PS_EPI0) ok = gemm_drain<SPLIT>(g, x, tmem, pp, status);
-  if (!ok) x.abort = 1;
-  return ok;
+// What the draining warps make of a tile of (i): step (ii), T2[w', s', a', b]
+// = 2^-e sum_{w, s} W'[w, w', s, s'] T1[w, a', s, b], into (iii)'s packed
+// operand. A half goes through its columns in rounds of bw = 16 b (d <= 2) or
+// 8 b: T1 of the round to shared memory, row (w, s, a') of bw floats; then a
+// thread takes 8 b of one a' and every ms-th output channel, four at a time.
+// Neighbouring lanes take the two halves of 16 b: whole 32-byte sectors.
+struct PsStepII {
+  uint8_t* hi;   // packed T2
+  int64_t lo;    // byte distance to the lo plane, 0: none
+  float inv;     // 2^-e
+  int32_t Da, Db, DbP, wa, wb, d, slabs, lg;
+  uint32_t rd;   // m / d = m * rd >> 16 (m < 8)
+};
+
+template <int HR>  // rounds of 8 HR columns
+__device__ __forceinline__ void step_ii_rounds(const PsStepII& q, const float4 (*Ws)[4], uint8_t* staged, int half,
+                                               int cells, int tpi, int tqi, const float* acc) {
+  const int tid = (threadIdx.x - PS_EPI0 * 32) & (PS_GROUP - 1);
+  const int lg = q.lg, d = q.d, wad = q.wa * d, wbd = q.wb * d;
+  const int rw = tid >> lg, ra = tid - (rw << lg);  // this thread's T1 row (w, a')
+  constexpr int CH = 2 * HR;                  // 16-byte chunks of a staged row
+  auto slot = [&](int k, int a, int c) -> uint8_t* {
+    const int sw = HR == 2 ? (a >> 1) & 3 : (a >> 2) & 1;
+    return staged + (((k << lg) + a) * CH + (c ^ sw)) * 16;
+  };
+  const int ib = HR == 2 ? tid & 1 : 0, rest = tid / HR, mh = rest >> lg, ia = rest - (mh << lg);
+  const int ms = (PS_GROUP / HR) >> lg, kst = CH * 16 << lg;
+  const int a = (tpi << lg) + ia;
+  for (int c = 0; c < cells; ++c) {
+    const int b0 = (((tqi * 2 + half) * cells) + c) * 16;
+    if (b0 >= q.Db) break;
+#pragma unroll
+    for (int hb = 0; hb < 2; hb += HR) {
+      // the group's readers of the previous round are done
+      ptx::named_barrier(1 + half, PS_GROUP);
+#pragma unroll
+      for (int gi = 0; gi < 4; ++gi) {
+        const int sk = gi - c * d;
+        if (sk >= 0 && sk < d && rw < q.wa) {
+#pragma unroll
+          for (int ch = 0; ch < CH; ++ch) {
+            const float* v = acc + 16 * gi + 8 * hb + 4 * ch;
+            *reinterpret_cast<float4*>(slot(rw * d + sk, ra, ch)) = make_float4(v[0], v[1], v[2], v[3]);
+          }
+        }
+      }
+      ptx::named_barrier(1 + half, PS_GROUP);
+      if (a < q.Da) {
+        for (int m0 = mh; m0 < wbd; m0 += 4 * ms) {
+          float2 o[4][4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) o[i][j] = make_float2(0.0f, 0.0f);
+          const uint8_t *row0 = slot(0, ia, 2 * ib), *row1 = slot(0, ia, 2 * ib + 1);
+#pragma unroll 4
+          for (int k = 0; k < wad; ++k) {
+            const float4 t0 = *reinterpret_cast<const float4*>(row0 + k * kst);
+            const float4 t1 = *reinterpret_cast<const float4*>(row1 + k * kst);
+            const float2 t[4] = {{t0.x, t0.y}, {t0.z, t0.w}, {t1.x, t1.y}, {t1.z, t1.w}};
+            const float4 w4 = Ws[k][ms == 1 ? m0 >> 2 : mh];
+            const float wv[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) o[i][j] = __ffma2_rn(make_float2(wv[i], wv[i]), t[j], o[i][j]);
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int m = m0 + i * ms;
+            if (m >= wbd) break;
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              v[2 * j] = o[i][j].x * q.inv;
+              v[2 * j + 1] = o[i][j].y * q.inv;
+            }
+            const int w2 = (int)((uint32_t)m * q.rd >> 16), s2 = m - w2 * d;
+            const int32_t r0 = w2 * q.DbP + b0 + (hb + ib) * 8, kx = a * d + s2;
+            const size_t off = ((size_t)(r0 >> 7) * q.slabs + (kx >> 6)) * PS_BLOCK +
+                               mn_block_chunk((r0 & 127) >> 3, kx & 63);
+            uint4 h, l;
+            split8(v, h, l);
+            *reinterpret_cast<uint4*>(q.hi + off) = h;
+            if (q.lo) *reinterpret_cast<uint4*>(q.hi + q.lo + off) = l;
+          }
+        }
+      }
+    }
+  }
+}
+
+// What the draining warps make of a tile of (iii): rows (w', b) of L', columns
+// b', packed as the next site's first operand of (i) (row (w', b') at shared
+// index b) with the largest magnitude. Lanes 2i and 2i + 1 hold rows b and b +
+// 1 and swap chunks, so that each store of the pair is one 32-byte sector.
+struct PsNext {
+  uint8_t* hi;
+  int64_t lo;
+  int32_t Db, DbP, wb, lg, slabs, cols;
+};
+
+__device__ __forceinline__ void pack_next(const PsNext& q, int half, int tpi, int tqi, const float* acc, float& mx) {
+  const int lane = threadIdx.x & 31, quad = (threadIdx.x >> 5) & 3, ng = q.cols >> 5;
+  const int row = tpi * 128 + quad * 32 + lane, odd = lane & 1;
+  const int wq = row / q.DbP, b = row - wq * q.DbP, b0 = b & ~1;
+  const bool live = wq < q.wb, valid = live && b < q.Db;  // DbP is even: the pair has one w'
+#pragma unroll
+  for (int gi = 0; gi < 4; ++gi) {
+    const int cb = tqi * q.cols + (half * ng + gi) * 16;
+    if (gi < ng && cb < q.Db) {
+      const float* v = acc + 16 * gi;
+      uint4 h[2], l[2];
+      split8(v, h[0], l[0]);
+      split8(v + 8, h[1], l[1]);
+      if (valid) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) mx = fmaxf(mx, fabsf(v[j]));
+      }
+      const int t = cb >> q.lg, mg = ((wq << q.lg) + cb - (t << q.lg)) >> 3;
+      uint8_t* blk = q.hi + (size_t)t * q.slabs * PS_BLOCK;
+      const size_t o0 = (size_t)(b0 >> 6) * PS_BLOCK + mn_block_chunk(mg + odd, b0 & 63);
+      const size_t o1 = (size_t)(b0 >> 6) * PS_BLOCK + mn_block_chunk(mg + odd, (b0 + 1) & 63);
+      // chunk `odd` of rows b0 (o0) and b0 + 1 (o1)
+      const uint4 hs = swap_pair(pick(odd, h[0], h[1])), ls = swap_pair(pick(odd, l[0], l[1]));
+      if (live && b0 < q.Db) {
+        *reinterpret_cast<uint4*>(blk + o0) = pick(odd, hs, h[0]);
+        if (q.lo) *reinterpret_cast<uint4*>(blk + q.lo + o0) = pick(odd, ls, l[0]);
+      }
+      if (live && b0 + 1 < q.Db) {
+        *reinterpret_cast<uint4*>(blk + o1) = pick(odd, h[1], hs);
+        if (q.lo) *reinterpret_cast<uint4*>(blk + q.lo + o1) = pick(odd, l[1], ls);
+      }
+    }
+  }
 }
 
 // The whole sweep. Grid: one CTA per SM (cooperative launch).
 template <int SPLIT>
 __global__ void __launch_bounds__(PS_THREADS, 1) expect_persistent_kernel(const __grid_constant__ PsParams p) {
-  using C = PsCfg<SPLIT>;
   extern __shared__ uint8_t ps_smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(ps_smem_raw) + 1023) & ~uintptr_t(1023));
-  PsAux& x = *reinterpret_cast<PsAux*>(smem + (size_t)C::STAGES * C::STAGE_BYTES);
-  const int warp = threadIdx.x >> 5;
+  uint8_t* staged = smem + PS_RING;
+  PsAux& x = *reinterpret_cast<PsAux*>(staged + 2 * PS_STAGED);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int st = 0; st < C::STAGES; ++st) {
+    for (int st = 0; st < p.stages; ++st) {
       ptx::mbar_init(ptx::smem_addr(&x.full[st]), 1);   // the producer's transaction arrival
       ptx::mbar_init(ptx::smem_addr(&x.empty[st]), 1);  // the MMA issuer's commit
     }
@@ -533,128 +620,160 @@ __global__ void __launch_bounds__(PS_THREADS, 1) expect_persistent_kernel(const 
   ptx::tc_fence_after();
   const uint32_t tmem = x.tmem_base, stage0 = ptx::smem_addr(smem);
   const int64_t gtid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, gstride = (int64_t)gridDim.x * blockDim.x;
-  const int32_t d = p.d;
-  PsPipe pp{0u, 0u, 0u};
+  const int32_t d = p.d, half = (warp - PS_EPI0) >> 2;
+  const int64_t Lp_lo = SPLIT ? p.Lp_lo : 0, T2p_lo = SPLIT ? p.T2p_lo : 0;
+  PsPipe pp{0u, 0u, 0u, 0u};
   uint32_t epoch = 0;
-  int cur = 0;
   // (0) every site's core in the two operand layouts, and the first
-  // environment (1 in each channel) as the first site's MN-major operand
-  for (int64_t e = gtid; e < p.chunks; e += gstride) {
-    int lo = 0, hi = p.n - 1;  // the site whose chunks hold e
+  // environment (1 in each channel) as the first site's operand
+  for (uint32_t e = blockIdx.x * (PS_THREADS / 32) + warp; e < p.units; e += gridDim.x * (PS_THREADS / 32)) {
+    int lo = 0, hi = p.n - 1;  // the site whose units hold e
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (p.site[mid].chunk0 <= e) lo = mid;
+      if (p.site[mid].unit0 <= e) lo = mid;
       else hi = mid - 1;
     }
     const PsSite& st = p.site[lo];
-    PsPack q;
-    core_packs(p, st, d, &q, nullptr);
-    const int64_t c1 = pack_chunks(q);
-    int64_t k = e - st.chunk0;
-    if (k >= c1) {
-      core_packs(p, st, d, nullptr, &q);
-      k -= c1;
-    }
-    pack_chunk(q, k, 0.0f);
+    uint32_t k = e - st.unit0;
+    const uint32_t c1 = pack_units(st.t[0]);
+    const int third = k >= c1;
+    if (third) k -= c1;
+    const PsTiles& tt = st.t[third];
+    pack_unit(PsPack{st.A, p.Cp + (size_t)tt.off * 1024, p.Cp_lo, tt.cols, tt.slabs, third ? d * st.Da : st.Da, st.Db,
+                     third ? 1 : d},
+              k);
   }
   {
     const PsSite& s0 = p.site[0];
-    const int32_t R = s0.wa * s0.Da, K = s0.Da, tiles = ceil_div(R, 128), slabs = ceil_div(K, 64);
+    const int32_t lg = group_shift(s0.wa), tiles = s0.t[0].tp, slabs = s0.t[0].slabs;
     for (int64_t e = gtid; e < (int64_t)tiles * slabs * 16 * 64; e += gstride)
-      pack_mn_chunk(p.L[0], s0.Da, R, K, slabs, p.Lp, SPLIT ? p.Lp_lo : 0, e);
+      pack_mn_chunk(p.L[0], s0.Da, s0.wa, lg, slabs, p.Lp, Lp_lo, e);
   }
   bool ok = grid_sync(p, epoch, x);
   for (int i = 0; i < p.n && ok; ++i) {
     const PsSite& st = p.site[i];
-    const int32_t Da = st.Da, Db = st.Db, wa = st.wa, wb = st.wb;
-    const int32_t slabs1 = ceil_div(Da, 64), slabs3 = ceil_div(d * Da, 64);
-    // (B) T1[(w, a'), (s, b)] = sum_a L[(w, a'), a] A[a, (s, b)]
+    const int32_t Da = st.Da, Db = st.Db, wa = st.wa, wb = st.wb, DbP = pad16(Db);
+    const int32_t slabs3 = st.t[1].slabs;
+    // (B) T1 and, from its tiles, T2 = 2^-e W' T1
     PsGemm g;
-    memset(&g, 0, sizeof(g));
+    auto tiles = [&](const PsTiles& t) {
+      g.Q = p.Cp + (size_t)t.off * 1024;
+      g.units = (int32_t)t.tp * t.tq;
+      g.tq = t.tq;
+      g.slabs = t.slabs;
+      g.cols = t.cols;
+      g.magic = t.magic;
+    };
+    tiles(st.t[0]);
     g.P = p.Lp;
-    g.Q = p.Cp + st.a1_off;
     g.P_lo = p.Lp_lo;
     g.Q_lo = p.Cp_lo;
-    g.C = p.T1;
-    g.ldc = d * Db;
-    g.R = wa * Da;
-    g.N = d * Db;
-    g.tp = ceil_div(g.R, 128);
-    g.tq = ceil_div(g.N, 128);
-    g.slabs = slabs1;
-    g.p_mn = 1;
-    gemm_phase<SPLIT>(g, stage0, x, tmem, pp, p.status);
-    if (!(ok = grid_sync(p, epoch, x))) break;
-    // (C) T2 = 2^-e W' T1, straight into (iii)'s packed first operand; zeros
-    // at the shared indices past Db of the next site's operand of (i)
-    StepIIPack q2;
-    q2.T1 = p.T1;
-    q2.W = p.Wx + st.woff;
-    q2.maxbits = i > 0 ? p.bits + i : nullptr;
-    q2.lg = p.lg;
-    q2.hi = p.T2p;
-    q2.lo = SPLIT ? p.T2p + p.T2p_lo : nullptr;
-    q2.Da = Da;
-    q2.Db = Db;
-    q2.wa = wa;
-    q2.wb = wb;
-    q2.d = d;
-    q2.tiles = ceil_div(wb * Db, 128);
-    q2.slabs = slabs3;
-    q2.ps = 1;
-    q2.pa = d;
-    q2.pad = 0;
-    step_ii_pack(q2, gtid, gstride, blockIdx.x == 0 && threadIdx.x == 0);
-    const int32_t nslabs = ceil_div(Db, 64), npad = nslabs * 64 - Db;
-    if (i + 1 < p.n && npad > 0) {
-      const int64_t nz = (int64_t)ceil_div(wb * Db, 128) * 16 * npad;
-      for (int64_t e = gtid; e < nz; e += gstride) {
-        const int32_t kk = Db + (int32_t)(e % npad);
-        const int64_t rest = e / npad;
-        const int32_t mg = (int32_t)(rest & 15), t = (int32_t)(rest >> 4);
-        const size_t off = ((size_t)t * nslabs + (kk >> 6)) * PS_BLOCK + mn_block_chunk(mg, kk & 63);
-        *reinterpret_cast<uint4*>(p.Lp + off) = make_uint4(0u, 0u, 0u, 0u);
-        if (SPLIT) *reinterpret_cast<uint4*>(p.Lp + p.Lp_lo + off) = make_uint4(0u, 0u, 0u, 0u);
+    if (threadIdx.x == 0) {
+      if (!gemm_copy<SPLIT>(g, p, stage0, x, pp)) x.abort = 1;
+    } else if (warp == 1) {
+      if (!gemm_issue<SPLIT>(g, p, stage0, x, tmem, pp)) x.abort = 1;
+    } else if (warp >= PS_EPI0) {
+      const int tid = threadIdx.x - PS_EPI0 * 32;
+      // each half's copy of W' (its readers wait at the half's barriers), by
+      // the order step_ii_rounds reads it: the four channels m of a thread's
+      // pass (m = mh, mh + ms, ...) as one 16-byte word
+      const int lg = group_shift(wa), lms = (d <= 2 ? 6 : 7) - lg;
+      if ((tid & (PS_GROUP - 1)) < 64) {
+        const int k = (tid >> 3) & 7, m = tid & 7;
+        float v = 0.0f;
+        if (k < wa * d && m < wb * d) {
+          const int w = k / d, sk = k - w * d, w2 = m / d, s2 = m - w2 * d;
+          v = __ldg(p.Wx + st.woff + ((w * wb + w2) * d + sk) * d + s2);
+        }
+        const int ms1 = (1 << lms) - 1;
+        reinterpret_cast<float*>(x.Ws[half][k])[lms == 0 ? m : (m & ms1) * 4 + (m >> lms)] = v;
+        if (lms == 2) reinterpret_cast<float*>(x.Ws[half][k])[(m & 3) * 4 + 2 + (m >> 2)] = 0.0f;
       }
+      int e = 0;
+      if (i > 0) e = pow2_exponent(__uint_as_float(__ldcg(p.bits + i)));
+      if (i > 0 && blockIdx.x == 0 && tid == 0) *p.lg += (double)e * 0.69314718055994530942;
+      PsStepII q;
+      q.hi = p.T2p;
+      q.lo = T2p_lo;
+      q.inv = __int_as_float((127 - e) << 23);
+      q.Da = Da;
+      q.Db = Db;
+      q.DbP = DbP;
+      q.wa = wa;
+      q.wb = wb;
+      q.d = d;
+      q.slabs = slabs3;
+      q.lg = lg;
+      q.rd = (uint32_t)(65536 + d - 1) / (uint32_t)d;
+      const int cells = (int)((uint32_t)(g.cols >> 5) * q.rd >> 16);
+      uint8_t* mine = staged + half * PS_STAGED;
+      const bool done = gemm_drain<SPLIT>(g, x, tmem, pp, p.status, [&](int tpi, int tqi, const float* acc) {
+        if (d <= 2) step_ii_rounds<2>(q, x.Ws[half], mine, half, cells, tpi, tqi, acc);
+        else step_ii_rounds<1>(q, x.Ws[half], mine, half, cells, tpi, tqi, acc);
+      });
+      if (!done) x.abort = 1;
+    } else if (warp >= 2) {
+      zero_shared_tail(p.T2p, T2p_lo, st.t[1].tp, slabs3, d * Da, blockIdx.x * 64 + threadIdx.x - 64, gridDim.x * 64);
     }
     if (!(ok = grid_sync(p, epoch, x))) break;
-    // (D) L'[(w', b), b'] = sum_{(a', s')} T2[(w', b), (a', s')] A[(a', s'), b'];
-    // L' also packed as the next site's operand of (i), with its largest magnitude
+    // (D) L'[(w', b), b'] = sum_{(a', s')} T2[(w', b), (a', s')] A[(a', s'), b']
+    tiles(st.t[1]);
     g.P = p.T2p;
-    g.Q = p.Cp + st.a3_off;
     g.P_lo = p.T2p_lo;
-    g.Q_lo = p.Cp_lo;
-    g.C = p.L[cur ^ 1];
-    g.ldc = Db;
-    g.R = wb * Db;
-    g.N = Db;
-    g.tp = q2.tiles;
-    g.tq = ceil_div(Db, 128);
-    g.slabs = slabs3;
-    g.p_mn = 1;
-    if (i + 1 < p.n) {
-      g.Pn = p.Lp;
-      g.Pn_lo = SPLIT ? p.Lp_lo : 0;
-      g.Db = Db;
-      g.pn_slabs = nslabs;
-      g.maxbits = p.bits + i + 1;
+    const bool last = i + 1 == p.n;
+    const int32_t slabsn = ceil_div(Db, 64);
+    if (threadIdx.x == 0) {
+      if (!gemm_copy<SPLIT>(g, p, stage0, x, pp)) x.abort = 1;
+    } else if (warp == 1) {
+      if (!gemm_issue<SPLIT>(g, p, stage0, x, tmem, pp)) x.abort = 1;
+    } else if (warp >= PS_EPI0) {
+      float mx = 0.0f;
+      PsNext q;
+      q.hi = p.Lp;
+      q.lo = Lp_lo;
+      q.Db = Db;
+      q.DbP = DbP;
+      q.wb = wb;
+      q.lg = group_shift(wb);
+      q.slabs = slabsn;
+      q.cols = g.cols;
+      const bool done = gemm_drain<SPLIT>(g, x, tmem, pp, p.status, [&](int tpi, int tqi, const float* acc) {
+        if (!last) {
+          pack_next(q, half, tpi, tqi, acc, mx);
+        } else if (tqi == 0 && half == 0) {
+          // Db = 1: the last environment, one value per channel
+          const int row = tpi * 128 + (warp & 3) * 32 + lane, wq = row / DbP;
+          if (wq < wb && row == wq * DbP) p.L[1][wq] = acc[0];
+        }
+      });
+      if (!done) x.abort = 1;
+      if (!last) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (lane == 0 && mx > 0.0f) atomicMax(p.bits + i + 1, __float_as_uint(mx));
+      }
+    } else if (warp >= 2 && !last) {
+      zero_shared_tail(p.Lp, Lp_lo, ceil_div(Db, 1 << group_shift(wb)), slabsn, Db, blockIdx.x * 64 + threadIdx.x - 64, gridDim.x * 64);
     }
-    gemm_phase<SPLIT>(g, stage0, x, tmem, pp, p.status);
     if (!(ok = grid_sync(p, epoch, x))) break;
-    cur ^= 1;
   }
   if (ok && blockIdx.x == 0 && threadIdx.x == 0) {
-    const float* L = p.L[cur];
-    p.result[0] = (double)L[0];
-    p.result[1] = *p.lg;
-    p.result[2] = (double)L[1];
-    p.result[3] = *p.lg;
+    const float* L = p.L[1];
+    p.result[0] = (double)__ldcg(L);
+    p.result[1] = __ldcg(p.lg);
+    p.result[2] = (double)__ldcg(L + 1);
+    p.result[3] = __ldcg(p.lg);
   }
   // wind down: copies still in flight land, every MMA completes, then TMEM is freed
   if (threadIdx.x == 0) {
-    for (uint32_t q = pp.consumed; q < pp.issued; ++q)
-      ptx::mbar_wait(ptx::smem_addr(&x.full[q % C::STAGES]), (q / C::STAGES) & 1u, p.status);
-    ptx::mma_commit(ptx::smem_addr(&x.final_bar));
+    const uint32_t S = (uint32_t)p.stages;
+    for (uint32_t q = pp.slab < S ? 0u : pp.slab - S; q < pp.slab; ++q)
+      ptx::mbar_wait(ptx::smem_addr(&x.full[q % S]), (q / S) & 1u, p.status);
+  }
+  __syncwarp();
+  if (warp == 1) {
+    if (ptx::elect_one()) ptx::mma_commit(ptx::smem_addr(&x.final_bar));  // the lane that issued the MMAs
+    __syncwarp();
     ptx::mbar_wait(ptx::smem_addr(&x.final_bar), 0u, p.status);
   }
   ptx::tc_fence_before();
@@ -667,18 +786,74 @@ __global__ void __launch_bounds__(PS_THREADS, 1) expect_persistent_kernel(const 
 
 }  // namespace
 
-size_t ps_blocks(int64_t R, int64_t K) { return (size_t)((R + 127) / 128) * (size_t)((K + 63) / 64) * PS_BLOCK; }
+// Bytes of one plane (hi or lo) of an operand in blocks of `rows` rows.
+size_t ps_bytes(int64_t tiles, int64_t K, int64_t rows) { return (size_t)tiles * (size_t)((K + 63) / 64) * (size_t)rows * 128; }
 
-// One plane (hi or lo) of every site's packed cores: the core as (i)'s
-// second operand (d Db rows, Da shared) then as (iii)'s (Db rows, d Da shared).
-size_t cores_plane_bytes(const tn_mps* psi) {
-  size_t b = 0;
-  for (int i = 0; i < psi->n; ++i)
-    b += ps_blocks(psi->d * psi->bond[i + 1], psi->bond[i]) + ps_blocks(psi->bond[i + 1], psi->d * psi->bond[i]);
-  return align256(b);
+int device_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return 152;
+  return sms;
 }
 
-size_t expect_persistent_cores_bytes(const tn_mps* psi) { return 2 * cores_plane_bytes(psi); }
+int64_t ceil64(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// Columns of a GEMM phase's tiles (step, 2 step, .. up to 128; step: the
+// columns that must stay together in both halves, 32 d for (i), 32 for
+// (iii)): the count that makes the phase shortest by a model of it, rounds of
+// units over the SMs, each the copies of its slabs (32 KB of P and 256 bytes
+// a column for BF16X3, at about 64 bytes a cycle; its MMAs, 40 to 64 cycles
+// each whatever the width, take about as long) and its epilogue (about 20
+// cycles a column). At bond 256 it takes 64 and 32 columns, 64 units in each
+// phase; at 512 128 and 64.
+int tile_cols(int64_t tp, int64_t total, int64_t K, int step, int64_t sms) {
+  const int64_t slabs = ceil64(K, 64);
+  int best = step;
+  int64_t best_cost = INT64_MAX;
+  for (int c = step; c <= 128; c *= 2) {
+    const int64_t units = tp * ceil64(total, c);
+    const int64_t cost = ceil64(units, sms) * (slabs * (512 + 4 * c) + 20 * c + 1000);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = c;
+    }
+  }
+  return best;
+}
+
+// Tiles of a site's phases: first operands' row tiles and the columns.
+struct SiteTiles {
+  int64_t t1, t3;
+  int n1, n3;
+};
+SiteTiles site_tiles(int64_t Da, int64_t Db, int64_t wa, int64_t wb, int64_t d, int64_t sms) {
+  SiteTiles t;
+  const int64_t DbP = pad16((int32_t)Db);
+  t.t1 = ceil64(Da, int64_t(1) << group_shift((int32_t)wa));
+  t.t3 = ceil64(wb * DbP, 128);
+  t.n1 = tile_cols(t.t1, d * DbP, Da, (int)(32 * d), sms);
+  t.n3 = tile_cols(t.t3, DbP, d * Da, 32, sms);
+  return t;
+}
+
+ExpectRegions expect_persistent_regions(const tn_mps* psi, const tn_mpo* H) {
+  ExpectRegions r{0, 0, 0};
+  const int64_t sms = device_sms();
+  const int64_t d = psi->d;
+  for (int i = 0; i < psi->n; ++i) {
+    const int64_t Da = psi->bond[i], Db = psi->bond[i + 1];
+    const SiteTiles t = site_tiles(Da, Db, H->bond[i] + 1, H->bond[i + 1] + 1, d, sms);
+    r.env = std::max(r.env, ps_bytes(t.t1, Da, 128));
+    r.t2 = std::max(r.t2, ps_bytes(t.t3, d * Da, 128));
+    const int64_t DbP = pad16((int32_t)Db);
+    r.cores += ps_bytes(ceil64(d * DbP, t.n1), Da, t.n1) + ps_bytes(ceil64(DbP, t.n3), d * Da, t.n3);
+  }
+  r.env = align256(r.env);
+  r.t2 = align256(r.t2);
+  r.cores = align256(r.cores);
+  return r;
+}
 
 bool expect_persistent_ok(const tn_mps* psi, const tn_mpo* H, int prec) {
   if (prec != TN_PREC_BF16 && prec != TN_PREC_BF16X3) return false;
@@ -699,57 +874,58 @@ int expect_persistent(const tn_mps* psi, const tn_mpo* H, int prec, const Expect
   p.Wx = w.Wx;
   p.L[0] = w.L0;
   p.L[1] = w.L1;
-  p.T1 = w.T1;
-  // packed regions, laid out for the largest bond: L (hi, lo) in scratch,
-  // T2 (hi, lo) in scratch3; every site's cores (hi plane, then lo) in cores
-  int64_t Wm = 1, D = 1;
-  for (int i = 0; i <= H->n; ++i) Wm = std::max(Wm, H->bond[i]);
-  for (int i = 0; i <= psi->n; ++i) D = std::max(D, psi->bond[i]);
-  const int64_t W1 = Wm + 1, d = psi->d;
-  const size_t bl = align256(ps_blocks(W1 * D, D)), bt = align256(ps_blocks(W1 * D, d * D));
-  const size_t bc = cores_plane_bytes(psi);
-  if (w.scratch_bytes < 2 * bl || w.scratch3_bytes < 2 * bt || w.cores_bytes < 2 * bc) return TN_ERR_WORKSPACE;
+  // packed regions (hi plane, then lo): L in scratch, T2 in scratch3, every
+  // site's cores in cores
+  const ExpectRegions need = expect_persistent_regions(psi, H);
+  if (w.scratch_bytes < 2 * need.env || w.scratch3_bytes < 2 * need.t2 || w.cores_bytes < 2 * need.cores)
+    return TN_ERR_WORKSPACE;
+  const int64_t d = psi->d;
   p.Lp = w.scratch;
-  p.Lp_lo = split ? (int64_t)bl : 0;
+  p.Lp_lo = split ? (int64_t)need.env : 0;
   p.T2p = w.scratch3;
-  p.T2p_lo = split ? (int64_t)bt : 0;
+  p.T2p_lo = split ? (int64_t)need.t2 : 0;
   p.Cp = w.cores;
-  p.Cp_lo = split ? (int64_t)bc : 0;
+  p.Cp_lo = split ? (int64_t)need.cores : 0;
   p.bits = w.bits;
   p.lg = w.lg;
   p.bar = w.bar;
   p.result = result;
   p.status = status_word();
-  for (int i = 0; i < psi->n; ++i) {
-    PsSite& st = p.site[i];
-    st.A = psi->cores[i];
-    st.Da = (int32_t)psi->bond[i];
-    st.Db = (int32_t)psi->bond[i + 1];
-    st.wa = (int32_t)(H->bond[i] + 1);
-    st.wb = (int32_t)(H->bond[i + 1] + 1);
-    st.woff = (int32_t)w.woff[(size_t)i];
-  }
-  // the cores' places and pack chunks, site by site
+  // the cores' places, pack units and tiles, site by site
   size_t off = 0;
-  int64_t chunks = 0;
+  uint32_t units = 0;
+  int widest = 0;
+  const int sms = device_sms();
   for (int i = 0; i < psi->n; ++i) {
     PsSite& st = p.site[i];
-    const int64_t Da = st.Da, Db = st.Db;
-    st.a1_off = (int64_t)off;
-    off += ps_blocks(d * Db, Da);
-    st.a3_off = (int64_t)off;
-    off += ps_blocks(Db, d * Da);
-    st.chunk0 = chunks;
-    chunks += (int64_t)(ps_blocks(d * Db, Da) + ps_blocks(Db, d * Da)) / PS_BLOCK * 1024;
+    const int64_t Da = psi->bond[i], Db = psi->bond[i + 1], DbP = pad16((int32_t)Db);
+    st.A = psi->cores[i];
+    st.Da = (int16_t)Da;
+    st.Db = (int16_t)Db;
+    st.wa = (int8_t)(H->bond[i] + 1);
+    st.wb = (int8_t)(H->bond[i + 1] + 1);
+    st.woff = (int32_t)w.woff[(size_t)i];
+    st.unit0 = units;
+    const SiteTiles t = site_tiles(Da, Db, st.wa, st.wb, d, sms);
+    for (int j = 0; j < 2; ++j) {
+      PsTiles& q = st.t[j];
+      const int cols = j ? t.n3 : t.n1;
+      const int64_t K = j ? d * Da : Da, tq = ceil64(j ? DbP : d * DbP, cols);
+      q.off = (uint32_t)(off / 1024);
+      q.tp = (uint16_t)(j ? t.t3 : t.t1);
+      q.tq = (uint16_t)tq;
+      q.magic = tq == 1 ? 0u : (uint32_t)(((uint64_t(1) << 32) + (uint64_t)tq - 1) / (uint64_t)tq);
+      q.cols = (int16_t)cols;
+      q.slabs = (int16_t)ceil64(K, 64);
+      off += ps_bytes(tq, K, cols);
+      units += pack_units(q);
+      widest = std::max(widest, cols);
+    }
   }
-  p.chunks = chunks;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
-                                                cudaSuccess)
-    return TN_ERR_CUDA;
-  const size_t smem = 1024 + (size_t)(split ? PsCfg<1>::STAGES * PsCfg<1>::STAGE_BYTES
-                                            : PsCfg<0>::STAGES * PsCfg<0>::STAGE_BYTES) +
-                      sizeof(PsAux);
+  p.units = units;
+  p.stage_bytes = (split ? 2 : 1) * (PS_BLOCK + widest * 128);
+  p.stages = std::min(PS_RING / p.stage_bytes, PS_MAX_STAGES);
+  const size_t smem = 1024 + (size_t)PS_RING + 2 * PS_STAGED + sizeof(PsAux);
   const void* fn = split ? (const void*)expect_persistent_kernel<1> : (const void*)expect_persistent_kernel<0>;
   static std::atomic<uint64_t> attr[2];
   if (!smem_limit_once(fn, smem, &attr[split ? 1 : 0])) return TN_ERR_CUDA;

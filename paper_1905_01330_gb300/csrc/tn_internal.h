@@ -182,12 +182,12 @@ void step_iii_places(int64_t Da, int64_t Db, int64_t d, const int64_t* kstrA, in
 // The energy sweep as one persistent cooperative launch (mps_persistent.cu):
 // BF16 / BF16X3, at most 512 sites, (extended MPO bond) x d <= 8. Buffers
 // from the energy sweep's workspace: environments L0 / L1 (with the first
-// site's L0 = 1 in its channels), T1, the extended MPO Wx (site i at
+// site's L0 = 1 in its channels), the extended MPO Wx (site i at
 // woff[i]), per-site max slots `bits` and the log-scale `lg` (zeroed), the
 // barrier counter `bar` (4 bytes), the packed regions `scratch` / `scratch3`
 // and `cores` (every site's core packed once per call).
 struct ExpectBuffers {
-  float *L0, *L1, *T1;
+  float *L0, *L1;
   const float* Wx;
   const int64_t* woff;
   unsigned* bits;
@@ -197,11 +197,16 @@ struct ExpectBuffers {
   size_t scratch_bytes;
   uint8_t* scratch3;
   size_t scratch3_bytes;
-  uint8_t* cores;  // every site's packed cores (expect_persistent_cores_bytes)
+  uint8_t* cores;  // every site's packed cores
   size_t cores_bytes;
 };
 bool expect_persistent_ok(const tn_mps* psi, const tn_mpo* H, int prec);
-size_t expect_persistent_cores_bytes(const tn_mps* psi);
+// Bytes of one plane (hi or lo) of its packed regions: the environment, T2,
+// every site's cores.
+struct ExpectRegions {
+  size_t env, t2, cores;
+};
+ExpectRegions expect_persistent_regions(const tn_mps* psi, const tn_mpo* H);
 int expect_persistent(const tn_mps* psi, const tn_mpo* H, int prec, const ExpectBuffers& w, double* result,
                       cudaStream_t s);
 

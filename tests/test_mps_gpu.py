@@ -171,6 +171,30 @@ def test_energy_long_chain_both_launch_forms(tn, n, prec):
     assert rel(val(r, 1), norm) <= tol(prec, 2 * n) + 2 * n * bias
 
 
+@pytest.mark.parametrize("d,w", [(1, 3), (1, 7), (2, 1), (2, 2), (2, 3), (3, 1), (4, 1)])
+@pytest.mark.parametrize("prec", ["bf16x3", "bf16"])
+def test_energy_tiles_of_the_one_launch_sweep(tn, d, w, prec):
+    # Every split of a 128-row tile among the channels (w + 1 = 2 .. 8) and
+    # both widths of a step (ii) round (d <= 2, d > 2), at bonds around the
+    # edges of cells (16), shared slabs (64) and tiles. All numbers positive:
+    # nothing cancels, so energy and norm are bounded like the norm above.
+    bonds = [1, 5, 16, 17, 64, 70, 130, 33, 3, 1]
+    n = len(bonds) - 1
+    rng = np.random.default_rng(100 * d + w)
+    cores = [(rng.uniform(0.5, 1.5, (bonds[i], d, bonds[i + 1])) / math.sqrt(bonds[i] * bonds[i + 1])).astype(np.float32)
+             for i in range(n)]
+    wb = [1] + [w] * (n - 1) + [1]
+    W = [rng.uniform(0.5, 1.5, (wb[i], wb[i + 1], d, d)).astype(np.float32) for i in range(n)]
+    e, le = oracle.mpo_expect(cores, W)
+    nv, ln = oracle.mps_inner(cores, cores)
+    r = tn.mps_expect(to_dev(cores), to_dev(W), prec=prec)
+    assert tn.sync_status() == 0
+    bias = {"bf16x3": 2.0 ** -18, "bf16": 2.0 ** -16}[prec]
+    bound = tol(prec, 2 * n) + 2 * n * bias
+    assert rel(val(r, 0), e * math.exp(le)) <= bound
+    assert rel(val(r, 1), nv * math.exp(ln)) <= bound
+
+
 @pytest.mark.parametrize("prec", ["fp32", "bf16x3", "bf16"])
 def test_energy_three_level_sites(tn, prec):
     # spin-1 sites (d = 3) with a bond-4 MPO: (bond + 1) d = 15, so the sweep
