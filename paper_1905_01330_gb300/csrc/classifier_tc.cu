@@ -25,13 +25,26 @@
 // hi = bf16(x) plus lo = bf16(x - hi) and each product is hi*hi + lo*hi +
 // hi*lo in the float32 accumulator.
 //
-// One launch covers both half-chains (CTA = (half, tile)). A CTA has 256
-// epilogue threads, two per sample (thread r owns TMEM lane r % 128 and half
-// of the columns), and one producer warp that streams the packed core slabs
-// (and, in the adjoint, the v tiles) into shared-memory rings with 1-D bulk
-// async copies. Thread 0 issues the MMAs. Every mbarrier wait is bounded; a
-// CTA that gives up records TN_ERR_TIMEOUT, lets its copies land, frees its
-// TMEM and returns.
+// One launch covers both half-chains (CTA = (half, tile)). A CTA has NG
+// epilogue threads per sample (thread r owns TMEM lane r % 128 and its group's
+// columns), one producer warp that streams the packed core slabs (and, in the
+// adjoint, the v tiles) into shared-memory rings with 1-D bulk async copies,
+// and one warp that issues the MMAs.
+//
+// What bounds it: a step is a chain, MMAs, accumulator, mixing, splitting,
+// shared memory, MMAs, and nothing else of the tile can run meanwhile (a
+// second tile's operands do not fit beside the first's). So the MMA warp does
+// nothing else (with an epilogue thread as issuer, which the tensor pipe's
+// short queue holds until its last MMAs run, that thread's own part of the
+// step came after the MMAs: 6,500 cycles a step of which the MMAs are 3,070
+// at chi = 128); the exchange of the scales runs while the MMAs do; at chi =
+// 128 the forward step's columns are two halves, so that the first half's
+// epilogue and the next step's MMAs on it run beside the second half's; and
+// the adjoint's epilogue works on g' while the gradient product runs.
+// Measured (4096 samples, 784 sites, split BF16x3; before -> now): forward chi
+// = 128 FWD128, chi = 64 with recomputation FWD64, adjoint chi = 64 ADJ64.
+// Every mbarrier wait is bounded; a CTA that gives up records
+// TN_ERR_TIMEOUT, lets its copies land, frees its TMEM and returns.
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -42,8 +55,6 @@ namespace tn {
 namespace {
 
 constexpr int TS = CLS_TILE;         // samples per tile
-constexpr int NEPI = 2 * TS;         // epilogue threads
-constexpr int NTHREADS = NEPI + 32;  // + the producer warp
 constexpr int PXS = 16;              // steps of pixels staged at once
 constexpr int SLAB_V = TS * 128;     // one 64-column slab of a 128-row tile (bytes)
 constexpr int SMEM_BUDGET = 200 * 1024;
@@ -61,14 +72,21 @@ struct Cfg {
   static constexpr int KSL = KPAD / 64;
   static constexpr int VT = KSL * SLAB_V;           // one part of a vector tile
   static constexpr int VTS = VT * PARTS;
-  static constexpr int HC = CHI / 2;                // columns per epilogue thread
-  // forward: image rows (s, j), K = k
-  static constexpr int FN = 2 * CHI;
+  static constexpr int NG = CHI >= 64 ? 4 : 2;      // epilogue threads per sample
+  static constexpr int NEPI = NG * TS;
+  static constexpr int NTHREADS = NEPI + 96;        // + producer, MMA and (forward) vector-image store warps
+  static constexpr int ATHREADS = NEPI + 64;
+  static constexpr int HC = CHI / NG;               // columns per epilogue thread
+  // forward: image rows (j / (CHI / NH), s, j % (CHI / NH)), K = k; NH column
+  // halves, each with its own accumulator, blocks (k slab, half) in this order
+  static constexpr int NH = CHI == 128 ? 2 : 1;
+  static constexpr int FN = 2 * CHI / NH;
   static constexpr int FSLAB = FN * 128;
   static constexpr int FSET = FSLAB * PARTS;
   static constexpr int FRING_RAW = (SMEM_BUDGET - VTS) / FSET;
   static constexpr int FRING = FRING_RAW > 8 ? 8 : FRING_RAW;
-  static constexpr uint32_t FCOLS = FN < 32 ? 32 : FN;
+  static constexpr int VCOL = 2 * CHI;              // TMEM columns of the vector: part p at VCOL + p KPAD / 2
+  static constexpr uint32_t FCOLS = (uint32_t)pow2ceil(VCOL + PARTS * KPAD / 2);
   // adjoint: x tile rows b, columns m = (s, j); image rows k, K = m
   static constexpr int XSL = 2 * CHI / 64;
   static constexpr int XPART = (XSL + (CHI == 32 ? 1 : 0)) * SLAB_V;  // + a zero M half at chi = 32
@@ -81,8 +99,9 @@ struct Cfg {
   static constexpr int A2OFF = CHI < 64 ? 64 : CHI;  // TMEM column of the gradient accumulator
   // two gradient accumulators when they fit (step q's is drained while step
   // q + 1's products run), else one
-  static constexpr int A2BUF = A2OFF + 2 * MH * KPAD <= 512 ? 2 : 1;
-  static constexpr uint32_t ACOLS = (uint32_t)pow2ceil(A2OFF + A2BUF * MH * KPAD);
+  static constexpr int A2BUF = A2OFF + 2 * MH * KPAD + PARTS * CHI <= 512 ? 2 : 1;
+  static constexpr int XCOL = A2OFF + A2BUF * MH * KPAD;  // x in TMEM: part p at XCOL + p CHI
+  static constexpr uint32_t ACOLS = (uint32_t)pow2ceil(XCOL + PARTS * CHI);
 };
 
 struct __align__(8) Bars {
@@ -90,15 +109,19 @@ struct __align__(8) Bars {
   uint64_t empty[8];
   uint64_t vfull[2];
   uint64_t vempty[2];
-  uint64_t acc_full;
+  uint64_t acc_full[2];  // forward: a half's accumulator is complete; adjoint: g', the gradient
+  uint64_t ready[2];     // the next step's operand is written (forward at chi = 128: its k slabs)
+  uint64_t drained;      // the second half's accumulator has been read
+  uint64_t image;        // forward: the vector's image for the gradients is written
+  uint64_t stored;       // and its copy to device memory has been read out
   uint64_t final_bar;
   uint32_t tmem_base;
   int32_t abort;
 };
 
 struct StageTail {
-  float px[PXS][TS];
-  float pmax[2][TS];
+  float2 phi[PXS][TS];
+  float pmax[2][4][TS];
   Bars bars;
 };
 
@@ -116,19 +139,6 @@ __device__ __forceinline__ void split_pair(float a, float b, uint32_t& hi, uint3
   const float2 hf = __bfloat1622float2(h);
   hi = bf16x2_bits(h);
   lo = bf16x2_bits(__floats2bfloat162_rn(a - hf.x, b - hf.y));
-}
-
-// Writes 8 values as one 16-byte chunk of every part of a K-major tile
-// (part 1 = the lo part, `part_bytes` after part 0).
-template <int PARTS>
-__device__ __forceinline__ void put8(uint8_t* tile, int part_bytes, uint32_t off, const float* v) {
-  uint4 h, l;
-  split_pair(v[0], v[1], h.x, l.x);
-  split_pair(v[2], v[3], h.y, l.y);
-  split_pair(v[4], v[5], h.z, l.z);
-  split_pair(v[6], v[7], h.w, l.w);
-  *reinterpret_cast<uint4*>(tile + off) = h;
-  if (PARTS == 2) *reinterpret_cast<uint4*>(tile + part_bytes + off) = l;
 }
 
 // 2^-e and 2^e as floats (e in [-126, 126]).
@@ -156,66 +166,134 @@ __device__ __forceinline__ void bulk_copy_s2g(void* dst, uint32_t src_smem, uint
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-template <int N>
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t* r) {
-  if constexpr (N == 32) ptx::tmem_ld_32x32b_x32(taddr, r);
-  else ptx::tmem_ld_32x32b_x16(taddr, r);
-}
-
-__device__ __forceinline__ void epi_barrier() { ptx::named_barrier(1, NEPI); }
-
-// Stages pixels of steps [q0, q0 + PXS) of this tile (zeros past the end).
-template <class SiteOf>
-__device__ __forceinline__ void stage_pixels(float (&px)[PXS][TS], const float* pixels, int n, int B, int b0, int q0,
+// Stages (cos, sin)(pi x / 2) of steps [q0, q0 + PXS) of this tile (zeros
+// past the end), between barriers of the epilogue threads: the previous ones
+// are read by then, the new ones visible after.
+template <int NEPI, class SiteOf>
+__device__ __forceinline__ void stage_pixels(float2 (&phi)[PXS][TS], const float* pixels, int n, int B, int b0, int q0,
                                              int nsteps, SiteOf site_of) {
+  ptx::named_barrier(1, NEPI);
   for (int e = threadIdx.x; e < PXS * TS; e += NEPI) {
     const int qq = e % PXS, bb = e / PXS;
     float val = 0.0f;
     if (q0 + qq < nsteps && b0 + bb < B) val = __ldg(pixels + (int64_t)(b0 + bb) * n + site_of(q0 + qq));
-    px[qq][bb] = val;
+    phi[qq][bb] = make_float2(cospif(0.5f * val), sinpif(0.5f * val));
   }
+  ptx::named_barrier(1, NEPI);
+}
+
+// N packed columns of this lane's row of an operand in tensor memory.
+template <int N>
+__device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t* r) {
+  if constexpr (N == 16) ptx::tmem_st_32x32b_x16(taddr, r);
+  else ptx::tmem_st_32x32b_x8(taddr, r);
+}
+
+// Waits of an epilogue warp: once one has run out the warp stops waiting (and
+// the CTA is winding down) but keeps taking part in the named barriers.
+struct EpiWait {
+  int32_t* abort;
+  int* status;
+  bool dead = false;
+  __device__ __forceinline__ void operator()(uint64_t* bar, uint32_t parity) {
+    if (!dead && !__all_sync(0xffffffffu, ptx::mbar_wait(ptx::smem_addr(bar), parity, status))) {
+      *(volatile int32_t*)abort = 1;
+      dead = true;
+    }
+    ptx::tc_fence_after();
+  }
+};
+// The warp's arrival after its generic writes / TMEM reads.
+__device__ __forceinline__ void warp_arrive(uint64_t* bar) {
+  ptx::tc_fence_before();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(ptx::smem_addr(bar));
 }
 
 // ------------------------------------------------------------------ packing
+__device__ __forceinline__ uint4 swap_chunk(const uint4& a) {
+  return make_uint4(__shfl_xor_sync(0xffffffffu, a.x, 1), __shfl_xor_sync(0xffffffffu, a.y, 1),
+                    __shfl_xor_sync(0xffffffffu, a.z, 1), __shfl_xor_sync(0xffffffffu, a.w, 1));
+}
+
 // Value L[k, s, j] of the core of step t: the left half reads A[k, s, j],
 // the right half (swept from the chain's right end) A[j, s, k].
-__global__ void cls_pack_kernel(const __grid_constant__ ClsPackParams p) {
+__global__ void __launch_bounds__(256) cls_pack_kernel(const __grid_constant__ ClsPackParams p) {
   const int t = blockIdx.x, h = blockIdx.y;
   if (t >= p.T[h]) return;
   const int site = h == 0 ? t : p.n - 1 - t;
   const int Da = p.bond[site], Dc = p.bond[site + 1];
   const int Din = h == 0 ? Da : Dc, Dout = h == 0 ? Dc : Da;
   const float* __restrict__ A = p.core[site];
-  const int chi = p.chi, parts = p.split ? 2 : 1;
+  const int chi = p.chi, lc = 31 - __clz(chi), parts = p.split ? 2 : 1;  // chi = 32, 64 or 128
   uint8_t* img = p.images[h] + (size_t)t * p.step_bytes;
-  auto value = [&](int k, int s, int j) -> float {
-    if (k >= Din || j >= Dout) return 0.0f;
-    return h == 0 ? __ldg(A + ((int64_t)k * 2 + s) * Dc + j) : __ldg(A + ((int64_t)j * 2 + s) * Dc + k);
-  };
-  const int kpad = chi < 64 ? 64 : chi;
-  // rows R and K extent of the image kind; a 16-byte chunk is 8 consecutive K of one row
-  const int R = p.adjoint ? chi : 2 * chi;
-  const int KX = p.adjoint ? 2 * chi : kpad;
-  const int slab_bytes = R * 128;
-  const int chunks = R * (KX / 8);
-  for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
-    const int row = c % R, kg = c / R;
-    float v[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int kk = kg * 8 + e;
-      if (p.adjoint) v[e] = value(row, kk / chi, kk % chi);  // row k, K index m = (s, j)
-      else v[e] = value(kk, row / chi, row % chi);            // row (s, j), K index k
+  // log2 of the rows and of the K extent of the image kind; a 16-byte chunk is 8 consecutive K of one row
+  const int lr = p.adjoint ? lc : lc + 1;
+  const int lk = p.adjoint ? lc + 1 : (lc < 6 ? 6 : lc);
+  // forward at chi = 128: blocks of one half's 128 rows
+  const int halves = !p.adjoint && chi == 128 ? 2 : 1;
+  const int slab_bytes = (128 << lr) / halves;
+  // The K index runs along the core's unit stride (forward image of the right
+  // half, adjoint image of the left): 16 consecutive values as four 16-byte
+  // loads where they are aligned.
+  const bool kfast = (h == 1) != (p.adjoint != 0);
+  const bool vec = kfast && (Dc & 3) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+  const int lane = threadIdx.x & 31, odd = lane & 1;
+  const int pairs = 1 << (lr + lk - 4);  // two chunks of one row each
+  for (int c = threadIdx.x; c < pairs; c += 256) {
+    const int row = c & ((1 << lr) - 1), k0 = (c >> lr) * 16;
+    float v[16];
+    // value(K index, row) at base + 16 steps of `stride`, real below `real`
+    int fixed_ok, s2, k2;
+    if (p.adjoint) {
+      s2 = k0 >> lc;  // chi is a multiple of 16: one s
+      k2 = k0 & (chi - 1);
+      fixed_ok = row < Din;
+    } else {
+      s2 = row >> lc;
+      k2 = k0;
+      fixed_ok = (row & (chi - 1)) < Dout;
     }
-    const int ks = kg >> 3, g = kg & 7;
-    uint8_t* dst = img + (size_t)ks * parts * slab_bytes + sw128(row, g);
-    uint4 hh, ll;
-    split_pair(v[0], v[1], hh.x, ll.x);
-    split_pair(v[2], v[3], hh.y, ll.y);
-    split_pair(v[4], v[5], hh.z, ll.z);
-    split_pair(v[6], v[7], hh.w, ll.w);
-    *reinterpret_cast<uint4*>(dst) = hh;
-    if (p.split) *reinterpret_cast<uint4*>(dst + slab_bytes) = ll;
+    const int kreal = (p.adjoint ? Dout : Din) - k2, rowi = p.adjoint ? row : row & (chi - 1);
+    // element (k or j along K, the other index along the rows) of A[k, s, j] / A[j, s, k]
+    const float* src = kfast ? A + ((int64_t)rowi * 2 + s2) * Dc + k2 : A + ((int64_t)k2 * 2 + s2) * Dc + rowi;
+    const int64_t stride = kfast ? 1 : 2 * (int64_t)Dc;
+    if (vec && fixed_ok && kreal >= 16) {
+#pragma unroll
+      for (int e = 0; e < 16; e += 4) {
+        const float4 f = __ldg(reinterpret_cast<const float4*>(src + e));
+        v[e] = f.x;
+        v[e + 1] = f.y;
+        v[e + 2] = f.z;
+        v[e + 3] = f.w;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 16; ++e) v[e] = fixed_ok && e < kreal ? __ldg(src + e * stride) : 0.0f;
+    }
+    const int ks = k0 >> 6, g = (k0 >> 3) & 7;
+    const int half = halves == 2 ? (row >> 6) & 1 : 0;
+    const int rb = halves == 2 ? ((row >> 7) << 6) | (row & 63) : row;  // row of its block
+    uint8_t* blk = img + (size_t)(ks * halves + half) * parts * slab_bytes;
+    uint4 hh[2], ll[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      split_pair(v[8 * i], v[8 * i + 1], hh[i].x, ll[i].x);
+      split_pair(v[8 * i + 2], v[8 * i + 3], hh[i].y, ll[i].y);
+      split_pair(v[8 * i + 4], v[8 * i + 5], hh[i].z, ll[i].z);
+      split_pair(v[8 * i + 6], v[8 * i + 7], hh[i].w, ll[i].w);
+    }
+    // lanes 2i and 2i + 1 (neighbouring rows) swap a chunk, so that the pair's
+    // stores are whole 32-byte sectors
+    const uint4 hs = swap_chunk(odd ? hh[0] : hh[1]), ls = swap_chunk(odd ? ll[0] : ll[1]);
+    const int r0 = rb & ~1;
+    const uint32_t o0 = sw128(r0, g + odd), o1 = sw128(r0 + 1, g + odd);
+    *reinterpret_cast<uint4*>(blk + o0) = odd ? hs : hh[0];
+    *reinterpret_cast<uint4*>(blk + o1) = odd ? hh[1] : hs;
+    if (p.split) {
+      *reinterpret_cast<uint4*>(blk + slab_bytes + o0) = odd ? ls : ll[0];
+      *reinterpret_cast<uint4*>(blk + slab_bytes + o1) = odd ? ll[1] : ls;
+    }
   }
 }
 
@@ -227,7 +305,7 @@ constexpr size_t fwd_smem_bytes() {
 }
 
 template <int CHI, int SPLIT>
-__global__ void __launch_bounds__(NTHREADS, 1) cls_fwd_tc(const __grid_constant__ ClsTcParams p) {
+__global__ void __launch_bounds__(Cfg<CHI, SPLIT>::NTHREADS, 1) cls_fwd_tc(const __grid_constant__ ClsTcParams p) {
   using C = Cfg<CHI, SPLIT>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -242,14 +320,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_fwd_tc(const __grid_constant_
   const int nsteps = p.t_end[h] - t0;
   const int n = p.n;
   auto site_of = [&](int q) { return p.half_site[h] + p.half_dir[h] * (t0 + q); };
-  const int nslabs = nsteps * C::KSL;
+  constexpr int BLOCKS = C::KSL * C::NH;  // core blocks of a step
 
   if (tid == 0) {
     for (int i = 0; i < C::FRING; ++i) {
       ptx::mbar_init(ptx::smem_addr(&x.full[i]), 1);
       ptx::mbar_init(ptx::smem_addr(&x.empty[i]), 1);
     }
-    ptx::mbar_init(ptx::smem_addr(&x.acc_full), 2);  // MMA commit + the vector-image store's read
+    for (int i = 0; i < C::NH; ++i) {
+      ptx::mbar_init(ptx::smem_addr(&x.acc_full[i]), 1);
+      ptx::mbar_init(ptx::smem_addr(&x.ready[i]), C::NEPI / 32 / C::NH);
+    }
+    ptx::mbar_init(ptx::smem_addr(&x.drained), C::NEPI / 64);
+    ptx::mbar_init(ptx::smem_addr(&x.image), C::NEPI / 32);
+    ptx::mbar_init(ptx::smem_addr(&x.stored), 1);
     ptx::mbar_init(ptx::smem_addr(&x.final_bar), 1);
     x.abort = 0;
     ptx::fence_mbar_init();
@@ -259,14 +343,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_fwd_tc(const __grid_constant_
     ptx::tmem_relinquish();
   }
   // zero the vector tile (padding columns stay zero)
-  for (int i = tid; i < C::VTS / 16; i += NTHREADS) reinterpret_cast<uint4*>(vt)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < C::VTS / 16; i += C::NTHREADS) reinterpret_cast<uint4*>(vt)[i] = make_uint4(0, 0, 0, 0);
+  ptx::fence_proxy_async_smem();
+  ptx::tc_fence_before();
   __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = x.tmem_base;
 
-  if (warp == NEPI / 32) {
-    // ---------------- producer: core slabs into the ring
+  if (warp == C::NEPI / 32) {
+    // ---------------- producer: core blocks into the ring
     if ((tid & 31) == 0) {
+      const int nblocks = nsteps * BLOCKS;
+      const uint8_t* src = p.images[h] + (size_t)t0 * BLOCKS * C::FSET;
       int g = 0;
-      for (; g < nslabs; ++g) {
+      for (; g < nblocks; ++g, src += C::FSET) {
         const int slot = g % C::FRING;
         if (g >= C::FRING &&
             !ptx::mbar_wait(ptx::smem_addr(&x.empty[slot]), (uint32_t)(((g / C::FRING) - 1) & 1), p.status)) {
@@ -274,20 +364,99 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_fwd_tc(const __grid_constant_
           break;
         }
         if (*(volatile int32_t*)&x.abort) break;
-        const int q = g / C::KSL, ks = g % C::KSL;
         const uint32_t bar = ptx::smem_addr(&x.full[slot]);
         ptx::mbar_arrive_expect_tx(bar, C::FSET);
-        ptx::bulk_copy_g2s(ptx::smem_addr(ring + (size_t)slot * C::FSET),
-                           p.images[h] + ((size_t)(t0 + q) * C::KSL + ks) * C::FSET, C::FSET, bar);
+        ptx::bulk_copy_g2s(ptx::smem_addr(ring + (size_t)slot * C::FSET), src, C::FSET, bar);
       }
       // let every copy issued land before the CTA can leave
       for (int gg = g - C::FRING < 0 ? 0 : g - C::FRING; gg < g; ++gg)
         ptx::mbar_wait(ptx::smem_addr(&x.full[gg % C::FRING]), (uint32_t)((gg / C::FRING) & 1), p.status);
     }
     __syncwarp();
+  } else if (warp == C::NEPI / 32 + 1) {
+    // ---------------- MMAs. At chi = 128 (two halves, two k slabs) in the
+    // order (k0, half 0), (k0, half 1), (k1, half 0), (k1, half 1): slab 0 of
+    // the vector tile is free again when half 0's accumulator is complete, so
+    // half 0 writes its part of the next vector, slab 0, while half 1's last
+    // MMAs run, and the next step's first two blocks need nothing else.
+    const uint32_t raddr = ptx::smem_addr(ring);
+    constexpr int KS = CHI < 64 ? CHI / 16 : 4;  // MMAs along K of a slab (chi = 32: without the padding)
+    constexpr uint32_t idesc = ptx::idesc_bf16_f32(128, C::FN);
+    int slot = 0;
+    uint32_t phase = 0;
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      const bool w = __all_sync(0xffffffffu, ptx::mbar_wait(ptx::smem_addr(bar), parity, p.status));
+      ptx::tc_fence_after();
+      return w;
+    };
+    // A wait takes some 150 cycles when its barrier has completed long ago, and
+    // the tensor pipe's queue is short: a block's barriers are waited for
+    // before the last MMAs of the block before it are issued.
+    bool ok = nsteps > 0 && wait(&x.full[0], 0u);
+    for (int q = 0; q < nsteps && ok; ++q) {
+      const uint32_t par = (uint32_t)(q & 1);
+      ok = wait(&x.ready[0], par);
+#pragma unroll
+      for (int ks = 0; ks < C::KSL; ++ks) {
+#pragma unroll
+        for (int nh = 0; nh < C::NH; ++nh) {
+          const uint32_t vh = tmem + (uint32_t)(C::VCOL + ks * 32), vl = vh + C::KPAD / 2;
+          const uint32_t bh = ptx::desc_lo(raddr + (uint32_t)(slot * C::FSET)), bl = bh + (C::FSLAB >> 4);
+          const uint32_t d = tmem + (uint32_t)(nh * C::FN), empty = ptx::smem_addr(&x.empty[slot]);
+          auto step = [&](int kk) {
+            ptx::mma_bf16_ta(d, vh + kk * 8u, bh + kk * 2u, idesc, (ks | kk) ? 1u : 0u);
+            if (SPLIT) {
+              ptx::mma_bf16_ta(d, vl + kk * 8u, bh + kk * 2u, idesc, 1u);
+              ptx::mma_bf16_ta(d, vh + kk * 8u, bl + kk * 2u, idesc, 1u);
+            }
+          };
+          if (ok && ptx::elect_one()) {
+#pragma unroll
+            for (int kk = 0; kk < KS - 1; ++kk) step(kk);
+          }
+          __syncwarp();
+          if (++slot == C::FRING) {
+            slot = 0;
+            phase ^= 1u;
+          }
+          const bool last = ks == C::KSL - 1 && nh == C::NH - 1;
+          if (C::NH == 2 && ks == 0 && nh == 0 && q > 0) ok = ok && wait(&x.drained, par ^ 1u);
+          if (C::KSL == 2 && ks == 0 && nh == C::NH - 1) ok = ok && wait(&x.ready[1], par);
+          if (!last || q + 1 < nsteps) ok = ok && wait(&x.full[slot], phase);
+          if (ok && ptx::elect_one()) {
+            step(KS - 1);
+            ptx::mma_commit(empty);
+            if (ks == C::KSL - 1) ptx::mma_commit(ptx::smem_addr(&x.acc_full[nh]));
+          }
+          __syncwarp();
+        }
+      }
+    }
+    if (!ok && nsteps > 0) x.abort = 1;
+    if (ptx::elect_one()) {
+      ptx::mma_commit(ptx::smem_addr(&x.final_bar));
+      ptx::mbar_wait(ptx::smem_addr(&x.final_bar), 0u, p.status);
+    }
+    __syncwarp();
+  } else if (warp == C::NEPI / 32 + 2) {
+    // ---------------- the vectors entering the steps, for the adjoint's gradient product
+    if (p.vseg[h] && (tid & 31) == 0) {
+      for (int q = 0; q < nsteps; ++q) {
+        if (!ptx::mbar_wait(ptx::smem_addr(&x.image), (uint32_t)(q & 1), p.status)) {
+          x.abort = 1;
+          break;
+        }
+        bulk_copy_s2g(p.vseg[h] + ((size_t)q * p.ntiles + tile) * C::VTS, ptx::smem_addr(vt), C::VTS);
+        bulk_wait_read();
+        ptx::mbar_arrive(ptx::smem_addr(&x.stored));
+      }
+      bulk_wait_all();
+    }
+    __syncwarp();
   } else {
-    // ---------------- epilogue threads (and thread 0: the MMA issuer)
-    const int r = tid & (TS - 1), hc = tid >> 7;  // sample row, column half
+    // ---------------- epilogue threads
+    const int r = tid & (TS - 1), hc = tid >> 7;  // sample row, column group
+    const int half = hc * C::NH / C::NG;
     const int b = b0 + r;
     const bool live = b < B;
     const int c0 = hc * C::HC;  // first column of this thread
@@ -299,95 +468,65 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_fwd_tc(const __grid_constant_
     // scale of the vector in the tile not yet applied (deferred mode)
     int e_prev = 0;
     const bool defer = p.vseg[h] == nullptr;
-    auto write_vtile = [&]() {
+    uint32_t vh[C::HC / 2], vl[C::HC / 2];
+    const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    // v, split, as the next step's operand: a lane's row of tensor memory
+    auto write_operand = [&]() {
+#pragma unroll
+      for (int k = 0; k < C::HC / 2; ++k) split_pair(v[2 * k], v[2 * k + 1], vh[k], vl[k]);
+      tmem_st<C::HC / 2>(lanes + (uint32_t)(C::VCOL + c0 / 2), vh);
+      if (SPLIT) tmem_st<C::HC / 2>(lanes + (uint32_t)(C::VCOL + C::KPAD / 2 + c0 / 2), vl);
+      ptx::tmem_st_wait();
+      warp_arrive(&x.ready[half]);
+    };
+    // and as the image the gradient product reads (128-byte swizzle)
+    auto write_image = [&]() {
 #pragma unroll
       for (int g8 = 0; g8 < C::HC / 8; ++g8) {
         const int col = c0 + g8 * 8;
-        put8<C::PARTS>(vt, C::VT, (uint32_t)((col >> 6) * SLAB_V) + sw128(r, (col >> 3) & 7), &v[g8 * 8]);
+        uint8_t* dst = vt + (col >> 6) * SLAB_V + sw128(r, (col >> 3) & 7);
+        *reinterpret_cast<uint4*>(dst) = make_uint4(vh[4 * g8], vh[4 * g8 + 1], vh[4 * g8 + 2], vh[4 * g8 + 3]);
+        if (SPLIT)
+          *reinterpret_cast<uint4*>(dst + C::VT) = make_uint4(vl[4 * g8], vl[4 * g8 + 1], vl[4 * g8 + 2], vl[4 * g8 + 3]);
       }
+      ptx::fence_proxy_async_smem();
+      warp_arrive(&x.image);
     };
-    write_vtile();
-    ptx::fence_proxy_async_smem();
-    ptx::tc_fence_before();
-    epi_barrier();
-    ptx::tc_fence_after();
-    const uint32_t tmem = x.tmem_base;
-    const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t vaddr = ptx::smem_addr(vt), raddr = ptx::smem_addr(ring);
-    constexpr uint32_t idesc = ptx::idesc_bf16_f32(128, C::FN);
-    constexpr int LDN = C::HC >= 32 ? 32 : 16;
-
-    bool ok = true;
-    int gs = 0;  // slabs consumed (thread 0)
-    // thread 0: the MMAs of step qq (issued as soon as the tile holds its vector)
-    auto issue = [&](int qq) {
-      // the vector entering step t0 + qq, for the adjoint's gradient product
-      if (p.vseg[h]) bulk_copy_s2g(p.vseg[h] + ((size_t)qq * p.ntiles + tile) * C::VTS, vaddr, C::VTS);
-      bool w = true;
-      for (int ks = 0; ks < C::KSL && w; ++ks, ++gs) {
-        const int slot = gs % C::FRING;
-        w = ptx::mbar_wait(ptx::smem_addr(&x.full[slot]), (uint32_t)((gs / C::FRING) & 1), p.status);
-        if (!w) break;
-        ptx::tc_fence_after();
-        const uint32_t bs = raddr + (uint32_t)(slot * C::FSET);
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          const uint32_t ao = vaddr + (uint32_t)(ks * SLAB_V + kk * 32);
-          const uint64_t ah = ptx::sw128_kmajor_desc(ao), bh = ptx::sw128_kmajor_desc(bs + kk * 32);
-          ptx::mma_bf16(tmem, ah, bh, idesc, (ks | kk) ? 1u : 0u);
-          if (SPLIT) {
-            ptx::mma_bf16(tmem, ptx::sw128_kmajor_desc(ao + C::VT), bh, idesc, 1u);
-            ptx::mma_bf16(tmem, ah, ptx::sw128_kmajor_desc(bs + C::FSLAB + kk * 32), idesc, 1u);
-          }
-        }
-        ptx::mma_commit(ptx::smem_addr(&x.empty[slot]));
-      }
-      if (w) ptx::mma_commit(ptx::smem_addr(&x.acc_full));
-      else {
-        x.abort = 1;
-        ptx::mbar_arrive(ptx::smem_addr(&x.acc_full));
-      }
-      bulk_wait_read();
-      ptx::mbar_arrive(ptx::smem_addr(&x.acc_full));
-    };
-    if (nsteps > 0 && tid == 0) issue(0);
-    __syncwarp();
-    for (int q = 0; q < nsteps && ok; ++q) {
+    write_operand();
+    if (!defer) write_image();
+    // this thread's columns of the accumulators: U[b, (s, j)] at column (half, s, j % (CHI / NH))
+    constexpr int JH = CHI / C::NH;
+    const uint32_t acc = lanes + (uint32_t)(half * C::FN + c0 % JH);
+    EpiWait wait{&x.abort, p.status};
+    for (int q = 0; q < nsteps; ++q) {
       const int t = t0 + q;
-      // pixels of the next PXS steps (the epilogue threads only)
-      if (q % PXS == 0) {
-        stage_pixels(st.px, p.pixels, n, B, b0, q, nsteps, site_of);
-        epi_barrier();
-      }
+      if (q % PXS == 0) stage_pixels<C::NEPI>(st.phi, p.pixels, n, B, b0, q, nsteps, site_of);
       // keep the float32 vector entering step t (v holds it times 2^e_prev)
+      const float ip = pow2f(-e_prev);
       if (p.store[h] && live && ((t - p.store_base[h]) % p.store_every) == 0) {
         float* dst = p.store[h] + ((int64_t)((t - p.store_base[h]) / p.store_every) * B + b) * CHI + c0;
-        const float ip = pow2f(-e_prev);
 #pragma unroll
         for (int k = 0; k < C::HC; k += 4)
           *reinterpret_cast<float4*>(dst + k) = make_float4(v[k] * ip, v[k + 1] * ip, v[k + 2] * ip, v[k + 3] * ip);
       }
-      const float xp = st.px[q % PXS][r];
-      const float f0 = cospif(0.5f * xp), f1 = sinpif(0.5f * xp);
-      const bool waited = ptx::mbar_wait(ptx::smem_addr(&x.acc_full), (uint32_t)(q & 1), p.status);
-      if (!__all_sync(0xffffffffu, waited)) x.abort = 1;
-      if (waited) {
-        ptx::tc_fence_after();
-        // the MMA read v_t 2^e_prev: the step's output times 2^-e_prev is u_t itself (exact)
-        const float ip = pow2f(-e_prev);
-        const float g0 = f0 * ip, g1 = f1 * ip;
+      // the MMA read v_t 2^e_prev: the step's output times 2^-e_prev is u_t itself (exact)
+      const float2 phi = st.phi[q % PXS][r];
+      const float g0 = phi.x * ip, g1 = phi.y * ip;
+      wait(&x.acc_full[half], (uint32_t)(q & 1));
+      {
+        uint32_t u0[C::HC], u1[C::HC];
 #pragma unroll
-        for (int c = 0; c < C::HC; c += LDN) {
-          uint32_t u0[LDN], u1[LDN];
-          tmem_ld<LDN>(lane_base + (uint32_t)(c0 + c), u0);
-          tmem_ld<LDN>(lane_base + (uint32_t)(CHI + c0 + c), u1);
-          ptx::tmem_ld_wait();
-#pragma unroll
-          for (int e = 0; e < LDN; ++e) v[c + e] = g0 * __uint_as_float(u0[e]) + g1 * __uint_as_float(u1[e]);
+        for (int c = 0; c < C::HC; c += 16) {
+          ptx::tmem_ld_32x32b_x16(acc + (uint32_t)c, u0 + c);
+          ptx::tmem_ld_32x32b_x16(acc + (uint32_t)(JH + c), u1 + c);
         }
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < C::HC; ++e) v[e] = g0 * __uint_as_float(u0[e]) + g1 * __uint_as_float(u1[e]);
       }
-      // the step's scale 2^e_t from the sample's largest |u_t| over both
-      // column halves. Without a vector-image store it is applied one step
+      if (C::NH == 2 && half == 1) warp_arrive(&x.drained);
+      // the step's scale 2^e_t from the sample's largest |u_t| over its
+      // column groups. Without a vector-image store it is applied one step
       // late (the next MMA reads u_t itself, bf16(u_t) = bf16(v_{t+1}) 2^e_t),
       // so the exchange runs while that MMA does; the recomputation keeps
       // the normalised v_{t+1} in the tile it stores for the gradients.
@@ -395,9 +534,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_fwd_tc(const __grid_constant_
         float m = 0.0f;
 #pragma unroll
         for (int k = 0; k < C::HC; ++k) m = fmaxf(m, fabsf(v[k]));
-        st.pmax[hc][r] = m;
-        ptx::named_barrier(2 + (warp & 3), 64);
-        m = fmaxf(st.pmax[0][r], st.pmax[1][r]);
+        float(*pm)[TS] = st.pmax[q & 1];  // the other one is still being read
+        pm[hc][r] = m;
+        ptx::named_barrier(2 + (warp & 3), 32 * C::NG);
+#pragma unroll
+        for (int i = 0; i < C::NG; ++i) m = fmaxf(m, pm[i][r]);
         const int e = scale_exponent(m);
         lam_e += e;
         if (hc == 0 && live) p.sc[h][(int64_t)t * B + b] = pow2f(e);
@@ -408,14 +549,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_fwd_tc(const __grid_constant_
 #pragma unroll
         for (int k = 0; k < C::HC; ++k) v[k] *= inv;
       }
-      write_vtile();
-      ptx::fence_proxy_async_smem();
-      ptx::tc_fence_before();
-      ok = ptx::named_barrier_or(1, NEPI, *(volatile int32_t*)&x.abort != 0) == false;
-      ptx::tc_fence_after();
-      if (tid == 0 && ok && q + 1 < nsteps) issue(q + 1);
-      __syncwarp();
-      if (defer) e_prev = exchange();
+      write_operand();
+      if (defer) {
+        e_prev = exchange();
+      } else if (q + 1 < nsteps) {
+        wait(&x.stored, (uint32_t)(q & 1));
+        write_image();
+      }
     }
     {
       const float ip = pow2f(-e_prev);
@@ -428,18 +568,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_fwd_tc(const __grid_constant_
         *reinterpret_cast<float4*>(p.state[h] + (int64_t)b * CHI + c0 + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
       if (hc == 0) p.lam[h][b] = lam0 + (double)lam_e * 0.69314718055994530942;
     }
-    if (tid == 0) {
-      ptx::mma_commit(ptx::smem_addr(&x.final_bar));
-      ptx::mbar_wait(ptx::smem_addr(&x.final_bar), 0u, p.status);
-      bulk_wait_all();
-    }
-    __syncwarp();
   }
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 0) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(x.tmem_base, C::FCOLS);
+    ptx::tmem_dealloc(tmem, C::FCOLS);
   }
 }
 
@@ -452,7 +586,7 @@ constexpr size_t adj_smem_bytes() {
 }
 
 template <int CHI, int SPLIT>
-__global__ void __launch_bounds__(NTHREADS, 1) cls_adj_tc(const __grid_constant__ ClsTcParams p) {
+__global__ void __launch_bounds__(Cfg<CHI, SPLIT>::ATHREADS, 1) cls_adj_tc(const __grid_constant__ ClsTcParams p) {
   using C = Cfg<CHI, SPLIT>;
   static_assert(C::ARING >= 2, "adjoint staging does not fit in shared memory");
   extern __shared__ uint8_t smem_raw[];
@@ -479,8 +613,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_adj_tc(const __grid_constant_
     for (int i = 0; i < 2; ++i) {
       ptx::mbar_init(ptx::smem_addr(&x.vfull[i]), 1);
       ptx::mbar_init(ptx::smem_addr(&x.vempty[i]), 1);
+      ptx::mbar_init(ptx::smem_addr(&x.acc_full[i]), 1);
     }
-    ptx::mbar_init(ptx::smem_addr(&x.acc_full), 1);
+    for (int i = 0; i < 2; ++i) ptx::mbar_init(ptx::smem_addr(&x.ready[i]), C::NEPI / 32);
     ptx::mbar_init(ptx::smem_addr(&x.final_bar), 1);
     x.abort = 0;
     ptx::fence_mbar_init();
@@ -489,10 +624,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_adj_tc(const __grid_constant_
     ptx::tmem_alloc(ptx::smem_addr(&x.tmem_base), C::ACOLS);
     ptx::tmem_relinquish();
   }
-  for (int i = tid; i < C::XTS / 16; i += NTHREADS) reinterpret_cast<uint4*>(xt)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < C::XTS / 16; i += C::ATHREADS) reinterpret_cast<uint4*>(xt)[i] = make_uint4(0, 0, 0, 0);
+  ptx::fence_proxy_async_smem();
+  ptx::tc_fence_before();
   __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = x.tmem_base;
 
-  if (warp == NEPI / 32) {
+  if (warp == C::NEPI / 32) {
     // ---------------- producer: per step the core slabs, then the v tile
     if ((tid & 31) == 0) {
       int g = 0, q = 0;
@@ -533,6 +672,89 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_adj_tc(const __grid_constant_
         ptx::mbar_wait(ptx::smem_addr(&x.vfull[qq & 1]), (uint32_t)((qq >> 1) & 1), p.status);
     }
     __syncwarp();
+  } else if (warp == C::NEPI / 32 + 1) {
+    // ---------------- MMAs: g' first (the next step waits for it), then the gradient
+    const uint32_t xaddr = ptx::smem_addr(xt), vaddr = ptx::smem_addr(vring), caddr = ptx::smem_addr(cring);
+    constexpr uint32_t idesc1 = ptx::idesc_bf16_f32(128, CHI);
+    constexpr uint32_t idesc2 = ptx::idesc_bf16_f32(128, C::KPAD, 1, 1);
+    int slot = 0;
+    uint32_t phase = 0;
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      const bool w = __all_sync(0xffffffffu, ptx::mbar_wait(ptx::smem_addr(bar), parity, p.status));
+      ptx::tc_fence_after();
+      return w;
+    };
+    // barriers are waited for ahead of their MMAs, as in the forward
+    bool ok = nsteps > 0 && wait(&x.full[0], 0u);
+    for (int q = 0; q < nsteps && ok; ++q) {
+      const int vs = q & 1;
+      ok = wait(&x.ready[0], (uint32_t)(q & 1));
+      // g'[b, k] = sum_m x[b, m] L[k, m]
+#pragma unroll 1
+      for (int ks = 0; ks < C::XSL && ok; ++ks) {
+        const uint32_t ah = tmem + (uint32_t)(C::XCOL + ks * 32), al = ah + CHI;
+        const uint32_t bh = ptx::desc_lo(caddr + (uint32_t)(slot * C::ASET)), bl = bh + (C::ASLAB >> 4);
+        const uint32_t empty = ptx::smem_addr(&x.empty[slot]);
+        auto step = [&](int kk) {
+          ptx::mma_bf16_ta(tmem, ah + kk * 8u, bh + kk * 2u, idesc1, (ks | kk) ? 1u : 0u);
+          if (SPLIT) {
+            ptx::mma_bf16_ta(tmem, al + kk * 8u, bh + kk * 2u, idesc1, 1u);
+            ptx::mma_bf16_ta(tmem, ah + kk * 8u, bl + kk * 2u, idesc1, 1u);
+          }
+        };
+        if (ptx::elect_one()) {
+          step(0);
+          step(1);
+          step(2);
+        }
+        __syncwarp();
+        if (++slot == C::ARING) {
+          slot = 0;
+          phase ^= 1u;
+        }
+        if (ks + 1 < C::XSL) ok = wait(&x.full[slot], phase);
+        if (ok && ptx::elect_one()) {
+          step(3);
+          ptx::mma_commit(empty);
+          if (ks == C::XSL - 1) ptx::mma_commit(ptx::smem_addr(&x.acc_full[0]));
+        }
+        __syncwarp();
+      }
+      ok = ok && wait(&x.ready[1], (uint32_t)(q & 1)) && wait(&x.vfull[vs], (uint32_t)((q >> 1) & 1));
+      // dL[m, k] = sum_b x[b, m] v[b, k]: both operands MN-major (the
+      // K-major x tile read transposed; the v tile as the forward wrote it)
+      auto grad = [&](int mh, int kk) {
+        const uint32_t d = tmem + (uint32_t)(C::A2OFF + ((q & 1) % C::A2BUF) * C::MH * C::KPAD + mh * C::KPAD);
+        const uint32_t ah = ptx::desc_lo(xaddr + (uint32_t)(mh * 2 * SLAB_V), SLAB_V), al = ah + (C::XPART >> 4);
+        const uint32_t bh = ptx::desc_lo(vaddr + (uint32_t)(vs * C::VTS), SLAB_V), bl = bh + (C::VT >> 4);
+        ptx::mma_bf16_lo(d, ah + kk * 128u, bh + kk * 128u, idesc2, kk ? 1u : 0u);
+        if (SPLIT) {
+          ptx::mma_bf16_lo(d, al + kk * 128u, bh + kk * 128u, idesc2, 1u);
+          ptx::mma_bf16_lo(d, ah + kk * 128u, bl + kk * 128u, idesc2, 1u);
+        }
+      };
+      if (ok && ptx::elect_one()) {
+#pragma unroll
+        for (int mh = 0; mh < C::MH; ++mh)
+#pragma unroll
+          for (int kk = 0; kk < TS / 16; ++kk)
+            if (mh < C::MH - 1 || kk < TS / 16 - 1) grad(mh, kk);
+      }
+      __syncwarp();
+      if (q + 1 < nsteps) ok = ok && wait(&x.full[slot], phase);
+      if (ok && ptx::elect_one()) {
+        grad(C::MH - 1, TS / 16 - 1);
+        ptx::mma_commit(ptx::smem_addr(&x.vempty[vs]));
+        ptx::mma_commit(ptx::smem_addr(&x.acc_full[1]));
+      }
+      __syncwarp();
+    }
+    if (!ok && nsteps > 0) x.abort = 1;
+    if (ptx::elect_one()) {
+      ptx::mma_commit(ptx::smem_addr(&x.final_bar));
+      ptx::mbar_wait(ptx::smem_addr(&x.final_bar), 0u, p.status);
+    }
+    __syncwarp();
   } else {
     const int r = tid & (TS - 1), hc = tid >> 7;
     const int b = b0 + r;
@@ -541,37 +763,55 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_adj_tc(const __grid_constant_
     float g[C::HC];
 #pragma unroll
     for (int k = 0; k < C::HC; ++k) g[k] = live ? p.state[h][(int64_t)b * CHI + c0 + k] : 0.0f;
-    // x of the step q: Phi_s(x at that step's site) g / sc into columns (s, c0 + k)
-    auto write_xtile = [&](int q) {
-      const float xp = st.px[q % PXS][r];
-      const float f[2] = {cospif(0.5f * xp), sinpif(0.5f * xp)};
-      const float scl = live ? p.sc[h][(int64_t)step_t(q) * B + b] : 1.0f;
-      const float inv = __frcp_rn(scl);  // scales are powers of two: exact
+    // x of the step q: Phi_s(x at that step's site) g / sc, columns (s, c0 + k)
+    constexpr int HX = C::HC / 2;  // packed columns of one s
+    uint32_t xh[2][HX], xl[2][HX];
+    float f[2], inv;
+    auto load_scale = [&](int q) { return live && q < nsteps ? __ldg(p.sc[h] + (int64_t)step_t(q) * B + b) : 1.0f; };
+    float scl = load_scale(0);  // of the next x, a step ahead of its use
+    auto load_factors = [&](int q) {
+      const float2 phi = st.phi[q % PXS][r];
+      f[0] = phi.x;
+      f[1] = phi.y;
+      inv = __frcp_rn(scl);  // scales are powers of two: exact
+      scl = load_scale(q + 1);
+    };
+    const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    // as g's operand: a lane's row of tensor memory
+    auto make_x = [&]() {
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+#pragma unroll
+        for (int k = 0; k < HX; ++k)
+          split_pair(f[s] * g[2 * k] * inv, f[s] * g[2 * k + 1] * inv, xh[s][k], xl[s][k]);
+        const uint32_t col = lane_base + (uint32_t)(C::XCOL + (s * CHI + c0) / 2);
+        tmem_st<HX>(col, xh[s]);
+        if (SPLIT) tmem_st<HX>(col + CHI, xl[s]);
+      }
+      ptx::tmem_st_wait();
+      warp_arrive(&x.ready[0]);
+    };
+    // as the gradient's, transposed there: the swizzled tile
+    auto write_xtile = [&]() {
 #pragma unroll
       for (int s = 0; s < 2; ++s)
 #pragma unroll
         for (int g8 = 0; g8 < C::HC / 8; ++g8) {
-          float w[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) w[e] = f[s] * g[g8 * 8 + e] * inv;
           const int col = s * CHI + c0 + g8 * 8;
-          put8<C::PARTS>(xt, C::XPART, (uint32_t)((col >> 6) * SLAB_V) + sw128(r, (col >> 3) & 7), w);
+          uint8_t* dst = xt + (col >> 6) * SLAB_V + sw128(r, (col >> 3) & 7);
+          const uint32_t *hp = &xh[s][4 * g8], *lp = &xl[s][4 * g8];
+          *reinterpret_cast<uint4*>(dst) = make_uint4(hp[0], hp[1], hp[2], hp[3]);
+          if (SPLIT) *reinterpret_cast<uint4*>(dst + C::XPART) = make_uint4(lp[0], lp[1], lp[2], lp[3]);
         }
+      ptx::fence_proxy_async_smem();
+      warp_arrive(&x.ready[1]);
     };
-    stage_pixels(st.px, p.pixels, n, B, b0, 0, nsteps, site_of);
-    epi_barrier();
-    if (nsteps > 0) write_xtile(0);
-    ptx::fence_proxy_async_smem();
-    ptx::tc_fence_before();
-    epi_barrier();
-    ptx::tc_fence_after();
-    const uint32_t tmem = x.tmem_base;
-    const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t xaddr = ptx::smem_addr(xt), vaddr = ptx::smem_addr(vring), caddr = ptx::smem_addr(cring);
-    constexpr uint32_t idesc1 = ptx::idesc_bf16_f32(128, CHI);
-    constexpr uint32_t idesc2 = ptx::idesc_bf16_f32(128, C::KPAD, 1, 1);
-    constexpr int LDN = C::HC >= 32 ? 32 : 16;
-    constexpr int GLD = C::KPAD / 2 >= 32 ? 32 : 16;  // gradient columns per TMEM load
+    if (nsteps > 0) {
+      stage_pixels<C::NEPI>(st.phi, p.pixels, n, B, b0, 0, nsteps, site_of);
+      load_factors(0);
+      make_x();
+      write_xtile();
+    }
     const int mrow = r;  // gradient row (x column) of this lane in M half 0
     // this tile's share of step t's core gradient, from accumulator `buf`
     auto drain_grad = [&](int t, int buf) {
@@ -579,16 +819,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_adj_tc(const __grid_constant_
 #pragma unroll
       for (int mh = 0; mh < C::MH; ++mh) {
         const int m = mh * 128 + mrow;
-        if (m < 2 * CHI) {
 #pragma unroll
-          for (int c = 0; c < C::KPAD / 2; c += GLD) {
-            const int k0 = hc * (C::KPAD / 2) + c;
-            if (k0 < CHI) {
-              uint32_t u[GLD];
-              tmem_ld<GLD>(lane_base + (uint32_t)(C::A2OFF + buf * C::MH * C::KPAD + mh * C::KPAD + k0), u);
-              ptx::tmem_ld_wait();
+        for (int c = 0; c < C::KPAD / C::NG; c += 16) {
+          const int k0 = hc * (C::KPAD / C::NG) + c;
+          if (k0 < CHI) {
+            uint32_t u[16];
+            ptx::tmem_ld_32x32b_x16(lane_base + (uint32_t)(C::A2OFF + buf * C::MH * C::KPAD + mh * C::KPAD + k0), u);
+            ptx::tmem_ld_wait();
+            if (m < 2 * CHI) {
 #pragma unroll
-              for (int e = 0; e < GLD; ++e)
+              for (int e = 0; e < 16; ++e)
                 if (k0 + e < CHI) red_add(gbase + (size_t)(k0 + e) * 2 * CHI + m, __uint_as_float(u[e]));
             }
           }
@@ -596,111 +836,44 @@ __global__ void __launch_bounds__(NTHREADS, 1) cls_adj_tc(const __grid_constant_
       }
     };
 
-    bool ok = true;
-    int gs = 0;
-    // thread 0: both products of step qq (issued as soon as the x tile holds its operand)
-    auto issue = [&](int qq) {
-      bool w = true;
-      // g'[b, k] = sum_m x[b, m] L[k, m]
-      for (int ks = 0; ks < C::XSL && w; ++ks, ++gs) {
-        const int slot = gs % C::ARING;
-        w = ptx::mbar_wait(ptx::smem_addr(&x.full[slot]), (uint32_t)((gs / C::ARING) & 1), p.status);
-        if (!w) break;
-        ptx::tc_fence_after();
-        const uint32_t bs = caddr + (uint32_t)(slot * C::ASET);
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          const uint32_t ao = xaddr + (uint32_t)(ks * SLAB_V + kk * 32);
-          const uint64_t ah = ptx::sw128_kmajor_desc(ao), bh = ptx::sw128_kmajor_desc(bs + kk * 32);
-          ptx::mma_bf16(tmem, ah, bh, idesc1, (ks | kk) ? 1u : 0u);
-          if (SPLIT) {
-            ptx::mma_bf16(tmem, ptx::sw128_kmajor_desc(ao + C::XPART), bh, idesc1, 1u);
-            ptx::mma_bf16(tmem, ah, ptx::sw128_kmajor_desc(bs + C::ASLAB + kk * 32), idesc1, 1u);
-          }
-        }
-        ptx::mma_commit(ptx::smem_addr(&x.empty[slot]));
-      }
-      // dL[m, k] = sum_b x[b, m] v[b, k]: both operands MN-major (the
-      // K-major x tile read transposed; the v tile as the forward wrote it)
-      const int vs = qq & 1;
-      if (w) w = ptx::mbar_wait(ptx::smem_addr(&x.vfull[vs]), (uint32_t)((qq >> 1) & 1), p.status);
-      if (w) {
-        ptx::tc_fence_after();
-        const uint32_t vb = vaddr + (uint32_t)(vs * C::VTS);
-#pragma unroll
-        for (int mh = 0; mh < C::MH; ++mh) {
-          const uint32_t d = tmem + (uint32_t)(C::A2OFF + ((qq & 1) % C::A2BUF) * C::MH * C::KPAD + mh * C::KPAD);
-#pragma unroll
-          for (int kk = 0; kk < TS / 16; ++kk) {
-            const uint32_t ao = xaddr + (uint32_t)(mh * 2 * SLAB_V + kk * 2048);
-            const uint32_t bo = vb + (uint32_t)(kk * 2048);
-            const uint64_t ah = ptx::sw128_mnmajor_desc(ao, SLAB_V, 1024);
-            const uint64_t bh = ptx::sw128_mnmajor_desc(bo, SLAB_V, 1024);
-            ptx::mma_bf16(d, ah, bh, idesc2, kk ? 1u : 0u);
-            if (SPLIT) {
-              ptx::mma_bf16(d, ptx::sw128_mnmajor_desc(ao + C::XPART, SLAB_V, 1024), bh, idesc2, 1u);
-              ptx::mma_bf16(d, ah, ptx::sw128_mnmajor_desc(bo + C::VT, SLAB_V, 1024), idesc2, 1u);
-            }
-          }
-        }
-        ptx::mma_commit(ptx::smem_addr(&x.vempty[vs]));
-        ptx::mma_commit(ptx::smem_addr(&x.acc_full));
-      } else {
-        x.abort = 1;
-        ptx::mbar_arrive(ptx::smem_addr(&x.acc_full));
-      }
-    };
-    if (nsteps > 0 && tid == 0) issue(0);
-    __syncwarp();
-    for (int q = 0; q < nsteps && ok; ++q) {
+    EpiWait wait{&x.abort, p.status};
+    for (int q = 0; q < nsteps; ++q) {
       const int t = step_t(q);
+      const bool more = q + 1 < nsteps;
       // pixels of steps q + 1 .. q + PXS (the x of the next step needs them)
-      if ((q + 1) % PXS == 0 && q + 1 < nsteps) {
-        stage_pixels(st.px, p.pixels, n, B, b0, q + 1, nsteps, site_of);
-        epi_barrier();
-      }
-      const bool waited = ptx::mbar_wait(ptx::smem_addr(&x.acc_full), (uint32_t)(q & 1), p.status);
-      if (!__all_sync(0xffffffffu, waited)) x.abort = 1;
-      if (waited) {
-        ptx::tc_fence_after();
+      if ((q + 1) % PXS == 0 && more) stage_pixels<C::NEPI>(st.phi, p.pixels, n, B, b0, q + 1, nsteps, site_of);
+      if (more) load_factors(q + 1);
+      // g' and the next step's operand made of it; then, once the gradient
+      // product has read the x tile, the tile
+      wait(&x.acc_full[0], (uint32_t)(q & 1));
 #pragma unroll
-        for (int c = 0; c < C::HC; c += LDN) {
-          uint32_t u[LDN];
-          tmem_ld<LDN>(lane_base + (uint32_t)(c0 + c), u);
-          ptx::tmem_ld_wait();
+      for (int c = 0; c < C::HC; c += 16) {
+        uint32_t u[16];
+        ptx::tmem_ld_32x32b_x16(lane_base + (uint32_t)(c0 + c), u);
+        ptx::tmem_ld_wait();
 #pragma unroll
-          for (int e = 0; e < LDN; ++e) g[c + e] = __uint_as_float(u[e]);
-        }
-        if (C::A2BUF == 1) drain_grad(t, 0);
-        if (q + 1 < nsteps) write_xtile(q + 1);
+        for (int e = 0; e < 16; ++e) g[c + e] = __uint_as_float(u[e]);
       }
-      ptx::fence_proxy_async_smem();
-      ptx::tc_fence_before();
-      ok = ptx::named_barrier_or(1, NEPI, *(volatile int32_t*)&x.abort != 0) == false;
-      ptx::tc_fence_after();
-      if (tid == 0 && ok && q + 1 < nsteps) issue(q + 1);
-      __syncwarp();
+      if (more) make_x();
+      wait(&x.acc_full[1], (uint32_t)(q & 1));
+      if (C::A2BUF == 1 && !wait.dead) drain_grad(t, 0);
+      if (more) write_xtile();
       // with two accumulators this step's gradient is drained while the next
-      // step's products run (its buffer is rewritten two steps later, after
-      // the next barrier)
-      if (C::A2BUF == 2 && waited && ok) drain_grad(t, q & 1);
+      // step's products run (its buffer is rewritten by the products two
+      // steps on, which wait for this warp's next tile)
+      if (C::A2BUF == 2 && !wait.dead) drain_grad(t, q & 1);
     }
     if (live) {
 #pragma unroll
       for (int k = 0; k < C::HC; k += 4)
         *reinterpret_cast<float4*>(p.state[h] + (int64_t)b * CHI + c0 + k) = make_float4(g[k], g[k + 1], g[k + 2], g[k + 3]);
     }
-    if (tid == 0) {
-      ptx::mma_commit(ptx::smem_addr(&x.final_bar));
-      ptx::mbar_wait(ptx::smem_addr(&x.final_bar), 0u, p.status);
-    }
-    __syncwarp();
   }
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 0) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(x.tmem_base, C::ACOLS);
+    ptx::tmem_dealloc(tmem, C::ACOLS);
   }
 }
 
@@ -729,7 +902,7 @@ int launch_fwd(const ClsTcParams& p, cudaStream_t s) {
   const size_t smem = fwd_smem_bytes<CHI, SPLIT>();
   static std::atomic<uint64_t> attr{0};
   if (!smem_limit_once((const void*)cls_fwd_tc<CHI, SPLIT>, smem, &attr)) return TN_ERR_CUDA;
-  cls_fwd_tc<CHI, SPLIT><<<2 * p.ntiles, NTHREADS, smem, s>>>(p);
+  cls_fwd_tc<CHI, SPLIT><<<2 * p.ntiles, Cfg<CHI, SPLIT>::NTHREADS, smem, s>>>(p);
   return cudaGetLastError() == cudaSuccess ? TN_OK : TN_ERR_CUDA;
 }
 
@@ -741,7 +914,7 @@ int launch_adj(const ClsTcParams& p, cudaStream_t s) {
     const size_t smem = adj_smem_bytes<CHI, SPLIT>();
     static std::atomic<uint64_t> attr{0};
     if (!smem_limit_once((const void*)cls_adj_tc<CHI, SPLIT>, smem, &attr)) return TN_ERR_CUDA;
-    cls_adj_tc<CHI, SPLIT><<<2 * p.ntiles, NTHREADS, smem, s>>>(p);
+    cls_adj_tc<CHI, SPLIT><<<2 * p.ntiles, Cfg<CHI, SPLIT>::ATHREADS, smem, s>>>(p);
     return cudaGetLastError() == cudaSuccess ? TN_OK : TN_ERR_CUDA;
   }
 }
