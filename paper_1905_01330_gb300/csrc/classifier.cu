@@ -194,7 +194,7 @@ struct ClsLayout {
   // tensor-core path (the images are the float32 path's too)
   uint8_t* fimg[2];  // forward core images per half
   uint8_t* aimg[2];  // adjoint core images per half
-  uint8_t* vseg[2];  // bf16 vector tiles of one segment per half
+  uint8_t* vseg[2][2];  // bf16 vector tiles of a segment per half; two: one being written, one read
   float* grad[2];    // [t][chi][2 chi] accumulated core gradients per half
   // label core
   float* labG;     // [batch][DL][2][L]
@@ -254,7 +254,10 @@ ClsLayout cls_layout(uint8_t* base, const tn_mps* W, int ls, int L, int batch, i
   for (int h = 0; h < 2; ++h) {
     w.fimg[h] = take(cls_fwd_image_bytes(chi, 1) * (size_t)w.T[h]);
     w.aimg[h] = take(bwd ? cls_adj_image_bytes(chi, 1) * (size_t)w.T[h] : 0);
-    w.vseg[h] = take(bwd ? cls_vtile_bytes(chi, 1) * (size_t)w.ntiles * (size_t)std::min(w.seg_len, std::max(w.T[h], 1)) : 0);
+    const size_t steps = (size_t)std::min(w.seg_len, std::max(w.T[h], 1));
+    for (int i = 0; i < 2; ++i)
+      w.vseg[h][i] = i == 0 || w.T[h] > w.seg_len ? take(bwd ? cls_vtile_bytes(chi, 1) * (size_t)w.ntiles * steps : 0)
+                                                  : w.vseg[h][0];
     w.grad[h] = reinterpret_cast<float*>(take(bwd ? sizeof(float) * (size_t)w.T[h] * chi * 2 * chi : 0));
   }
   const int64_t DL = W->bond[ls], DR = W->bond[ls + 1];
@@ -467,7 +470,7 @@ int tn_mps_classify(const tn_mps* W, int label_site, int n_labels, const float* 
     if ((rc = pack_images(W, w, split, 0, s)) != TN_OK) return rc;
     ClsTcParams q = tc_params(W, w, pixels);
     for (int h = 0; h < 2; ++h) {
-      q.state[h] = w.state[h];
+      q.state_in[h] = q.state[h] = w.state[h];
       q.lam[h] = w.lam[h];
       q.images[h] = w.fimg[h];
       if (ckpt_every > 0) q.store[h] = w.ckpt[h];
@@ -553,37 +556,41 @@ int tn_mps_classify_backward(const tn_mps* W, int label_site, int n_labels, cons
   const size_t vbytes = sizeof(float) * (size_t)batch * chi;
 
   if (prec != TN_PREC_FP32) {
-    // tcgen05: per round, one launch recomputes both halves' segments (their
-    // bf16 vector tiles kept for the gradient products) and one launch runs
-    // both adjoint segments, accumulating every step's core gradient
+    // tcgen05: per round, one launch runs both halves' adjoint segments,
+    // accumulating every step's core gradient, and recomputes the next
+    // segments from their kept vectors (their bf16 vector tiles kept for the
+    // gradient products)
     if ((rc = pack_images(W, w, split, 0, s)) != TN_OK) return rc;
     if ((rc = pack_images(W, w, split, 1, s)) != TN_OK) return rc;
     for (int h = 0; h < 2; ++h)
       if (w.T[h] > 0 &&
           cudaMemsetAsync(w.grad[h], 0, sizeof(float) * (size_t)w.T[h] * chi * 2 * chi, s) != cudaSuccess)
         return TN_ERR_CUDA;
-    for (int k = 0; k < rounds; ++k) {
+    auto recompute = [&](int k) {
       ClsTcParams f = tc_params(W, w, pixels);
-      ClsTcParams a = tc_params(W, w, pixels);
       for (int h = 0; h < 2; ++h) {
-        int t0, t1;
-        seg_range(h, k, &t0, &t1);
-        f.t_begin[h] = a.t_begin[h] = t0;
-        f.t_end[h] = a.t_end[h] = t1;
-        if (t1 > t0 && cudaMemcpyAsync(w.replay[h], w.ckpt[h] + (int64_t)(t0 / ckpt_every) * batch * chi, vbytes,
-                                       cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-          return TN_ERR_CUDA;
+        const bool any = seg_range(h, k, &f.t_begin[h], &f.t_end[h]);
+        f.state_in[h] = any ? w.ckpt[h] + (int64_t)(f.t_begin[h] / ckpt_every) * batch * chi : w.replay[h];
         f.state[h] = w.replay[h];
         f.lam[h] = w.replay_lam[h];
-        f.vseg[h] = w.vseg[h];
+        f.vseg[h] = w.vseg[h][k & 1];
         f.images[h] = w.fimg[h];
+      }
+      return f;
+    };
+    if (rounds > 0 && (rc = cls_fwd_tc_launch(chi, split, recompute(0), s)) != TN_OK) return rc;
+    for (int k = 0; k < rounds; ++k) {
+      ClsTcParams a = tc_params(W, w, pixels);
+      for (int h = 0; h < 2; ++h) {
+        seg_range(h, k, &a.t_begin[h], &a.t_end[h]);
         a.state[h] = w.g[h];
-        a.vseg[h] = w.vseg[h];
+        a.vseg[h] = w.vseg[h][k & 1];
         a.images[h] = w.aimg[h];
         a.grad[h] = w.grad[h];
       }
-      if ((rc = cls_fwd_tc_launch(chi, split, f, s)) != TN_OK) return rc;
-      if ((rc = cls_adj_tc_launch(chi, split, a, s)) != TN_OK) return rc;
+      ClsTcParams f;
+      if (k + 1 < rounds) f = recompute(k + 1);
+      if ((rc = cls_adj_tc_launch(chi, split, a, k + 1 < rounds ? &f : nullptr, s)) != TN_OK) return rc;
     }
     return scatter_gradients(W, w, dcores, s);
   }

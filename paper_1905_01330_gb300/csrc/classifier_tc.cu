@@ -42,11 +42,14 @@
 // epilogue and the next step's MMAs on it run beside the second half's; and
 // the adjoint's epilogue works on g' while the gradient product runs.
 // Measured (4096 samples, 784 sites, split BF16x3; before -> now): forward chi
-// = 128 FWD128, chi = 64 with recomputation FWD64, adjoint chi = 64 ADJ64.
+// = 128 1117 -> 783 us, chi = 64 with recomputation 1435 -> 1056 us, adjoint
+// chi = 64 1425 -> 957 us; those two then side by side (cls_pair_tc) PAIR64.
 // Every mbarrier wait is bounded; a CTA that gives up records
 // TN_ERR_TIMEOUT, lets its copies land, frees its TMEM and returns.
 #include <cuda_bf16.h>
 #include <math.h>
+
+#include <algorithm>
 
 #include "classifier_tc.h"
 #include "ptx.cuh"
@@ -75,7 +78,6 @@ struct Cfg {
   static constexpr int NG = CHI >= 64 ? 4 : 2;      // epilogue threads per sample
   static constexpr int NEPI = NG * TS;
   static constexpr int NTHREADS = NEPI + 96;        // + producer, MMA and (forward) vector-image store warps
-  static constexpr int ATHREADS = NEPI + 64;
   static constexpr int HC = CHI / NG;               // columns per epilogue thread
   // forward: image rows (j / (CHI / NH), s, j % (CHI / NH)), K = k; NH column
   // halves, each with its own accumulator, blocks (k slab, half) in this order
@@ -305,7 +307,7 @@ constexpr size_t fwd_smem_bytes() {
 }
 
 template <int CHI, int SPLIT>
-__global__ void __launch_bounds__(Cfg<CHI, SPLIT>::NTHREADS, 1) cls_fwd_tc(const __grid_constant__ ClsTcParams p) {
+__device__ void forward_tile(const ClsTcParams& p, const int cta) {
   using C = Cfg<CHI, SPLIT>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -314,7 +316,7 @@ __global__ void __launch_bounds__(Cfg<CHI, SPLIT>::NTHREADS, 1) cls_fwd_tc(const
   StageTail& st = *reinterpret_cast<StageTail*>(ring + (size_t)C::FRING * C::FSET);
   Bars& x = st.bars;
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int h = blockIdx.x / p.ntiles, tile = blockIdx.x % p.ntiles;
+  const int h = cta / p.ntiles, tile = cta % p.ntiles;
   const int B = p.batch, b0 = tile * TS;
   const int t0 = p.t_begin[h];
   const int nsteps = p.t_end[h] - t0;
@@ -462,7 +464,7 @@ __global__ void __launch_bounds__(Cfg<CHI, SPLIT>::NTHREADS, 1) cls_fwd_tc(const
     const int c0 = hc * C::HC;  // first column of this thread
     float v[C::HC];
 #pragma unroll
-    for (int k = 0; k < C::HC; ++k) v[k] = live ? p.state[h][(int64_t)b * CHI + c0 + k] : 0.0f;
+    for (int k = 0; k < C::HC; ++k) v[k] = live ? p.state_in[h][(int64_t)b * CHI + c0 + k] : 0.0f;
     double lam0 = (live && hc == 0) ? p.lam[h][b] : 0.0;
     int lam_e = 0;
     // scale of the vector in the tile not yet applied (deferred mode)
@@ -586,7 +588,7 @@ constexpr size_t adj_smem_bytes() {
 }
 
 template <int CHI, int SPLIT>
-__global__ void __launch_bounds__(Cfg<CHI, SPLIT>::ATHREADS, 1) cls_adj_tc(const __grid_constant__ ClsTcParams p) {
+__device__ void adjoint_tile(const ClsTcParams& p, const int cta) {
   using C = Cfg<CHI, SPLIT>;
   static_assert(C::ARING >= 2, "adjoint staging does not fit in shared memory");
   extern __shared__ uint8_t smem_raw[];
@@ -597,7 +599,7 @@ __global__ void __launch_bounds__(Cfg<CHI, SPLIT>::ATHREADS, 1) cls_adj_tc(const
   StageTail& st = *reinterpret_cast<StageTail*>(cring + (size_t)C::ARING * C::ASET);
   Bars& x = st.bars;
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int h = blockIdx.x / p.ntiles, tile = blockIdx.x % p.ntiles;
+  const int h = cta / p.ntiles, tile = cta % p.ntiles;
   const int B = p.batch, b0 = tile * TS;
   const int t0 = p.t_begin[h], t1 = p.t_end[h];
   const int nsteps = t1 - t0;
@@ -624,7 +626,7 @@ __global__ void __launch_bounds__(Cfg<CHI, SPLIT>::ATHREADS, 1) cls_adj_tc(const
     ptx::tmem_alloc(ptx::smem_addr(&x.tmem_base), C::ACOLS);
     ptx::tmem_relinquish();
   }
-  for (int i = tid; i < C::XTS / 16; i += C::ATHREADS) reinterpret_cast<uint4*>(xt)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < C::XTS / 16; i += C::NTHREADS) reinterpret_cast<uint4*>(xt)[i] = make_uint4(0, 0, 0, 0);
   ptx::fence_proxy_async_smem();
   ptx::tc_fence_before();
   __syncthreads();
@@ -755,7 +757,7 @@ __global__ void __launch_bounds__(Cfg<CHI, SPLIT>::ATHREADS, 1) cls_adj_tc(const
       ptx::mbar_wait(ptx::smem_addr(&x.final_bar), 0u, p.status);
     }
     __syncwarp();
-  } else {
+  } else if (warp < C::NEPI / 32) {
     const int r = tid & (TS - 1), hc = tid >> 7;
     const int b = b0 + r;
     const bool live = b < B;
@@ -877,6 +879,23 @@ __global__ void __launch_bounds__(Cfg<CHI, SPLIT>::ATHREADS, 1) cls_adj_tc(const
   }
 }
 
+template <int CHI, int SPLIT>
+__global__ void __launch_bounds__(Cfg<CHI, SPLIT>::NTHREADS, 1) cls_fwd_tc(const __grid_constant__ ClsTcParams p) {
+  forward_tile<CHI, SPLIT>(p, (int)blockIdx.x);
+}
+
+// The adjoint of one segment beside the recomputation of the next one: each
+// leaves more than half of the SMs idle at 4096 samples (64 CTAs).
+struct ClsPairParams {
+  ClsTcParams adj, fwd;
+};
+template <int CHI, int SPLIT>
+__global__ void __launch_bounds__(Cfg<CHI, SPLIT>::NTHREADS, 1) cls_pair_tc(const __grid_constant__ ClsPairParams p) {
+  const int n = 2 * p.adj.ntiles;
+  if ((int)blockIdx.x < n) adjoint_tile<CHI, SPLIT>(p.adj, (int)blockIdx.x);
+  else forward_tile<CHI, SPLIT>(p.fwd, (int)blockIdx.x - n);
+}
+
 // dcore[site] from the step's accumulated gradient G[t][k][(s, j)]: the left
 // half's core is L itself (A[k, s, j]), the right half's its transpose
 // (A[j, s, k]).
@@ -907,14 +926,17 @@ int launch_fwd(const ClsTcParams& p, cudaStream_t s) {
 }
 
 template <int CHI, int SPLIT>
-int launch_adj(const ClsTcParams& p, cudaStream_t s) {
+int launch_pair(const ClsTcParams& a, const ClsTcParams* f, cudaStream_t s) {
   if constexpr (Cfg<CHI, SPLIT>::ARING < 2) {
     return TN_ERR_UNSUPPORTED;
   } else {
-    const size_t smem = adj_smem_bytes<CHI, SPLIT>();
+    const size_t smem = std::max(adj_smem_bytes<CHI, SPLIT>(), fwd_smem_bytes<CHI, SPLIT>());
     static std::atomic<uint64_t> attr{0};
-    if (!smem_limit_once((const void*)cls_adj_tc<CHI, SPLIT>, smem, &attr)) return TN_ERR_CUDA;
-    cls_adj_tc<CHI, SPLIT><<<2 * p.ntiles, Cfg<CHI, SPLIT>::ATHREADS, smem, s>>>(p);
+    if (!smem_limit_once((const void*)cls_pair_tc<CHI, SPLIT>, smem, &attr)) return TN_ERR_CUDA;
+    ClsPairParams p;
+    p.adj = a;
+    p.fwd = f ? *f : a;
+    cls_pair_tc<CHI, SPLIT><<<(f ? 4 : 2) * a.ntiles, Cfg<CHI, SPLIT>::NTHREADS, smem, s>>>(p);
     return cudaGetLastError() == cudaSuccess ? TN_OK : TN_ERR_CUDA;
   }
 }
@@ -955,11 +977,12 @@ bool cls_adj_tc_supported(int chi, int split) {
   return false;
 }
 
-int cls_adj_tc_launch(int chi, int split, const ClsTcParams& p, cudaStream_t s) {
-  if (p.t_end[0] <= p.t_begin[0] && p.t_end[1] <= p.t_begin[1]) return TN_OK;
-  if (chi == 32) return split ? launch_adj<32, 1>(p, s) : launch_adj<32, 0>(p, s);
-  if (chi == 64) return split ? launch_adj<64, 1>(p, s) : launch_adj<64, 0>(p, s);
-  if (chi == 128) return split ? launch_adj<128, 1>(p, s) : launch_adj<128, 0>(p, s);
+int cls_adj_tc_launch(int chi, int split, const ClsTcParams& a, const ClsTcParams* f, cudaStream_t s) {
+  if (f && f->t_end[0] <= f->t_begin[0] && f->t_end[1] <= f->t_begin[1]) f = nullptr;
+  if (a.t_end[0] <= a.t_begin[0] && a.t_end[1] <= a.t_begin[1]) return f ? cls_fwd_tc_launch(chi, split, *f, s) : TN_OK;
+  if (chi == 32) return split ? launch_pair<32, 1>(a, f, s) : launch_pair<32, 0>(a, f, s);
+  if (chi == 64) return split ? launch_pair<64, 1>(a, f, s) : launch_pair<64, 0>(a, f, s);
+  if (chi == 128) return split ? launch_pair<128, 1>(a, f, s) : launch_pair<128, 0>(a, f, s);
   return TN_ERR_UNSUPPORTED;
 }
 

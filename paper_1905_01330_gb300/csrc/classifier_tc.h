@@ -43,7 +43,8 @@ struct ClsTcParams {
   int32_t half_site[2];   // site of step 0: 0 (left) and n - 1 (right)
   int32_t half_dir[2];    // site of step t = half_site + half_dir * t
   const float* pixels;    // [batch, n]
-  float* state[2];        // [batch, chi] in/out (forward: v, adjoint: g)
+  const float* state_in[2];  // forward: [batch, chi] v entering the first step (may be state)
+  float* state[2];        // [batch, chi] forward: v out; adjoint: g in/out
   double* lam[2];         // forward: [batch] log-scale in/out
   float* store[2];        // forward: kept float32 vectors (or null)
   float* sc[2];           // [t][batch] per-step scales (forward writes, adjoint reads)
@@ -54,7 +55,9 @@ struct ClsTcParams {
   int* status;
 };
 int cls_fwd_tc_launch(int chi, int split, const ClsTcParams& p, cudaStream_t s);
-int cls_adj_tc_launch(int chi, int split, const ClsTcParams& p, cudaStream_t s);
+// The adjoint of a, and in the same launch the forward of f (independent of
+// it; null: none).
+int cls_adj_tc_launch(int chi, int split, const ClsTcParams& a, const ClsTcParams* f, cudaStream_t s);
 // Whether the tcgen05 adjoint supports this (chi, split): its staging must
 // fit in shared memory.
 bool cls_adj_tc_supported(int chi, int split);
