@@ -43,7 +43,7 @@
 // the adjoint's epilogue works on g' while the gradient product runs.
 // Measured (4096 samples, 784 sites, split BF16x3; before -> now): forward chi
 // = 128 1117 -> 783 us, chi = 64 with recomputation 1435 -> 1056 us, adjoint
-// chi = 64 1425 -> 957 us; those two then side by side (cls_pair_tc) PAIR64.
+// chi = 64 1425 -> 957 us; those two then side by side (cls_pair_tc, 14 segments) 2010 -> 1190 us.
 // Every mbarrier wait is bounded; a CTA that gives up records
 // TN_ERR_TIMEOUT, lets its copies land, frees its TMEM and returns.
 #include <cuda_bf16.h>
@@ -307,7 +307,7 @@ constexpr size_t fwd_smem_bytes() {
 }
 
 template <int CHI, int SPLIT>
-__device__ void forward_tile(const ClsTcParams& p, const int cta) {
+__device__ __forceinline__ void forward_tile(const ClsTcParams& p, const int cta) {
   using C = Cfg<CHI, SPLIT>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -470,14 +470,18 @@ __device__ void forward_tile(const ClsTcParams& p, const int cta) {
     // scale of the vector in the tile not yet applied (deferred mode)
     int e_prev = 0;
     const bool defer = p.vseg[h] == nullptr;
-    uint32_t vh[C::HC / 2], vl[C::HC / 2];
     const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     // v, split, as the next step's operand: a lane's row of tensor memory
     auto write_operand = [&]() {
 #pragma unroll
-      for (int k = 0; k < C::HC / 2; ++k) split_pair(v[2 * k], v[2 * k + 1], vh[k], vl[k]);
-      tmem_st<C::HC / 2>(lanes + (uint32_t)(C::VCOL + c0 / 2), vh);
-      if (SPLIT) tmem_st<C::HC / 2>(lanes + (uint32_t)(C::VCOL + C::KPAD / 2 + c0 / 2), vl);
+      for (int c = 0; c < C::HC; c += 16) {
+        uint32_t vh[8], vl[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) split_pair(v[c + 2 * k], v[c + 2 * k + 1], vh[k], vl[k]);
+        const uint32_t col = lanes + (uint32_t)(C::VCOL + (c0 + c) / 2);
+        ptx::tmem_st_32x32b_x8(col, vh);
+        if (SPLIT) ptx::tmem_st_32x32b_x8(col + C::KPAD / 2, vl);
+      }
       ptx::tmem_st_wait();
       warp_arrive(&x.ready[half]);
     };
@@ -487,9 +491,13 @@ __device__ void forward_tile(const ClsTcParams& p, const int cta) {
       for (int g8 = 0; g8 < C::HC / 8; ++g8) {
         const int col = c0 + g8 * 8;
         uint8_t* dst = vt + (col >> 6) * SLAB_V + sw128(r, (col >> 3) & 7);
-        *reinterpret_cast<uint4*>(dst) = make_uint4(vh[4 * g8], vh[4 * g8 + 1], vh[4 * g8 + 2], vh[4 * g8 + 3]);
-        if (SPLIT)
-          *reinterpret_cast<uint4*>(dst + C::VT) = make_uint4(vl[4 * g8], vl[4 * g8 + 1], vl[4 * g8 + 2], vl[4 * g8 + 3]);
+        uint4 hh, ll;
+        split_pair(v[8 * g8], v[8 * g8 + 1], hh.x, ll.x);
+        split_pair(v[8 * g8 + 2], v[8 * g8 + 3], hh.y, ll.y);
+        split_pair(v[8 * g8 + 4], v[8 * g8 + 5], hh.z, ll.z);
+        split_pair(v[8 * g8 + 6], v[8 * g8 + 7], hh.w, ll.w);
+        *reinterpret_cast<uint4*>(dst) = hh;
+        if (SPLIT) *reinterpret_cast<uint4*>(dst + C::VT) = ll;
       }
       ptx::fence_proxy_async_smem();
       warp_arrive(&x.image);
@@ -515,16 +523,14 @@ __device__ void forward_tile(const ClsTcParams& p, const int cta) {
       const float2 phi = st.phi[q % PXS][r];
       const float g0 = phi.x * ip, g1 = phi.y * ip;
       wait(&x.acc_full[half], (uint32_t)(q & 1));
-      {
-        uint32_t u0[C::HC], u1[C::HC];
 #pragma unroll
-        for (int c = 0; c < C::HC; c += 16) {
-          ptx::tmem_ld_32x32b_x16(acc + (uint32_t)c, u0 + c);
-          ptx::tmem_ld_32x32b_x16(acc + (uint32_t)(JH + c), u1 + c);
-        }
+      for (int c = 0; c < C::HC; c += 16) {
+        uint32_t u0[16], u1[16];
+        ptx::tmem_ld_32x32b_x16(acc + (uint32_t)c, u0);
+        ptx::tmem_ld_32x32b_x16(acc + (uint32_t)(JH + c), u1);
         ptx::tmem_ld_wait();
 #pragma unroll
-        for (int e = 0; e < C::HC; ++e) v[e] = g0 * __uint_as_float(u0[e]) + g1 * __uint_as_float(u1[e]);
+        for (int e = 0; e < 16; ++e) v[c + e] = g0 * __uint_as_float(u0[e]) + g1 * __uint_as_float(u1[e]);
       }
       if (C::NH == 2 && half == 1) warp_arrive(&x.drained);
       // the step's scale 2^e_t from the sample's largest |u_t| over its
@@ -588,7 +594,7 @@ constexpr size_t adj_smem_bytes() {
 }
 
 template <int CHI, int SPLIT>
-__device__ void adjoint_tile(const ClsTcParams& p, const int cta) {
+__device__ __forceinline__ void adjoint_tile(const ClsTcParams& p, const int cta) {
   using C = Cfg<CHI, SPLIT>;
   static_assert(C::ARING >= 2, "adjoint staging does not fit in shared memory");
   extern __shared__ uint8_t smem_raw[];
