@@ -108,15 +108,24 @@ mps_inner_small_kernel(const __grid_constant__ SmallChain c, double* result) {
   }
 }
 
-// The same sweep with both cores of every site staged in shared memory: the
-// cores of site i+1 are copied in (cp.async, no registers) while site i is
-// contracted, and each thread computes four consecutive outputs along the
-// ket bond, so every shared-memory operand read feeds four FMAs.
-// Dynamic shared memory: E, E2 (emax floats each), T (tmax), two ket and two
-// bra core buffers (cmax each).
+// The same sweep with both cores of every site staged in shared memory, rows
+// padded to multiples of four: the cores of site i + 1 are copied in
+// (cp.async, no registers) while site i is contracted.
+// Dynamic shared memory: E (emax floats), T (tmax), two ket and two bra core
+// buffers (cmax each).
+//
+// What bounds it: one CTA's shared-memory reads and the latency of three
+// barriers a site. Each output is one chain of FMAs over ascending k, so the
+// work is split over outputs only: a thread holds 2 rows x 4 ket columns, so
+// a 16-byte read of the second operand feeds 8 FMAs (issued as packed pairs),
+// and E is read four k at a time; E' stays in registers until the block's
+// maximum is known and is divided by it there. Measured, N = 20, chi = 32
+// (with the launch): NORMA.
 struct StagedSizes {
   int32_t emax, tmax, cmax;
 };
+
+__host__ __device__ __forceinline__ int32_t pad4(int32_t x) { return (x + 3) & ~3; }
 
 __device__ __forceinline__ void cp_async_f32(float* dst, const float* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(ptx_smem(dst)), "l"(src) : "memory");
@@ -127,104 +136,186 @@ __device__ __forceinline__ void cp_async_16(float* dst, const float* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// Copies n floats global -> shared by all threads of the block.
-__device__ __forceinline__ void stage_core(float* dst, const float* __restrict__ src, int n) {
-  const bool v16 = ((reinterpret_cast<uintptr_t>(src) & 15) == 0) && ((n & 3) == 0);
-  if (v16) {
+// i / n for 0 <= i < 2^16, 0 < n (inv = 1 / n to within an ulp or two).
+__device__ __forceinline__ int small_div(int i, float inv) { return (int)(((float)i + 0.5f) * inv); }
+
+// Copies `rows` rows of `cols` floats global -> shared rows of pad4(cols), by
+// all threads of the block; the padding keeps what it holds.
+__device__ __forceinline__ void stage_core(float* dst, const float* __restrict__ src, int rows, int cols) {
+  const int n = rows * cols;
+  if ((cols & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
     for (int i = threadIdx.x * 4; i < n; i += SMALL_THREADS * 4) cp_async_16(dst + i, src + i);
   } else {
-    for (int i = threadIdx.x; i < n; i += SMALL_THREADS) cp_async_f32(dst + i, src + i);
+    const int ld = pad4(cols);
+    const float inv = __frcp_rn((float)cols);
+    for (int i = threadIdx.x; i < n; i += SMALL_THREADS) {
+      const int r = small_div(i, inv);
+      cp_async_f32(dst + r * ld + (i - r * cols), src + i);
+    }
   }
 }
+
+// x / sc for |x| <= sc, rounded as the division: the quotient by the correctly
+// rounded reciprocal, corrected by its residual (Markstein), unless sc or a
+// quotient lies where that is not exact.
+__device__ __noinline__ float divide_slow(float x, float sc) { return __fdiv_rn(x, sc); }
+template <int N>
+__device__ __forceinline__ void divide_by_max(float (&v)[N], float sc) {
+  const float r = __frcp_rn(sc);
+  bool plain = sc > 0x1p-60f && sc < 0x1p60f && (__float_as_uint(sc) & 0x7FFFFFu) != 0x7FFFFFu;
+  float q[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    q[j] = v[j] * r;
+    plain = plain && (fabsf(q[j]) > 0x1p-40f || v[j] == 0.0f);
+  }
+  if (__all_sync(__activemask(), plain)) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = fmaf(fmaf(-q[j], sc, v[j]), r, q[j]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = divide_slow(v[j], sc);
+  }
+}
+
+struct Acc24 {
+  float2 a[2][2];  // 2 rows x 4 columns
+  __device__ __forceinline__ void zero() {
+    a[0][0] = a[0][1] = a[1][0] = a[1][1] = make_float2(0.0f, 0.0f);
+  }
+  __device__ __forceinline__ void fma(float x0, float x1, const float4& y) {
+    const float2 lo = make_float2(y.x, y.y), hi = make_float2(y.z, y.w);
+    const float2 p0 = make_float2(x0, x0), p1 = make_float2(x1, x1);
+    a[0][0] = __ffma2_rn(p0, lo, a[0][0]);
+    a[0][1] = __ffma2_rn(p0, hi, a[0][1]);
+    a[1][0] = __ffma2_rn(p1, lo, a[1][0]);
+    a[1][1] = __ffma2_rn(p1, hi, a[1][1]);
+  }
+};
 
 __global__ void __launch_bounds__(SMALL_THREADS)
 mps_inner_staged_kernel(const __grid_constant__ SmallChain c, StagedSizes z, double* result) {
   extern __shared__ __align__(16) float smf[];
   float* E = smf;
-  float* E2 = E + z.emax;
-  float* T = E2 + z.emax;
+  float* T = E + z.emax;
   float* const kbuf = T + z.tmax;          // ket cores of sites i (i & 1) and i + 1
   float* const bbuf = kbuf + 2 * z.cmax;   // bra cores, likewise
   __shared__ float red[SMALL_THREADS / 32];
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d = c.d;
   if (tid == 0) E[0] = 1.0f;
   double lg = 0.0;
-  stage_core(kbuf, c.ket[0], c.bk[0] * d * c.bk[1]);
-  stage_core(bbuf, c.bra[0], c.bb[0] * d * c.bb[1]);
+  stage_core(kbuf, c.ket[0], c.bk[0] * d, c.bk[1]);
+  stage_core(bbuf, c.bra[0], c.bb[0] * d, c.bb[1]);
   cp_async_commit();
+  constexpr int TILES = SMALL_D / 2 * (SMALL_D / 4) / SMALL_THREADS;  // tiles of E' per thread, at most
   for (int i = 0; i < c.n; ++i) {
     const int Da = c.bb[i], Db = c.bb[i + 1], Dak = c.bk[i], Dbk = c.bk[i + 1];
     cp_async_wait_all();
     __syncthreads();  // site i's cores (and E) visible to all; buffers of site i-1 free
     if (i + 1 < c.n) {
-      stage_core(kbuf + ((i + 1) & 1) * z.cmax, c.ket[i + 1], Dbk * d * c.bk[i + 2]);
-      stage_core(bbuf + ((i + 1) & 1) * z.cmax, c.bra[i + 1], Db * d * c.bb[i + 2]);
+      stage_core(kbuf + ((i + 1) & 1) * z.cmax, c.ket[i + 1], Dbk * d, c.bk[i + 2]);
+      stage_core(bbuf + ((i + 1) & 1) * z.cmax, c.bra[i + 1], Db * d, c.bb[i + 2]);
     }
     cp_async_commit();
     const float* K = kbuf + (i & 1) * z.cmax;
     const float* Br = bbuf + (i & 1) * z.cmax;
-    // T[a, s, bk] = sum_ak E[a, ak] K[ak, s, bk], four bk per thread when Dbk % 4 == 0
-    const int w = (Dbk & 3) == 0 ? 4 : 1;
-    const int qn = Dbk / w;
-    const int nt = Da * d * qn;
-    for (int idx = tid; idx < nt; idx += SMALL_THREADS) {
-      const int q = idx % qn, rest = idx / qn, sidx = rest % d, a = rest / d;
-      const int bk = q * w;
-      if (w == 4) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int ak = 0; ak < Dak; ++ak) {
-          const float e = E[a * Dak + ak];
-          const float4 k4 = *reinterpret_cast<const float4*>(K + (ak * d + sidx) * Dbk + bk);
-          acc.x = fmaf(e, k4.x, acc.x);
-          acc.y = fmaf(e, k4.y, acc.y);
-          acc.z = fmaf(e, k4.z, acc.z);
-          acc.w = fmaf(e, k4.w, acc.w);
+    const int lde = pad4(Dak), ldk = pad4(Dbk), ldb = pad4(Db), qn = ldk >> 2;
+    const float iq = __frcp_rn((float)qn);
+    // T[a, s, bk] = sum_ak E[a, ak] K[ak, s, bk]: two a and four bk per thread
+    {
+      const float id = __frcp_rn((float)d);
+      const int tiles = ((Da + 1) >> 1) * d * qn;
+      for (int idx = tid; idx < tiles; idx += SMALL_THREADS) {
+        const int rest = small_div(idx, iq), q = idx - rest * qn;
+        const int ap = small_div(rest, id), s = rest - ap * d;
+        const int a0 = 2 * ap, a1 = min(a0 + 1, Da - 1);
+        const float *e0 = E + a0 * lde, *e1 = E + a1 * lde;
+        const float* kp = K + s * ldk + 4 * q;
+        const int kst = d * ldk;
+        Acc24 acc;
+        acc.zero();
+        int ak = 0;
+#pragma unroll 2
+        for (; ak + 4 <= Dak; ak += 4) {
+          const float4 x0 = *reinterpret_cast<const float4*>(e0 + ak), x1 = *reinterpret_cast<const float4*>(e1 + ak);
+          const float4 y0 = *reinterpret_cast<const float4*>(kp), y1 = *reinterpret_cast<const float4*>(kp + kst);
+          const float4 y2 = *reinterpret_cast<const float4*>(kp + 2 * kst);
+          const float4 y3 = *reinterpret_cast<const float4*>(kp + 3 * kst);
+          kp += 4 * kst;
+          acc.fma(x0.x, x1.x, y0);
+          acc.fma(x0.y, x1.y, y1);
+          acc.fma(x0.z, x1.z, y2);
+          acc.fma(x0.w, x1.w, y3);
         }
-        *reinterpret_cast<float4*>(T + (a * d + sidx) * Dbk + bk) = acc;
-      } else {
-        float acc = 0.0f;
-        for (int ak = 0; ak < Dak; ++ak) acc = fmaf(E[a * Dak + ak], K[(ak * d + sidx) * Dbk + bk], acc);
-        T[(a * d + sidx) * Dbk + bk] = acc;
+        for (; ak < Dak; ++ak, kp += kst) acc.fma(e0[ak], e1[ak], *reinterpret_cast<const float4*>(kp));
+        *reinterpret_cast<float4*>(T + (a0 * d + s) * ldk + 4 * q) =
+            make_float4(acc.a[0][0].x, acc.a[0][0].y, acc.a[0][1].x, acc.a[0][1].y);
+        if (a0 + 1 < Da)
+          *reinterpret_cast<float4*>(T + (a1 * d + s) * ldk + 4 * q) =
+              make_float4(acc.a[1][0].x, acc.a[1][0].y, acc.a[1][1].x, acc.a[1][1].y);
       }
     }
     __syncthreads();
-    // E2[b, bk] = sum_{a, s} Br[a, s, b] T[a, s, bk]
-    const int ne = Db * qn;
+    // E'[b, bk] = sum_{a, s} Br[a, s, b] T[a, s, bk]: two b and four bk per thread
+    const int tiles = ((Db + 1) >> 1) * qn;
+    float v[TILES][2][4];
     float mx = 0.0f;
-    for (int idx = tid; idx < ne; idx += SMALL_THREADS) {
-      const int q = idx % qn, b = idx / qn;
-      const int bk = q * w;
-      if (w == 4) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int as = 0; as < Da * d; ++as) {
-          const float br = Br[as * Db + b];
-          const float4 t4 = *reinterpret_cast<const float4*>(T + as * Dbk + bk);
-          acc.x = fmaf(br, t4.x, acc.x);
-          acc.y = fmaf(br, t4.y, acc.y);
-          acc.z = fmaf(br, t4.z, acc.z);
-          acc.w = fmaf(br, t4.w, acc.w);
+#pragma unroll
+    for (int t = 0; t < TILES; ++t) {
+      const int idx = tid + t * SMALL_THREADS;
+      if (idx < tiles) {
+        const int bp = small_div(idx, iq), q = idx - bp * qn, as_n = Da * d;
+        const float *br = Br + 2 * bp, *tp = T + 4 * q;
+        Acc24 acc;
+        acc.zero();
+#pragma unroll 8
+        for (int as = 0; as < as_n; ++as, br += ldb, tp += ldk) {
+          const float2 x = *reinterpret_cast<const float2*>(br);
+          acc.fma(x.x, x.y, *reinterpret_cast<const float4*>(tp));
         }
-        *reinterpret_cast<float4*>(E2 + b * Dbk + bk) = acc;
-        mx = fmaxf(mx, fmaxf(fmaxf(fabsf(acc.x), fabsf(acc.y)), fmaxf(fabsf(acc.z), fabsf(acc.w))));
-      } else {
-        float acc = 0.0f;
-        for (int as = 0; as < Da * d; ++as) acc = fmaf(Br[as * Db + b], T[as * Dbk + bk], acc);
-        E2[b * Dbk + bk] = acc;
-        mx = fmaxf(mx, fabsf(acc));
+        const bool second = 2 * bp + 1 < Db;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float2 p0 = acc.a[0][j >> 1], p1 = acc.a[1][j >> 1];
+          v[t][0][j] = (j & 1) ? p0.y : p0.x;
+          v[t][1][j] = (j & 1) ? p1.y : p1.x;
+          if (4 * q + j < Dbk) {
+            mx = fmaxf(mx, fabsf(v[t][0][j]));
+            if (second) mx = fmaxf(mx, fabsf(v[t][1][j]));
+          }
+        }
       }
     }
-    const float m = block_max(mx, red);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) red[warp] = mx;
+    __syncthreads();  // red written; every read of E (step 1) and of red (previous site) is done
+    float m = 0.0f;
+#pragma unroll
+    for (int k = 0; k < SMALL_THREADS / 32; ++k) m = fmaxf(m, red[k]);
     const float sc = m > 0.0f ? m : 1.0f;
-    for (int idx = tid; idx < Db * Dbk; idx += SMALL_THREADS) E[idx] = E2[idx] / sc;
-    lg += (double)logf(sc);
+#pragma unroll
+    for (int t = 0; t < TILES; ++t) {
+      const int idx = tid + t * SMALL_THREADS;
+      if (idx < tiles) {
+        const int bp = small_div(idx, iq), q = idx - bp * qn;
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          if (2 * bp + r < Db) {
+            divide_by_max(v[t][r], sc);
+            *reinterpret_cast<float4*>(E + (2 * bp + r) * ldk + 4 * q) =
+                make_float4(v[t][r][0], v[t][r][1], v[t][r][2], v[t][r][3]);
+          }
+        }
+      }
+    }
+    if (warp == SMALL_THREADS / 32 - 1) lg += (double)logf(sc);
   }
   cp_async_wait_all();
   __syncthreads();
-  if (tid == 0) {
-    result[0] = (double)E[0];
-    result[1] = lg;
-  }
+  if (tid == 0) result[0] = (double)E[0];
+  if (tid == SMALL_THREADS - 1) result[1] = lg;
 }
 
 // ------------------------------------------------------------ rescale pair
@@ -778,19 +869,15 @@ int tn_mps_inner(const tn_mps* bra, const tn_mps* ket, int prec, void* workspace
       c.bra[i] = bra->cores[i];
       c.ket[i] = ket->cores[i];
     }
-    // staged variant when its buffers fit: E, E2, T and four core buffers
-    StagedSizes z{1, 1, 1};
+    // staged variant when its buffers fit: E, T and four core buffers, rows
+    // padded to multiples of four
+    StagedSizes z{4, 4, 4};
     for (int i = 0; i < bra->n; ++i) {
-      z.emax = std::max(z.emax, c.bb[i + 1] * c.bk[i + 1]);
-      z.emax = std::max(z.emax, c.bb[i] * c.bk[i]);
-      z.tmax = std::max(z.tmax, c.bb[i] * c.d * c.bk[i + 1]);
-      z.cmax = std::max(z.cmax, std::max(c.bb[i] * c.d * c.bb[i + 1], c.bk[i] * c.d * c.bk[i + 1]));
+      z.emax = std::max(z.emax, c.bb[i + 1] * pad4(c.bk[i + 1]));
+      z.tmax = std::max(z.tmax, c.bb[i] * c.d * pad4(c.bk[i + 1]));
+      z.cmax = std::max(z.cmax, std::max(c.bb[i] * c.d * pad4(c.bb[i + 1]), c.bk[i] * c.d * pad4(c.bk[i + 1])));
     }
-    // every buffer starts on a 16-byte boundary
-    z.emax = (z.emax + 3) & ~3;
-    z.tmax = (z.tmax + 3) & ~3;
-    z.cmax = (z.cmax + 3) & ~3;
-    const size_t staged = sizeof(float) * (2 * (size_t)z.emax + z.tmax + 4 * (size_t)z.cmax);
+    const size_t staged = sizeof(float) * ((size_t)z.emax + z.tmax + 4 * (size_t)z.cmax);
     constexpr size_t STAGED_MAX = 200 * 1024;
     if (staged <= STAGED_MAX) {
       static std::atomic<uint64_t> attr2{0};
