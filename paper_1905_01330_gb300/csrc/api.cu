@@ -153,7 +153,8 @@ int tn_sync_status(void* stream) {
 
 int tn_contract(const tn_tensor* A, const int* legsA, const tn_tensor* B, const int* legsB,
                 int nshared, const tn_tensor* C, int prec, void* stream) {
-  return tn::contract_internal(A, legsA, B, legsB, nshared, C, prec, static_cast<cudaStream_t>(stream));
+  return tn::contract_internal(A, legsA, B, legsB, nshared, C, prec, static_cast<cudaStream_t>(stream), nullptr, 0,
+                               true);
 }
 
 size_t tn_contract_workspace_bytes(const tn_tensor* A, const int* legsA, const tn_tensor* B, const int* legsB,
@@ -169,20 +170,20 @@ size_t tn_contract_workspace_bytes(const tn_tensor* A, const int* legsA, const t
 int tn_contract_ws(const tn_tensor* A, const int* legsA, const tn_tensor* B, const int* legsB, int nshared,
                    const tn_tensor* C, int prec, void* workspace, size_t bytes, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (!workspace) return tn::contract_internal(A, legsA, B, legsB, nshared, C, prec, s);
+  if (!workspace) return tn::contract_internal(A, legsA, B, legsB, nshared, C, prec, s, nullptr, 0, true);
   if (reinterpret_cast<uintptr_t>(workspace) & 255) return TN_ERR_WORKSPACE;
   if (prec == TN_PREC_BF16 || prec == TN_PREC_BF16X3) {
     const size_t need = tn_contract_workspace_bytes(A, legsA, B, legsB, nshared, C, prec);
     if (bytes < need) return TN_ERR_WORKSPACE;
   }
-  return tn::contract_internal(A, legsA, B, legsB, nshared, C, prec, s, workspace, bytes);
+  return tn::contract_internal(A, legsA, B, legsB, nshared, C, prec, s, workspace, bytes, true);
 }
 
 }  // extern "C"
 
 int tn::contract_internal(const tn_tensor* A, const int* legsA, const tn_tensor* B, const int* legsB,
                           int nshared, const tn_tensor* C, int prec, cudaStream_t s, void* scratch,
-                          size_t scratch_bytes) {
+                          size_t scratch_bytes, bool any_order) {
   if (prec != TN_PREC_FP32 && prec != TN_PREC_BF16 && prec != TN_PREC_BF16X3) return TN_ERR_ARG;
   ContractDesc d;
   int rc = plan_contract(A, legsA, B, legsB, nshared, C, &d);
@@ -195,6 +196,8 @@ int tn::contract_internal(const tn_tensor* A, const int* legsA, const tn_tensor*
   // against an environment): one thread per result column
   if (prec == TN_PREC_FP32 && d.M <= SKINNY_MAX && d.K <= SKINNY_MAX && d.N >= 4096)
     return launch_contract_skinny(d, s);
+  if (prec == TN_PREC_FP32 && outer_ok(d)) return launch_outer(d, s);
+  if (prec == TN_PREC_FP32 && any_order && matvec_ok(d)) return launch_matvec(d, s);
   plan_units(&d, min_units_single());
   if (prec == TN_PREC_FP32) plan_simt(&d, SimtPlan::alone);
   if (prec != TN_PREC_FP32 && scratch && packed_single_bytes(d, prec) <= scratch_bytes)

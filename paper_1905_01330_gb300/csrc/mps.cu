@@ -120,7 +120,7 @@ mps_inner_small_kernel(const __grid_constant__ SmallChain c, double* result) {
 // a 16-byte read of the second operand feeds 8 FMAs (issued as packed pairs),
 // and E is read four k at a time; E' stays in registers until the block's
 // maximum is known and is divided by it there. Measured, N = 20, chi = 32
-// (with the launch): NORMA.
+// (kernel): 66 -> 47 us.
 struct StagedSizes {
   int32_t emax, tmax, cmax;
 };

@@ -63,6 +63,12 @@ int launch_contract_skinny(const ContractDesc& d, cudaStream_t stream);
 // The same over an uploaded list of `count` such contractions (max_n: the
 // largest N among them).
 int launch_contract_skinny_grouped(const ContractDesc* descs, int count, int64_t max_n, cudaStream_t stream);
+// FP32: outer products (K <= 8; sums in the general kernel's order) and a
+// matrix times a vector (M or N = 1; its own order).
+bool outer_ok(const ContractDesc& d);
+int launch_outer(const ContractDesc& d, cudaStream_t stream);
+bool matvec_ok(const ContractDesc& d);
+int launch_matvec(const ContractDesc& d, cudaStream_t stream);
 
 // Tile shapes of the kernels (used by the planner to count tiles).
 constexpr int TC_BM = 128, TC_BN = 128;
@@ -101,7 +107,7 @@ int launch_zero(const ZeroRange* ranges, int n, cudaStream_t stream);
 // contraction runs as pack + GEMM; otherwise on the single-pass kernels.
 int contract_internal(const tn_tensor* A, const int* legsA, const tn_tensor* B, const int* legsB,
                       int nshared, const tn_tensor* C, int prec, cudaStream_t stream, void* scratch = nullptr,
-                      size_t scratch_bytes = 0);
+                      size_t scratch_bytes = 0, bool any_order = false);
 
 // tn_group_plan_create; allow_packed = false keeps BF16 / BF16X3 plans on
 // the single-launch kernel, whose workspace holds only the work list.

@@ -346,6 +346,34 @@ def test_fp32_tiles_and_gathers(tn, M, N, K):
                 check(tn.contract(At, la, Bt, lb, prec="fp32"), A, la, B, lb, "fp32")
 
 
+@pytest.mark.parametrize("M,N,K", [(16, 1024, 1), (129, 130, 2), (64, 256, 7), (333, 65, 8), (1024, 1024, 2)])
+def test_fp32_outer_products(tn, M, N, K):
+    # K <= 8: edges of the 64 x 64 tiles, both layouts of both operands, the
+    # unaligned result rows of an odd N
+    for ta in (0, 1):
+        for tb in (0, 1):
+            A, B = rand(71 + ta, (K, M) if ta else (M, K)), rand(81 + tb, (K, N) if tb else (N, K))
+            la, lb = [0 if ta else 1], [0 if tb else 1]
+            r = tn.contract(torch.from_numpy(A).cuda(), la, torch.from_numpy(B).cuda(), lb, prec="fp32")
+            check(r, A, la, B, lb, "fp32")
+
+
+@pytest.mark.parametrize("R,K1,K2", [(64, 8, 8), (65, 1, 67), (1024, 32, 32), (260, 5, 40), (7000, 2, 1024)])
+def test_fp32_matrix_times_vector(tn, R, K1, K2):
+    # one free index on one side only: the vector first or second, the
+    # matrix's free leg or a shared leg of unit stride, two shared legs, in
+    # 16-byte or single loads, one to eight parts of the shared index
+    x = rand(91, (K1, K2))
+    xt = torch.from_numpy(x).cuda()
+    for shape, legs in [((K1, K2, R), [0, 1]), ((R, K1, K2), [1, 2]), ((K1, R, K2), [0, 2])]:
+        for off in (0, 1):
+            M = rand(92, shape)
+            Mt = torch.zeros(shape[0], shape[1], shape[2] + 3 * off, device="cuda")[:, :, off:off + shape[2]]
+            Mt.copy_(torch.from_numpy(M))
+            check(tn.contract(xt, [0, 1], Mt, legs, prec="fp32"), x, [0, 1], M, legs, "fp32")
+            check(tn.contract(Mt, legs, xt, [0, 1], prec="fp32"), M, legs, x, [0, 1], "fp32")
+
+
 def test_fp32_group_with_long_k_ranges(tn):
     # a group large enough that a contraction of 20 or more tiles keeps its k
     # ranges in one unit (chains of 2048 added up in shared memory), beside
