@@ -32,7 +32,6 @@ namespace tn {
 namespace {
 
 constexpr int SMALL_D = 64;      // largest bond of the one-CTA sweep
-constexpr int64_t PERSISTENT_MAX_BOND = 512;  // largest bond of the persistent energy sweep
 constexpr int SMALL_PHYS = 4;    // largest physical dim of the one-CTA sweep
 constexpr int SMALL_MAXN = 1024; // sites passed by value to the one-CTA sweep
 constexpr int SMALL_THREADS = 256;

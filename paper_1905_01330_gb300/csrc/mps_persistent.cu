@@ -40,6 +40,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <vector>
 
 #include "mpo_step.cuh"
 #include "packed.h"
@@ -105,6 +106,8 @@ struct __align__(8) PsAux {
   uint64_t final_bar;     // every MMA of the launch is complete
   uint32_t tmem_base;
   volatile int32_t abort;
+  uint4 unit[2][2][4];      // batch, per half and parity of the unit: its chain's words,
+  unsigned unit_max[2][4];  // the bits of the largest |L| entering, and the chain's number
   float4 Ws[2][8][4];     // per half: the site's W' as [(w, s)][(w', s') by reader], zero past the MPO
 };
 
@@ -199,6 +202,8 @@ struct PsPack {
   uint8_t* hi;
   int64_t lo;  // byte distance to the lo plane, 0: none
   int32_t cols, slabs, K, Db, ns;  // ns: d for (i), 1 for (iii)
+  int32_t run;  // (iii) with shared index (s', a'): Da, and the core rows run by d; else 0
+  int32_t d;
 };
 
 __device__ __forceinline__ uint4 pick(bool c, const uint4& a, const uint4& b) {
@@ -226,8 +231,21 @@ __device__ __forceinline__ void pack_unit(const PsPack& q, uint32_t u) {
 #pragma unroll 2
   for (int g = 0; g < 8; g += 2) {
     float v[16];
+    if (q.run == 0) {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = 8 * g + j < kn ? __ldg(src + (8 * g + j) * ks) : 0.0f;
+      for (int j = 0; j < 16; ++j) v[j] = 8 * g + j < kn ? __ldg(src + (8 * g + j) * ks) : 0.0f;
+    } else {
+      // k = s' Da + a': row a' d + s'
+      int s1 = (k0 + 8 * g) / q.run, a1 = k0 + 8 * g - s1 * q.run;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        v[j] = 8 * g + j < kn ? __ldg(q.src + ((int64_t)a1 * q.d + s1) * q.Db + b) : 0.0f;
+        if (++a1 == q.run) {
+          a1 = 0;
+          ++s1;
+        }
+      }
+    }
     uint4 h[2], l[2];
     split8(v, h[0], l[0]);
     split8(v + 8, h[1], l[1]);
@@ -294,33 +312,66 @@ struct PsGemm {
   int32_t units, tq, slabs, cols;
   uint32_t magic;
 };
-__device__ __forceinline__ void unit_tile(const PsGemm& g, int u, int& tpi, int& tqi) {
-  tpi = g.magic ? (int)__umulhi((uint32_t)u, g.magic) : u;
-  tqi = u - tpi * g.tq;
-}
+
+// What the roles of a phase need of a unit.
+struct UnitOps {  // the copies
+  const uint8_t *P, *Q;
+  int64_t P_lo, Q_lo;
+  int32_t slabs, cols;
+};
+struct UnitShape {
+  int32_t slabs, cols, tpi, tqi;
+  bool cross;  // BF16X3: lo*hi before hi*lo
+};
+
+// The units of one chain's phase: CTA c takes c, c + grid, ...
+struct OneUnits {
+  const PsGemm& g;
+  int u;
+  __device__ __forceinline__ explicit OneUnits(const PsGemm& gg) : g(gg), u((int)blockIdx.x) {}
+  __device__ __forceinline__ bool valid() const { return u < g.units; }
+  __device__ __forceinline__ void advance() { u += (int)gridDim.x; }
+  __device__ __forceinline__ UnitShape shape() const {
+    UnitShape s;
+    s.slabs = g.slabs;
+    s.cols = g.cols;
+    s.tpi = g.magic ? (int)__umulhi((uint32_t)u, g.magic) : u;
+    s.tqi = u - s.tpi * g.tq;
+    s.cross = false;
+    return s;
+  }
+  __device__ __forceinline__ UnitOps ops() const {
+    const UnitShape s = shape();
+    return UnitOps{g.P + (size_t)s.tpi * g.slabs * PS_BLOCK, g.Q + (size_t)s.tqi * g.slabs * (size_t)(g.cols * 128),
+                   g.P_lo, g.Q_lo, g.slabs, g.cols};
+  }
+  __device__ __forceinline__ void stage(int) const {}
+};
 
 // Pipeline positions kept across the phases of the launch: slabs through the
 // stage ring (the copying thread's and the MMA issuer's own counts) and
 // accumulator chunks (issuer and draining warps).
+struct PsRing {
+  int32_t stages, stage_bytes;
+  int* status;
+};
 struct PsPipe {
   uint32_t slab, stage, phase, gc;  // phase: rounds of the ring, stage: slab % stages
 };
 
 // Copies of a GEMM phase (one thread): every slab of its units into the ring,
 // as soon as its stage is free. A stage holds P hi, (P lo,) Q hi, (Q lo).
-template <int SPLIT>
-__device__ bool gemm_copy(const PsGemm& g, const PsParams& p, uint32_t stage0, PsAux& x, PsPipe& pp) {
-  const uint32_t S = (uint32_t)p.stages, stage_bytes = (uint32_t)p.stage_bytes;
-  const uint32_t qbytes = (uint32_t)g.cols * 128u, qoff = (SPLIT ? 2 : 1) * PS_BLOCK;
+template <int SPLIT, class Units>
+__device__ __forceinline__ bool gemm_copy(Units it, const PsRing& rg, uint32_t stage0, PsAux& x, PsPipe& pp) {
+  const uint32_t S = (uint32_t)rg.stages, stage_bytes = (uint32_t)rg.stage_bytes, qoff = (SPLIT ? 2 : 1) * PS_BLOCK;
   uint32_t st = pp.stage, round = pp.phase;
-  for (int u = blockIdx.x; u < g.units; u += gridDim.x) {
-    int tpi, tqi;
-    unit_tile(g, u, tpi, tqi);
-    const uint8_t* pb = g.P + (size_t)tpi * g.slabs * PS_BLOCK;
-    const uint8_t* qb = g.Q + (size_t)tqi * g.slabs * qbytes;
+  for (; it.valid(); it.advance()) {
+    const UnitOps g = it.ops();
+    const uint8_t *pb = g.P, *qb = g.Q;
+    const uint32_t qbytes = (uint32_t)g.cols * 128u;
     for (int ks = 0; ks < g.slabs; ++ks, pb += PS_BLOCK, qb += qbytes) {
       // the stage's previous contents: read by MMAs that must be complete
-      if (round && !ptx::mbar_wait(ptx::smem_addr(&x.empty[st]), (round - 1u) & 1u, p.status)) return false;
+      if (round && !ptx::mbar_wait(ptx::smem_addr(&x.empty[st]), (round - 1u) & 1u, rg.status)) return false;
       const uint32_t full = ptx::smem_addr(&x.full[st]), dst = stage0 + st * stage_bytes;
       ptx::mbar_arrive_expect_tx(full, (SPLIT ? 2u : 1u) * (PS_BLOCK + qbytes));
       ptx::bulk_copy_g2s(dst, pb, PS_BLOCK, full);
@@ -345,13 +396,11 @@ __device__ bool gemm_copy(const PsGemm& g, const PsParams& p, uint32_t stage0, P
 // thread took it 2,000 cycles a slab, the MMAs themselves 500): the warp runs
 // the loop together and one lane issues, so that the descriptors stay in
 // uniform registers.
-template <int SPLIT>
-__device__ bool gemm_issue(const PsGemm& g, const PsParams& p, uint32_t stage0, PsAux& x, uint32_t tmem, PsPipe& pp) {
-  const uint32_t S = (uint32_t)p.stages, stage_bytes = (uint32_t)p.stage_bytes;
-  int* status = p.status;
-  const uint32_t idesc = ptx::idesc_bf16_f32(128, g.cols, 1, 0);
-  const uint32_t qbytes = (uint32_t)g.cols * 128u, qoff = (SPLIT ? 2 : 1) * PS_BLOCK;
-  const int nks = g.slabs, chunk = SPLIT ? PS_KC : nks;
+template <int SPLIT, class Units>
+__device__ __forceinline__ bool gemm_issue(Units it, const PsRing& rg, uint32_t stage0, PsAux& x, uint32_t tmem,
+                                           PsPipe& pp) {
+  const uint32_t S = (uint32_t)rg.stages, stage_bytes = (uint32_t)rg.stage_bytes, qoff = (SPLIT ? 2 : 1) * PS_BLOCK;
+  int* status = rg.status;
   uint32_t st = pp.stage, phase = pp.phase;
   auto wait_full = [&]() {
     const bool w = ptx::mbar_wait(ptx::smem_addr(&x.full[st]), phase, status);
@@ -359,7 +408,10 @@ __device__ bool gemm_issue(const PsGemm& g, const PsParams& p, uint32_t stage0, 
     ptx::tc_fence_after();
     return true;
   };
-  for (int u = blockIdx.x; u < g.units; u += gridDim.x) {
+  for (; it.valid(); it.advance()) {
+    const UnitShape g = it.shape();
+    const uint32_t idesc = ptx::idesc_bf16_f32(128, g.cols, 1, 0), qbytes = (uint32_t)g.cols * 128u;
+    const int nks = g.slabs, chunk = SPLIT ? PS_KC : nks;
     for (int k0 = 0; k0 < nks; k0 += chunk) {
       // the accumulator this chunk overwrites has been drained
       const uint32_t b = pp.gc & 1u, dt = tmem + b * 128u;
@@ -374,8 +426,10 @@ __device__ bool gemm_issue(const PsGemm& g, const PsParams& p, uint32_t stage0, 
         auto step = [&](int kk) {
           ptx::mma_bf16_lo(dt, ph + kk * 128u, qh + kk * 2u, idesc, (ks != k0 || kk != 0) ? 1u : 0u);
           if (SPLIT) {
-            ptx::mma_bf16_lo(dt, ph + kk * 128u, ql + kk * 2u, idesc, 1u);
-            ptx::mma_bf16_lo(dt, pl + kk * 128u, qh + kk * 2u, idesc, 1u);
+            const uint32_t c0 = g.cross ? pl : ph, d0 = g.cross ? qh : ql;
+            const uint32_t c1 = g.cross ? ph : pl, d1 = g.cross ? ql : qh;
+            ptx::mma_bf16_lo(dt, c0 + kk * 128u, d0 + kk * 2u, idesc, 1u);
+            ptx::mma_bf16_lo(dt, c1 + kk * 128u, d1 + kk * 2u, idesc, 1u);
           }
         };
         if (ptx::elect_one()) {
@@ -413,14 +467,15 @@ __device__ bool gemm_issue(const PsGemm& g, const PsParams& p, uint32_t stage0, 
 // sums into float32 registers. fin(row tile, column tile, values) finishes a
 // unit; it is entered by a whole half together, and a wait that ran out in one
 // of its warps ends all four.
-template <int SPLIT, class Fin>
-__device__ bool gemm_drain(const PsGemm& g, PsAux& x, uint32_t tmem, PsPipe& pp, int* status, Fin fin) {
+template <int SPLIT, class Units, class Fin>
+__device__ __forceinline__ bool gemm_drain(Units it, PsAux& x, uint32_t tmem, PsPipe& pp, int* status, Fin fin) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int quad = warp & 3, half = (warp - PS_EPI0) >> 2, ng = g.cols >> 5;
-  const int nks = g.slabs, nchunks = SPLIT ? (nks + PS_KC - 1) / PS_KC : 1;
-  for (int u = blockIdx.x; u < g.units; u += gridDim.x) {
-    int tpi, tqi;
-    unit_tile(g, u, tpi, tqi);
+  const int quad = warp & 3, half = (warp - PS_EPI0) >> 2;
+  for (int i = 0; it.valid(); it.advance(), ++i) {
+    const UnitShape g = it.shape();
+    const int ng = g.cols >> 5;
+    const int nks = g.slabs, nchunks = SPLIT ? (nks + PS_KC - 1) / PS_KC : 1;
+    it.stage(i & 1);
     float acc[64];
 #pragma unroll
     for (int j = 0; j < 64; ++j) acc[j] = 0.0f;
@@ -448,7 +503,7 @@ __device__ bool gemm_drain(const PsGemm& g, PsAux& x, uint32_t tmem, PsPipe& pp,
       if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&x.acc_empty[b]));
       ++pp.gc;
     }
-    fin(tpi, tqi, acc);
+    fin(g.tpi, g.tqi, i & 1, acc);
   }
   return true;
 }
@@ -464,6 +519,7 @@ struct PsStepII {
   int64_t lo;    // byte distance to the lo plane, 0: none
   float inv;     // 2^-e
   int32_t Da, Db, DbP, wa, wb, d, slabs, lg;
+  int32_t ps, pa;  // shared index of (iii): s' ps + a' pa
   uint32_t rd;   // m / d = m * rd >> 16 (m < 8)
 };
 
@@ -531,7 +587,7 @@ __device__ __forceinline__ void step_ii_rounds(const PsStepII& q, const float4 (
               v[2 * j + 1] = o[i][j].y * q.inv;
             }
             const int w2 = (int)((uint32_t)m * q.rd >> 16), s2 = m - w2 * d;
-            const int32_t r0 = w2 * q.DbP + b0 + (hb + ib) * 8, kx = a * d + s2;
+            const int32_t r0 = w2 * q.DbP + b0 + (hb + ib) * 8, kx = a * q.pa + s2 * q.ps;
             const size_t off = ((size_t)(r0 >> 7) * q.slabs + (kx >> 6)) * PS_BLOCK +
                                mn_block_chunk((r0 & 127) >> 3, kx & 63);
             uint4 h, l;
@@ -590,6 +646,45 @@ __device__ __forceinline__ void pack_next(const PsNext& q, int half, int tpi, in
   }
 }
 
+// Copies still in flight land, every MMA completes, then TMEM is freed.
+__device__ __forceinline__ void wind_down(PsAux& x, const PsPipe& pp, const PsRing& rg, uint32_t tmem) {
+  const int warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    const uint32_t S = (uint32_t)rg.stages;
+    for (uint32_t q = pp.slab < S ? 0u : pp.slab - S; q < pp.slab; ++q)
+      ptx::mbar_wait(ptx::smem_addr(&x.full[q % S]), (q / S) & 1u, rg.status);
+  }
+  __syncwarp();
+  if (warp == 1) {
+    if (ptx::elect_one()) ptx::mma_commit(ptx::smem_addr(&x.final_bar));  // the lane that issued the MMAs
+    __syncwarp();
+    ptx::mbar_wait(ptx::smem_addr(&x.final_bar), 0u, rg.status);
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, PS_TMEM_COLS);
+  }
+}
+
+// Each half's copy of W' (its readers wait at the half's barriers), by the
+// order step_ii_rounds reads it: the four channels m of a thread's pass (m =
+// mh, mh + ms, ...) as one 16-byte word.
+__device__ __forceinline__ void load_site_mpo(const float* W, int wa, int wb, int d, PsAux& x, int half) {
+  const int tid = threadIdx.x - PS_EPI0 * 32, lms = (d <= 2 ? 6 : 7) - group_shift(wa);
+  if ((tid & (PS_GROUP - 1)) >= 64) return;
+  const int k = (tid >> 3) & 7, m = tid & 7;
+  float v = 0.0f;
+  if (k < wa * d && m < wb * d) {
+    const int w = k / d, sk = k - w * d, w2 = m / d, s2 = m - w2 * d;
+    v = __ldg(W + ((w * wb + w2) * d + sk) * d + s2);
+  }
+  float* row = reinterpret_cast<float*>(x.Ws[half][k]);
+  row[lms == 0 ? m : (m & ((1 << lms) - 1)) * 4 + (m >> lms)] = v;
+  if (lms == 2) row[(m & 3) * 4 + 2 + (m >> 2)] = 0.0f;
+}
+
 // The whole sweep. Grid: one CTA per SM (cooperative launch).
 template <int SPLIT>
 __global__ void __launch_bounds__(PS_THREADS, 1) expect_persistent_kernel(const __grid_constant__ PsParams p) {
@@ -623,6 +718,7 @@ __global__ void __launch_bounds__(PS_THREADS, 1) expect_persistent_kernel(const 
   const int32_t d = p.d, half = (warp - PS_EPI0) >> 2;
   const int64_t Lp_lo = SPLIT ? p.Lp_lo : 0, T2p_lo = SPLIT ? p.T2p_lo : 0;
   PsPipe pp{0u, 0u, 0u, 0u};
+  const PsRing rg{p.stages, p.stage_bytes, p.status};
   uint32_t epoch = 0;
   // (0) every site's core in the two operand layouts, and the first
   // environment (1 in each channel) as the first site's operand
@@ -640,7 +736,7 @@ __global__ void __launch_bounds__(PS_THREADS, 1) expect_persistent_kernel(const 
     if (third) k -= c1;
     const PsTiles& tt = st.t[third];
     pack_unit(PsPack{st.A, p.Cp + (size_t)tt.off * 1024, p.Cp_lo, tt.cols, tt.slabs, third ? d * st.Da : st.Da, st.Db,
-                     third ? 1 : d},
+                     third ? 1 : d, 0, d},
               k);
   }
   {
@@ -669,26 +765,13 @@ __global__ void __launch_bounds__(PS_THREADS, 1) expect_persistent_kernel(const 
     g.P_lo = p.Lp_lo;
     g.Q_lo = p.Cp_lo;
     if (threadIdx.x == 0) {
-      if (!gemm_copy<SPLIT>(g, p, stage0, x, pp)) x.abort = 1;
+      if (!gemm_copy<SPLIT>(OneUnits(g), rg, stage0, x, pp)) x.abort = 1;
     } else if (warp == 1) {
-      if (!gemm_issue<SPLIT>(g, p, stage0, x, tmem, pp)) x.abort = 1;
+      if (!gemm_issue<SPLIT>(OneUnits(g), rg, stage0, x, tmem, pp)) x.abort = 1;
     } else if (warp >= PS_EPI0) {
       const int tid = threadIdx.x - PS_EPI0 * 32;
-      // each half's copy of W' (its readers wait at the half's barriers), by
-      // the order step_ii_rounds reads it: the four channels m of a thread's
-      // pass (m = mh, mh + ms, ...) as one 16-byte word
-      const int lg = group_shift(wa), lms = (d <= 2 ? 6 : 7) - lg;
-      if ((tid & (PS_GROUP - 1)) < 64) {
-        const int k = (tid >> 3) & 7, m = tid & 7;
-        float v = 0.0f;
-        if (k < wa * d && m < wb * d) {
-          const int w = k / d, sk = k - w * d, w2 = m / d, s2 = m - w2 * d;
-          v = __ldg(p.Wx + st.woff + ((w * wb + w2) * d + sk) * d + s2);
-        }
-        const int ms1 = (1 << lms) - 1;
-        reinterpret_cast<float*>(x.Ws[half][k])[lms == 0 ? m : (m & ms1) * 4 + (m >> lms)] = v;
-        if (lms == 2) reinterpret_cast<float*>(x.Ws[half][k])[(m & 3) * 4 + 2 + (m >> 2)] = 0.0f;
-      }
+      load_site_mpo(p.Wx + st.woff, wa, wb, d, x, half);
+      const int lg = group_shift(wa);
       int e = 0;
       if (i > 0) e = pow2_exponent(__uint_as_float(__ldcg(p.bits + i)));
       if (i > 0 && blockIdx.x == 0 && tid == 0) *p.lg += (double)e * 0.69314718055994530942;
@@ -704,10 +787,12 @@ __global__ void __launch_bounds__(PS_THREADS, 1) expect_persistent_kernel(const 
       q.d = d;
       q.slabs = slabs3;
       q.lg = lg;
+      q.ps = 1;
+      q.pa = d;
       q.rd = (uint32_t)(65536 + d - 1) / (uint32_t)d;
       const int cells = (int)((uint32_t)(g.cols >> 5) * q.rd >> 16);
       uint8_t* mine = staged + half * PS_STAGED;
-      const bool done = gemm_drain<SPLIT>(g, x, tmem, pp, p.status, [&](int tpi, int tqi, const float* acc) {
+      const bool done = gemm_drain<SPLIT>(OneUnits(g), x, tmem, pp, p.status, [&](int tpi, int tqi, int, const float* acc) {
         if (d <= 2) step_ii_rounds<2>(q, x.Ws[half], mine, half, cells, tpi, tqi, acc);
         else step_ii_rounds<1>(q, x.Ws[half], mine, half, cells, tpi, tqi, acc);
       });
@@ -723,9 +808,9 @@ __global__ void __launch_bounds__(PS_THREADS, 1) expect_persistent_kernel(const 
     const bool last = i + 1 == p.n;
     const int32_t slabsn = ceil_div(Db, 64);
     if (threadIdx.x == 0) {
-      if (!gemm_copy<SPLIT>(g, p, stage0, x, pp)) x.abort = 1;
+      if (!gemm_copy<SPLIT>(OneUnits(g), rg, stage0, x, pp)) x.abort = 1;
     } else if (warp == 1) {
-      if (!gemm_issue<SPLIT>(g, p, stage0, x, tmem, pp)) x.abort = 1;
+      if (!gemm_issue<SPLIT>(OneUnits(g), rg, stage0, x, tmem, pp)) x.abort = 1;
     } else if (warp >= PS_EPI0) {
       float mx = 0.0f;
       PsNext q;
@@ -737,7 +822,7 @@ __global__ void __launch_bounds__(PS_THREADS, 1) expect_persistent_kernel(const 
       q.lg = group_shift(wb);
       q.slabs = slabsn;
       q.cols = g.cols;
-      const bool done = gemm_drain<SPLIT>(g, x, tmem, pp, p.status, [&](int tpi, int tqi, const float* acc) {
+      const bool done = gemm_drain<SPLIT>(OneUnits(g), x, tmem, pp, p.status, [&](int tpi, int tqi, int, const float* acc) {
         if (!last) {
           pack_next(q, half, tpi, tqi, acc, mx);
         } else if (tqi == 0 && half == 0) {
@@ -764,24 +849,268 @@ __global__ void __launch_bounds__(PS_THREADS, 1) expect_persistent_kernel(const 
     p.result[2] = (double)__ldcg(L + 1);
     p.result[3] = __ldcg(p.lg);
   }
-  // wind down: copies still in flight land, every MMA completes, then TMEM is freed
-  if (threadIdx.x == 0) {
-    const uint32_t S = (uint32_t)p.stages;
-    for (uint32_t q = pp.slab < S ? 0u : pp.slab - S; q < pp.slab; ++q)
-      ptx::mbar_wait(ptx::smem_addr(&x.full[q % S]), (q / S) & 1u, p.status);
+  wind_down(x, pp, rg, tmem);
+}
+
+// ------------------------------------------------------------ many chains
+// The same sweep for a batch of chains with one MPO: every phase works on the
+// units of all of them, in lists the host made (largest first, dealt out to
+// the CTAs back and forth), so the device-wide barriers, the copies' latency
+// and the ragged tiles of a site are shared. Warps 2 and 3 pack the next
+// site's cores meanwhile, into the other of two regions. Sums run in the order
+// of the grouped contractions: (iii)'s shared index is (s', a'), and where
+// those would have the core as the first operand of (i) the cross terms of
+// BF16x3 swap places.
+struct PbChain {   // a chain at a site
+  const float* A;  // core (Da, d, Db), row-major
+  uint32_t unit0;  // its first pack unit of the site
+  int16_t Da, Db;
+  PsTiles t[2];    // (i), (iii); off: in the site's region
+  uint32_t lp, lp_lo, t2, t2_lo;  // packed L and T2 (hi planes and distances to lo), in 1024 bytes
+};
+static_assert(sizeof(PbChain) == 64, "loaded as four 16-byte words");
+
+struct PbUnit {
+  uint16_t chain;
+  uint8_t tpi, tqi, slabs, cols16, cross, pad;
+};
+static_assert(sizeof(PbUnit) == 8, "");
+
+struct PbParams {
+  int32_t n, d, count;
+  int32_t stages, stage_bytes;
+  const float* Wx;
+  uint8_t* base;          // of the packed regions
+  uint8_t* Cp[2];         // packed cores of a site (even, odd)
+  int64_t Cp_lo;
+  const PbChain* chains;  // [site][chain]
+  const PbUnit* units;
+  const int32_t* first;   // [site][phase][CTA]: its first unit (one more at the end)
+  float* const* last;     // per chain: its last environment (one value per channel)
+  unsigned* bits;         // [site - 1][chain]: largest |L| entering the site
+  double* lg;
+  unsigned* bar;
+  int* status;
+  int32_t woff[PS_MAX_SITES];
+  uint32_t pack[PS_MAX_SITES];  // pack units of the site
+  int8_t w[PS_MAX_SITES + 1];   // extended MPO bonds
+};
+
+// This CTA's units of a phase.
+struct ListUnits {
+  const PbUnit* u;
+  const PbUnit* end;
+  const PbChain* chains;
+  const PbParams& p;
+  int phase, site;
+  uint4 (*slot)[4];      // draining half: the chain's words, for fin
+  unsigned* slot_max;
+  uint2 cur;
+  __device__ __forceinline__ ListUnits(const PbParams& pp, int st, int ph, uint4 (*sl)[4] = nullptr,
+                                       unsigned* mx = nullptr)
+      : p(pp), phase(ph), site(st), slot(sl), slot_max(mx) {
+    const int32_t* f = pp.first + ((size_t)st * 2 + ph) * gridDim.x + blockIdx.x;
+    u = pp.units + __ldg(f);
+    end = pp.units + __ldg(f + 1);
+    chains = pp.chains + (size_t)st * pp.count;
+    load();
   }
-  __syncwarp();
+  __device__ __forceinline__ void load() {
+    cur = u < end ? __ldg(reinterpret_cast<const uint2*>(u)) : make_uint2(0u, 0u);
+  }
+  __device__ __forceinline__ bool valid() const { return u < end; }
+  __device__ __forceinline__ void advance() {
+    ++u;
+    load();
+  }
+  __device__ __forceinline__ UnitShape shape() const {
+    return UnitShape{(int32_t)(cur.y & 0xFF), (int32_t)((cur.y >> 8) & 0xFF) * 16, (int32_t)((cur.x >> 16) & 0xFF),
+                     (int32_t)(cur.x >> 24), ((cur.y >> 16) & 1) != 0};
+  }
+  __device__ __forceinline__ UnitOps ops() const {
+    const UnitShape s = shape();
+    const uint4* c = reinterpret_cast<const uint4*>(chains + (cur.x & 0xFFFF));
+    const uint4 r = __ldg(c + 3);                       // lp, lp_lo, t2, t2_lo
+    const uint32_t off = __ldg(&chains[cur.x & 0xFFFF].t[phase].off);
+    const size_t P = (size_t)(phase ? r.z : r.x) * 1024;
+    return UnitOps{p.base + P + (size_t)s.tpi * s.slabs * PS_BLOCK,
+                   p.Cp[site & 1] + (size_t)off * 1024 + (size_t)s.tqi * s.slabs * (size_t)(s.cols * 128),
+                   (int64_t)(phase ? r.w : r.y) * 1024, p.Cp_lo, s.slabs, s.cols};
+  }
+  // the chain's words into the half's slot (the half's barrier before fin makes them visible)
+  __device__ __forceinline__ void stage(int which) const {
+    const int t = threadIdx.x & (PS_GROUP - 1), k = (int)(cur.x & 0xFFFF);
+    if (t < 4) slot[which][t] = __ldg(reinterpret_cast<const uint4*>(chains + k) + t);
+    if (t == 4) slot_max[2 * which] = site > 0 ? __ldcg(p.bits + (size_t)(site - 1) * p.count + k) : 0u;
+    if (t == 5) slot_max[2 * which + 1] = (unsigned)k;
+  }
+};
+
+// Pack units [e0, e1) of a site's cores, by `nwarps` warps.
+__device__ __forceinline__ void pack_site(const PbParams& p, int site, uint32_t e0, uint32_t e1, uint32_t wid,
+                                          uint32_t nwarps) {
+  const PbChain* chains = p.chains + (size_t)site * p.count;
+  for (uint32_t e = e0 + wid; e < e1; e += nwarps) {
+    int lo = 0, hi = p.count - 1;  // the chain whose units hold e
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (__ldg(&chains[mid].unit0) <= e) lo = mid;
+      else hi = mid - 1;
+    }
+    const PbChain& c = chains[lo];
+    uint32_t k = e - c.unit0;
+    const uint32_t c1 = pack_units(c.t[0]);
+    const int third = k >= c1;
+    if (third) k -= c1;
+    const PsTiles& tt = c.t[third];
+    pack_unit(PsPack{c.A, p.Cp[site & 1] + (size_t)tt.off * 1024, p.Cp_lo, tt.cols, tt.slabs,
+                     third ? p.d * c.Da : c.Da, c.Db, third ? 1 : p.d, third ? c.Da : 0, p.d},
+              k);
+  }
+}
+
+template <int SPLIT>
+__global__ void __launch_bounds__(PS_THREADS, 1) expect_batch_kernel(const __grid_constant__ PbParams p) {
+  extern __shared__ uint8_t ps_smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(ps_smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* staged = smem + PS_RING;
+  PsAux& x = *reinterpret_cast<PsAux*>(staged + 2 * PS_STAGED);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int st = 0; st < p.stages; ++st) {
+      ptx::mbar_init(ptx::smem_addr(&x.full[st]), 1);
+      ptx::mbar_init(ptx::smem_addr(&x.empty[st]), 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      ptx::mbar_init(ptx::smem_addr(&x.acc_full[b]), 1);
+      ptx::mbar_init(ptx::smem_addr(&x.acc_empty[b]), PS_EPI);
+    }
+    ptx::mbar_init(ptx::smem_addr(&x.final_bar), 1);
+    x.abort = 0;
+    ptx::fence_mbar_init();
+  }
   if (warp == 1) {
-    if (ptx::elect_one()) ptx::mma_commit(ptx::smem_addr(&x.final_bar));  // the lane that issued the MMAs
-    __syncwarp();
-    ptx::mbar_wait(ptx::smem_addr(&x.final_bar), 0u, p.status);
+    ptx::tmem_alloc(ptx::smem_addr(&x.tmem_base), PS_TMEM_COLS);
+    ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
   __syncthreads();
-  if (warp == 1) {
-    ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem, PS_TMEM_COLS);
+  ptx::tc_fence_after();
+  const uint32_t tmem = x.tmem_base, stage0 = ptx::smem_addr(smem);
+  const int32_t d = p.d, half = (warp - PS_EPI0) >> 2;
+  PsPipe pp{0u, 0u, 0u, 0u};
+  const PsRing rg{p.stages, p.stage_bytes, p.status};
+  uint32_t epoch = 0;
+  // (0) the first site's cores, and the first environments: 1 in each channel
+  pack_site(p, 0, 0u, p.pack[0], blockIdx.x * (PS_THREADS / 32) + warp, gridDim.x * (PS_THREADS / 32));
+  for (int c = blockIdx.x; c < p.count; c += gridDim.x) {
+    const PbChain& ch = p.chains[c];
+    uint8_t* hi = p.base + (size_t)ch.lp * 1024;
+    const int lg = group_shift(p.w[0]);
+    for (int e = threadIdx.x; e < 1024; e += PS_THREADS) {  // one block: row (w, 0) at shared index 0
+      const int kk = e & 63, mg = e >> 6, w = (mg * 8) >> lg;
+      const bool one = kk == 0 && w < p.w[0] && (w << lg) == mg * 8;
+      *reinterpret_cast<uint4*>(hi + mn_block_chunk(mg, kk)) = make_uint4(one ? 0x3F80u : 0u, 0u, 0u, 0u);
+      if (SPLIT) *reinterpret_cast<uint4*>(hi + (size_t)ch.lp_lo * 1024 + mn_block_chunk(mg, kk)) = make_uint4(0u, 0u, 0u, 0u);
+    }
   }
+  bool ok = grid_barrier(p.bar, epoch, p.status, ptx::kWaitLimitNs, &x.abort);
+  const uint32_t bw = blockIdx.x * 2 + warp - 2, nbw = gridDim.x * 2;  // the packing warps
+  for (int i = 0; i < p.n && ok; ++i) {
+    const int32_t wa = p.w[i], wb = p.w[i + 1];
+    const bool last = i + 1 == p.n;
+    // (B) T1 and, from its tiles, T2 = 2^-e W' T1
+    if (threadIdx.x == 0) {
+      if (!gemm_copy<SPLIT>(ListUnits(p, i, 0), rg, stage0, x, pp)) x.abort = 1;
+    } else if (warp == 1) {
+      if (!gemm_issue<SPLIT>(ListUnits(p, i, 0), rg, stage0, x, tmem, pp)) x.abort = 1;
+    } else if (warp >= PS_EPI0) {
+      load_site_mpo(p.Wx + p.woff[i], wa, wb, d, x, half);
+      uint8_t* mine = staged + half * PS_STAGED;
+      const uint32_t rd = (uint32_t)(65536 + d - 1) / (uint32_t)d;
+      const bool done = gemm_drain<SPLIT>(
+          ListUnits(p, i, 0, x.unit[half], x.unit_max[half]), x, tmem, pp, p.status,
+          [&](int tpi, int tqi, int which, const float* acc) {
+            const PbChain& ch = *reinterpret_cast<const PbChain*>(x.unit[half][which]);
+            const int e = i > 0 ? pow2_exponent(__uint_as_float(x.unit_max[half][2 * which])) : 0;
+            // one unit of the chain adds the site's exponent to its log-scale
+            if (i > 0 && tpi == 0 && tqi == 0 && threadIdx.x == PS_EPI0 * 32) {
+              double* l = p.lg + x.unit_max[half][2 * which + 1];
+              __stcg(l, __ldcg(l) + (double)e * 0.69314718055994530942);
+            }
+            PsStepII q;
+            q.hi = p.base + (size_t)ch.t2 * 1024;
+            q.lo = SPLIT ? (int64_t)ch.t2_lo * 1024 : 0;
+            q.inv = __int_as_float((127 - e) << 23);
+            q.Da = ch.Da;
+            q.Db = ch.Db;
+            q.DbP = pad16(ch.Db);
+            q.wa = wa;
+            q.wb = wb;
+            q.d = d;
+            q.slabs = ch.t[1].slabs;
+            q.lg = group_shift(wa);
+            q.ps = ch.Da;
+            q.pa = 1;
+            q.rd = rd;
+            const int cells = (int)((uint32_t)(ch.t[0].cols >> 5) * rd >> 16);
+            if (d <= 2) step_ii_rounds<2>(q, x.Ws[half], mine, half, cells, tpi, tqi, acc);
+            else step_ii_rounds<1>(q, x.Ws[half], mine, half, cells, tpi, tqi, acc);
+          });
+      if (!done) x.abort = 1;
+    } else if (warp >= 2) {
+      for (int c = blockIdx.x; c < p.count; c += gridDim.x) {
+        const PbChain& ch = p.chains[(size_t)i * p.count + c];
+        zero_shared_tail(p.base + (size_t)ch.t2 * 1024, SPLIT ? (int64_t)ch.t2_lo * 1024 : 0, ch.t[1].tp,
+                         ch.t[1].slabs, d * ch.Da, threadIdx.x - 64, 64);
+      }
+      if (!last) pack_site(p, i + 1, 0u, p.pack[i + 1] / 2, bw, nbw);
+    }
+    if (!(ok = grid_barrier(p.bar, epoch, p.status, ptx::kWaitLimitNs, &x.abort))) break;
+    // (D) L' from T2 and the core
+    if (threadIdx.x == 0) {
+      if (!gemm_copy<SPLIT>(ListUnits(p, i, 1), rg, stage0, x, pp)) x.abort = 1;
+    } else if (warp == 1) {
+      if (!gemm_issue<SPLIT>(ListUnits(p, i, 1), rg, stage0, x, tmem, pp)) x.abort = 1;
+    } else if (warp >= PS_EPI0) {
+      const bool done = gemm_drain<SPLIT>(
+          ListUnits(p, i, 1, x.unit[half], x.unit_max[half]), x, tmem, pp, p.status,
+          [&](int tpi, int tqi, int which, const float* acc) {
+            const PbChain& ch = *reinterpret_cast<const PbChain*>(x.unit[half][which]);
+            const unsigned k = x.unit_max[half][2 * which + 1];
+            PsNext q;
+            q.hi = p.base + (size_t)ch.lp * 1024;
+            q.lo = SPLIT ? (int64_t)ch.lp_lo * 1024 : 0;
+            q.Db = ch.Db;
+            q.DbP = pad16(ch.Db);
+            q.wb = wb;
+            q.lg = group_shift(wb);
+            q.slabs = ceil_div(ch.Db, 64);
+            q.cols = ch.t[1].cols;
+            if (!last) {
+              float mx = 0.0f;
+              pack_next(q, half, tpi, tqi, acc, mx);
+#pragma unroll
+              for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+              if (lane == 0 && mx > 0.0f) atomicMax(p.bits + (size_t)i * p.count + k, __float_as_uint(mx));
+            } else if (tqi == 0 && half == 0) {
+              // Db = 1: the last environment, one value per channel
+              const int row = tpi * 128 + (warp & 3) * 32 + lane, wq = row / q.DbP;
+              if (wq < wb && row == wq * q.DbP) p.last[k][wq] = acc[0];
+            }
+          });
+      if (!done) x.abort = 1;
+    } else if (warp >= 2 && !last) {
+      for (int c = blockIdx.x; c < p.count; c += gridDim.x) {
+        const PbChain& ch = p.chains[(size_t)i * p.count + c];
+        zero_shared_tail(p.base + (size_t)ch.lp * 1024, SPLIT ? (int64_t)ch.lp_lo * 1024 : 0,
+                         ceil_div(ch.Db, 1 << group_shift(wb)), ceil_div(ch.Db, 64), ch.Db, threadIdx.x - 64, 64);
+      }
+      pack_site(p, i + 1, p.pack[i + 1] / 2, p.pack[i + 1], bw, nbw);
+    }
+    if (!(ok = grid_barrier(p.bar, epoch, p.status, ptx::kWaitLimitNs, &x.abort))) break;
+  }
+  wind_down(x, pp, rg, tmem);
 }
 
 }  // namespace
@@ -855,6 +1184,39 @@ ExpectRegions expect_persistent_regions(const tn_mps* psi, const tn_mpo* H) {
   return r;
 }
 
+// Raises a sweep kernel's shared-memory limit, once per device.
+bool smem_limit_sweep(const void* fn, size_t smem) {
+  static std::atomic<uint64_t> attr[4];
+  const void* all[4] = {(const void*)expect_persistent_kernel<0>, (const void*)expect_persistent_kernel<1>,
+                        (const void*)expect_batch_kernel<0>, (const void*)expect_batch_kernel<1>};
+  for (int i = 0; i < 4; ++i)
+    if (all[i] == fn) return smem_limit_once(fn, smem, &attr[i]);
+  return false;
+}
+
+// One CTA per SM, all resident.
+template <class P>
+int launch_sweep(void (*fn)(const P), const P& p, cudaStream_t s) {
+  const size_t smem = 1024 + (size_t)PS_RING + 2 * PS_STAGED + sizeof(PsAux);
+  if (!smem_limit_sweep((const void*)fn, smem)) return TN_ERR_CUDA;
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, PS_THREADS, smem) != cudaSuccess ||
+      per_sm < 1)
+    return TN_ERR_UNSUPPORTED;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3((unsigned)device_sms());
+  cfg.blockDim = dim3(PS_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, p) == cudaSuccess ? TN_OK : TN_ERR_CUDA;
+}
+
 bool expect_persistent_ok(const tn_mps* psi, const tn_mpo* H, int prec) {
   if (prec != TN_PREC_BF16 && prec != TN_PREC_BF16X3) return false;
   if (psi->n > PS_MAX_SITES) return false;
@@ -925,29 +1287,209 @@ int expect_persistent(const tn_mps* psi, const tn_mpo* H, int prec, const Expect
   p.units = units;
   p.stage_bytes = (split ? 2 : 1) * (PS_BLOCK + widest * 128);
   p.stages = std::min(PS_RING / p.stage_bytes, PS_MAX_STAGES);
-  const size_t smem = 1024 + (size_t)PS_RING + 2 * PS_STAGED + sizeof(PsAux);
-  const void* fn = split ? (const void*)expect_persistent_kernel<1> : (const void*)expect_persistent_kernel<0>;
-  static std::atomic<uint64_t> attr[2];
-  if (!smem_limit_once(fn, smem, &attr[split ? 1 : 0])) return TN_ERR_CUDA;
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, PS_THREADS, smem) != cudaSuccess || per_sm < 1)
-    return TN_ERR_UNSUPPORTED;
   // the device-wide barrier counts arrivals from zero
   if (cudaMemsetAsync(w.bar, 0, sizeof(unsigned), s) != cudaSuccess) return TN_ERR_CUDA;
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((unsigned)sms);
-  cfg.blockDim = dim3(PS_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeCooperative;
-  at[0].val.cooperative = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  const cudaError_t e = split ? cudaLaunchKernelEx(&cfg, expect_persistent_kernel<1>, p)
-                              : cudaLaunchKernelEx(&cfg, expect_persistent_kernel<0>, p);
-  return e == cudaSuccess ? TN_OK : TN_ERR_CUDA;
+  return split ? launch_sweep(expect_persistent_kernel<1>, p, s) : launch_sweep(expect_persistent_kernel<0>, p, s);
+}
+
+// ------------------------------------------------------------ many chains
+namespace {
+
+// Unit costs in cycles, as in tile_cols.
+double unit_cost(int slabs, int cols) { return slabs * (512.0 + 4.0 * cols) + 20.0 * cols + 1000.0; }
+
+// Columns of a tile when many chains share the SMs: the least padded work.
+int batch_cols(int64_t total, int64_t K, int step) {
+  int best = step;
+  double best_cost = 1e30;
+  for (int c = step; c <= 128; c *= 2) {
+    const double cost = (double)ceil64(total, c) * unit_cost((int)ceil64(K, 64), c);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = c;
+    }
+  }
+  return best;
+}
+
+}  // namespace
+
+struct BatchSweep::Tables {
+  std::vector<PbChain> chains;
+  std::vector<PbUnit> units;
+  std::vector<int32_t> first;
+  std::vector<float*> last;
+  PbParams p;
+};
+
+BatchSweep::BatchSweep() : t(new Tables()) {}
+BatchSweep::~BatchSweep() { delete t; }
+
+bool batch_sweep_ok(const tn_mps* psis, int count, const tn_mpo* H, int prec) {
+  if (count > PB_MAX_CHAINS) return false;
+  for (int k = 0; k < count; ++k) {
+    if (!expect_persistent_ok(&psis[k], H, prec)) return false;
+    for (int i = 0; i <= psis[k].n; ++i)
+      if (psis[k].bond[i] > PERSISTENT_MAX_BOND) return false;
+  }
+  return true;
+}
+
+int BatchSweep::build(const tn_mps* psis, int cnt, const tn_mpo* H, int prec) {
+  count = cnt;
+  split = prec == TN_PREC_BF16X3;
+  const int n = psis[0].n, planes = split ? 2 : 1;
+  const int64_t d = psis[0].d;
+  const int grid = device_sms();
+  PbParams& p = t->p;
+  memset(&p, 0, sizeof(p));
+  p.n = n;
+  p.d = (int32_t)d;
+  p.count = count;
+  for (int i = 0; i <= n; ++i) p.w[i] = (int8_t)(H->bond[i] + 1);
+  // per chain: one packed environment and one packed T2, sized for its sites
+  size_t off = 0;
+  std::vector<size_t> lp((size_t)count), t2((size_t)count), lpb((size_t)count), t2b((size_t)count);
+  for (int k = 0; k < count; ++k) {
+    for (int i = 0; i < n; ++i) {
+      const int64_t Da = psis[k].bond[i], Db = psis[k].bond[i + 1];
+      lpb[k] = std::max(lpb[k], ps_bytes(ceil64(Da, int64_t(1) << group_shift(p.w[i])), Da, 128));
+      t2b[k] = std::max(t2b[k], ps_bytes(ceil64(p.w[i + 1] * (int64_t)pad16((int32_t)Db), 128), d * Da, 128));
+    }
+    lp[k] = off;
+    off += lpb[k] * planes;
+    t2[k] = off;
+    off += t2b[k] * planes;
+  }
+  if (off / 1024 > 0xFFFFFFFFull) return TN_ERR_UNSUPPORTED;
+  off_cores = off;
+  t->chains.resize((size_t)n * count);
+  t->first.assign((size_t)n * 2 * grid + 1, 0);
+  t->last.resize((size_t)count);
+  size_t cores = 0;
+  int widest = 0;
+  struct Cost {
+    double c;
+    PbUnit u;
+  };
+  std::vector<Cost> list;
+  for (int i = 0; i < n; ++i) {
+    size_t co = 0;
+    uint32_t pu = 0;
+    for (int k = 0; k < count; ++k) {
+      PbChain& c = t->chains[(size_t)i * count + k];
+      memset(&c, 0, sizeof(c));
+      const int64_t Da = psis[k].bond[i], Db = psis[k].bond[i + 1], DbP = pad16((int32_t)Db);
+      c.A = psis[k].cores[i];
+      c.Da = (int16_t)Da;
+      c.Db = (int16_t)Db;
+      c.unit0 = pu;
+      c.lp = (uint32_t)(lp[k] / 1024);
+      c.lp_lo = split ? (uint32_t)(lpb[k] / 1024) : 0u;
+      c.t2 = (uint32_t)(t2[k] / 1024);
+      c.t2_lo = split ? (uint32_t)(t2b[k] / 1024) : 0u;
+      for (int j = 0; j < 2; ++j) {
+        PsTiles& q = c.t[j];
+        const int64_t total = j ? DbP : d * DbP, K = j ? d * Da : Da;
+        const int cols = batch_cols(total, K, j ? 32 : (int)(32 * d));
+        q.off = (uint32_t)(co / 1024);
+        q.tp = (uint16_t)(j ? ceil64(p.w[i + 1] * DbP, 128) : ceil64(Da, int64_t(1) << group_shift(p.w[i])));
+        q.tq = (uint16_t)ceil64(total, cols);
+        q.cols = (int16_t)cols;
+        q.slabs = (int16_t)ceil64(K, 64);
+        co += ps_bytes(q.tq, K, cols);
+        pu += pack_units(q);
+        widest = std::max(widest, cols);
+      }
+    }
+    if (co / 1024 > 0xFFFFFFFFull) return TN_ERR_UNSUPPORTED;
+    cores = std::max(cores, co);
+    p.pack[i] = pu;
+    for (int j = 0; j < 2; ++j) {
+      list.clear();
+      for (int k = 0; k < count; ++k) {
+        const PbChain& c = t->chains[(size_t)i * count + k];
+        const PsTiles& q = c.t[j];
+        // the grouped contraction's first operand: the core when the
+        // environment has fewer than 128 rows and fewer than the core
+        const int64_t M = (int64_t)p.w[i] * c.Da, N = d * c.Db;
+        PbUnit u;
+        memset(&u, 0, sizeof(u));
+        u.chain = (uint16_t)k;
+        u.slabs = (uint8_t)q.slabs;
+        u.cols16 = (uint8_t)(q.cols / 16);
+        u.cross = j == 0 && N > M && M < 128;
+        for (int a = 0; a < q.tp; ++a)
+          for (int b = 0; b < q.tq; ++b) {
+            u.tpi = (uint8_t)a;
+            u.tqi = (uint8_t)b;
+            list.push_back(Cost{unit_cost(q.slabs, q.cols), u});
+          }
+      }
+      std::stable_sort(list.begin(), list.end(), [](const Cost& a, const Cost& b) { return a.c > b.c; });
+      // dealt out back and forth: CTA c's units lie together
+      for (int c = 0; c < grid; ++c) {
+        t->first[((size_t)i * 2 + j) * grid + c] = (int32_t)t->units.size();
+        for (size_t r = 0;; ++r) {
+          const size_t at = r * grid + (r & 1 ? (size_t)(grid - 1 - c) : (size_t)c);
+          if (r * (size_t)grid >= list.size()) break;
+          if (at < list.size()) t->units.push_back(list[at].u);
+        }
+      }
+    }
+  }
+  t->first.back() = (int32_t)t->units.size();
+  p.stage_bytes = planes * (PS_BLOCK + widest * 128);
+  p.stages = std::min(PS_RING / p.stage_bytes, PS_MAX_STAGES);
+  cores = align256(cores);
+  p.Cp_lo = split ? (int64_t)cores : 0;
+  site_bytes = cores * planes;
+  off = off_cores + 2 * site_bytes;
+  off_chains = off;
+  off += align256(sizeof(PbChain) * t->chains.size());
+  off_units = off;
+  off += align256(sizeof(PbUnit) * std::max<size_t>(t->units.size(), 1));
+  off_first = off;
+  off += align256(sizeof(int32_t) * t->first.size());
+  off_last = off;
+  off += align256(sizeof(float*) * (size_t)count);
+  off_bar = off;
+  off += 256;
+  bytes = off;
+  return TN_OK;
+}
+
+int BatchSweep::upload(uint8_t* region, float* const* last, const float* Wx, const int64_t* woff, unsigned* bits,
+                       double* lg, cudaStream_t s) {
+  PbParams& p = t->p;
+  p.base = region;
+  p.Cp[0] = region + off_cores;
+  p.Cp[1] = region + off_cores + site_bytes;
+  p.chains = reinterpret_cast<const PbChain*>(region + off_chains);
+  p.units = reinterpret_cast<const PbUnit*>(region + off_units);
+  p.first = reinterpret_cast<const int32_t*>(region + off_first);
+  p.last = reinterpret_cast<float* const*>(region + off_last);
+  p.bar = reinterpret_cast<unsigned*>(region + off_bar);
+  p.Wx = Wx;
+  p.bits = bits;
+  p.lg = lg;
+  p.status = status_word();
+  for (int i = 0; i < p.n; ++i) p.woff[i] = (int32_t)woff[i];
+  for (int k = 0; k < count; ++k) t->last[(size_t)k] = last[k];
+  auto up = [&](size_t at, const void* src, size_t b) {
+    return b == 0 || cudaMemcpyAsync(region + at, src, b, cudaMemcpyHostToDevice, s) == cudaSuccess;
+  };
+  return up(off_chains, t->chains.data(), sizeof(PbChain) * t->chains.size()) &&
+                 up(off_units, t->units.data(), sizeof(PbUnit) * t->units.size()) &&
+                 up(off_first, t->first.data(), sizeof(int32_t) * t->first.size()) &&
+                 up(off_last, t->last.data(), sizeof(float*) * t->last.size())
+             ? TN_OK
+             : TN_ERR_CUDA;
+}
+
+int BatchSweep::run(cudaStream_t s) const {
+  if (cudaMemsetAsync(t->p.bar, 0, sizeof(unsigned), s) != cudaSuccess) return TN_ERR_CUDA;
+  return split ? launch_sweep(expect_batch_kernel<1>, t->p, s) : launch_sweep(expect_batch_kernel<0>, t->p, s);
 }
 
 }  // namespace tn

@@ -216,6 +216,34 @@ ExpectRegions expect_persistent_regions(const tn_mps* psi, const tn_mpo* H);
 int expect_persistent(const tn_mps* psi, const tn_mpo* H, int prec, const ExpectBuffers& w, double* result,
                       cudaStream_t s);
 
+// The same for a batch of chains and one MPO (mps_persistent.cu): bonds at most
+// PERSISTENT_MAX_BOND, at most PB_MAX_CHAINS chains. Built once; upload() puts
+// its tables into a region of `bytes` (256-byte aligned) and names the chains'
+// last environments, the extended MPO, the max slots and log-scales (both
+// zeroed before run()); run() is one memset and one launch.
+constexpr int64_t PERSISTENT_MAX_BOND = 512;  // largest bond of the persistent energy sweeps
+constexpr int PB_MAX_CHAINS = 1024;
+bool batch_sweep_ok(const tn_mps* psis, int count, const tn_mpo* H, int prec);
+class BatchSweep {
+ public:
+  BatchSweep();
+  ~BatchSweep();
+  BatchSweep(const BatchSweep&) = delete;
+  BatchSweep& operator=(const BatchSweep&) = delete;
+  int build(const tn_mps* psis, int count, const tn_mpo* H, int prec);
+  int upload(uint8_t* region, float* const* last, const float* Wx, const int64_t* woff, unsigned* bits, double* lg,
+             cudaStream_t s);
+  int run(cudaStream_t s) const;
+  size_t bytes = 0;
+
+ private:
+  struct Tables;
+  Tables* t;
+  int count = 0;
+  bool split = false;
+  size_t off_cores = 0, site_bytes = 0, off_chains = 0, off_units = 0, off_first = 0, off_last = 0, off_bar = 0;
+};
+
 // wad, wbd: (extended MPO bond) x d on either side of the site.
 int launch_mpo_step_ii_grouped(const StepII* descs, int count, int64_t max_cols, int64_t wad, int64_t wbd,
                                cudaStream_t s);

@@ -195,6 +195,31 @@ def test_energy_tiles_of_the_one_launch_sweep(tn, d, w, prec):
     assert rel(val(r, 1), nv * math.exp(ln)) <= bound
 
 
+@pytest.mark.parametrize("d,w", [(1, 7), (2, 1), (2, 2), (2, 3), (3, 1), (4, 1)])
+@pytest.mark.parametrize("prec", ["bf16x3", "bf16"])
+def test_energy_batch_in_one_launch(tn, d, w, prec):
+    # the batch's one-launch sweep over the same edges, chains of very
+    # different bonds beside one another (units of unequal cost, chains with
+    # no padded shared index beside ones with some). Bounds as above.
+    lists = [[1, 5, 16, 17, 64, 70, 130, 33, 3, 1], [1, 1, 1, 1, 1, 1, 1, 1, 1, 1], [1, 2, 4, 8, 300, 256, 8, 4, 2, 1],
+             [1, 128, 128, 64, 64, 192, 96, 32, 16, 1]]
+    n = len(lists[0]) - 1
+    rng = np.random.default_rng(1000 * d + w)
+    wb = [1] + [w] * (n - 1) + [1]
+    W = [rng.uniform(0.5, 1.5, (wb[i], wb[i + 1], d, d)).astype(np.float32) for i in range(n)]
+    states = [[(rng.uniform(0.5, 1.5, (b[i], d, b[i + 1])) / math.sqrt(b[i] * b[i + 1])).astype(np.float32)
+               for i in range(n)] for b in lists]
+    r = tn.mps_expect_grouped([to_dev(c) for c in states], to_dev(W), prec=prec)
+    assert tn.sync_status() == 0
+    bias = {"bf16x3": 2.0 ** -18, "bf16": 2.0 ** -16}[prec]
+    bound = tol(prec, 2 * n) + 2 * n * bias
+    for k, cores in enumerate(states):
+        e, le = oracle.mpo_expect(cores, W)
+        nv, ln = oracle.mps_inner(cores, cores)
+        assert rel(val(r[k], 0), e * math.exp(le)) <= bound
+        assert rel(val(r[k], 1), nv * math.exp(ln)) <= bound
+
+
 @pytest.mark.parametrize("prec", ["fp32", "bf16x3", "bf16"])
 def test_energy_three_level_sites(tn, prec):
     # spin-1 sites (d = 3) with a bond-4 MPO: (bond + 1) d = 15, so the sweep
