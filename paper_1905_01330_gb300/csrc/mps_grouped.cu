@@ -13,7 +13,7 @@
 // MN-major blocks), so that plan packs only the cores. Of these, batches of at
 // most PB_MAX_CHAINS chains with bonds up to PERSISTENT_MAX_BOND run as one
 // launch for the whole sweep (BatchSweep; 16 states of up to 512, N = 100,
-// BF16x3: 14.5 ms as launches per site, 8.5 as one), with the same results;
+// BF16x3: 14.5 ms as launches per site, 8.2 as one), with the same results;
 // the launches per site remain for longer chains, wider bonds and FP32.
 #include <math.h>
 #include <string.h>

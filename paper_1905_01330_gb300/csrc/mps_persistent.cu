@@ -40,6 +40,9 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
+#include <queue>
+#include <utility>
 #include <vector>
 
 #include "mpo_step.cuh"
@@ -228,24 +231,27 @@ __device__ __forceinline__ void pack_unit(const PsPack& q, uint32_t u) {
   const float* src = q.src + k0 * ks + (int64_t)sk * q.Db + b;
   uint8_t* blk = q.hi + ((size_t)t * q.slabs + sl) * (size_t)(q.cols * 128) + (size_t)(rr >> 3) * 1024;
   const int r0 = rr & 6;  // row of the pair's even lane, in its group of 8
-#pragma unroll 2
-  for (int g = 0; g < 8; g += 2) {
-    float v[16];
-    if (q.run == 0) {
+  // the whole unit's loads before anything waits on one: beside a GEMM phase
+  // each takes thousands of cycles
+  float all[64];
+  if (q.run == 0) {
 #pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = 8 * g + j < kn ? __ldg(src + (8 * g + j) * ks) : 0.0f;
-    } else {
-      // k = s' Da + a': row a' d + s'
-      int s1 = (k0 + 8 * g) / q.run, a1 = k0 + 8 * g - s1 * q.run;
+    for (int j = 0; j < 64; ++j) all[j] = j < kn ? __ldg(src + j * ks) : 0.0f;
+  } else {
+    // k = s' Da + a': row a' d + s'
+    int s1 = k0 / q.run, a1 = k0 - s1 * q.run;
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        v[j] = 8 * g + j < kn ? __ldg(q.src + ((int64_t)a1 * q.d + s1) * q.Db + b) : 0.0f;
-        if (++a1 == q.run) {
-          a1 = 0;
-          ++s1;
-        }
+    for (int j = 0; j < 64; ++j) {
+      all[j] = j < kn ? __ldg(q.src + ((int64_t)a1 * q.d + s1) * q.Db + b) : 0.0f;
+      if (++a1 == q.run) {
+        a1 = 0;
+        ++s1;
       }
     }
+  }
+#pragma unroll
+  for (int g = 0; g < 8; g += 2) {
+    const float* v = all + 8 * g;
     uint4 h[2], l[2];
     split8(v, h[0], l[0]);
     split8(v + 8, h[1], l[1]);
@@ -854,8 +860,8 @@ __global__ void __launch_bounds__(PS_THREADS, 1) expect_persistent_kernel(const 
 
 // ------------------------------------------------------------ many chains
 // The same sweep for a batch of chains with one MPO: every phase works on the
-// units of all of them, in lists the host made (largest first, dealt out to
-// the CTAs back and forth), so the device-wide barriers, the copies' latency
+// units of all of them, in lists the host made (largest first, each to the CTA
+// with the least so far), so the device-wide barriers, the copies' latency
 // and the ragged tiles of a site are shared. Warps 2 and 3 pack the next
 // site's cores meanwhile, into the other of two regions. Sums run in the order
 // of the grouped contractions: (iii)'s shared index is (s', a'), and where
@@ -885,7 +891,7 @@ struct PbParams {
   int64_t Cp_lo;
   const PbChain* chains;  // [site][chain]
   const PbUnit* units;
-  const int32_t* first;   // [site][phase][CTA]: its first unit (one more at the end)
+  const int32_t* first;   // [site][phase][CTA]: its first unit; one more: the end
   float* const* last;     // per chain: its last environment (one value per channel)
   unsigned* bits;         // [site - 1][chain]: largest |L| entering the site
   double* lg;
@@ -909,7 +915,7 @@ struct ListUnits {
   __device__ __forceinline__ ListUnits(const PbParams& pp, int st, int ph, uint4 (*sl)[4] = nullptr,
                                        unsigned* mx = nullptr)
       : p(pp), phase(ph), site(st), slot(sl), slot_max(mx) {
-    const int32_t* f = pp.first + ((size_t)st * 2 + ph) * gridDim.x + blockIdx.x;
+    const int32_t* f = pp.first + ((size_t)st * 2 + ph) * (gridDim.x + 1) + blockIdx.x;
     u = pp.units + __ldg(f);
     end = pp.units + __ldg(f + 1);
     chains = pp.chains + (size_t)st * pp.count;
@@ -950,12 +956,13 @@ struct ListUnits {
 __device__ __forceinline__ void pack_site(const PbParams& p, int site, uint32_t e0, uint32_t e1, uint32_t wid,
                                           uint32_t nwarps) {
   const PbChain* chains = p.chains + (size_t)site * p.count;
+  int lo = -1, lane = threadIdx.x & 31;  // the chain whose units hold e: e only grows
   for (uint32_t e = e0 + wid; e < e1; e += nwarps) {
-    int lo = 0, hi = p.count - 1;  // the chain whose units hold e
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (__ldg(&chains[mid].unit0) <= e) lo = mid;
-      else hi = mid - 1;
+    for (;;) {  // 32 chains a look: those whose first unit is not past e
+      const int at = lo + 1 + lane;
+      const unsigned m = __ballot_sync(0xffffffffu, at < p.count && __ldg(&chains[at].unit0) <= e);
+      lo += __popc(m);
+      if (m != 0xffffffffu) break;
     }
     const PbChain& c = chains[lo];
     uint32_t k = e - c.unit0;
@@ -1295,15 +1302,20 @@ int expect_persistent(const tn_mps* psi, const tn_mpo* H, int prec, const Expect
 // ------------------------------------------------------------ many chains
 namespace {
 
-// Unit costs in cycles, as in tile_cols.
-double unit_cost(int slabs, int cols) { return slabs * (512.0 + 4.0 * cols) + 20.0 * cols + 1000.0; }
+// Cycles of a unit: its copies and MMAs as in tile_cols; the epilogue of (i),
+// step (ii), about as long as 8 slabs of a 128-column tile, overlaps the next
+// unit's.
+double unit_cost(int slabs, int cols, int phase) {
+  const double gemm = slabs * (512.0 + 4.0 * cols);
+  return phase == 0 ? std::max(gemm, 90.0 * cols) + 1000.0 : gemm + 20.0 * cols + 1000.0;
+}
 
 // Columns of a tile when many chains share the SMs: the least padded work.
-int batch_cols(int64_t total, int64_t K, int step) {
+int batch_cols(int64_t total, int64_t K, int step, int phase) {
   int best = step;
   double best_cost = 1e30;
   for (int c = step; c <= 128; c *= 2) {
-    const double cost = (double)ceil64(total, c) * unit_cost((int)ceil64(K, 64), c);
+    const double cost = (double)ceil64(total, c) * unit_cost((int)ceil64(K, 64), c, phase);
     if (cost < best_cost) {
       best_cost = cost;
       best = c;
@@ -1364,7 +1376,7 @@ int BatchSweep::build(const tn_mps* psis, int cnt, const tn_mpo* H, int prec) {
   if (off / 1024 > 0xFFFFFFFFull) return TN_ERR_UNSUPPORTED;
   off_cores = off;
   t->chains.resize((size_t)n * count);
-  t->first.assign((size_t)n * 2 * grid + 1, 0);
+  t->first.assign((size_t)n * 2 * (grid + 1), 0);
   t->last.resize((size_t)count);
   size_t cores = 0;
   int widest = 0;
@@ -1391,7 +1403,7 @@ int BatchSweep::build(const tn_mps* psis, int cnt, const tn_mpo* H, int prec) {
       for (int j = 0; j < 2; ++j) {
         PsTiles& q = c.t[j];
         const int64_t total = j ? DbP : d * DbP, K = j ? d * Da : Da;
-        const int cols = batch_cols(total, K, j ? 32 : (int)(32 * d));
+        const int cols = batch_cols(total, K, j ? 32 : (int)(32 * d), j);
         q.off = (uint32_t)(co / 1024);
         q.tp = (uint16_t)(j ? ceil64(p.w[i + 1] * DbP, 128) : ceil64(Da, int64_t(1) << group_shift(p.w[i])));
         q.tq = (uint16_t)ceil64(total, cols);
@@ -1405,6 +1417,15 @@ int BatchSweep::build(const tn_mps* psis, int cnt, const tn_mpo* H, int prec) {
     if (co / 1024 > 0xFFFFFFFFull) return TN_ERR_UNSUPPORTED;
     cores = std::max(cores, co);
     p.pack[i] = pu;
+    // a site like the one before it, as most of a chain's are, has its units
+    bool same = i > 0 && p.w[i] == p.w[i - 1] && p.w[i + 1] == p.w[i];
+    for (int k = 0; k < count && same; ++k)
+      same = psis[k].bond[i] == psis[k].bond[i - 1] && psis[k].bond[i + 1] == psis[k].bond[i];
+    if (same) {
+      const auto before = t->first.begin() + (ptrdiff_t)(i - 1) * 2 * (grid + 1);
+      std::copy(before, before + 2 * (grid + 1), before + 2 * (grid + 1));
+      continue;
+    }
     for (int j = 0; j < 2; ++j) {
       list.clear();
       for (int k = 0; k < count; ++k) {
@@ -1423,22 +1444,28 @@ int BatchSweep::build(const tn_mps* psis, int cnt, const tn_mpo* H, int prec) {
           for (int b = 0; b < q.tq; ++b) {
             u.tpi = (uint8_t)a;
             u.tqi = (uint8_t)b;
-            list.push_back(Cost{unit_cost(q.slabs, q.cols), u});
+            list.push_back(Cost{unit_cost(q.slabs, q.cols, j), u});
           }
       }
       std::stable_sort(list.begin(), list.end(), [](const Cost& a, const Cost& b) { return a.c > b.c; });
-      // dealt out back and forth: CTA c's units lie together
-      for (int c = 0; c < grid; ++c) {
-        t->first[((size_t)i * 2 + j) * grid + c] = (int32_t)t->units.size();
-        for (size_t r = 0;; ++r) {
-          const size_t at = r * grid + (r & 1 ? (size_t)(grid - 1 - c) : (size_t)c);
-          if (r * (size_t)grid >= list.size()) break;
-          if (at < list.size()) t->units.push_back(list[at].u);
-        }
+      // each to the CTA with the least so far; a CTA's units lie together
+      std::vector<std::vector<PbUnit>> mine((size_t)grid);
+      std::priority_queue<std::pair<double, int>, std::vector<std::pair<double, int>>, std::greater<>> load;
+      for (int c = 0; c < grid; ++c) load.push({0.0, c});
+      for (const Cost& e : list) {
+        const auto least = load.top();
+        load.pop();
+        mine[(size_t)least.second].push_back(e.u);
+        load.push({least.first + e.c, least.second});
       }
+      int32_t* first = t->first.data() + ((size_t)i * 2 + j) * (grid + 1);
+      for (int c = 0; c < grid; ++c) {
+        first[c] = (int32_t)t->units.size();
+        t->units.insert(t->units.end(), mine[(size_t)c].begin(), mine[(size_t)c].end());
+      }
+      first[grid] = (int32_t)t->units.size();
     }
   }
-  t->first.back() = (int32_t)t->units.size();
   p.stage_bytes = planes * (PS_BLOCK + widest * 128);
   p.stages = std::min(PS_RING / p.stage_bytes, PS_MAX_STAGES);
   cores = align256(cores);
