@@ -286,6 +286,7 @@ __global__ void __launch_bounds__(PACK_THREADS)
 pack_pair_kernel(const __grid_constant__ PackPair pp) {
   extern __shared__ __align__(16) uint8_t pack_smem_raw[];
   PackSmem& sm = *reinterpret_cast<PackSmem*>(pack_smem_raw);
+  ptx::launch_dependents();  // the GEMM's set-up may start once every CTA here runs
   const int blk = (int)blockIdx.x;
   const int which = blk < pp.units_a ? 0 : (blk < pp.units_a + pp.units_b ? 1 : 2);
   stage_job(which == 0 ? pp.a : (which == 1 ? pp.b : pp.c), sm);
@@ -1010,6 +1011,7 @@ packed_gemm_kernel(const __grid_constant__ GemmDesc single, const GemmDesc* __re
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
+  ptx::wait_dependencies();  // launched beside the pack: its blocks are written
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = x.tmem_base;
@@ -1536,12 +1538,31 @@ int sm_count() {
 
 template <int SPLIT, int FUSE>
 int launch_gemm(const GemmDesc& single, const GemmDesc* descs, const int32_t* map, const PackJob* jobs,
-                int64_t units, cudaStream_t s, uint32_t* unit_ctr = nullptr) {
+                int64_t units, cudaStream_t s, uint32_t* unit_ctr = nullptr, bool overlap = false) {
   const size_t smem = gemm_smem_bytes<SPLIT, FUSE>();
   static std::atomic<uint64_t> attr{0};
   if (!smem_limit_once((const void*)packed_gemm_kernel<SPLIT, FUSE>, smem, &attr)) return TN_ERR_CUDA;
   const int64_t sms = sm_count();
   const unsigned grid = (unsigned)(units < sms ? units : sms);
+  if (overlap) {
+    // started as the kernel before it ends: its set-up runs meanwhile, and it
+    // waits for that kernel's results before it reads anything
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(GCfg<SPLIT, FUSE>::THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, packed_gemm_kernel<SPLIT, FUSE>, single, descs, map, jobs, units, unit_ctr,
+                              status_word()) == cudaSuccess
+               ? TN_OK
+               : TN_ERR_CUDA;
+  }
   packed_gemm_kernel<SPLIT, FUSE>
       <<<grid, GCfg<SPLIT, FUSE>::THREADS, smem, s>>>(single, descs, map, jobs, units, unit_ctr, status_word());
   return cudaGetLastError() == cudaSuccess ? TN_OK : TN_ERR_CUDA;
@@ -2107,8 +2128,8 @@ int launch_gemm_single(const GemmDesc& g, int prec, cudaStream_t s) {
     return TN_ERR_CUDA;
   const int64_t units = (int64_t)g.tiles_p * g.tiles_q * g.splits;
   if (units <= 0) return TN_OK;
-  if (prec == TN_PREC_BF16) return launch_gemm<0, 0>(g, nullptr, nullptr, nullptr, units, s);
-  if (prec == TN_PREC_BF16X3) return launch_gemm<1, 0>(g, nullptr, nullptr, nullptr, units, s);
+  if (prec == TN_PREC_BF16) return launch_gemm<0, 0>(g, nullptr, nullptr, nullptr, units, s, nullptr, true);
+  if (prec == TN_PREC_BF16X3) return launch_gemm<1, 0>(g, nullptr, nullptr, nullptr, units, s, nullptr, true);
   return TN_ERR_ARG;
 }
 

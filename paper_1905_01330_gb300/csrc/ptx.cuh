@@ -197,6 +197,12 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
       : "memory");
 }
 
+// Programmatic dependent launch: lets the next kernel of the stream, if it was
+// launched so, begin; waits until the kernels before this one have completed
+// and their results are visible (returns at once in an ordinary launch).
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_dependencies() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // True in one lane of the (converged) warp.
 __device__ __forceinline__ bool elect_one() {
   uint32_t r;
