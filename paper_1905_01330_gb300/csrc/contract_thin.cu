@@ -5,8 +5,8 @@
 // Outer products, K <= 8: bound by writing C. A CTA gathers its 64 rows and 64
 // columns of the operands once into shared memory; a thread makes 4 x 4
 // results and stores rows of 16 bytes. Sums are one chain over ascending k, as
-// in the general kernel. Measured, on the general kernel and here: 1024
-// x 1024 x 2 6.4 -> 2.7 us, 4096 x 4096 x 8 27.7 -> 24.9.
+// in the general kernel. Measured in a row of launches, on the general kernel
+// and here: 1024 x 1024 x 2 6.4 -> 2.2 us, 4096 x 4096 x 8 27.7 -> 23.4.
 //
 // Matrix times vector: bound by reading the matrix, and at the sizes of a
 // network's environments (1024 x 1024) by the latency of the loads in flight.
@@ -14,13 +14,15 @@
 // columns at one k, a CTA takes 64 columns and a part of the shared index, and
 // the (up to 8) parts are CTAs of one cluster that add up through distributed
 // shared memory: no zeroed result, no atomics, one order. With the shared leg
-// of unit stride a warp takes a row. Measured (columns / rows): 1024 x 1024
-// 49.2 -> 4.3 / 4.7 us, 64 x 64 13.3 -> 3.3 / 2.4, 20000 x 2048 427 -> 32 / 33 us (5 TB/s).
+// of unit stride a warp takes a row. Measured likewise (columns / rows): 1024 x
+// 1024 49.2 -> 3.1 / 2.7 us, 64 x 64 13.3 -> 1.9 / 1.4, 20000 x 2048 427 -> 28 /
+// 36 us (4.5 to 5.8 TB/s).
 #include <cooperative_groups.h>
 
 #include <algorithm>
 
 #include "gather.cuh"
+#include "ptx.cuh"
 #include "tn_internal.h"
 
 namespace tn {
@@ -37,6 +39,7 @@ constexpr int MV_ROWK = 2048;  // longest shared index of the row form
 
 __global__ void __launch_bounds__(THREADS) outer_kernel(const __grid_constant__ ContractDesc d) {
   __shared__ __align__(16) float As[OUT_K][OUT_T], Bs[OUT_K][OUT_T];
+  ptx::launch_dependents();
   const int t = threadIdx.x, K = (int)d.K;
   const int64_t m0 = (int64_t)(blockIdx.x / d.tiles_n) * OUT_T, n0 = (int64_t)(blockIdx.x % d.tiles_n) * OUT_T;
   {
@@ -45,9 +48,17 @@ __global__ void __launch_bounds__(THREADS) outer_kernel(const __grid_constant__ 
     const bool in = row < (side ? d.N : d.M);
     const float* src = side ? d.B : d.A;
     if (in) src += side ? leg_offset((uint32_t)row, d.nn, d.ndim, d.nstr) : leg_offset((uint32_t)row, d.nm, d.mdim, d.mstr);
-    for (int k = t >> 7; k < K; k += 2) {
-      const int64_t ko = leg_offset((uint32_t)k, d.nk, d.kdim, side ? d.kstrB : d.kstrA);
-      (side ? Bs : As)[k][r] = in ? __ldg(src + ko) : 0.0f;
+    int64_t ko[OUT_K / 2];
+#pragma unroll
+    for (int i = 0; i < OUT_K / 2; ++i) {
+      const int k = (t >> 7) + 2 * i;
+      ko[i] = k < K ? leg_offset((uint32_t)k, d.nk, d.kdim, side ? d.kstrB : d.kstrA) : 0;
+    }
+    ptx::wait_dependencies();
+#pragma unroll
+    for (int i = 0; i < OUT_K / 2; ++i) {
+      const int k = (t >> 7) + 2 * i;
+      if (k < K) (side ? Bs : As)[k][r] = in ? src[ko[i]] : 0.0f;
     }
   }
   __syncthreads();
@@ -91,12 +102,17 @@ __global__ void __launch_bounds__(THREADS) matvec_columns(const __grid_constant_
   __shared__ int64_t ko[MV_PART];
   __shared__ __align__(16) float sums[16][MV_COLS];
   __shared__ float mine[MV_COLS];
+  ptx::launch_dependents();
   cg::cluster_group cl = cg::this_cluster();
   const int t = threadIdx.x, ranks = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int k0 = rank * d.part, kn = max(0, min(d.K - k0, d.part));
-  for (int k = t; k < kn; k += THREADS) {
+  int64_t xo[MV_PART / THREADS];
+#pragma unroll
+  for (int i = 0; i < MV_PART / THREADS; ++i) {
+    const int k = t + i * THREADS;
+    if (k >= kn) break;
     ko[k] = leg_offset((uint32_t)(k0 + k), d.nk, d.kdim, d.kstr);
-    xs[k] = __ldg(d.x + leg_offset((uint32_t)(k0 + k), d.nk, d.kdim, d.xstr));
+    xo[i] = leg_offset((uint32_t)(k0 + k), d.nk, d.kdim, d.xstr);
   }
   // this thread's four columns: c0 .. c0 + 3, or c0 + 16 j
   const int l = t & 15, kg = t >> 4;
@@ -109,6 +125,13 @@ __global__ void __launch_bounds__(THREADS) matvec_columns(const __grid_constant_
     in[j] = r < d.R;
     if (!VEC || j == 0) col[j] = d.mat + (in[j] ? leg_offset((uint32_t)r, d.nr, d.rdim, d.rstr) : 0);
   }
+  ptx::wait_dependencies();
+#pragma unroll
+  for (int i = 0; i < MV_PART / THREADS; ++i) {
+    const int k = t + i * THREADS;
+    if (k >= kn) break;
+    xs[k] = d.x[xo[i]];
+  }
   __syncthreads();
   float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
   if (in[0]) {
@@ -116,7 +139,7 @@ __global__ void __launch_bounds__(THREADS) matvec_columns(const __grid_constant_
     for (int k = kg; k < kn; k += 16) {
       const float xv = xs[k];
       if (VEC) {
-        const float4 b = __ldg(reinterpret_cast<const float4*>(col[0] + ko[k]));
+        const float4 b = *reinterpret_cast<const float4*>(col[0] + ko[k]);
         acc[0] = fmaf(xv, b.x, acc[0]);
         acc[1] = fmaf(xv, b.y, acc[1]);
         acc[2] = fmaf(xv, b.z, acc[2]);
@@ -124,7 +147,7 @@ __global__ void __launch_bounds__(THREADS) matvec_columns(const __grid_constant_
       } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if (in[j]) acc[j] = fmaf(xv, __ldg(col[j] + ko[k]), acc[j]);
+          if (in[j]) acc[j] = fmaf(xv, col[j][ko[k]], acc[j]);
       }
     }
   }
@@ -153,33 +176,68 @@ __global__ void __launch_bounds__(THREADS) matvec_rows(const __grid_constant__ M
   constexpr int W = VEC ? 4 : 1;
   __shared__ __align__(16) float xs[MV_ROWK];
   __shared__ int64_t ko[MV_ROWK / W];
+  ptx::launch_dependents();
   const int t = threadIdx.x, lane = t & 31;
-  for (int k = t; k < d.K; k += THREADS) {
-    xs[k] = __ldg(d.x + leg_offset((uint32_t)k, d.nk, d.kdim, d.xstr));
+  int64_t xo[MV_ROWK / THREADS];
+#pragma unroll
+  for (int i = 0; i < MV_ROWK / THREADS; ++i) {
+    const int k = t + i * THREADS;
+    if (k >= d.K) break;
+    xo[i] = leg_offset((uint32_t)k, d.nk, d.kdim, d.xstr);
     if (k % W == 0) ko[k / W] = leg_offset((uint32_t)k, d.nk, d.kdim, d.kstr);
   }
-  __syncthreads();
   const int r = (int)blockIdx.x * (THREADS / 32) + (t >> 5);
+  const float* row = d.mat + (r < d.R ? leg_offset((uint32_t)r, d.nr, d.rdim, d.rstr) : 0);
+  ptx::wait_dependencies();
+#pragma unroll
+  for (int i = 0; i < MV_ROWK / THREADS; ++i) {
+    const int k = t + i * THREADS;
+    if (k >= d.K) break;
+    xs[k] = d.x[xo[i]];
+  }
+  __syncthreads();
   if (r >= d.R) return;
-  const float* row = d.mat + leg_offset((uint32_t)r, d.nr, d.rdim, d.rstr);
   float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 8
   for (int k = lane; k < d.K / W; k += 32) {
     if (VEC) {
-      const float4 b = __ldg(reinterpret_cast<const float4*>(row + ko[k]));
+      const float4 b = *reinterpret_cast<const float4*>(row + ko[k]);
       const float4 xv = *reinterpret_cast<const float4*>(&xs[4 * k]);
       acc[0] = fmaf(xv.x, b.x, acc[0]);
       acc[1] = fmaf(xv.y, b.y, acc[1]);
       acc[2] = fmaf(xv.z, b.z, acc[2]);
       acc[3] = fmaf(xv.w, b.w, acc[3]);
     } else {
-      acc[0] = fmaf(xs[k], __ldg(row + ko[k]), acc[0]);
+      acc[0] = fmaf(xs[k], row[ko[k]], acc[0]);
     }
   }
   float s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) d.y[r] = s;
+}
+
+// A launch that may begin while the kernel before it ends (each kernel here
+// waits for it before it reads an operand): a network's products run one after
+// another, and the offsets are worked out meanwhile.
+template <class P>
+int launch_overlapped(void (*fn)(const P), const P& p, int64_t ctas, int cluster, cudaStream_t s) {
+  if (ctas > 0x7FFFFFFF) return TN_ERR_UNSUPPORTED;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3((unsigned)ctas);
+  cfg.blockDim = dim3(THREADS);
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  memset(at, 0, sizeof(at));
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, fn, p) == cudaSuccess ? TN_OK : TN_ERR_CUDA;
 }
 
 // The innermost leg (dims > 1) of a list has unit stride; *vec: its runs of
@@ -207,9 +265,7 @@ int launch_outer(const ContractDesc& d, cudaStream_t s) {
   q.tiles_m = (int32_t)((d.M + OUT_T - 1) / OUT_T);
   q.tiles_n = (int32_t)((d.N + OUT_T - 1) / OUT_T);
   const int64_t ctas = (int64_t)q.tiles_m * q.tiles_n;
-  if (ctas > 0x7FFFFFFF) return TN_ERR_UNSUPPORTED;
-  outer_kernel<<<(unsigned)ctas, THREADS, 0, s>>>(q);
-  return cudaGetLastError() == cudaSuccess ? TN_OK : TN_ERR_CUDA;
+  return launch_overlapped(outer_kernel, q, ctas, 1, s);
 }
 
 bool matvec_ok(const ContractDesc& d) {
@@ -240,10 +296,8 @@ int launch_matvec(const ContractDesc& d, cudaStream_t s) {
   }
   bool vec = false;
   if (unit_inner(v.nk, v.kdim, v.kstr, v.nr, v.rstr, v.rdim, v.mat, &vec)) {
-    const unsigned grid = (unsigned)((v.R + THREADS / 32 - 1) / (THREADS / 32));
-    if (vec) matvec_rows<true><<<grid, THREADS, 0, s>>>(v);
-    else matvec_rows<false><<<grid, THREADS, 0, s>>>(v);
-    return cudaGetLastError() == cudaSuccess ? TN_OK : TN_ERR_CUDA;
+    return launch_overlapped(vec ? matvec_rows<true> : matvec_rows<false>, v, (v.R + THREADS / 32 - 1) / (THREADS / 32), 1,
+                             s);
   }
   unit_inner(v.nr, v.rdim, v.rstr, v.nk, v.kstr, v.kdim, v.mat, &vec);
   // parts of the shared index: enough CTAs for the SMs, at least 64 indices each
@@ -251,20 +305,7 @@ int launch_matvec(const ContractDesc& d, cudaStream_t s) {
   int parts = (v.K + MV_PART - 1) / MV_PART;
   while (parts < 8 && groups * parts < 152 && v.K / (2 * parts) >= 64) parts *= 2;
   v.part = (v.K + parts - 1) / parts;
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((unsigned)(groups * parts));
-  cfg.blockDim = dim3(THREADS);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)parts;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  const cudaError_t e = vec ? cudaLaunchKernelEx(&cfg, matvec_columns<true>, v)
-                            : cudaLaunchKernelEx(&cfg, matvec_columns<false>, v);
-  return e == cudaSuccess ? TN_OK : TN_ERR_CUDA;
+  return launch_overlapped(vec ? matvec_columns<true> : matvec_columns<false>, v, groups * parts, parts, s);
 }
 
 }  // namespace tn
