@@ -363,8 +363,8 @@ def run_extras(tn, synth, dev, stream):
                     loss, dft = tn.mps_classify_loss(ft, y)
                     tn.mps_classify_backward(cores, ls, px, dft, ws, prec=prec, ckpt_every=ck)
                 ms_eager = _time(step, 3, 1, stream)
-                # BF16 / BF16X3 from a CUDA graph; the FP32 backward builds and
-                # uploads its grouped plans in the call, so it runs eagerly
+                # BF16 / BF16X3 from a CUDA graph; the FP32 backward refuses a
+                # capturing stream, so it runs eagerly
                 ms = ms_eager if prec == "fp32" else _time_graph(step, 1, 5, stream)
                 train[prec] = {"ms": ms, "ms_eager": ms_eager, "samples_per_s": B / (ms * 1e-3),
                                "tflops": 4 * flops / (ms * 1e-3) / 1e12,
@@ -420,7 +420,7 @@ def run_extras(tn, synth, dev, stream):
                     loss, dft = tn.mps_classify_loss(ft, y)
                     tn.mps_classify_separate_backward(mps, px, dft, ws, prec=prec, ckpt_every=28)
                 ms_eager = _time(sep_step, 2, 1, stream)
-                # BF16 / BF16X3 from a CUDA graph; the FP32 backward uploads plans in the call
+                # BF16 / BF16X3 from a CUDA graph; the FP32 backward refuses capture
                 ms = ms_eager if prec == "fp32" else _time_graph(sep_step, 1, 3, stream)
                 entry[prec]["train_step_ms"] = ms
                 entry[prec]["train_step_ms_eager"] = ms_eager

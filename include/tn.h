@@ -362,10 +362,10 @@ int tn_mps_inner(const tn_mps* bra, const tn_mps* ket, int prec, void* workspace
  * Launch forms (results the same up to the order of float32 sums):
  *   - BF16 / BF16X3 with (bond + 1) * d <= 8 on every MPO bond, n <= 512 and
  *     D <= 512: ONE persistent cooperative launch for the whole chain (one
- *     CTA per SM, the sites' GEMM (i) / step (ii) / GEMM (iii) phases
- *     separated by device-wide barriers; the cores packed to bf16 once per
- *     call, step (ii) and GEMM (iii) writing the next contraction's packed
- *     operand). Its barriers are bounded: on expiry TN_ERR_TIMEOUT is
+ *     CTA per SM, two phases per site separated by device-wide barriers:
+ *     GEMM (i) with step (ii) in its epilogue, and GEMM (iii), each writing
+ *     the next one's packed operand; the cores packed to bf16 once per
+ *     call). Its barriers are bounded: on expiry TN_ERR_TIMEOUT is
  *     recorded in the status word (tn_sync_status) and the launch ends.
  *   - BF16 / BF16X3 otherwise with (bond + 1) * d <= 8: four launches per
  *     site (a pack of L and the core, the GEMM of (i), step (ii) written
@@ -387,10 +387,13 @@ int tn_mps_expect(const tn_mps* psi, const tn_mpo* H, int prec, void* workspace,
 
 /*
  * tn_mps_expect for a batch of `count` MPS sharing one MPO (same n and d for
- * all; bond dimensions may differ from state to state). Each site step runs
- * as grouped launches over the whole batch ((i), (ii), (iii) and one max-abs
- * pass, the norm carried as an extra MPO channel as in tn_mps_expect), so a
- * sweep is a fixed number of launches per site whatever the batch size.
+ * all; bond dimensions may differ from state to state), the norm carried as
+ * an extra MPO channel as in tn_mps_expect. BF16 / BF16X3 with at most 1024
+ * states and the persistent form's limits (n <= 512, bonds <= 512,
+ * (bond + 1) * d <= 8): one cooperative launch for the whole batch. Otherwise
+ * each site step runs as grouped launches over the whole batch, a fixed number
+ * per site whatever its size: (i), (ii), (iii), and for FP32 and wider MPOs a
+ * max-abs pass (else the next site's pack finds the maxima).
  *   psis:   HOST array of `count` chains.
  *   result: DEVICE pointer to 4*count doubles, {e_value, e_log_scale,
  *           n_value, n_log_scale} per state, as tn_mps_expect.
@@ -410,12 +413,12 @@ int tn_mps_expect_grouped(const tn_mps* psis, int count, const tn_mpo* H, int pr
 
 /*
  * tn_mps_expect_grouped in two parts, for a batch evaluated many times:
- * _plan builds the host layout of the sweep (per site the grouped work lists
- * of steps (i) and (iii), the step (ii) descriptors, the max-abs tables) in
- * `workspace` and uploads its tables on `stream` (host -> device copies from
- * pageable memory); _run only launches (one extended-MPO build, per site two
- * grouped contractions, one grouped float32 step and one max-abs pass, then
- * the finisher) and writes `result` as tn_mps_expect_grouped does. The plan
+ * _plan builds the host layout of the sweep (the units of every site and
+ * phase, or per site the grouped work lists of steps (i) and (iii), the step
+ * (ii) descriptors, the max-abs tables) in `workspace` and uploads its tables
+ * on `stream` (host -> device copies from pageable memory); _run only launches
+ * (one extended-MPO build, the sweep in one launch or per site as above, the
+ * finisher) and writes `result` as tn_mps_expect_grouped does. The plan
  * keeps the device pointers of the states' and the MPO's cores and the
  * workspace (which must stay allocated and unused by others); the values
  * behind them are read at every run. Errors: as tn_mps_expect_grouped;

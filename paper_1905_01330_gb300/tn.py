@@ -49,20 +49,12 @@ class TnNconStep(ctypes.Structure):
                 ("legs_b", ctypes.c_int32 * TN_MAX_RANK), ("shape", ctypes.c_int64 * TN_MAX_RANK)]
 
 
-def _check_cores(cores, message: str):
-    """Every core a contiguous float32 CUDA tensor (attribute by attribute: a
-    784-core chain's check is on the path of every call)."""
-    if (any([c.dtype is not torch.float32 for c in cores]) or not all([c.is_cuda for c in cores])
-            or not all(map(torch.Tensor.is_contiguous, cores))):
-        raise TypeError(message)
-
-
 def _chain(cores, bonds, d):
     """(TnChain, its host arrays). The arrays are filled through `array`: ctypes
-    converts a list element by element (784 cores: the description 411 -> 250 us)."""
+    converts a list element by element (784 cores: the description 411 -> 280 us)."""
     n = len(cores)
     bond_arr = (ctypes.c_int64 * (n + 1)).from_buffer(array("q", bonds))
-    ptr_arr = (ctypes.c_void_p * n).from_buffer(array("Q", map(torch.Tensor.data_ptr, cores)))
+    ptr_arr = (ctypes.c_void_p * n).from_buffer(array("Q", [c.data_ptr() for c in cores]))
     ch = TnChain()
     ch.n = n
     ch.d = d
@@ -74,7 +66,10 @@ def _chain(cores, bonds, d):
 def chain_desc(cores, phys_axis: int = 1):
     """(TnChain, keepalive) for a list of contiguous float32 CUDA tensors; bonds
     are the first axis of each core plus the last core's second bond axis."""
-    _check_cores(cores, "MPS/MPO cores must be contiguous float32 CUDA tensors")
+    f32 = torch.float32
+    for c in cores:
+        if c.dtype is not f32 or not c.is_cuda or not c.is_contiguous():
+            raise TypeError("MPS/MPO cores must be contiguous float32 CUDA tensors")
     right_axis = 2 if cores[-1].dim() == 3 else 1
     return _chain(cores, [c.shape[0] for c in cores] + [cores[-1].shape[right_axis]], cores[0].shape[phys_axis])
 
@@ -707,7 +702,10 @@ def classifier_workspace(cores, label_site: int, n_labels: int, batch: int, ckpt
 
 def chain_desc_classifier(cores, label_site: int):
     """tn_mps of a classifier MPS: the label core (D, 2, L, D') keeps its bonds."""
-    _check_cores(cores, "classifier cores must be contiguous float32 CUDA tensors")
+    f32 = torch.float32
+    for c in cores:
+        if c.dtype is not f32 or not c.is_cuda or not c.is_contiguous():
+            raise TypeError("classifier cores must be contiguous float32 CUDA tensors")
     return _chain(cores, [c.shape[0] for c in cores] + [cores[-1].shape[-1]], cores[0].shape[1])
 
 
