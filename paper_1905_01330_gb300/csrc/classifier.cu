@@ -201,7 +201,7 @@ struct ClsLayout {
   float* labG;     // [batch][DL][2][L]
   float* labH;     // [batch][DL][2][L]
   float* gR;       // [batch][DR]
-  uint8_t* scratch;  // packed operands of the label core's BF16X3 contractions
+  uint8_t* scratch;  // packed operands of G = vR C (BF16X3), or none
   size_t scratch_bytes;
   size_t bytes;
 };
@@ -268,12 +268,12 @@ ClsLayout cls_layout(uint8_t* base, const tn_mps* W, int ls, int L, int batch, i
   w.labG = reinterpret_cast<float*>(take(lab));
   w.labH = reinterpret_cast<float*>(take(bwd ? lab : 0));
   w.gR = reinterpret_cast<float*>(take(bwd ? sizeof(float) * (size_t)batch * DR : 0));
-  // in place their gathers bound them (4096 samples, chi = 128: 66 us; packed and multiplied by the grouped kernel 36)
-  const int64_t SL = DL * 2 * L;
-  w.scratch_bytes = packed_scratch_bound(batch, SL, DR, TN_PREC_BF16X3);
-  if (bwd)
-    w.scratch_bytes = std::max({w.scratch_bytes, packed_scratch_bound(batch, DR, SL, TN_PREC_BF16X3),
-                                packed_scratch_bound(SL, DR, batch, TN_PREC_BF16X3)});
+  // G = vR C on packed operands (in place its gather bounds it: 4096 samples, chi =
+  // 128: 66 us, packed and multiplied by the grouped kernel 36). Only where that
+  // gives the same bits: a batch of 128 or more is the first operand there too,
+  // and K <= 128 is one accumulation. The backward's two (K up to a batch) would
+  // add in other pieces, which a BF16 adjoint's roundings blow up.
+  w.scratch_bytes = batch >= 128 ? packed_scratch_bound(batch, DL * 2 * L, DR, TN_PREC_BF16X3) : 0;
   w.scratch = take(w.scratch_bytes);
   w.bytes = off;
   return w;
@@ -425,7 +425,7 @@ int label_G(const tn_mps* W, const ClsLayout& w, int prec, cudaStream_t s) {
   tn_tensor tc = strided(const_cast<float*>(W->cores[w.ls]), 4, shc, stc);
   tn_tensor tg = strided(w.labG, 4, shg, stg);
   const int lv[1] = {1}, lc[1] = {3};
-  return contract_internal(&tv, lv, &tc, lc, 1, &tg, label_prec(prec), s, w.scratch, w.scratch_bytes);
+  return contract_internal(&tv, lv, &tc, lc, 1, &tg, label_prec(prec), s, w.scratch_bytes ? w.scratch : nullptr, w.scratch_bytes);
 }
 
 }  // namespace
@@ -538,14 +538,14 @@ int tn_mps_classify_backward(const tn_mps* W, int label_site, int n_labels, cons
     tn_tensor tc = strided(const_cast<float*>(W->cores[ls]), 4, shc, stc);
     tn_tensor tr = strided(w.gR, 2, shr, str);
     const int lh[3] = {1, 2, 3}, lc[3] = {0, 1, 2};
-    if ((rc = contract_internal(&th, lh, &tc, lc, 3, &tr, label_prec(prec), s, w.scratch, w.scratch_bytes)) != TN_OK) return rc;
+    if ((rc = contract_internal(&th, lh, &tc, lc, 3, &tr, label_prec(prec), s)) != TN_OK) return rc;
     const int64_t nvec = B * chi;
     cls_pad_rows<<<(unsigned)((nvec + 255) / 256), 256, 0, s>>>(w.gR, (int)DR, w.g[1], batch, chi);
     if (cudaGetLastError() != cudaSuccess) return TN_ERR_CUDA;
     tn_tensor tv = strided(w.state[1], 2, shv, stv);
     tn_tensor td = strided(dcores[ls], 4, shc, stc);
     const int l0[1] = {0};
-    if ((rc = contract_internal(&th, l0, &tv, l0, 1, &td, label_prec(prec), s, w.scratch, w.scratch_bytes)) != TN_OK) return rc;
+    if ((rc = contract_internal(&th, l0, &tv, l0, 1, &td, label_prec(prec), s)) != TN_OK) return rc;
   }
 
   const int seg = ckpt_every <= 1 ? std::max(std::max(w.T[0], w.T[1]), 1) : ckpt_every;
