@@ -108,10 +108,10 @@ mps_inner_small_kernel(const __grid_constant__ SmallChain c, double* result) {
 }
 
 // The same sweep with both cores of every site staged in shared memory, rows
-// padded to multiples of four: the cores of site i + 1 are copied in
+// padded to multiples of four: the cores of the next sites are copied in
 // (cp.async, no registers) while site i is contracted.
-// Dynamic shared memory: E (emax floats), T (tmax), two ket and two bra core
-// buffers (cmax each).
+// Dynamic shared memory: E (emax floats), T (tmax), `ring` ket and `ring` bra
+// core buffers (cmax each).
 //
 // What bounds it: one CTA's shared-memory reads and the latency of three
 // barriers a site. Each output is one chain of FMAs over ascending k, so the
@@ -119,9 +119,12 @@ mps_inner_small_kernel(const __grid_constant__ SmallChain c, double* result) {
 // a 16-byte read of the second operand feeds 8 FMAs (issued as packed pairs),
 // and E is read four k at a time; E' stays in registers until the block's
 // maximum is known and is divided by it there. Measured, N = 20, chi = 32
-// (kernel): 66 -> 47 us.
+// (kernel): 66 -> 47 us; n = 200, chi = 4 327 -> 260 us, 60 x 64 1457 -> 705.
 struct StagedSizes {
   int32_t emax, tmax, cmax;
+  int32_t ring;  // core buffers of each chain: sites up to ring - 1 ahead are on their way (4, else 2)
+  int32_t apart; // no site has more than 128 tiles: the other 128 threads copy (bonds up to 16: a
+                 // tenth of a site's time)
 };
 
 __host__ __device__ __forceinline__ int32_t pad4(int32_t x) { return (x + 3) & ~3; }
@@ -134,20 +137,22 @@ __device__ __forceinline__ void cp_async_16(float* dst, const float* src) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_but_two() { asm volatile("cp.async.wait_group 2;" ::: "memory"); }
 
 // i / n for 0 <= i < 2^16, 0 < n (inv = 1 / n to within an ulp or two).
 __device__ __forceinline__ int small_div(int i, float inv) { return (int)(((float)i + 0.5f) * inv); }
 
 // Copies `rows` rows of `cols` floats global -> shared rows of pad4(cols), by
-// all threads of the block; the padding keeps what it holds.
-__device__ __forceinline__ void stage_core(float* dst, const float* __restrict__ src, int rows, int cols) {
+// thread t of nt; the padding keeps what it holds.
+__device__ __forceinline__ void stage_core(float* dst, const float* __restrict__ src, int rows, int cols, int t,
+                                           int nt) {
   const int n = rows * cols;
   if ((cols & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
-    for (int i = threadIdx.x * 4; i < n; i += SMALL_THREADS * 4) cp_async_16(dst + i, src + i);
+    for (int i = t * 4; i < n; i += nt * 4) cp_async_16(dst + i, src + i);
   } else {
     const int ld = pad4(cols);
-    const float inv = __frcp_rn((float)cols);
-    for (int i = threadIdx.x; i < n; i += SMALL_THREADS) {
+    const float inv = __fdividef(1.0f, (float)cols);
+    for (int i = t; i < n; i += nt) {
       const int r = small_div(i, inv);
       cp_async_f32(dst + r * ld + (i - r * cols), src + i);
     }
@@ -197,33 +202,39 @@ mps_inner_staged_kernel(const __grid_constant__ SmallChain c, StagedSizes z, dou
   extern __shared__ __align__(16) float smf[];
   float* E = smf;
   float* T = E + z.emax;
-  float* const kbuf = T + z.tmax;          // ket cores of sites i (i & 1) and i + 1
-  float* const bbuf = kbuf + 2 * z.cmax;   // bra cores, likewise
+  float* const kbuf = T + z.tmax;  // ket cores of site i (i % ring) and of the ones after it
+  float* const bbuf = kbuf + z.ring * z.cmax;  // bra cores, likewise
   __shared__ float red[SMALL_THREADS / 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int d = c.d;
   if (tid == 0) E[0] = 1.0f;
   double lg = 0.0;
-  stage_core(kbuf, c.ket[0], c.bk[0] * d, c.bk[1]);
-  stage_core(bbuf, c.bra[0], c.bb[0] * d, c.bb[1]);
-  cp_async_commit();
+  const int ring = z.ring, mask = ring - 1;
+  auto stage = [&](int i) {
+    if (i < c.n) {
+      const int t = z.apart ? tid - SMALL_THREADS / 2 : tid, nt = z.apart ? SMALL_THREADS / 2 : SMALL_THREADS;
+      if (t >= 0) {
+        stage_core(kbuf + (i & mask) * z.cmax, c.ket[i], c.bk[i] * d, c.bk[i + 1], t, nt);
+        stage_core(bbuf + (i & mask) * z.cmax, c.bra[i], c.bb[i] * d, c.bb[i + 1], t, nt);
+      }
+    }
+    cp_async_commit();  // a group a site, empty past the end
+  };
+  for (int i = 0; i + 1 < ring; ++i) stage(i);
   constexpr int TILES = SMALL_D / 2 * (SMALL_D / 4) / SMALL_THREADS;  // tiles of E' per thread, at most
   for (int i = 0; i < c.n; ++i) {
     const int Da = c.bb[i], Db = c.bb[i + 1], Dak = c.bk[i], Dbk = c.bk[i + 1];
-    cp_async_wait_all();
+    if (ring == 4) cp_async_wait_but_two();
+    else cp_async_wait_all();
     __syncthreads();  // site i's cores (and E) visible to all; buffers of site i-1 free
-    if (i + 1 < c.n) {
-      stage_core(kbuf + ((i + 1) & 1) * z.cmax, c.ket[i + 1], Dbk * d, c.bk[i + 2]);
-      stage_core(bbuf + ((i + 1) & 1) * z.cmax, c.bra[i + 1], Db * d, c.bb[i + 2]);
-    }
-    cp_async_commit();
-    const float* K = kbuf + (i & 1) * z.cmax;
-    const float* Br = bbuf + (i & 1) * z.cmax;
+    stage(i + ring - 1);
+    const float* K = kbuf + (i & mask) * z.cmax;
+    const float* Br = bbuf + (i & mask) * z.cmax;
     const int lde = pad4(Dak), ldk = pad4(Dbk), ldb = pad4(Db), qn = ldk >> 2;
-    const float iq = __frcp_rn((float)qn);
+    const float iq = __fdividef(1.0f, (float)qn);
     // T[a, s, bk] = sum_ak E[a, ak] K[ak, s, bk]: two a and four bk per thread
     {
-      const float id = __frcp_rn((float)d);
+      const float id = __fdividef(1.0f, (float)d);
       const int tiles = ((Da + 1) >> 1) * d * qn;
       for (int idx = tid; idx < tiles; idx += SMALL_THREADS) {
         const int rest = small_div(idx, iq), q = idx - rest * qn;
@@ -282,6 +293,8 @@ mps_inner_staged_kernel(const __grid_constant__ SmallChain c, StagedSizes z, dou
           if (4 * q + j < Dbk) {
             mx = fmaxf(mx, fabsf(v[t][0][j]));
             if (second) mx = fmaxf(mx, fabsf(v[t][1][j]));
+          } else {
+            v[t][0][j] = v[t][1][j] = 0.0f;  // made of padding
           }
         }
       }
@@ -870,14 +883,18 @@ int tn_mps_inner(const tn_mps* bra, const tn_mps* ket, int prec, void* workspace
     }
     // staged variant when its buffers fit: E, T and four core buffers, rows
     // padded to multiples of four
-    StagedSizes z{4, 4, 4};
+    StagedSizes z{4, 4, 4, 4, 1};
     for (int i = 0; i < bra->n; ++i) {
+      const int32_t qn = pad4(c.bk[i + 1]) / 4;
+      if (std::max((c.bb[i] + 1) / 2 * c.d, (c.bb[i + 1] + 1) / 2) * qn > SMALL_THREADS / 2) z.apart = 0;
       z.emax = std::max(z.emax, c.bb[i + 1] * pad4(c.bk[i + 1]));
       z.tmax = std::max(z.tmax, c.bb[i] * c.d * pad4(c.bk[i + 1]));
       z.cmax = std::max(z.cmax, std::max(c.bb[i] * c.d * pad4(c.bb[i + 1]), c.bk[i] * c.d * pad4(c.bk[i + 1])));
     }
-    const size_t staged = sizeof(float) * ((size_t)z.emax + z.tmax + 4 * (size_t)z.cmax);
     constexpr size_t STAGED_MAX = 200 * 1024;
+    auto need = [&](int ring) { return sizeof(float) * ((size_t)z.emax + z.tmax + 2 * ring * (size_t)z.cmax); };
+    if (need(z.ring) > STAGED_MAX) z.ring = 2;
+    const size_t staged = need(z.ring);
     if (staged <= STAGED_MAX) {
       static std::atomic<uint64_t> attr2{0};
       if (!smem_limit_once((const void*)mps_inner_staged_kernel, STAGED_MAX, &attr2)) return TN_ERR_CUDA;

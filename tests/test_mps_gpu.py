@@ -171,6 +171,22 @@ def test_energy_long_chain_both_launch_forms(tn, n, prec):
     assert rel(val(r, 1), norm) <= tol(prec, 2 * n) + 2 * n * bias
 
 
+@pytest.mark.parametrize("d,lo,hi", [(2, 1, 3), (2, 5, 7), (2, 15, 18), (2, 61, 64), (3, 1, 40), (4, 30, 33)])
+def test_inner_one_cta_bond_edges(tn, d, lo, hi):
+    # the one-CTA sweep's padded rows (bonds off a multiple of four, bra and
+    # ket different), its copying threads apart (up to 128 tiles) or not, four
+    # or two core buffers, and the unstaged form past them. All numbers
+    # positive, so nothing cancels: the float32 tolerance of a sweep.
+    n = 14
+    rng = np.random.default_rng(10 * d + hi)
+    bonds = [[1] + [int(x) for x in rng.integers(lo, hi + 1, n - 1)] + [1] for _ in range(2)]
+    a, b = [[(rng.uniform(0.5, 1.5, (c[i], d, c[i + 1])) / math.sqrt(c[i] * c[i + 1])).astype(np.float32)
+             for i in range(n)] for c in bonds]
+    v, lg = oracle.mps_inner(a, b)
+    r = tn.mps_inner(to_dev(a), to_dev(b), prec="fp32")
+    assert rel(val(r), v * math.exp(lg)) <= 1e-5
+
+
 @pytest.mark.parametrize("d,w", [(1, 3), (1, 7), (2, 1), (2, 2), (2, 3), (3, 1), (4, 1)])
 @pytest.mark.parametrize("prec", ["bf16x3", "bf16"])
 def test_energy_tiles_of_the_one_launch_sweep(tn, d, w, prec):
