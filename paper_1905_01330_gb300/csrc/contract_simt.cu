@@ -327,6 +327,7 @@ __device__ __forceinline__ void multiply(SimtSmem& s, float* ring, int subs, int
             acc[i][j] = make_float2(f.x + acc[i][j].x, f.y + acc[i][j].y);
             acc[i][j + 1] = make_float2(f.z + acc[i][j + 1].x, f.w + acc[i][j + 1].y);
           }
+        __syncwarp();  // the rows below lie over other lanes' sums
       }
       if (ke < s.uc.k_end) {
 #pragma unroll

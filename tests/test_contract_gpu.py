@@ -394,3 +394,17 @@ def test_fp32_group_with_long_k_ranges(tn):
         check(C, A, [1], B, [0], "fp32")
     for sp in specs[:10]:
         assert torch.equal(sp[4], torch.full_like(sp[4], 64.0))
+
+
+@pytest.mark.parametrize("M,N,K", [(2048, 512, 1024), (1024, 256, 1024), (20000, 16, 1100)])
+def test_fp32_chunks_of_a_unit(tn, M, N, K):
+    # several chains added up in the shared-memory region that the result's
+    # rows then pass through, in each tile shape (64 x 128, 32 x 128, 16 x 256
+    # with the operands exchanged): no lane's rows before another's sums are
+    # read. At most two addends reach a result, so a repeat has the same bits.
+    A, B = rand(101, (M, K)), rand(102, (K, N))
+    At, Bt = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    C = tn.contract(At, [1], Bt, [0], prec="fp32")
+    check(C, A, [1], B, [0], "fp32")
+    for _ in range(4):
+        assert torch.equal(tn.contract(At, [1], Bt, [0], prec="fp32"), C)
