@@ -199,7 +199,7 @@ int tn::contract_internal(const tn_tensor* A, const int* legsA, const tn_tensor*
   if (prec == TN_PREC_FP32 && outer_ok(d)) return launch_outer(d, s);
   if (prec == TN_PREC_FP32 && any_order && matvec_ok(d)) return launch_matvec(d, s);
   plan_units(&d, min_units_single());
-  if (prec == TN_PREC_FP32) plan_simt(&d, SimtPlan::alone);
+  if (prec == TN_PREC_FP32) plan_simt(&d, any_order ? SimtPlan::alone : SimtPlan::sweep);
   if (prec != TN_PREC_FP32 && scratch && packed_single_bytes(d, prec) <= scratch_bytes)
     return contract_packed_single(d, prec, scratch, scratch_bytes, s);
   if (d.splits > 1 &&

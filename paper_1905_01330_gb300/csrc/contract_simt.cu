@@ -493,6 +493,9 @@ void plan_simt(ContractDesc* d, SimtPlan how) {
         for (int64_t c = 1; c <= d->splits; ++c) {  // chunks of a unit
           const int64_t sp = (slabs + c * chunk - 1) / (c * chunk), u = (tiles * sp + 151) / 152;
           if (sp > 2 && tiles >= 16) continue;  // two addends commute: such results do not vary from run to run
+          // a sweep's results stay sums of the k ranges one by one, in whatever
+          // order: all ranges in ascending order in one unit, or a unit each
+          if (how == SimtPlan::sweep && c > 1 && c < d->splits) continue;
           const double t = (double)((u + 1) / 2) * 8000.0 +
                            (double)u * (double)(4 * std::min(slabs, c * chunk)) * slab[k] + (sp > 1 ? 6000.0 : 0.0);
           if (best < 0.0 || t < best) {

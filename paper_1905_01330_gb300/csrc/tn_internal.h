@@ -87,8 +87,11 @@ void plan_units(ContractDesc* d, int64_t min_units);
 // Tile shape, orientation, load widths and k ranges of an FP32 contraction
 // planned by plan_units, whose k ranges become the chains a result is summed
 // in: alone (a unit may run several of them, so that the tiles fill the SMs),
-// in a group (the k ranges as given) or as 128 x 128 units (as given).
-enum class SimtPlan { alone, group, pairs };
+// in a sweep over a chain (all of them in a unit or one, so that a result is
+// the sum of the chains added one by one, as it always was: its float64
+// energies show such sums in the seventh digit), in
+// a group (the k ranges as given) or as 128 x 128 units (as given).
+enum class SimtPlan { alone, sweep, group, pairs };
 void plan_simt(ContractDesc* d, SimtPlan how);
 // Work units a lone contraction asks plan_units for (two per SM).
 int64_t min_units_single();

@@ -97,3 +97,58 @@ def test_clock_sampler_keeps_samples_of_the_timed_region(tmp_path, monkeypatch):
     s = bench.ClockSampler(0)
     s.start()
     assert s.stop() is None
+
+
+SUM_ORDER = r"""
+#include <cstdio>
+#include "tn_internal.h"
+using namespace tn;
+int main() {
+  long long M, N, K, ta, tb;
+  while (scanf("%lld %lld %lld %lld %lld", &M, &N, &K, &ta, &tb) == 5) {
+    tn_tensor A{}, B{}, C{};
+    A.data = B.data = C.data = (void*)4096;
+    A.rank = B.rank = C.rank = 2;
+    A.dtype = B.dtype = C.dtype = TN_F32;
+    A.shape[0] = ta ? K : M; A.shape[1] = ta ? M : K;
+    B.shape[0] = tb ? N : K; B.shape[1] = tb ? K : N;
+    C.shape[0] = M; C.shape[1] = N;
+    const int la = ta ? 0 : 1, lb = tb ? 1 : 0;
+    ContractDesc d;
+    if (plan_contract(&A, &la, &B, &lb, 1, &C, &d) != TN_OK) return 1;
+    plan_units(&d, 304);
+    const long long ranges = d.splits, range = d.k_per_split;
+    plan_simt(&d, SimtPlan::sweep);
+    printf("%lld %lld %d %lld %d\n", ranges, range, (int)d.splits, (long long)d.k_per_split, (int)d.chunk);
+  }
+}
+"""
+
+
+def test_sweep_results_are_sums_of_the_k_ranges_one_by_one(built, tmp_path):
+    """A float32 contraction of a sweep adds the chains of plan_units' k ranges
+    (at most 2048 shared indices each) to a result one by one: a unit runs one
+    of them, or all in ascending order. Sums of sums, which no order of such
+    additions gives, are for lone contractions only. Over the bonds an energy
+    or norm sweep meets, rising, level and falling, and MPO bonds 1 to 5."""
+    src, exe = tmp_path / "order.cpp", tmp_path / "order"
+    src.write_text(SUM_ORDER)
+    subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "paper_1905_01330_gb300", "csrc"),
+                    "-I", "/usr/local/cuda/include", str(src), built, "-Wl,-rpath," + os.path.dirname(built),
+                    "-o", str(exe)], check=True, timeout=300)
+    bonds = [(a, b) for c in (100, 256, 300, 383, 384, 400, 512, 640, 1024) for a, b in ((c, c), (c, c // 2), (c // 2, c))]
+    cases = []
+    for a, b in bonds:
+        for d in (2, 3):
+            cases += [(a, d * b, a, 1, 0), (b, b, d * a, 1, 0)]                       # norm
+            for w in (2, 4, 6):
+                cases += [(w * a, d * b, a, 1, 0), (w * b, b, d * a, 0, 0)]           # energy
+    out = subprocess.run([str(exe)], input="".join("%d %d %d %d %d\n" % c for c in cases), capture_output=True, text=True,
+                         check=True, timeout=300).stdout.split("\n")
+    several = 0
+    for case, line in zip(cases, out):
+        ranges, rng, units, per, chunk = map(int, line.split())
+        assert chunk * 64 == min(rng, 2048) and per % (chunk * 64) == 0, (case, line)
+        assert units == 1 or (units == ranges and per == rng), (case, line)
+        several += ranges > 2
+    assert several >= 20

@@ -340,3 +340,24 @@ def test_grouped_energy_plan_runs_like_the_one_shot_call(tn):
     for j in (0, 2):
         assert rel(c[1, j] * math.exp(c[1, j + 1]), 4.0 * a[1, j] * math.exp(a[1, j + 1])) <= 1e-5
         assert rel(c[0, j] * math.exp(c[0, j + 1]), a[0, j] * math.exp(a[0, j + 1])) <= 1e-12
+
+
+def test_fp32_energy_repeats_its_bits(tn):
+    # bonds at which step (iii) sums its shared index in four chains, and the
+    # falling bond behind them: the chains are added in one order, so a second
+    # pass has the same bits
+    bonds = [1, 256, 512, 512, 256, 128, 1]
+    n = len(bonds) - 1
+    rng = np.random.default_rng(61)
+    cores = [(rng.uniform(0.5, 1.5, (bonds[i], 2, bonds[i + 1])) / math.sqrt(bonds[i] * bonds[i + 1])).astype(np.float32)
+             for i in range(n)]
+    wb = [1] + [3] * (n - 1) + [1]
+    W = [rng.uniform(0.5, 1.5, (wb[i], wb[i + 1], 2, 2)).astype(np.float32) for i in range(n)]
+    e, le = oracle.mpo_expect(cores, W)
+    nv, ln = oracle.mps_inner(cores, cores)
+    dc, dw = to_dev(cores), to_dev(W)
+    first = tn.mps_expect(dc, dw, prec="fp32").cpu()
+    assert rel(val(first, 0), e * math.exp(le)) <= 1e-5
+    assert rel(val(first, 1), nv * math.exp(ln)) <= 1e-5
+    for _ in range(8):
+        assert torch.equal(tn.mps_expect(dc, dw, prec="fp32").cpu(), first)
