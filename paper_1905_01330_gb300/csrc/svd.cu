@@ -49,6 +49,13 @@ constexpr int SVD_MAX_SWEEPS = 40;
 constexpr int SVD_B = 16;      // columns of a block
 constexpr int SVD_CH = 256;    // rows staged at once
 constexpr int SVD_CLUSTER = 8; // most CTAs that share out a pair's rows
+// W is the matrix times a power of two that brings the sum of its squares to
+// 2^80 at most; a column whose squared norm is 2^-100 or less there (2^-90 of
+// the matrix) is left as it is. So a rotation's quotients stay normal numbers
+// whatever the node's scale: squares of 2^-126 and less would count as 0 in
+// the approximate roots.
+constexpr int SVD_TOP = 40;
+constexpr float SVD_NULL = 0x1p-100f;
 
 // The node's matrix view: element (i, j) at A + loff(i) + roff(j).
 struct SplitView {
@@ -71,9 +78,30 @@ __device__ __forceinline__ int64_t leg_offset(int64_t idx, int n, const int32_t*
   return off;
 }
 
+// *bits: the bits of the node's largest magnitude (0 before).
+__global__ void svd_largest(SplitView v, unsigned* bits) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  unsigned m = 0u;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < v.M * v.N; e += stride) {
+    const int64_t i = e / v.N, j = e - i * v.N;
+    const float x = v.A[leg_offset(i, v.nl, v.ldim, v.lstr) + leg_offset(j, v.nr, v.rdim, v.rstr)];
+    m = max(m, __float_as_uint(fabsf(x)));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(bits, m);
+}
+
+// The exponent of the power of two W is scaled by; 0 for zeros, infinities and
+// NaN. half: (log2 of the matrix's entries) / 2, rounded up.
+__device__ __forceinline__ int svd_shift(unsigned bits, int half) {
+  return bits == 0u || bits >= 0x7F800000u ? 0 : SVD_TOP - half - 1 - ilogbf(__uint_as_float(bits));
+}
+
 // W in blocks of 16 columns, [block][row][16] (zeros past column r), V = I
 // likewise.
-__global__ void svd_gather(SplitView v, float* __restrict__ W, float* __restrict__ V, int64_t L, int64_t r, int64_t cols) {
+__global__ void svd_gather(SplitView v, const unsigned* bits, int half, float* __restrict__ W, float* __restrict__ V, int64_t L,
+                           int64_t r, int64_t cols) {
+  const int shift = svd_shift(*bits, half);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   for (int64_t w = first; w < L * cols; w += stride) {
     // neighbouring threads walk the view's own rows where those are columns of W
@@ -82,7 +110,7 @@ __global__ void svd_gather(SplitView v, float* __restrict__ W, float* __restrict
     float x = 0.0f;
     if (col < r) {
       const int64_t i = v.wide ? col : row, j = v.wide ? row : col;
-      x = v.A[leg_offset(i, v.nl, v.ldim, v.lstr) + leg_offset(j, v.nr, v.rdim, v.rstr)];
+      x = ldexpf(v.A[leg_offset(i, v.nl, v.ldim, v.lstr) + leg_offset(j, v.nr, v.rdim, v.rstr)], shift);
     }
     W[w] = x;
   }
@@ -172,11 +200,12 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
 // The rotations (Hestenes) of one round on the Gram matrix in s.G[0], and
 // their product in s.Q: for a pair with a = g_pp, b = g_qq, g = g_pq the
 // tangent t is the smaller root, h sign(d) / (|d| + sqrt(d^2 + h^2)) for d = (b
-// - a) / sqrt(ab) and h = 2 g / sqrt(ab); c = 1 / sqrt(1 + t^2), s = c t, and the columns become (c p -
-// s q, s p + c q). Pairs orthogonal to within tol (|g| <= tol sqrt(ab)) are
-// left alone, but counted only above 16 tol: the sweeps end when none is, and
-// what the last one still found below that is rotated away. FULL: all pairs of the 32 columns by the circle method, else
-// the pairs across the two blocks. Every warp computes the step's 16 angles
+// - a) / sqrt(ab) and h = 2 g / sqrt(ab); c = 1 / sqrt(1 + t^2), s = c t, and
+// the columns become (c p - s q, s p + c q). Pairs orthogonal to within tol
+// (|g| <= tol sqrt(ab)) are left alone, as are columns of SVD_NULL; counted are
+// only those above 16 tol: the sweeps end when none is, and what the last one
+// still found below that is rotated away. FULL: all pairs of the 32 columns by
+// the circle method, else the pairs across the two blocks. Every warp computes the step's 16 angles
 // (lanes 0-15; approximate quotients and roots: they only move the angle, the
 // next rounds see what is left); thread (u, v) updates the 2 x 2 block of pairs
 // u and v and two rows of Q. Returns whether it rotated anything, and adds to
@@ -200,9 +229,12 @@ __device__ __forceinline__ bool svd_rotate(SvdSmem& s, float tol, int& count) {
     const float b00 = g[pu][pv], b01 = g[pu][qv], b10 = g[qu][pv], b11 = g[qu][qv];
     // scaled by the two norms, so that no square leaves the exponent range
     const float ia = rsqrt_approx(al), ib = rsqrt_approx(be), co = ga * ia * ib;
-    const bool go = al > 0.0f && be > 0.0f && fabsf(co) > tol;
+    const bool go = al > SVD_NULL && be > SVD_NULL && fabsf(co) > tol;
     const float d = (be - al) * ia * ib, h = co + co;
-    const float tt = fminf(fabsf(h) * rcp_approx(fabsf(d) + sqrt_approx(fmaf(d, d, h * h))), 1.0f);
+    // the root is at most |d| + |h|, which it gives way to where d^2 overflows
+    // (norms far apart: a pair turned by 0 for it would be counted for ever)
+    const float root = fminf(sqrt_approx(fmaf(d, d, h * h)), fabsf(d) + fabsf(h));
+    const float tt = fminf(fabsf(h) * rcp_approx(fabsf(d) + root), 1.0f);
     const float ts = (d < 0.0f) != (h < 0.0f) ? -tt : tt;
     float c = rsqrt_approx(fmaf(tt, tt, 1.0f)), sn = c * ts;
     // c^2 + s^2 = 1 to the rounding of c and s: a bias here would drift the
@@ -423,12 +455,13 @@ __device__ __forceinline__ int64_t blocked(int64_t row, int64_t col, int64_t n) 
   return ((col / SVD_B) * n + row) * SVD_B + col % SVD_B;
 }
 
-// Column j (CTA j): vnorm[j] = |V[:, j]| and sigma[j] = |W[:, j]| / vnorm[j].
-// Both blocks took the same products with Q, so what these left of the unit
-// length of V's columns is also in W's and cancels.
+// Column j (CTA j): vnorm[j] = |V[:, j]|, wnorm[j] = |W[:, j]| and sigma[j] =
+// their quotient, without W's power of two. Both blocks took the same products
+// with Q, so what these left of the unit length of V's columns is also in W's
+// and cancels.
 __global__ void __launch_bounds__(SVD_THREADS)
-svd_norms(const float* __restrict__ W, const float* __restrict__ V, int64_t L, int64_t r, float* __restrict__ sigma,
-          float* __restrict__ vnorm) {
+svd_norms(const float* __restrict__ W, const float* __restrict__ V, int64_t L, int64_t r, const unsigned* bits, int half,
+          float* __restrict__ sigma, float* __restrict__ vnorm, float* __restrict__ wnorm) {
   const float* w = W + blocked(0, blockIdx.x, L);
   const float* v = V + blocked(0, blockIdx.x, r);
   float a = 0.0f, b = 0.0f;
@@ -436,9 +469,10 @@ svd_norms(const float* __restrict__ W, const float* __restrict__ V, int64_t L, i
   for (int64_t i = threadIdx.x; i < r; i += SVD_THREADS) b = fmaf(v[i * SVD_B], v[i * SVD_B], b);
   const double sa = block_sum(a), sb = block_sum(b);
   if (threadIdx.x == 0) {
-    const double vn = sqrt(sb);
+    const double vn = sqrt(sb), wn = sqrt(sa);
     vnorm[blockIdx.x] = (float)vn;
-    sigma[blockIdx.x] = (float)(sqrt(sa) / vn);
+    wnorm[blockIdx.x] = (float)wn;
+    sigma[blockIdx.x] = (float)ldexp(wn / vn, -svd_shift(*bits, half));
   }
 }
 
@@ -459,16 +493,14 @@ __global__ void svd_sort(const float* __restrict__ sigma, int r, int32_t* __rest
   sorted[rank] = sigma[j];
 }
 
-// The outputs for the k kept values. Columns of V give singular vectors scaled
-// by vnorm, columns of W scaled by sigma vnorm (w_j = sigma_j vnorm_j u_j). Left (M x k,
-// row-major): W's columns when M >= N, else V's; right (k x N, row-major):
+// The outputs for the k kept values: columns of V and W over their norms. Left
+// (M x k, row-major): W's columns when M >= N, else V's; right (k x N, row-major):
 // the other one. absorb: both sides carry sqrt(sigma) (split_node), else
 // neither (full SVD). A W column of a zero singular value has no direction:
 // its vector is written as zeros (not completed to an orthonormal basis).
 __global__ void svd_write(const float* __restrict__ W, const float* __restrict__ V, const int32_t* __restrict__ order,
-                          const float* __restrict__ sorted, const float* __restrict__ vnorm, int64_t M, int64_t N,
-                          int64_t L, int r, int k,
-                          int wide, int absorb, float* __restrict__ U, float* __restrict__ S, float* __restrict__ Vt,
+                          const float* __restrict__ sorted, const float* __restrict__ vnorm,
+                          const float* __restrict__ wnorm, int64_t M, int64_t N, int64_t L, int r, int k, int wide, int absorb, float* __restrict__ U, float* __restrict__ S, float* __restrict__ Vt,
                           float* __restrict__ dropped) {
   const int64_t nl = M * k, nr = (int64_t)k * N, stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -479,14 +511,13 @@ __global__ void svd_write(const float* __restrict__ W, const float* __restrict__
     const int64_t i = left ? f / k : f % N;  // row of the left node, column of the right one
     const int j = min(max(order[c], 0), r - 1);
     const float sg = sorted[c];
-    const float vn = vnorm[j];
     const bool from_w = left != (wide != 0);  // left from W iff M >= N
     float x;
     if (from_w) {
-      const float sc = sg > 0.0f ? (absorb ? 1.0f / (sqrtf(sg) * vn) : 1.0f / (sg * vn)) : 0.0f;
+      const float sc = sg > 0.0f ? (absorb ? sqrtf(sg) / wnorm[j] : 1.0f / wnorm[j]) : 0.0f;
       x = W[blocked(i, j, L)] * sc;
     } else {
-      x = V[blocked(i, j, r)] * (absorb ? sqrtf(fmaxf(sg, 0.0f)) / vn : 1.0f / vn);
+      x = V[blocked(i, j, r)] * (absorb ? sqrtf(fmaxf(sg, 0.0f)) / vnorm[j] : 1.0f / vnorm[j]);
     }
     if (left)
       U[f] = x;
@@ -504,7 +535,7 @@ static size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 struct SplitLayout {
   SplitView v;
   int64_t L, r, ns;  // ns: blocks of 16 columns
-  size_t w_off, v_off, sig_off, vn_off, ord_off, sorted_off, cnt_off, total;
+  size_t w_off, v_off, sig_off, vn_off, wn_off, ord_off, sorted_off, cnt_off, total;
 };
 
 static int plan_split(const tn_tensor* A, const int* left, int nleft, const int* right, int nright,
@@ -559,10 +590,11 @@ static int plan_split(const tn_tensor* A, const int* left, int nleft, const int*
   o.v_off = al256(sizeof(float) * (size_t)(o.L * o.ns * SVD_B));
   o.sig_off = o.v_off + al256(sizeof(float) * (size_t)(o.r * o.ns * SVD_B));
   o.vn_off = o.sig_off + al256(sizeof(float) * (size_t)o.r);
-  o.ord_off = o.vn_off + al256(sizeof(float) * (size_t)o.r);
+  o.wn_off = o.vn_off + al256(sizeof(float) * (size_t)o.r);
+  o.ord_off = o.wn_off + al256(sizeof(float) * (size_t)o.r);
   o.sorted_off = o.ord_off + al256(sizeof(int32_t) * (size_t)o.r);
   o.cnt_off = o.sorted_off + al256(sizeof(float) * (size_t)(o.r + 1));  // the values, then the sweep count
-  o.total = o.cnt_off + 256;  // barrier counter, rotations per sweep
+  o.total = o.cnt_off + 256;  // barrier counter, rotations per sweep, the largest magnitude
   return TN_OK;
 }
 
@@ -619,6 +651,7 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
   float* V = reinterpret_cast<float*>(base + lay.v_off);
   float* sigma = reinterpret_cast<float*>(base + lay.sig_off);
   float* vnorm = reinterpret_cast<float*>(base + lay.vn_off);
+  float* wnorm = reinterpret_cast<float*>(base + lay.wn_off);
   int32_t* order = reinterpret_cast<int32_t*>(base + lay.ord_off);
   float* sorted = reinterpret_cast<float*>(base + lay.sorted_off);
   const int64_t L = lay.L, cols = lay.ns * SVD_B;
@@ -636,11 +669,15 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
   P.counts = reinterpret_cast<int*>(base + lay.cnt_off) + 1;
   P.sweeps = reinterpret_cast<int*>(sorted + r);
   P.status = status_word();
-  static_assert(sizeof(int) * (SVD_MAX_SWEEPS + 1) <= 256, "barrier counter and rotation counts");
+  static_assert(sizeof(int) * (SVD_MAX_SWEEPS + 2) <= 256, "barrier counter, rotation counts, largest magnitude");
+  unsigned* bits = P.bar + SVD_MAX_SWEEPS + 1;
+  int half = 0;  // 4^half >= M N
+  while (half < 31 && (int64_t(1) << (2 * half)) < L * r) ++half;
   if (cudaMemsetAsync(base + lay.cnt_off, 0, 256, s) != cudaSuccess ||
       cudaMemsetAsync(P.sweeps, 0, sizeof(int), s) != cudaSuccess)
     return TN_ERR_CUDA;
-  svd_gather<<<grid_for(L * cols, 256), 256, 0, s>>>(lay.v, W, V, L, lay.r, cols);
+  svd_largest<<<grid_for(L * r, 256), 256, 0, s>>>(lay.v, bits);
+  svd_gather<<<grid_for(L * cols, 256), 256, 0, s>>>(lay.v, bits, half, W, V, L, lay.r, cols);
   if (cudaGetLastError() != cudaSuccess) return TN_ERR_CUDA;
   static std::atomic<uint64_t> attr{0};
   if (!smem_limit_once((const void*)svd_jacobi, sizeof(SvdSmem), &attr)) return TN_ERR_CUDA;
@@ -671,7 +708,7 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
       break;
   }
   if (cudaLaunchKernelEx(&cfg, svd_jacobi, P) != cudaSuccess) return TN_ERR_CUDA;
-  svd_norms<<<r, SVD_THREADS, 0, s>>>(W, V, L, r, sigma, vnorm);
+  svd_norms<<<r, SVD_THREADS, 0, s>>>(W, V, L, r, bits, half, sigma, vnorm, wnorm);
   svd_sort<<<(r + 255) / 256, 256, 0, s>>>(sigma, r, order, sorted);
   if (cudaGetLastError() != cudaSuccess) return TN_ERR_CUDA;
   std::vector<float> host_sorted((size_t)r + 1);
@@ -684,9 +721,9 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
   if (used == 0) return TN_ERR_TIMEOUT;  // the barrier's wait expired
   if (sweeps) *sweeps = used;
   const int64_t k = tn_split_truncation(host_sorted.data(), r, max_singular_values, max_truncation_err);
-  svd_write<<<grid_for((lay.v.M + lay.v.N) * k + r, 256), 256, 0, s>>>(W, V, order, sorted, vnorm, lay.v.M, lay.v.N, L,
-                                                                        r, (int)k, lay.v.wide, absorb ? 1 : 0, U, S, Vt,
-                                                                        dropped);
+  svd_write<<<grid_for((lay.v.M + lay.v.N) * k + r, 256), 256, 0, s>>>(W, V, order, sorted, vnorm, wnorm, lay.v.M,
+                                                                        lay.v.N, L, r, (int)k, lay.v.wide, absorb ? 1 : 0,
+                                                                        U, S, Vt, dropped);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return TN_ERR_CUDA;
   *kept = k;
   return TN_OK;

@@ -168,3 +168,49 @@ def test_block_edges(tn, shape, scale):
     # come near the ends of the exponent range; tolerances as above
     A = (rand(31, shape) * np.float32(scale)).astype(np.float32)
     check(tn, A, [0], [1])
+
+
+def node_kinds():
+    """Nodes whose columns (of the matrix, or what rotations leave of them) have
+    norms far apart, or whose squares leave the exponent range: low rank, few
+    non-zero rows, zero-padded bonds, blocks beside tiny entries, graded columns."""
+    out = []
+    for scale in (1.0, 1e-8, 1e-12, 1e-13, 1e-15, 1e-18, 1e18):
+        for rank in (1, 4):
+            out.append(("rank", (32, 32), rank, scale))
+    out += [("rank", (256, 256), 3, 1e-13), ("rank", (40, 600), 2, 1e-14)]
+    for size in (4, 16):
+        for tiny in (1e-12, 1e-19, 1e-20, 1e-22):
+            out.append(("block", (32, 32), size, tiny))
+    for rows in (1, 2, 3, 4, 6, 8):
+        out += [("rows", (32, 16), rows, 1.0), ("rows", (48, 40), rows, 1e-10)]
+    for z in (1, 2, 3, 4):
+        out.append(("bond", (8, 2, 2, 8), z, 1.0))
+    for last in (1e-12, 1e-22, 1e-30):
+        out.append(("graded", (40, 40), 0, last))
+    out += [("full", (32, 32), 0, scale) for scale in (1e-18, 1e-20, 1e-25, 1e18, 1e25)]
+    return out
+
+
+@pytest.mark.parametrize("kind,shape,count,size", node_kinds())
+@pytest.mark.parametrize("seed", [0, 1, 2])
+def test_norms_far_apart(tn, kind, shape, count, size, seed):
+    # singular values and products as above, and the sweeps end by themselves
+    rng = np.random.default_rng(1000 * seed + count)
+    A = rng.standard_normal(shape)
+    if kind == "rank":
+        A = rng.standard_normal((shape[0], count)) @ rng.standard_normal((count, shape[1])) * size
+    elif kind == "block":
+        A[count:] *= size
+        A[:count, count:] *= size
+    elif kind == "rows":
+        A[count:] = 0.0
+        A *= size
+    elif kind == "bond":
+        A[count:] = 0.0
+    elif kind == "graded":
+        A *= np.logspace(0, np.log10(size), shape[1])
+    else:
+        A *= size
+    legs = ([0, 1], [2, 3]) if len(shape) == 4 else ([0], [1])
+    check(tn, A.astype(np.float32), *legs)
