@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import warnings
 from array import array
 
 import numpy as np
@@ -385,7 +386,8 @@ def split_node(A: torch.Tensor, left_legs, right_legs, max_singular_values: int 
     dropped singular values -- or, with full_svd, (u, s, vh, dropped) with s
     the k kept singular values (the diagonal of the singular-value node).
     Synchronises the stream (k decides the output shapes). info, if given,
-    receives the Jacobi sweep count."""
+    receives the Jacobi sweep count, negative if the limit was reached; that
+    also raises a RuntimeWarning."""
     lib = load()
     left, right = [int(p) for p in left_legs], [int(p) for p in right_legs]
     ad = tensor_desc(A)
@@ -416,6 +418,9 @@ def split_node(A: torch.Tensor, left_legs, right_legs, max_singular_values: int 
     k = kept.value
     if info is not None:
         info["sweeps"] = sweeps.value
+    if sweeps.value < 0:
+        warnings.warn("split_node: %d sweeps left column pairs that are not orthogonal" % -sweeps.value, RuntimeWarning,
+                      stacklevel=2)
     u = U[:M * k].view(ldims + [k])
     vh = Vt[:k * N].view([k] + rdims)
     dropped = D[:r - k]

@@ -152,3 +152,32 @@ def test_sweep_results_are_sums_of_the_k_ranges_one_by_one(built, tmp_path):
         assert units == 1 or (units == ranges and per == rng), (case, line)
         several += ranges > 2
     assert several >= 20
+
+
+@pytest.mark.parametrize("sweeps", [13, -40])
+def test_split_node_warns_at_the_sweep_limit(monkeypatch, sweeps):
+    """The binding says so when the library reports that the sweeps ran out
+    (a negative count), whether or not the caller asked for the count."""
+    import ctypes
+    import warnings
+    import torch
+    from paper_1905_01330_gb300 import tn
+
+    class Lib:
+        def tn_split_node_workspace_bytes(self, *a):
+            return 256
+
+        def tn_split_node(self, *a):
+            ctypes.cast(a[12], ctypes.POINTER(ctypes.c_int64))[0] = 2
+            ctypes.cast(a[13], ctypes.POINTER(ctypes.c_int32))[0] = sweeps
+            return 0
+
+    monkeypatch.setattr(tn, "load", lambda: Lib())
+    monkeypatch.setattr(tn, "tensor_desc", lambda t: ctypes.c_int(0))
+    monkeypatch.setattr(tn, "_workspace", lambda n, dev: torch.empty(n, dtype=torch.uint8))
+    monkeypatch.setattr(tn, "_stream", lambda s: None)
+    with warnings.catch_warnings(record=True) as got:
+        warnings.simplefilter("always")
+        u, vh, dropped = tn.split_node(torch.ones(3, 4), [0], [1])
+    assert u.shape == (3, 2) and vh.shape == (2, 4) and dropped.shape == (1,)
+    assert [w.category for w in got] == ([RuntimeWarning] if sweeps < 0 else [])
