@@ -133,7 +133,7 @@ struct SvdParams {
   int32_t r, ns, nb;   // columns; blocks; blocks rounded up to even (the added one is zeros, not stored)
   int32_t cluster;     // CTAs sharing out a pair's rows
   float tol;
-  unsigned* bar;       // barrier counter (zero)
+  unsigned long long* bar;  // barrier word (zero)
   int* counts;         // rotations per sweep (zero)
   int* sweeps;         // out: sweeps used, negative if the limit was reached
   int* status;
@@ -397,6 +397,32 @@ __device__ __forceinline__ unsigned svd_load_acquire(const unsigned* p) {
   return v;
 }
 
+// Device-wide barrier, by one thread of every CTA, arrival `epoch` (from 1).
+// Low half of *bar: arrivals; high half: the epoch at which a wait ran out.
+// Bounded, and all CTAs get the same answer: only a barrier that is not
+// complete can be given up, and one given up stays so when late CTAs arrive.
+// So all leave behind the same round, and none reads the shared memory of a CTA
+// of its cluster that has left.
+__device__ __forceinline__ bool svd_barrier(unsigned long long* bar, unsigned epoch, int* status) {
+  __threadfence();
+  atomicAdd(bar, 1ull);
+  const unsigned target = epoch * gridDim.x;
+  const uint64_t start = ptx::globaltimer();
+  for (unsigned i = 1;; ++i) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(bar) : "memory");
+    if ((unsigned)(v >> 32) == epoch) return false;
+    if ((unsigned)v >= target) break;
+    if ((i & 63u) == 0u && ptx::globaltimer() - start > ptx::kWaitLimitNs &&
+        atomicCAS(bar, v, v | ((unsigned long long)epoch << 32)) == v) {
+      ptx::set_status(status, TN_ERR_TIMEOUT);
+      return false;
+    }
+  }
+  __threadfence();
+  return true;
+}
+
 // All sweeps: one cooperative launch.
 __global__ void __launch_bounds__(SVD_THREADS) svd_jacobi(const __grid_constant__ SvdParams P) {
   extern __shared__ __align__(16) uint8_t raw[];
@@ -415,18 +441,7 @@ __global__ void __launch_bounds__(SVD_THREADS) svd_jacobi(const __grid_constant_
       __syncthreads();
       if (tid == 0) {
         if (rotations && blockIdx.x % P.cluster == 0) atomicAdd(P.counts + used, rotations);
-        __threadfence();
-        ++epoch;
-        atomicAdd(P.bar, 1u);
-        const unsigned target = epoch * gridDim.x;
-        const uint64_t start = ptx::globaltimer();
-        for (unsigned i = 1; svd_load_acquire(P.bar) < target; ++i)
-          if ((i & 63u) == 0u && ptx::globaltimer() - start > ptx::kWaitLimitNs) {
-            ptx::set_status(P.status, TN_ERR_TIMEOUT);
-            s.abort = 1;
-            break;
-          }
-        __threadfence();
+        if (!svd_barrier(P.bar, ++epoch, P.status)) s.abort = 1;
       }
       __syncthreads();
       if (s.abort) return;
@@ -594,7 +609,7 @@ static int plan_split(const tn_tensor* A, const int* left, int nleft, const int*
   o.ord_off = o.wn_off + al256(sizeof(float) * (size_t)o.r);
   o.sorted_off = o.ord_off + al256(sizeof(int32_t) * (size_t)o.r);
   o.cnt_off = o.sorted_off + al256(sizeof(float) * (size_t)(o.r + 1));  // the values, then the sweep count
-  o.total = o.cnt_off + 256;  // barrier counter, rotations per sweep, the largest magnitude
+  o.total = o.cnt_off + 256;  // barrier word, rotations per sweep, the largest magnitude
   return TN_OK;
 }
 
@@ -665,12 +680,12 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
   P.nb = P.ns + (P.ns & 1);
   // counted above 16 tol, a few times the float32 rounding of a length-L dot product
   P.tol = 0.25f * sqrtf((float)L) * 5.9604645e-8f;
-  P.bar = reinterpret_cast<unsigned*>(base + lay.cnt_off);
-  P.counts = reinterpret_cast<int*>(base + lay.cnt_off) + 1;
+  P.bar = reinterpret_cast<unsigned long long*>(base + lay.cnt_off);
+  P.counts = reinterpret_cast<int*>(base + lay.cnt_off) + 2;
   P.sweeps = reinterpret_cast<int*>(sorted + r);
   P.status = status_word();
-  static_assert(sizeof(int) * (SVD_MAX_SWEEPS + 2) <= 256, "barrier counter, rotation counts, largest magnitude");
-  unsigned* bits = P.bar + SVD_MAX_SWEEPS + 1;
+  static_assert(sizeof(int) * (SVD_MAX_SWEEPS + 3) <= 256, "barrier word, rotation counts, largest magnitude");
+  unsigned* bits = reinterpret_cast<unsigned*>(P.counts) + SVD_MAX_SWEEPS;
   int half = 0;  // 4^half >= M N
   while (half < 31 && (int64_t(1) << (2 * half)) < L * r) ++half;
   if (cudaMemsetAsync(base + lay.cnt_off, 0, 256, s) != cudaSuccess ||
