@@ -27,7 +27,15 @@
 // other entries broadcast from shared memory, for the Gram matrix (lane j: its
 // column of it) and for the product with Q alike. The rows are shared out over
 // the CTAs of a cluster, which add up their Gram matrices and rotate alike.
-// Measured (two-site node of bond 128, r = 256, 13 sweeps): 18.7 -> 2.2 ms; a
+// The angles are float32, from approximate roots: an angle that is a little off
+// leaves a little for the next round, while the values come from the columns'
+// norms (in 64 bits) and c^2 + s^2 = 1 holds to rounding. Error against 64 bits
+// of two-site nodes of bond 6 to 160, half and all of the values kept, one pair
+// at a time with 64-bit angles -> here: values 1.4e-7 .. 5.4e-7 -> 0.7e-7 ..
+// 1.2e-7, the product 3.4e-7 .. 3.8e-6 -> 2.5e-7 .. 2.1e-6, 0.2 to 0.84 of the
+// former at every size. Gram sums over warps and CTAs that keep their roundings
+// (two-sum) took 10 % longer for the same errors.
+// Measured (two-site node of bond 128, r = 256, 13 sweeps): 18.7 -> 2.3 ms; a
 // round takes ~19,000 cycles: Gram matrix 1,300, its sum over 8 warps and 8
 // CTAs 4,800, the 17 rotation steps 9,800 (a dependent chain of ~370 cycles
 // each), W and V 2,300, the barrier 2,600. r = 1000: 98 -> 14 ms, 2048: 380 ->
@@ -452,8 +460,8 @@ __global__ void __launch_bounds__(SVD_THREADS) svd_jacobi(const __grid_constant_
   if (blockIdx.x == 0 && tid == 0) *P.sweeps = done ? used : -used;
 }
 
-// Sum of a per-thread value over the CTA, in double across warps.
-__device__ __forceinline__ double block_sum(float a) {
+// Sum of a per-thread value over the CTA.
+__device__ __forceinline__ double block_sum(double a) {
   __shared__ double part[SVD_WARPS];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
@@ -479,9 +487,9 @@ svd_norms(const float* __restrict__ W, const float* __restrict__ V, int64_t L, i
           float* __restrict__ sigma, float* __restrict__ vnorm, float* __restrict__ wnorm) {
   const float* w = W + blocked(0, blockIdx.x, L);
   const float* v = V + blocked(0, blockIdx.x, r);
-  float a = 0.0f, b = 0.0f;
-  for (int64_t i = threadIdx.x; i < L; i += SVD_THREADS) a = fmaf(w[i * SVD_B], w[i * SVD_B], a);
-  for (int64_t i = threadIdx.x; i < r; i += SVD_THREADS) b = fmaf(v[i * SVD_B], v[i * SVD_B], b);
+  double a = 0.0, b = 0.0;
+  for (int64_t i = threadIdx.x; i < L; i += SVD_THREADS) a = fma((double)w[i * SVD_B], (double)w[i * SVD_B], a);
+  for (int64_t i = threadIdx.x; i < r; i += SVD_THREADS) b = fma((double)v[i * SVD_B], (double)v[i * SVD_B], b);
   const double sa = block_sum(a), sb = block_sum(b);
   if (threadIdx.x == 0) {
     const double vn = sqrt(sb), wn = sqrt(sa);
