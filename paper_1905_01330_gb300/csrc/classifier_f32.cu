@@ -31,6 +31,7 @@
 #include <math.h>
 
 #include "classifier_f32.h"
+#include "divide.cuh"
 #include "ptx.cuh"
 
 namespace tn {
@@ -87,35 +88,6 @@ struct SweepCfg {
 struct SweepBars {
   uint64_t full[8], empty[8];
 };
-
-// v[i][:] / sc[i]: away from the ends of the exponent range an estimate of the
-// quotient corrected once by its own residual (Markstein's iteration), within
-// an ulp of it, at a third of the division's instructions; a warp with a
-// scale elsewhere divides, out of line (a step divides a thread's whole tile,
-// and the divisions inline cost it 1,000 cycles).
-__device__ __noinline__ float divide_any(float x, float sc) { return x / sc; }
-template <int RS>
-__device__ __forceinline__ void divide(float (&v)[RS][4], const float (&sc)[RS]) {
-  bool plain = true;
-#pragma unroll
-  for (int i = 0; i < RS; ++i) plain = plain && sc[i] > 0x1p-100f && sc[i] < 0x1p100f;
-  if (__all_sync(0xffffffffu, plain)) {
-#pragma unroll
-    for (int i = 0; i < RS; ++i) {
-      const float r = __fdividef(1.0f, sc[i]);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float q = v[i][j] * r;
-        v[i][j] = fmaf(fmaf(-q, sc[i], v[i][j]), r, q);
-      }
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < RS; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) v[i][j] = divide_any(v[i][j], sc[i]);
-  }
-}
 
 template <int CHI, int RS, int ADJ>
 __global__ void __launch_bounds__(SweepCfg<CHI, RS>::NT)
@@ -244,7 +216,7 @@ cls_f32_sweep_kernel(const __grid_constant__ ClsF32Params p) {
       float sc[RS];
 #pragma unroll
       for (int i = 0; i < RS; ++i) sc[i] = scl[q & 1][f0 + i];
-      divide(out, sc);
+      divide_rows<false>(out, sc);
     }
     float* keep = nullptr;
     if (ADJ) {
@@ -377,7 +349,7 @@ cls_f32_sweep_kernel(const __grid_constant__ ClsF32Params p) {
         if (!(m[i] > 0.0f)) m[i] = 1.0f;
         if (og == 0) scl[q & 1][f0 + i] = m[i];
       }
-      divide(out, m);
+      divide_rows<true>(out, m);
     }
     if (q + 1 < nsteps) publish(q + 1);
     // the next vector, features and scales are in place for every warp; a

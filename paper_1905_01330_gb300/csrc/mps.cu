@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "divide.cuh"
 #include "mpo_step.cuh"
 #include "packed.h"
 #include "tn_internal.h"
@@ -156,29 +157,6 @@ __device__ __forceinline__ void stage_core(float* dst, const float* __restrict__
       const int r = small_div(i, inv);
       cp_async_f32(dst + r * ld + (i - r * cols), src + i);
     }
-  }
-}
-
-// x / sc for |x| <= sc, rounded as the division: the quotient by the correctly
-// rounded reciprocal, corrected by its residual (Markstein), unless sc or a
-// quotient lies where that is not exact.
-__device__ __noinline__ float divide_slow(float x, float sc) { return __fdiv_rn(x, sc); }
-template <int N>
-__device__ __forceinline__ void divide_by_max(float (&v)[N], float sc) {
-  const float r = __frcp_rn(sc);
-  bool plain = sc > 0x1p-60f && sc < 0x1p60f && (__float_as_uint(sc) & 0x7FFFFFu) != 0x7FFFFFu;
-  float q[N];
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-    q[j] = v[j] * r;
-    plain = plain && (fabsf(q[j]) > 0x1p-40f || v[j] == 0.0f);
-  }
-  if (__all_sync(__activemask(), plain)) {
-#pragma unroll
-    for (int j = 0; j < N; ++j) v[j] = fmaf(fmaf(-q[j], sc, v[j]), r, q[j]);
-  } else {
-#pragma unroll
-    for (int j = 0; j < N; ++j) v[j] = divide_slow(v[j], sc);
   }
 }
 
