@@ -99,11 +99,14 @@ def test_clock_sampler_keeps_samples_of_the_timed_region(tmp_path, monkeypatch):
     assert s.stop() is None
 
 
-SUM_ORDER = r"""
+PLANS = r"""
+#include <chrono>
 #include <cstdio>
+#include <cstring>
 #include "tn_internal.h"
 using namespace tn;
-int main() {
+int main(int argc, char** argv) {
+  const SimtPlan how = strcmp(argv[1], "sweep") ? SimtPlan::alone : SimtPlan::sweep;
   long long M, N, K, ta, tb;
   while (scanf("%lld %lld %lld %lld %lld", &M, &N, &K, &ta, &tb) == 5) {
     tn_tensor A{}, B{}, C{};
@@ -118,11 +121,26 @@ int main() {
     if (plan_contract(&A, &la, &B, &lb, 1, &C, &d) != TN_OK) return 1;
     plan_units(&d, 304);
     const long long ranges = d.splits, range = d.k_per_split;
-    plan_simt(&d, SimtPlan::sweep);
-    printf("%lld %lld %d %lld %d\n", ranges, range, (int)d.splits, (long long)d.k_per_split, (int)d.chunk);
+    const auto t0 = std::chrono::steady_clock::now();
+    plan_simt(&d, how);
+    const double us = std::chrono::duration<double, std::micro>(std::chrono::steady_clock::now() - t0).count();
+    printf("%lld %lld %d %lld %d %.2f\n", ranges, range, (int)d.splits, (long long)d.k_per_split, (int)d.chunk, us);
   }
 }
 """
+
+
+def simt_plans(built, tmp_path, how, cases):
+    """(k ranges of plan_units, their length, k ranges and length of plan_simt, its chunk, microseconds) per (M, N, K, A
+    transposed, B transposed)."""
+    src, exe = tmp_path / "plans.cpp", tmp_path / "plans"
+    src.write_text(PLANS)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", os.path.join(ROOT, "paper_1905_01330_gb300", "csrc"),
+                    "-I", "/usr/local/cuda/include", str(src), built, "-Wl,-rpath," + os.path.dirname(built),
+                    "-o", str(exe)], check=True, timeout=300)
+    out = subprocess.run([str(exe), how], input="".join("%d %d %d %d %d\n" % c for c in cases), capture_output=True,
+                         text=True, check=True, timeout=300).stdout.split("\n")
+    return [[float(x) for x in line.split()] for line in out if line]
 
 
 def test_sweep_results_are_sums_of_the_k_ranges_one_by_one(built, tmp_path):
@@ -131,11 +149,6 @@ def test_sweep_results_are_sums_of_the_k_ranges_one_by_one(built, tmp_path):
     of them, or all in ascending order. Sums of sums, which no order of such
     additions gives, are for lone contractions only. Over the bonds an energy
     or norm sweep meets, rising, level and falling, and MPO bonds 1 to 5."""
-    src, exe = tmp_path / "order.cpp", tmp_path / "order"
-    src.write_text(SUM_ORDER)
-    subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "paper_1905_01330_gb300", "csrc"),
-                    "-I", "/usr/local/cuda/include", str(src), built, "-Wl,-rpath," + os.path.dirname(built),
-                    "-o", str(exe)], check=True, timeout=300)
     bonds = [(a, b) for c in (100, 256, 300, 383, 384, 400, 512, 640, 1024) for a, b in ((c, c), (c, c // 2), (c // 2, c))]
     cases = []
     for a, b in bonds:
@@ -143,15 +156,22 @@ def test_sweep_results_are_sums_of_the_k_ranges_one_by_one(built, tmp_path):
             cases += [(a, d * b, a, 1, 0), (b, b, d * a, 1, 0)]                       # norm
             for w in (2, 4, 6):
                 cases += [(w * a, d * b, a, 1, 0), (w * b, b, d * a, 0, 0)]           # energy
-    out = subprocess.run([str(exe)], input="".join("%d %d %d %d %d\n" % c for c in cases), capture_output=True, text=True,
-                         check=True, timeout=300).stdout.split("\n")
     several = 0
-    for case, line in zip(cases, out):
-        ranges, rng, units, per, chunk = map(int, line.split())
-        assert chunk * 64 == min(rng, 2048) and per % (chunk * 64) == 0, (case, line)
-        assert units == 1 or (units == ranges and per == rng), (case, line)
+    for case, (ranges, rng, units, per, chunk, _) in zip(cases, simt_plans(built, tmp_path, "sweep", cases)):
+        assert chunk * 64 == min(rng, 2048) and per % (chunk * 64) == 0, case
+        assert units == 1 or (units == ranges and per == rng), case
         several += ranges > 2
     assert several >= 20
+
+
+def test_planning_a_long_shared_index_is_quick(built, tmp_path):
+    """A lone float32 contraction's plan takes microseconds whatever the length
+    of its shared index (tens of thousands of k ranges), and covers it."""
+    cases = [(m, n, k, 0, 0) for m, n in ((1, 1), (2, 5), (3, 1)) for k in (10 ** 6, 10 ** 7, 10 ** 8, 2 * 10 ** 8 + 1)]
+    plans = simt_plans(built, tmp_path, "alone", cases * 5)
+    for case, (_, _, units, per, chunk, _) in zip(cases * 5, plans):
+        assert units * per >= case[2] > (units - 1) * per and per % (64 * chunk) == 0, (case, units, per)
+    assert min(max(p[5] for p in plans[i * len(cases):(i + 1) * len(cases)]) for i in range(5)) <= 100.0
 
 
 @pytest.mark.parametrize("sweeps", [13, -40])
