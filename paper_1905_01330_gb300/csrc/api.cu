@@ -28,9 +28,7 @@ int* status_word() {
   return ptrs[dev];
 }
 
-// One contraction alone should still fill the GPU when its K allows: ask for
-// at least two work units per SM.
-int64_t min_units_single() {
+int sm_count() {
   static int sms = 0;
   if (!sms) {
     int dev = 0;
@@ -38,8 +36,12 @@ int64_t min_units_single() {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       sms = 152;
   }
-  return 2 * (int64_t)sms;
+  return sms;
 }
+
+// One contraction alone should still fill the GPU when its K allows: ask for
+// at least two work units per SM.
+int64_t min_units_single() { return 2 * (int64_t)sm_count(); }
 
 static int launch_one(const ContractDesc& d, int prec, cudaStream_t stream) {
   const int64_t tiles = (int64_t)d.tiles_m * d.tiles_n * d.splits;

@@ -378,11 +378,12 @@ int launch_sweep(const ClsF32Params& p, cudaStream_t s) {
 template <int CHI, int ADJ>
 int launch_sweep_chi(const ClsF32Params& p, cudaStream_t s) {
   // a step takes about as long as its tile has samples, so the tile is the
-  // smallest with which both halves still fit the 152 SMs in one wave
+  // smallest with which both halves still fit the SMs in one wave
   constexpr int SG = SweepCfg<CHI, 2>::SG;
   auto ctas = [&](int rs) { return 2 * ((p.batch + rs * SG - 1) / (rs * SG)); };
-  if (ctas(2) <= 152) return launch_sweep<CHI, 2, ADJ>(p, s);
-  if (ctas(4) <= 152) return launch_sweep<CHI, 4, ADJ>(p, s);
+  const int sms = sm_count();
+  if (ctas(2) <= sms) return launch_sweep<CHI, 2, ADJ>(p, s);
+  if (ctas(4) <= sms) return launch_sweep<CHI, 4, ADJ>(p, s);
   return launch_sweep<CHI, 8, ADJ>(p, s);
 }
 
@@ -502,7 +503,8 @@ int launch_grad(const ClsF32GradParams& p0, cudaStream_t s) {
   // wave (few cuts: each adds its whole tile to the gradient), a segment with
   // more tiles in four parts, so that the last wave is short
   const int jparts = CHI / C::JW, tiles = (n0 + n1) * jparts;
-  int want = tiles <= 152 * 4 ? 152 * 4 / tiles : 4;
+  const int room = 4 * sm_count();
+  int want = tiles <= room ? room / tiles : 4;
   const int most = (p.batch + 127) / 128;
   if (want > most) want = most;
   p.chunk = ((p.batch + want - 1) / want + C::GB - 1) / C::GB * C::GB;

@@ -494,10 +494,10 @@ void plan_simt(ContractDesc* d, SimtPlan how) {
         // shared index of 1e8 took 2.1 ms on the host), and all of them. In a
         // sweep one or all, so that a result is the sum of the k ranges one by
         // one, in whatever order.
-        const int64_t most = d->splits;
+        const int64_t most = d->splits, sms = sm_count();
         for (int64_t c = 1, next; c <= most; c = next) {
           next = c == most ? most + 1 : std::min(most, how == SimtPlan::sweep ? most : c + 1 + (c >= 8 ? c / 4 : 0));
-          const int64_t sp = (slabs + c * chunk - 1) / (c * chunk), u = (tiles * sp + 151) / 152;
+          const int64_t sp = (slabs + c * chunk - 1) / (c * chunk), u = (tiles * sp + sms - 1) / sms;
           if (sp > 2 && tiles >= 16) continue;  // two addends commute: such results do not vary from run to run
           const double t = (double)((u + 1) / 2) * 8000.0 +
                            (double)u * (double)(4 * std::min(slabs, c * chunk)) * slab[k] + (sp > 1 ? 6000.0 : 0.0);

@@ -553,17 +553,6 @@ tc_contract_kernel(const __grid_constant__ ContractDesc single, const ContractDe
   }
 }
 
-int sm_count() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      sms = 152;
-  }
-  return sms;
-}
-
 template <int SPLIT>
 int launch_tc(const ContractDesc& single, const ContractDesc* group, const int32_t* unit_desc, int64_t units,
               cudaStream_t stream) {

@@ -303,7 +303,7 @@ int launch_matvec(const ContractDesc& d, cudaStream_t s) {
   // parts of the shared index: enough CTAs for the SMs, at least 64 indices each
   const int64_t groups = (v.R + MV_COLS - 1) / MV_COLS;
   int parts = (v.K + MV_PART - 1) / MV_PART;
-  while (parts < 8 && groups * parts < 152 && v.K / (2 * parts) >= 64) parts *= 2;
+  while (parts < 8 && groups * parts < sm_count() && v.K / (2 * parts) >= 64) parts *= 2;
   v.part = (v.K + parts - 1) / parts;
   return launch_overlapped(vec ? matvec_columns<true> : matvec_columns<false>, v, groups * parts, parts, s);
 }

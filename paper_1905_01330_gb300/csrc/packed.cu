@@ -1525,17 +1525,6 @@ bool pack_attr() {
   return true;
 }
 
-int sm_count() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      sms = 152;
-  }
-  return sms;
-}
-
 template <int SPLIT, int FUSE>
 int launch_gemm(const GemmDesc& single, const GemmDesc* descs, const int32_t* map, const PackJob* jobs,
                 int64_t units, cudaStream_t s, uint32_t* unit_ctr = nullptr, bool overlap = false) {

@@ -718,7 +718,7 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
   cfg.numAttrs = 2;
   // one CTA per SM; the rows of a pair over as many CTAs (up to 8, at least
   // 32 rows each) as all pairs leave room for
-  const int64_t pairs = P.nb / 2, sms = min_units_single() / 2;
+  const int64_t pairs = P.nb / 2, sms = sm_count();
   P.cluster = 1;
   while (P.cluster < SVD_CLUSTER && pairs * P.cluster * 2 <= sms && L >= 64 * P.cluster) P.cluster *= 2;
   for (;; P.cluster /= 2) {

@@ -93,6 +93,8 @@ void plan_units(ContractDesc* d, int64_t min_units);
 // a group (the k ranges as given) or as 128 x 128 units (as given).
 enum class SimtPlan { alone, sweep, group, pairs };
 void plan_simt(ContractDesc* d, SimtPlan how);
+// SMs of the current device (152 where there is none).
+int sm_count();
 // Work units a lone contraction asks plan_units for (two per SM).
 int64_t min_units_single();
 // The same for the packed GEMM (longer k ranges when a spec has many tiles).
