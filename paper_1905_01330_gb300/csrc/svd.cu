@@ -35,6 +35,12 @@
 // 1.2e-7, the product 3.4e-7 .. 3.8e-6 -> 2.5e-7 .. 2.1e-6, 0.2 to 0.84 of the
 // former at every size. Gram sums over warps and CTAs that keep their roundings
 // (two-sum) took 10 % longer for the same errors.
+// At most two blocks of columns and many rows (svd_tall): the rows are shared
+// out over the whole grid, Gram sums go through device memory, and rows are
+// stored only as wide as they are (4, 8 or 16 columns). One cluster for such a
+// pair took longer than one CTA per two columns: 4e6 x 1 0.69 ms that way, 8.7
+// by a cluster, 0.47 now; 4e6 x 2 1.31, 14.5, 0.50; 1e6 x 5 7.1, 9.6, 0.46;
+// 2e5 x 32 22.7, 3.5, 0.77.
 // Measured (two-site node of bond 128, r = 256, 13 sweeps): 18.7 -> 2.3 ms; a
 // round takes ~19,000 cycles: Gram matrix 1,300, its sum over 8 warps and 8
 // CTAs 4,800, the 17 rotation steps 9,800 (a dependent chain of ~370 cycles
@@ -79,9 +85,11 @@ struct SplitView {
 __device__ __forceinline__ int64_t leg_offset(int64_t idx, int n, const int32_t* dim, const int64_t* str) {
   int64_t off = 0;
   for (int p = n - 1; p >= 0; --p) {
-    const int64_t d = dim[p];
-    off += (idx % d) * str[p];
-    idx /= d;
+    int64_t hi;
+    if (idx <= 0xFFFFFFFFll) hi = (uint32_t)idx / (uint32_t)dim[p];
+    else hi = idx / dim[p];
+    off += (idx - hi * dim[p]) * str[p];
+    idx = hi;
   }
   return off;
 }
@@ -91,7 +99,7 @@ __global__ void svd_largest(SplitView v, unsigned* bits) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   unsigned m = 0u;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < v.M * v.N; e += stride) {
-    const int64_t i = e / v.N, j = e - i * v.N;
+    const int64_t i = e <= 0xFFFFFFFFll && v.N <= 0xFFFFFFFFll ? (uint32_t)e / (uint32_t)v.N : e / v.N, j = e - i * v.N;
     const float x = v.A[leg_offset(i, v.nl, v.ldim, v.lstr) + leg_offset(j, v.nr, v.rdim, v.rstr)];
     m = max(m, __float_as_uint(fabsf(x)));
   }
@@ -105,16 +113,16 @@ __device__ __forceinline__ int svd_shift(unsigned bits, int half) {
   return bits == 0u || bits >= 0x7F800000u ? 0 : SVD_TOP - half - 1 - ilogbf(__uint_as_float(bits));
 }
 
-// W in blocks of 16 columns, [block][row][16] (zeros past column r), V = I
-// likewise.
-__global__ void svd_gather(SplitView v, const unsigned* bits, int half, float* __restrict__ W, float* __restrict__ V, int64_t L,
-                           int64_t r, int64_t cols) {
+// W in blocks of 2^lw columns (16; a tall node's one block may have fewer),
+// [block][row][column] (zeros past column r), V = I likewise.
+__global__ void svd_gather(SplitView v, const unsigned* bits, int half, int lw, float* __restrict__ W, float* __restrict__ V,
+                           int64_t L, int64_t r, int64_t cols) {
   const int shift = svd_shift(*bits, half);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   for (int64_t w = first; w < L * cols; w += stride) {
     // neighbouring threads walk the view's own rows where those are columns of W
-    const int64_t blk = w / (L * SVD_B), in = w - blk * L * SVD_B;
-    const int64_t row = in / SVD_B, col = blk * SVD_B + in % SVD_B;
+    const int64_t blk = (cols >> lw) == 1 ? 0 : w / (L << lw), in = w - ((blk * L) << lw);
+    const int64_t row = in >> lw, col = (blk << lw) + (in & ((1 << lw) - 1));
     float x = 0.0f;
     if (col < r) {
       const int64_t i = v.wide ? col : row, j = v.wide ? row : col;
@@ -123,8 +131,8 @@ __global__ void svd_gather(SplitView v, const unsigned* bits, int half, float* _
     W[w] = x;
   }
   for (int64_t e = first; e < r * cols; e += stride) {
-    const int64_t blk = e / (r * SVD_B), in = e - blk * r * SVD_B;
-    V[e] = in / SVD_B == blk * SVD_B + in % SVD_B ? 1.0f : 0.0f;
+    const int64_t blk = e / (r << lw), in = e - ((blk * r) << lw);
+    V[e] = in >> lw == (blk << lw) + (in & ((1 << lw) - 1)) ? 1.0f : 0.0f;
   }
 }
 
@@ -144,6 +152,7 @@ struct SvdParams {
   unsigned long long* bar;  // barrier word (zero)
   int* counts;         // rotations per sweep (zero)
   int* sweeps;         // out: sweeps used, negative if the limit was reached
+  float* parts;        // tall nodes: the CTAs' Gram sums, two sets in turn
   int* status;
 };
 
@@ -460,42 +469,217 @@ __global__ void __launch_bounds__(SVD_THREADS) svd_jacobi(const __grid_constant_
   if (blockIdx.x == 0 && tid == 0) *P.sweeps = done ? used : -used;
 }
 
-// Sum of a per-thread value over the CTA.
-__device__ __forceinline__ double block_sum(double a) {
-  __shared__ double part[SVD_WARPS];
+// s + x, s a sum (x) and what its roundings left (y) (Knuth's two-sum).
+__device__ __forceinline__ void add_exact(float2& s, float x) {
+  const float t = s.x + x, u = t - s.x;
+  s.y += (s.x - (t - u)) + (x - u);
+  s.x = t;
+}
+
+// All sweeps of a node of at most two blocks (COLS columns stored: one block of
+// 4, 8 or 16, or two of 16), its rows shared out over the grid: cooperative
+// launch. A warp takes 32 / COLS rows at once. Every CTA adds up all Gram sums
+// in the same order and rotates alike, so one barrier a sweep is enough (the
+// sums are written to the other set meanwhile) and the count needs no adding.
+template <int COLS>
+__global__ void __launch_bounds__(SVD_THREADS) svd_tall(const __grid_constant__ SvdParams P) {
+  constexpr int C = 2 * SVD_B, BW = COLS < SVD_B ? COLS : SVD_B, Q4 = COLS / 4, SUB = 32 / COLS;
+  constexpr int CH = 2 * SVD_CH * SVD_B / COLS;  // rows staged at once
+  constexpr int E = COLS * COLS, NP = E < SVD_THREADS ? SVD_THREADS / E : 1;  // threads adding up one entry
+  extern __shared__ __align__(16) uint8_t raw[];
+  SvdSmem& s = *reinterpret_cast<SvdSmem*>(raw);
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, col = lane % COLS, sub = lane / COLS;
+  const int rank = (int)blockIdx.x, cs = (int)gridDim.x;
+  const int64_t lp = (P.L + cs - 1) / cs, w0 = min(P.L, lp * rank), wn = min(P.L, w0 + lp) - w0;
+  const int nw = (int)((wn + CH - 1) / CH), items = nw + (rank == 0 ? 1 : 0);  // W's chunks; the first CTA: V
+  float* X = &s.X[0][0][0];
+  auto rows_of = [&](int i) { return i < nw ? (int)min((int64_t)CH, wn - (int64_t)i * CH) : P.r; };
+  // element (row, c) of item i's first row on
+  auto at = [&](int i, int row, int c) -> float* {
+    const int64_t n = i < nw ? P.L : P.r, row0 = i < nw ? w0 + (int64_t)i * CH : 0;
+    return (i < nw ? P.W : P.V) + ((c / BW) * n + row0 + row) * BW + c % BW;
+  };
+  auto stage = [&](int i) {
+    float* x = X + (i & 1) * CH * COLS;
+    const int words = rows_of(i) * Q4;
+    for (int e = tid; e < words; e += SVD_THREADS)
+      ptx::cp_async16(ptx::smem_addr(x + e * 4), at(i, e / Q4, e % Q4 * 4));
+    ptx::cp_async_commit();
+  };
+  if (tid == 0) s.abort = 0;
+  unsigned epoch = 0;
+  bool done = false;
+  int used = 0;
+  while (!done && used < SVD_MAX_SWEEPS) {
+    float2 acc[COLS / 2];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = a;
-  __syncthreads();
-  double s = 0.0;
-  for (int w = 0; w < SVD_WARPS; ++w) s += part[w];
-  return s;
+    for (int m = 0; m < COLS / 2; ++m) acc[m] = make_float2(0.f, 0.f);
+    if (nw > 0) stage(0);
+    for (int c = 0; c < nw; ++c) {
+      ptx::cp_async_wait<0>();
+      __syncthreads();
+      if (c + 1 < nw) stage(c + 1);
+      const float* x = X + (c & 1) * CH * COLS;
+      const int rows = rows_of(c);
+#pragma unroll 4
+      for (int row = w * SUB + sub; row < rows; row += SVD_WARPS * SUB) {
+        const float mine = x[row * COLS + col];
+        const float2 mm = make_float2(mine, mine);
+#pragma unroll
+        for (int m = 0; m < Q4; ++m) {
+          const float4 f = *reinterpret_cast<const float4*>(x + row * COLS + 4 * m);
+          acc[2 * m] = __ffma2_rn(make_float2(f.x, f.y), mm, acc[2 * m]);
+          acc[2 * m + 1] = __ffma2_rn(make_float2(f.z, f.w), mm, acc[2 * m + 1]);
+        }
+      }
+    }
+#pragma unroll
+    for (int m = 0; m < COLS / 2; ++m) {
+#pragma unroll
+      for (int o = COLS; o < 32; o <<= 1) {
+        acc[m].x += __shfl_xor_sync(0xffffffffu, acc[m].x, o);
+        acc[m].y += __shfl_xor_sync(0xffffffffu, acc[m].y, o);
+      }
+      if (sub == 0) {
+        s.red[w][2 * m][col] = acc[m].x;
+        s.red[w][2 * m + 1][col] = acc[m].y;
+      }
+    }
+    __syncthreads();
+    float* parts = P.parts + (size_t)(used & 1) * cs * E;
+    for (int e = tid; e < E; e += SVD_THREADS) {
+      float2 g = make_float2(s.red[0][e / COLS][e % COLS], 0.0f);
+      for (int u = 1; u < SVD_WARPS; ++u) add_exact(g, s.red[u][e / COLS][e % COLS]);
+      __stcg(parts + (size_t)rank * E + e, g.x + g.y);
+    }
+    for (int e = tid; e < C * C; e += SVD_THREADS) {
+      s.Q[e / C][e % C] = e / C == e % C ? 1.0f : 0.0f;
+      s.G[0][e / C][e % C] = 0.0f;
+    }
+    __syncthreads();
+    if (tid == 0 && !svd_barrier(P.bar, ++epoch, P.status)) s.abort = 1;
+    __syncthreads();
+    if (s.abort) return;
+    float2* sums = reinterpret_cast<float2*>(X);  // [NP][E]
+    for (int e = tid; e < E * NP; e += SVD_THREADS) {
+      float2 g = make_float2(0.f, 0.f);
+#pragma unroll 8
+      for (int k = e / E; k < cs; k += NP) add_exact(g, __ldcg(parts + (size_t)k * E + e % E));
+      if (NP == 1) s.G[0][e / COLS][e % COLS] = g.x + g.y;
+      else sums[e] = g;
+    }
+    __syncthreads();
+    if (NP > 1 && tid < E) {
+      float2 g = sums[tid];
+      for (int k = 1; k < NP; ++k) {
+        add_exact(g, sums[k * E + tid].x);
+        g.y += sums[k * E + tid].y;
+      }
+      s.G[0][tid / COLS][tid % COLS] = g.x + g.y;
+    }
+    __syncthreads();
+    int count = 0;
+    if (svd_rotate<true>(s, P.tol, count)) {
+      float2 qc[COLS / 2];
+#pragma unroll
+      for (int m = 0; m < COLS / 2; ++m) qc[m] = make_float2(s.Q[2 * m][col], s.Q[2 * m + 1][col]);
+      if (items > 0) stage(0);
+      for (int i = 0; i < items; ++i) {
+        ptx::cp_async_wait<0>();
+        __syncthreads();
+        if (i + 1 < items) stage(i + 1);
+        const float* x = X + (i & 1) * CH * COLS;
+        const int rows = rows_of(i);
+#pragma unroll 4
+        for (int row = w * SUB + sub; row < rows; row += SVD_WARPS * SUB) {
+          float2 o = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int m = 0; m < Q4; ++m) {
+            const float4 f = *reinterpret_cast<const float4*>(x + row * COLS + 4 * m);
+            o = __ffma2_rn(make_float2(f.x, f.y), qc[2 * m], o);
+            o = __ffma2_rn(make_float2(f.z, f.w), qc[2 * m + 1], o);
+          }
+          *at(i, row, col) = o.x + o.y;
+        }
+      }
+      __syncthreads();  // the rows are written and the buffers read
+    }
+    done = count == 0;
+    ++used;
+  }
+  if (rank == 0 && tid == 0) *P.sweeps = done ? used : -used;
 }
 
-// Element (row, col) of a matrix kept in blocks of 16 columns, n rows.
-__device__ __forceinline__ int64_t blocked(int64_t row, int64_t col, int64_t n) {
-  return ((col / SVD_B) * n + row) * SVD_B + col % SVD_B;
+// Element (row, col) of a matrix kept in blocks of 2^lw columns, n rows.
+__device__ __forceinline__ int64_t blocked(int64_t row, int64_t col, int64_t n, int lw) {
+  return ((((col >> lw) * n) + row) << lw) + (col & ((1 << lw) - 1));
 }
 
-// Column j (CTA j): vnorm[j] = |V[:, j]|, wnorm[j] = |W[:, j]| and sigma[j] =
-// their quotient, without W's power of two. Both blocks took the same products
-// with Q, so what these left of the unit length of V's columns is also in W's
-// and cancels.
+// Column j's values from its sums of squares: vnorm[j] = |V[:, j]|, wnorm[j] =
+// |W[:, j]| and sigma[j] = their quotient, without W's power of two. Both blocks
+// took the same products with Q, so what these left of the unit length of V's
+// columns is also in W's and cancels.
+struct SvdNorms {
+  const unsigned* bits;
+  int half;
+  float *sigma, *vnorm, *wnorm;
+  __device__ __forceinline__ void put(int64_t j, double a, double b) const {
+    const double vn = sqrt(b), wn = sqrt(a);
+    vnorm[j] = (float)vn;
+    wnorm[j] = (float)wn;
+    sigma[j] = (float)ldexp(wn / vn, -svd_shift(*bits, half));
+  }
+};
+
+// Sums of squares of a block's columns over part blockIdx.y of the rows: the
+// values of one part, else the parts' sums [part][column][W, V] (svd_values).
 __global__ void __launch_bounds__(SVD_THREADS)
-svd_norms(const float* __restrict__ W, const float* __restrict__ V, int64_t L, int64_t r, const unsigned* bits, int half,
-          float* __restrict__ sigma, float* __restrict__ vnorm, float* __restrict__ wnorm) {
-  const float* w = W + blocked(0, blockIdx.x, L);
-  const float* v = V + blocked(0, blockIdx.x, r);
+svd_norms(const float* __restrict__ W, const float* __restrict__ V, int64_t L, int64_t r, int lw, SvdNorms out,
+          double* __restrict__ parts) {
+  __shared__ double sa[SVD_THREADS], sb[SVD_THREADS];
+  const int tid = threadIdx.x, width = 1 << lw, c = tid & (width - 1), step = SVD_THREADS >> lw;
+  const int64_t j = ((int64_t)blockIdx.x << lw) + c;
+  const int64_t lp = (L + gridDim.y - 1) / gridDim.y, l1 = min(L, lp * (blockIdx.y + 1));
   double a = 0.0, b = 0.0;
-  for (int64_t i = threadIdx.x; i < L; i += SVD_THREADS) a = fma((double)w[i * SVD_B], (double)w[i * SVD_B], a);
-  for (int64_t i = threadIdx.x; i < r; i += SVD_THREADS) b = fma((double)v[i * SVD_B], (double)v[i * SVD_B], b);
-  const double sa = block_sum(a), sb = block_sum(b);
-  if (threadIdx.x == 0) {
-    const double vn = sqrt(sb), wn = sqrt(sa);
-    vnorm[blockIdx.x] = (float)vn;
-    wnorm[blockIdx.x] = (float)wn;
-    sigma[blockIdx.x] = (float)ldexp(wn / vn, -svd_shift(*bits, half));
+#pragma unroll 4
+  for (int64_t i = lp * blockIdx.y + (tid >> lw); i < l1; i += step) {
+    const double x = W[blocked(i, j, L, lw)];
+    a = fma(x, x, a);
+  }
+  if (blockIdx.y == 0)
+    for (int64_t i = tid >> lw; i < r; i += step) {
+      const double x = V[blocked(i, j, r, lw)];
+      b = fma(x, x, b);
+    }
+  sa[tid] = a;
+  sb[tid] = b;
+  __syncthreads();
+  for (int o = SVD_THREADS / 2; o >= width; o >>= 1) {
+    if (tid < o) {
+      sa[tid] += sa[tid + o];
+      sb[tid] += sb[tid + o];
+    }
+    __syncthreads();
+  }
+  if (tid >= width || j >= r) return;
+  if (gridDim.y == 1) {
+    out.put(j, sa[tid], sb[tid]);
+  } else {
+    double* p = parts + 2 * (blockIdx.y * r + j);
+    p[0] = sa[tid];
+    p[1] = sb[tid];
+  }
+}
+// The values from `n` parts.
+__global__ void svd_values(const double* __restrict__ parts, int n, int r, SvdNorms out) {
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < r; j += gridDim.x * blockDim.x) {
+    double a = 0.0, b = 0.0;
+#pragma unroll 8
+    for (int k = 0; k < n; ++k) {
+      a += parts[2 * ((int64_t)k * r + j)];
+      b += parts[2 * ((int64_t)k * r + j) + 1];
+    }
+    out.put(j, a, b);
   }
 }
 
@@ -523,7 +707,7 @@ __global__ void svd_sort(const float* __restrict__ sigma, int r, int32_t* __rest
 // its vector is written as zeros (not completed to an orthonormal basis).
 __global__ void svd_write(const float* __restrict__ W, const float* __restrict__ V, const int32_t* __restrict__ order,
                           const float* __restrict__ sorted, const float* __restrict__ vnorm,
-                          const float* __restrict__ wnorm, int64_t M, int64_t N, int64_t L, int r, int k, int wide, int absorb, float* __restrict__ U, float* __restrict__ S, float* __restrict__ Vt,
+                          const float* __restrict__ wnorm, int lw, int64_t M, int64_t N, int64_t L, int r, int k, int wide, int absorb, float* __restrict__ U, float* __restrict__ S, float* __restrict__ Vt,
                           float* __restrict__ dropped) {
   const int64_t nl = M * k, nr = (int64_t)k * N, stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -538,9 +722,9 @@ __global__ void svd_write(const float* __restrict__ W, const float* __restrict__
     float x;
     if (from_w) {
       const float sc = sg > 0.0f ? (absorb ? sqrtf(sg) / wnorm[j] : 1.0f / wnorm[j]) : 0.0f;
-      x = W[blocked(i, j, L)] * sc;
+      x = W[blocked(i, j, L, lw)] * sc;
     } else {
-      x = V[blocked(i, j, r)] * (absorb ? sqrtf(fmaxf(sg, 0.0f)) / vnorm[j] : 1.0f / vnorm[j]);
+      x = V[blocked(i, j, r, lw)] * (absorb ? sqrtf(fmaxf(sg, 0.0f)) / vnorm[j] : 1.0f / vnorm[j]);
     }
     if (left)
       U[f] = x;
@@ -557,8 +741,10 @@ static size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 
 struct SplitLayout {
   SplitView v;
-  int64_t L, r, ns;  // ns: blocks of 16 columns
-  size_t w_off, v_off, sig_off, vn_off, wn_off, ord_off, sorted_off, cnt_off, total;
+  int64_t L, r, ns;  // ns: blocks of 2^lw columns
+  int lw, ctas;      // ctas: CTAs of svd_tall, 0: svd_jacobi
+  int parts;         // row parts of svd_norms
+  size_t w_off, v_off, sig_off, vn_off, wn_off, ord_off, sorted_off, cnt_off, parts_off, total;
 };
 
 static int plan_split(const tn_tensor* A, const int* left, int nleft, const int* right, int nright,
@@ -609,15 +795,28 @@ static int plan_split(const tn_tensor* A, const int* left, int nleft, const int*
   if (o.r > 0x3FFFFFFF) return TN_ERR_UNSUPPORTED;
   if (o.r > 0 && !o.v.A) return TN_ERR_ARG;
   o.ns = (o.r + SVD_B - 1) / SVD_B;
+  // rows shared out over the grid, 1024 or more each, where that makes more
+  // CTAs than the widest cluster has
+  if (o.ns <= 2 && o.L >= 1024 * (SVD_CLUSTER + 1)) {
+    const int64_t most = sm_count();
+    o.ctas = (int)(o.L / 1024 < most ? o.L / 1024 : most);
+  }
+  o.lw = o.ctas && o.r <= 4 ? 2 : o.ctas && o.r <= 8 ? 3 : 4;
+  const int64_t cols = o.ns << o.lw, norm_parts = (o.L + 4095) / 4096;
+  o.parts = (int)(norm_parts < 256 ? (norm_parts < 1 ? 1 : norm_parts) : 256);
   o.w_off = 0;
-  o.v_off = al256(sizeof(float) * (size_t)(o.L * o.ns * SVD_B));
-  o.sig_off = o.v_off + al256(sizeof(float) * (size_t)(o.r * o.ns * SVD_B));
+  o.v_off = al256(sizeof(float) * (size_t)(o.L * cols));
+  o.sig_off = o.v_off + al256(sizeof(float) * (size_t)(o.r * cols));
   o.vn_off = o.sig_off + al256(sizeof(float) * (size_t)o.r);
   o.wn_off = o.vn_off + al256(sizeof(float) * (size_t)o.r);
   o.ord_off = o.wn_off + al256(sizeof(float) * (size_t)o.r);
   o.sorted_off = o.ord_off + al256(sizeof(int32_t) * (size_t)o.r);
   o.cnt_off = o.sorted_off + al256(sizeof(float) * (size_t)(o.r + 1));  // the values, then the sweep count
-  o.total = o.cnt_off + 256;  // barrier word, rotations per sweep, the largest magnitude
+  o.parts_off = o.cnt_off + 256;  // barrier word, rotations per sweep, the largest magnitude
+  // Gram sums of svd_tall's CTAs (two sets), or the norms' parts
+  const size_t gram = sizeof(float) * 2 * (size_t)o.ctas * (size_t)(cols * cols);
+  const size_t norms = o.parts > 1 ? sizeof(double) * 2 * (size_t)o.parts * (size_t)o.r : 0;
+  o.total = o.parts_off + al256(gram > norms ? gram : norms);
   return TN_OK;
 }
 
@@ -677,7 +876,7 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
   float* wnorm = reinterpret_cast<float*>(base + lay.wn_off);
   int32_t* order = reinterpret_cast<int32_t*>(base + lay.ord_off);
   float* sorted = reinterpret_cast<float*>(base + lay.sorted_off);
-  const int64_t L = lay.L, cols = lay.ns * SVD_B;
+  const int64_t L = lay.L, cols = lay.ns << lay.lw;
   const int r = (int)lay.r;
   SvdParams P;
   P.W = W;
@@ -700,10 +899,17 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
       cudaMemsetAsync(P.sweeps, 0, sizeof(int), s) != cudaSuccess)
     return TN_ERR_CUDA;
   svd_largest<<<grid_for(L * r, 256), 256, 0, s>>>(lay.v, bits);
-  svd_gather<<<grid_for(L * cols, 256), 256, 0, s>>>(lay.v, bits, half, W, V, L, lay.r, cols);
+  svd_gather<<<grid_for(L * cols, 256), 256, 0, s>>>(lay.v, bits, half, lay.lw, W, V, L, lay.r, cols);
   if (cudaGetLastError() != cudaSuccess) return TN_ERR_CUDA;
-  static std::atomic<uint64_t> attr{0};
-  if (!smem_limit_once((const void*)svd_jacobi, sizeof(SvdSmem), &attr)) return TN_ERR_CUDA;
+  P.parts = reinterpret_cast<float*>(base + lay.parts_off);
+  void (*kernel)(const SvdParams) = svd_jacobi;
+  static std::atomic<uint64_t> attr[5];
+  std::atomic<uint64_t>* limit = &attr[0];
+  if (lay.ctas) {
+    kernel = cols == 4 ? svd_tall<4> : cols == 8 ? svd_tall<8> : cols == 16 ? svd_tall<16> : svd_tall<32>;
+    limit = &attr[cols == 4 ? 1 : cols == 8 ? 2 : cols == 16 ? 3 : 4];
+  }
+  if (!smem_limit_once((const void*)kernel, sizeof(SvdSmem), limit)) return TN_ERR_CUDA;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.blockDim = dim3(SVD_THREADS);
@@ -716,22 +922,30 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
   at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  // one CTA per SM; the rows of a pair over as many CTAs (up to 8, at least
-  // 32 rows each) as all pairs leave room for
-  const int64_t pairs = P.nb / 2, sms = sm_count();
-  P.cluster = 1;
-  while (P.cluster < SVD_CLUSTER && pairs * P.cluster * 2 <= sms && L >= 64 * P.cluster) P.cluster *= 2;
-  for (;; P.cluster /= 2) {
-    const int64_t ctas = pairs * P.cluster < sms ? pairs * P.cluster : sms / P.cluster * P.cluster;
-    cfg.gridDim = dim3((unsigned)ctas);
-    at[1].val.clusterDim.x = (unsigned)P.cluster;
-    int fit = 0;
-    if (P.cluster == 1 || (cudaOccupancyMaxActiveClusters(&fit, svd_jacobi, &cfg) == cudaSuccess &&
-                           (int64_t)fit * P.cluster >= ctas))
-      break;
+  if (lay.ctas) {
+    cfg.gridDim = dim3((unsigned)lay.ctas);
+    cfg.numAttrs = 1;
+  } else {
+    // one CTA per SM; the rows of a pair over as many CTAs (up to 8, at least
+    // 32 rows each) as all pairs leave room for
+    const int64_t pairs = P.nb / 2, sms = sm_count();
+    P.cluster = 1;
+    while (P.cluster < SVD_CLUSTER && pairs * P.cluster * 2 <= sms && L >= 64 * P.cluster) P.cluster *= 2;
+    for (;; P.cluster /= 2) {
+      const int64_t ctas = pairs * P.cluster < sms ? pairs * P.cluster : sms / P.cluster * P.cluster;
+      cfg.gridDim = dim3((unsigned)ctas);
+      at[1].val.clusterDim.x = (unsigned)P.cluster;
+      int fit = 0;
+      if (P.cluster == 1 || (cudaOccupancyMaxActiveClusters(&fit, svd_jacobi, &cfg) == cudaSuccess &&
+                             (int64_t)fit * P.cluster >= ctas))
+        break;
+    }
   }
-  if (cudaLaunchKernelEx(&cfg, svd_jacobi, P) != cudaSuccess) return TN_ERR_CUDA;
-  svd_norms<<<r, SVD_THREADS, 0, s>>>(W, V, L, r, bits, half, sigma, vnorm, wnorm);
+  if (cudaLaunchKernelEx(&cfg, kernel, P) != cudaSuccess) return TN_ERR_CUDA;
+  const SvdNorms norms{bits, half, sigma, vnorm, wnorm};
+  double* nparts = reinterpret_cast<double*>(base + lay.parts_off);
+  svd_norms<<<dim3((unsigned)lay.ns, (unsigned)lay.parts), SVD_THREADS, 0, s>>>(W, V, L, r, lay.lw, norms, nparts);
+  if (lay.parts > 1) svd_values<<<grid_for(r, 256), 256, 0, s>>>(nparts, lay.parts, r, norms);
   svd_sort<<<(r + 255) / 256, 256, 0, s>>>(sigma, r, order, sorted);
   if (cudaGetLastError() != cudaSuccess) return TN_ERR_CUDA;
   std::vector<float> host_sorted((size_t)r + 1);
@@ -744,7 +958,7 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
   if (used == 0) return TN_ERR_TIMEOUT;  // the barrier's wait expired
   if (sweeps) *sweeps = used;
   const int64_t k = tn_split_truncation(host_sorted.data(), r, max_singular_values, max_truncation_err);
-  svd_write<<<grid_for((lay.v.M + lay.v.N) * k + r, 256), 256, 0, s>>>(W, V, order, sorted, vnorm, wnorm, lay.v.M,
+  svd_write<<<grid_for((lay.v.M + lay.v.N) * k + r, 256), 256, 0, s>>>(W, V, order, sorted, vnorm, wnorm, lay.lw, lay.v.M,
                                                                         lay.v.N, L, r, (int)k, lay.v.wide, absorb ? 1 : 0,
                                                                         U, S, Vt, dropped);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return TN_ERR_CUDA;

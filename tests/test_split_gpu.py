@@ -214,3 +214,19 @@ def test_norms_far_apart(tn, kind, shape, count, size, seed):
         A *= size
     legs = ([0, 1], [2, 3]) if len(shape) == 4 else ([0], [1])
     check(tn, A.astype(np.float32), *legs)
+
+
+@pytest.mark.parametrize("shape", [(9215, 3), (9216, 1), (9217, 3), (10000, 4), (20001, 5), (9300, 8), (12001, 9),
+                                   (30000, 16), (9216, 17), (100003, 32), (9999, 33), (2, 20000), (17, 9999), (1, 300000)])
+def test_tall_nodes(tn, shape):
+    # rows shared out over the grid from 9216 on, stored 4, 8, 16 or 32 columns
+    # wide, ragged last parts and chunks, either side the long one; and the
+    # norms' row parts (4096); tolerances as above
+    check(tn, rand(51, shape), [0], [1])
+
+
+@pytest.mark.parametrize("count,rank,scale", [(4, 1, 1.0), (7, 2, 1e-13), (16, 3, 1e15), (31, 4, 1.0), (12, 12, 1e-20)])
+def test_tall_nodes_of_low_rank(tn, count, rank, scale):
+    rng = np.random.default_rng(60 + count)
+    A = rng.standard_normal((11000, rank)) @ rng.standard_normal((rank, count)) * scale
+    check(tn, A.astype(np.float32), [0], [1])
