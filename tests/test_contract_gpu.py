@@ -396,7 +396,7 @@ def test_fp32_group_with_long_k_ranges(tn):
         assert torch.equal(sp[4], torch.full_like(sp[4], 64.0))
 
 
-@pytest.mark.parametrize("M,N,K", [(2048, 512, 1024), (1024, 256, 1024), (20000, 16, 1100)])
+@pytest.mark.parametrize("M,N,K", [(2048, 512, 1024), (600, 512, 1024), (20000, 16, 1100)])
 def test_fp32_chunks_of_a_unit(tn, M, N, K):
     # several chains added up in the shared-memory region that the result's
     # rows then pass through, in each tile shape (64 x 128, 32 x 128, 16 x 256

@@ -174,6 +174,15 @@ def test_planning_a_long_shared_index_is_quick(built, tmp_path):
     assert min(max(p[5] for p in plans[i * len(cases):(i + 1) * len(cases)]) for i in range(5)) <= 100.0
 
 
+def test_lone_contractions_spread_a_long_shared_index(built, tmp_path):
+    """A lone float32 contraction of a few dozen tiles cuts its shared index
+    into as many ranges as the SMs take, not two at most."""
+    cases = [(885, 150, 2862, 0, 0), (150, 885, 2862, 1, 1), (1951, 367, 1797, 0, 1), (640, 640, 5000, 0, 1),
+             (128, 2048, 4000, 0, 0), (118, 1361, 1417, 1, 1)]
+    for case, (_, _, units, *_) in zip(cases, simt_plans(built, tmp_path, "alone", cases)):
+        assert units >= 3, case
+
+
 @pytest.mark.parametrize("sweeps", [13, -40])
 def test_split_node_warns_at_the_sweep_limit(monkeypatch, sweeps):
     """The binding says so when the library reports that the sweeps ran out
