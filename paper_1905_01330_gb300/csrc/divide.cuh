@@ -47,9 +47,16 @@ template <bool BOUNDED, int R, int N>
 __device__ __forceinline__ void divide_rows(float (&v)[R][N], const float (&s)[R]) {
   static_assert(R == 2 || R == 4 || R == 8, "rows");
   const int lane = threadIdx.x & 31;
-  float mine = s[0];
+  // row lane % R's scale, by bits of the lane (an indexed choice goes through
+  // local memory)
+  float pick[R];
 #pragma unroll
-  for (int i = 1; i < R; ++i) mine = (lane & (R - 1)) == i ? s[i] : mine;
+  for (int i = 0; i < R; ++i) pick[i] = s[i];
+#pragma unroll
+  for (int n = R / 2, bit = 1; n > 0; n /= 2, bit *= 2)
+#pragma unroll
+    for (int i = 0; i < n; ++i) pick[i] = (lane & bit) ? pick[2 * i + 1] : pick[2 * i];
+  const float mine = pick[0];
   bool plain = mine > 0x1p-24f && mine < 0x1p24f && !full_mantissa(mine);
   unsigned least = 0xFFFFFFFFu;  // of the values without their signs, times 2, less 1: zeros come last
   float most = 0.0f;
