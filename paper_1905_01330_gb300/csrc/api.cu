@@ -409,20 +409,14 @@ int tn::group_plan_create_ex(const tn_contract_spec* specs, int nspecs, int prec
     }
   }
   if (prec == TN_PREC_FP32 && !p->skinny) {
-    // a large group keeps a tile's k ranges (2048 shared indices each) in one
-    // unit, up to four of them, where a contraction has 16 tiles or more: no
-    // zeroing pass and no atomics, and the units still outnumber the CTAs
-    // that run at once eight times over
+    // a large group keeps a tile's k ranges (2048 shared indices at most, of
+    // even lengths: each is one chain of sums) in one unit, up to four of them,
+    // where a contraction has 16 tiles or more: no zeroing pass and no atomics,
+    // and the units still outnumber the CTAs that run at once eight times over
     int64_t units = 0;
     for (const auto& d : p->descs) units += (int64_t)d.tiles_m * d.tiles_n * d.splits;
-    for (auto& d : p->descs) {
-      if (units >= 8 * min_units_single() && (int64_t)d.tiles_m * d.tiles_n >= 16) {
-        const int64_t range = 4 * 64 * MAX_SLABS_PER_UNIT;
-        d.splits = (int32_t)((d.K + range - 1) / range);
-        d.k_per_split = range;
-      }
-      plan_simt(&d, SimtPlan::group);
-    }
+    for (auto& d : p->descs)
+      plan_simt(&d, SimtPlan::group, units >= 8 * min_units_single() && (int64_t)d.tiles_m * d.tiles_n >= 16 ? 4 : 1);
   }
   auto unit_work = [&](const ContractDesc& d) {
     const bool simt = prec == TN_PREC_FP32 && !p->skinny;

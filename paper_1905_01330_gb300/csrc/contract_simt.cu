@@ -463,13 +463,13 @@ bool vector_gather(const float* X, bool kfast, int nr, const int32_t* rdim, cons
 
 }  // namespace
 
-void plan_simt(ContractDesc* d, SimtPlan how) {
+void plan_simt(ContractDesc* d, SimtPlan how, int chains) {
   // A unit's chain lengths are those of the k ranges plan_units gave; a lone
   // contraction may run several of them in one unit.
   const int64_t slabs = (d->K + 63) / 64, chunk = d->k_per_split < 2048 ? d->k_per_split / 64 : 32;
   d->chunk = (int16_t)chunk;
   int tile = SIMT_TILE_PAIR, swap = 0;
-  int64_t per = d->k_per_split;
+  int64_t per = std::min<int64_t>(chains, d->splits) * d->k_per_split;
   if (how != SimtPlan::pairs) {
     // cycles of a 16-wide slab (two CTAs an SM), measured at 2048^3 and, for
     // the thin tiles, in proportion to their FMAs and shared-memory reads

@@ -88,11 +88,11 @@ void plan_units(ContractDesc* d, int64_t min_units);
 // planned by plan_units, whose k ranges become the chains a result is summed
 // in: alone (a unit may run several of them, so that the tiles fill the SMs),
 // in a sweep over a chain (all of them in a unit or one, so that a result is
-// the sum of the chains added one by one, as it always was: its float64
-// energies show such sums in the seventh digit), in
-// a group (the k ranges as given) or as 128 x 128 units (as given).
+// the sum of the chains added one by one: a sum of sums shows in the seventh
+// digit of a float64 energy), in a group (`chains` of them in a unit) or as 128
+// x 128 units (one).
 enum class SimtPlan { alone, sweep, group, pairs };
-void plan_simt(ContractDesc* d, SimtPlan how);
+void plan_simt(ContractDesc* d, SimtPlan how, int chains = 1);
 // SMs of the current device (152 where there is none).
 int sm_count();
 // Work units a lone contraction asks plan_units for (two per SM).

@@ -106,7 +106,8 @@ PLANS = r"""
 #include "tn_internal.h"
 using namespace tn;
 int main(int argc, char** argv) {
-  const SimtPlan how = strcmp(argv[1], "sweep") ? SimtPlan::alone : SimtPlan::sweep;
+  const bool group = !strcmp(argv[1], "group");
+  const SimtPlan how = group ? SimtPlan::group : !strcmp(argv[1], "sweep") ? SimtPlan::sweep : SimtPlan::alone;
   long long M, N, K, ta, tb;
   while (scanf("%lld %lld %lld %lld %lld", &M, &N, &K, &ta, &tb) == 5) {
     tn_tensor A{}, B{}, C{};
@@ -119,10 +120,10 @@ int main(int argc, char** argv) {
     const int la = ta ? 0 : 1, lb = tb ? 1 : 0;
     ContractDesc d;
     if (plan_contract(&A, &la, &B, &lb, 1, &C, &d) != TN_OK) return 1;
-    plan_units(&d, 304);
+    plan_units(&d, group ? 1 : 304);
     const long long ranges = d.splits, range = d.k_per_split;
     const auto t0 = std::chrono::steady_clock::now();
-    plan_simt(&d, how);
+    plan_simt(&d, how, group ? 4 : 1);
     const double us = std::chrono::duration<double, std::micro>(std::chrono::steady_clock::now() - t0).count();
     printf("%lld %lld %d %lld %d %.2f\n", ranges, range, (int)d.splits, (long long)d.k_per_split, (int)d.chunk, us);
   }
@@ -172,6 +173,15 @@ def test_planning_a_long_shared_index_is_quick(built, tmp_path):
     for case, (_, _, units, per, chunk, _) in zip(cases * 5, plans):
         assert units * per >= case[2] > (units - 1) * per and per % (64 * chunk) == 0, (case, units, per)
     assert min(max(p[5] for p in plans[i * len(cases):(i + 1) * len(cases)]) for i in range(5)) <= 100.0
+
+
+def test_a_group_keeps_the_lengths_of_its_chains(built, tmp_path):
+    """A large float32 group runs up to four k ranges of a tile in one unit, as
+    chains of the lengths plan_units gave them (even ones: 36 slabs are 18 + 18,
+    not 32 + 4, whose longer chain rounds worse)."""
+    cases = [(640, 512, k, 0, 0) for k in (40, 64, 2048, 2049, 2304, 4200, 6145, 9000, 50000)]
+    for case, (ranges, rng, units, per, chunk, _) in zip(cases, simt_plans(built, tmp_path, "group", cases)):
+        assert chunk * 64 == rng and per == min(4, ranges) * rng and units == -(-case[2] // per), case
 
 
 def test_lone_contractions_spread_a_long_shared_index(built, tmp_path):
