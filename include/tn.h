@@ -89,6 +89,11 @@ int tn_tensor_init(tn_tensor* t, void* data, int rank, const int64_t* shape);
  *   C      output tensor: float32, row-major contiguous, shape as above; it
  *          must not overlap A or B
  *   prec   TN_PREC_FP32 / TN_PREC_BF16 / TN_PREC_BF16X3
+ * A long shared index may be cut into ranges whose sums are added to C with
+ * float32 atomics: where more than two meet, results agree between runs to
+ * rounding, not bit for bit. The kernels' waits within a CTA are bounded (2 s,
+ * every prec): on expiry TN_ERR_TIMEOUT is recorded in the status word
+ * (tn_sync_status) and C is incomplete.
  * Errors: TN_ERR_ARG, TN_ERR_SHAPE, TN_ERR_UNSUPPORTED, TN_ERR_CUDA.
  */
 int tn_contract(const tn_tensor* A, const int* legsA, const tn_tensor* B, const int* legsB,
@@ -371,7 +376,9 @@ int tn_mps_inner(const tn_mps* bra, const tn_mps* ket, int prec, void* workspace
  *     site (a pack of L and the core, the GEMM of (i), step (ii) written
  *     straight into (iii)'s packed operand, the GEMM of (iii)).
  *   - FP32 and wider MPOs: three contractions, a float32 step (ii) and a
- *     max-abs pass per site.
+ *     max-abs pass per site. FP32 sums run in one order (unless a shared
+ *     index of 768 or more meets fewer than 16 result tiles of 32 x 128): a
+ *     call repeated on the same device gives the same bits.
  *   result: DEVICE pointer to 4 doubles {e_value, e_log_scale, n_value,
  *           n_log_scale}: <psi|H|psi> = e_value * exp(e_log_scale) and
  *           <psi|psi> = n_value * exp(n_log_scale); the energy per the
@@ -498,8 +505,10 @@ int tn_mps_classify(const tn_mps* W, int label_site, int n_labels, const float* 
  *           otherwise). TN_PREC_BF16X3 needs chi <=
  *           64 (its staging at chi = 128 does not fit in shared memory).
  * Errors: as tn_mps_classify, plus TN_ERR_UNSUPPORTED for TN_PREC_BF16X3 at
- * chi = 128. The gradient reductions are float32 atomics: results agree
- * between runs to rounding, not bit for bit.
+ * chi = 128. The gradient reductions are float32 atomics (TN_PREC_FP32: a
+ * core's gradient is the sum of several parts of the batch, 128 samples or
+ * more each, added in any order): results agree between runs to rounding, not
+ * bit for bit.
  */
 int tn_mps_classify_backward(const tn_mps* W, int label_site, int n_labels, const float* pixels,
                              int batch, int prec, int ckpt_every, const float* dftilde,
@@ -592,7 +601,9 @@ int tn_mps_classify_separate_backward(const tn_mps* Ws, int n_mps, const float* 
  * Arithmetic: float32 one-sided Jacobi (Hestenes) on the r columns of
  * length max(M, N), in blocks of 16 columns (the rotations of a block pair on
  * its Gram matrix, their product applied to the columns); singular values are
- * the column norms over the accumulated rotations' own. The singular vectors
+ * the column norms (64-bit sums) over the accumulated rotations' own. The
+ * columns are scaled by a power of two, so the node's scale does not matter;
+ * columns below 2^-90 of the node's norm are not rotated. The singular vectors
  * of a zero singular value on the longer side (columns of U when M >= N, rows
  * of V^T when M < N) are zeros. The sweeps are one cooperative launch with
  * bounded device-wide barriers. Workspace: tn_split_node_workspace_bytes

@@ -511,7 +511,7 @@ int tn_mps_classify_backward(const tn_mps* W, int label_site, int n_labels, cons
   const int chi = w.chi, n = W->n, ls = label_site, L = n_labels;
   const int split = prec == TN_PREC_BF16X3;
   if (prec != TN_PREC_FP32 && !cls_adj_tc_supported(chi, split)) return TN_ERR_UNSUPPORTED;
-  if (prec == TN_PREC_FP32 && batch > 0 && stream_capturing(s)) return TN_ERR_UNSUPPORTED;  // as documented
+  if (prec == TN_PREC_FP32 && batch > 0 && stream_capturing(s)) return TN_ERR_UNSUPPORTED;  // by the entry point's contract; nothing below needs it
   if (batch == 0) {
     for (int i = 0; i < n; ++i) {
       const int64_t e = W->bond[i] * 2 * W->bond[i + 1] * (i == ls ? L : 1);

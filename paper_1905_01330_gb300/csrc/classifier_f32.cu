@@ -26,8 +26,8 @@
 // conflicts. A step at chi = 64 takes ~7,300 cycles for 64 samples, 5,070 of
 // them the products (the FMA pipe's own 4,096), the rest the wait for the slab
 // (~250), the maximum, the division and the publishing.
-// Measured (784 sites, batch 4096, chi = 64): forward 10.9 -> 1.4 ms, training
-// step 53.2 -> 6.2 ms.
+// Measured (784 sites, batch 4096, chi = 64): forward 10.9 -> 1.5 ms, training
+// step 53.2 -> 6.3 ms.
 #include <math.h>
 
 #include "classifier_f32.h"

@@ -9,7 +9,7 @@ separated. Singular vectors are unique only up to sign, so they are checked
 for what must hold instead: orthonormal columns of U and rows of V^T (for
 non-zero values) and sqrt(S) carried on both sides by split_node.
 
-Tolerances (float32 one-sided Jacobi, rotation angles in float64): singular
+Tolerances (float32 one-sided Jacobi, column norms in float64): singular
 values within 5e-5 of the largest one; products within 5e-5 of |A|_F;
 orthonormality within 1e-4.
 """
