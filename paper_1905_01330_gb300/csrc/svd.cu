@@ -721,8 +721,8 @@ __global__ void svd_write(const float* __restrict__ W, const float* __restrict__
     const bool from_w = left != (wide != 0);  // left from W iff M >= N
     float x;
     if (from_w) {
-      const float sc = sg > 0.0f ? (absorb ? sqrtf(sg) / wnorm[j] : 1.0f / wnorm[j]) : 0.0f;
-      x = W[blocked(i, j, L, lw)] * sc;
+      // by the norm itself: a column of rounding noise may be too small for its reciprocal
+      x = sg > 0.0f ? W[blocked(i, j, L, lw)] / wnorm[j] * (absorb ? sqrtf(sg) : 1.0f) : 0.0f;
     } else {
       x = V[blocked(i, j, r, lw)] * (absorb ? sqrtf(fmaxf(sg, 0.0f)) / vnorm[j] : 1.0f / vnorm[j]);
     }

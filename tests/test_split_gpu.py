@@ -188,6 +188,7 @@ def node_kinds():
         out.append(("bond", (8, 2, 2, 8), z, 1.0))
     for last in (1e-12, 1e-22, 1e-30):
         out.append(("graded", (40, 40), 0, last))
+    out += [("ones", shape, 0, scale) for shape in ((100, 20), (48, 50), (100, 50)) for scale in (1e8, 1e25, 1e32)]
     out += [("full", (32, 32), 0, scale) for scale in (1e-18, 1e-20, 1e-25, 1e18, 1e25)]
     return out
 
@@ -208,6 +209,8 @@ def test_norms_far_apart(tn, kind, shape, count, size, seed):
         A *= size
     elif kind == "bond":
         A[count:] = 0.0
+    elif kind == "ones":  # null columns of rounding noise far below a large value
+        A = np.full(shape, size)
     elif kind == "graded":
         A *= np.logspace(0, np.log10(size), shape[1])
     else:
