@@ -603,7 +603,9 @@ int tn_mps_classify_separate_backward(const tn_mps* Ws, int n_mps, const float* 
  * its Gram matrix, their product applied to the columns); singular values are
  * the column norms (64-bit sums) over the accumulated rotations' own. The
  * columns are scaled by a power of two, so the node's scale does not matter;
- * columns below 2^-90 of the node's norm are not rotated. The singular vectors
+ * columns below 2^-90 of the node's norm are not rotated, and a column (of the
+ * shorter side) with an infinite or NaN entry takes no part: its value is
+ * infinite (the first) or NaN (the last), the others' are theirs. The singular vectors
  * of a zero singular value on the longer side (columns of U when M >= N, rows
  * of V^T when M < N) are zeros. The sweeps are one cooperative launch with
  * bounded device-wide barriers. Workspace: tn_split_node_workspace_bytes

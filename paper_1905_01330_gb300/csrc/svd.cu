@@ -94,28 +94,32 @@ __device__ __forceinline__ int64_t leg_offset(int64_t idx, int n, const int32_t*
   return off;
 }
 
-// *bits: the bits of the node's largest magnitude (0 before).
-__global__ void svd_largest(SplitView v, unsigned* bits) {
+// *bits: the bits of the node's largest finite magnitude (0 before); odd[c]:
+// bit 0 an infinity, bit 1 a NaN in column c of W (0 before). Such a column
+// takes no part: a product with it would spread over its block.
+__global__ void svd_largest(SplitView v, unsigned* bits, unsigned* odd) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   unsigned m = 0u;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < v.M * v.N; e += stride) {
     const int64_t i = e <= 0xFFFFFFFFll && v.N <= 0xFFFFFFFFll ? (uint32_t)e / (uint32_t)v.N : e / v.N, j = e - i * v.N;
     const float x = v.A[leg_offset(i, v.nl, v.ldim, v.lstr) + leg_offset(j, v.nr, v.rdim, v.rstr)];
-    m = max(m, __float_as_uint(fabsf(x)));
+    const unsigned b = __float_as_uint(fabsf(x));
+    if (b < 0x7F800000u) m = max(m, b);
+    else atomicOr(odd + (v.wide ? i : j), b == 0x7F800000u ? 1u : 2u);
   }
   m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0 && m) atomicMax(bits, m);
 }
 
-// The exponent of the power of two W is scaled by; 0 for zeros, infinities and
-// NaN. half: (log2 of the matrix's entries) / 2, rounded up.
+// The exponent of the power of two W is scaled by; 0 without a finite entry but
+// zeros. half: (log2 of the matrix's entries) / 2, rounded up.
 __device__ __forceinline__ int svd_shift(unsigned bits, int half) {
-  return bits == 0u || bits >= 0x7F800000u ? 0 : SVD_TOP - half - 1 - ilogbf(__uint_as_float(bits));
+  return bits == 0u ? 0 : SVD_TOP - half - 1 - ilogbf(__uint_as_float(bits));
 }
 
 // W in blocks of 2^lw columns (16; a tall node's one block may have fewer),
-// [block][row][column] (zeros past column r), V = I likewise.
-__global__ void svd_gather(SplitView v, const unsigned* bits, int half, int lw, float* __restrict__ W, float* __restrict__ V,
+// [block][row][column] (zeros past column r and for `odd` ones), V = I likewise.
+__global__ void svd_gather(SplitView v, const unsigned* bits, const unsigned* odd, int half, int lw, float* __restrict__ W, float* __restrict__ V,
                            int64_t L, int64_t r, int64_t cols) {
   const int shift = svd_shift(*bits, half);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -124,7 +128,7 @@ __global__ void svd_gather(SplitView v, const unsigned* bits, int half, int lw, 
     const int64_t blk = (cols >> lw) == 1 ? 0 : w / (L << lw), in = w - ((blk * L) << lw);
     const int64_t row = in >> lw, col = (blk << lw) + (in & ((1 << lw) - 1));
     float x = 0.0f;
-    if (col < r) {
+    if (col < r && odd[col] == 0u) {
       const int64_t i = v.wide ? col : row, j = v.wide ? row : col;
       x = ldexpf(v.A[leg_offset(i, v.nl, v.ldim, v.lstr) + leg_offset(j, v.nr, v.rdim, v.rstr)], shift);
     }
@@ -618,13 +622,13 @@ __device__ __forceinline__ int64_t blocked(int64_t row, int64_t col, int64_t n, 
 // Column j's values from its sums of squares: vnorm[j] = |V[:, j]|, wnorm[j] =
 // |W[:, j]| and sigma[j] = their quotient, without W's power of two. Both blocks
 // took the same products with Q, so what these left of the unit length of V's
-// columns is also in W's and cancels.
+// columns is also in W's and cancels. An odd column has the norm its entries have.
 struct SvdNorms {
-  const unsigned* bits;
+  const unsigned *bits, *odd;
   int half;
   float *sigma, *vnorm, *wnorm;
   __device__ __forceinline__ void put(int64_t j, double a, double b) const {
-    const double vn = sqrt(b), wn = sqrt(a);
+    const double vn = sqrt(b), wn = odd[j] == 0u ? sqrt(a) : (odd[j] & 2u) ? (double)NAN : (double)INFINITY;
     vnorm[j] = (float)vn;
     wnorm[j] = (float)wn;
     sigma[j] = (float)ldexp(wn / vn, -svd_shift(*bits, half));
@@ -744,7 +748,7 @@ struct SplitLayout {
   int64_t L, r, ns;  // ns: blocks of 2^lw columns
   int lw, ctas;      // ctas: CTAs of svd_tall, 0: svd_jacobi
   int parts;         // row parts of svd_norms
-  size_t w_off, v_off, sig_off, vn_off, wn_off, ord_off, sorted_off, cnt_off, parts_off, total;
+  size_t w_off, v_off, sig_off, vn_off, wn_off, ord_off, sorted_off, cnt_off, odd_off, parts_off, total;
 };
 
 static int plan_split(const tn_tensor* A, const int* left, int nleft, const int* right, int nright,
@@ -812,7 +816,8 @@ static int plan_split(const tn_tensor* A, const int* left, int nleft, const int*
   o.ord_off = o.wn_off + al256(sizeof(float) * (size_t)o.r);
   o.sorted_off = o.ord_off + al256(sizeof(int32_t) * (size_t)o.r);
   o.cnt_off = o.sorted_off + al256(sizeof(float) * (size_t)(o.r + 1));  // the values, then the sweep count
-  o.parts_off = o.cnt_off + 256;  // barrier word, rotations per sweep, the largest magnitude
+  o.odd_off = o.cnt_off + 256;  // barrier word, rotations per sweep, the largest magnitude
+  o.parts_off = o.odd_off + al256(sizeof(unsigned) * (size_t)o.r);
   // Gram sums of svd_tall's CTAs (two sets), or the norms' parts
   const size_t gram = sizeof(float) * 2 * (size_t)o.ctas * (size_t)(cols * cols);
   const size_t norms = o.parts > 1 ? sizeof(double) * 2 * (size_t)o.parts * (size_t)o.r : 0;
@@ -895,11 +900,12 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
   unsigned* bits = reinterpret_cast<unsigned*>(P.counts) + SVD_MAX_SWEEPS;
   int half = 0;  // 4^half >= M N
   while (half < 31 && (int64_t(1) << (2 * half)) < L * r) ++half;
-  if (cudaMemsetAsync(base + lay.cnt_off, 0, 256, s) != cudaSuccess ||
+  unsigned* odd = reinterpret_cast<unsigned*>(base + lay.odd_off);
+  if (cudaMemsetAsync(base + lay.cnt_off, 0, lay.parts_off - lay.cnt_off, s) != cudaSuccess ||
       cudaMemsetAsync(P.sweeps, 0, sizeof(int), s) != cudaSuccess)
     return TN_ERR_CUDA;
-  svd_largest<<<grid_for(L * r, 256), 256, 0, s>>>(lay.v, bits);
-  svd_gather<<<grid_for(L * cols, 256), 256, 0, s>>>(lay.v, bits, half, lay.lw, W, V, L, lay.r, cols);
+  svd_largest<<<grid_for(L * r, 256), 256, 0, s>>>(lay.v, bits, odd);
+  svd_gather<<<grid_for(L * cols, 256), 256, 0, s>>>(lay.v, bits, odd, half, lay.lw, W, V, L, lay.r, cols);
   if (cudaGetLastError() != cudaSuccess) return TN_ERR_CUDA;
   P.parts = reinterpret_cast<float*>(base + lay.parts_off);
   void (*kernel)(const SvdParams) = svd_jacobi;
@@ -942,7 +948,7 @@ int tn_split_node(const tn_tensor* A, const int* left, int nleft, const int* rig
     }
   }
   if (cudaLaunchKernelEx(&cfg, kernel, P) != cudaSuccess) return TN_ERR_CUDA;
-  const SvdNorms norms{bits, half, sigma, vnorm, wnorm};
+  const SvdNorms norms{bits, odd, half, sigma, vnorm, wnorm};
   double* nparts = reinterpret_cast<double*>(base + lay.parts_off);
   svd_norms<<<dim3((unsigned)lay.ns, (unsigned)lay.parts), SVD_THREADS, 0, s>>>(W, V, L, r, lay.lw, norms, nparts);
   if (lay.parts > 1) svd_values<<<grid_for(r, 256), 256, 0, s>>>(nparts, lay.parts, r, norms);

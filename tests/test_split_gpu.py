@@ -233,3 +233,22 @@ def test_tall_nodes_of_low_rank(tn, count, rank, scale):
     rng = np.random.default_rng(60 + count)
     A = rng.standard_normal((11000, rank)) @ rng.standard_normal((rank, count)) * scale
     check(tn, A.astype(np.float32), [0], [1])
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("shape", [(40, 24), (24, 40), (300, 65), (11000, 5), (3, 20000)])
+def test_an_infinite_or_nan_entry_stays_in_its_column(tn, shape, value):
+    # the column (of the shorter side) that holds it has no finite value: first
+    # among the values if infinite, last if NaN; the others' are theirs
+    A = rand(71, shape)
+    short = int(shape[0] >= shape[1])
+    at = (shape[0] // 2, shape[1] // 3)
+    A[at] = value
+    info = {}
+    _, s, _, d = tn.split_node(torch.from_numpy(A).cuda(), [0], [1], full_svd=True, info=info)
+    got = s.cpu().numpy().astype(np.float64)
+    assert info["sweeps"] > 0 and len(got) == min(shape) and d.numel() == 0
+    rest = np.linalg.svd(np.delete(A.astype(np.float64), at[short], axis=short), compute_uv=False)
+    odd, others = (got[-1], got[:-1]) if np.isnan(value) else (got[0], got[1:])
+    assert np.isnan(odd) if np.isnan(value) else odd == np.inf
+    assert np.abs(others - rest).max() <= 5e-5 * rest[0]
