@@ -50,12 +50,22 @@ class TnNconStep(ctypes.Structure):
                 ("legs_b", ctypes.c_int32 * TN_MAX_RANK), ("shape", ctypes.c_int64 * TN_MAX_RANK)]
 
 
+SHORT_CHAIN = 16
+
+
 def _chain(cores, bonds, d):
-    """(TnChain, its host arrays). The arrays are filled through `array`: ctypes
-    converts a list element by element (784 cores: the description 411 -> 280 us)."""
+    """(TnChain, its host arrays). Long chains' arrays are filled through `array`:
+    ctypes converts a list element by element (784 cores: the description 411 ->
+    280 us). Short ones take the list: the buffers behind `array` are more
+    objects for the garbage collector (a norm of 6 cores 40.5 us, 39 by lists)."""
     n = len(cores)
-    bond_arr = (ctypes.c_int64 * (n + 1)).from_buffer(array("q", bonds))
-    ptr_arr = (ctypes.c_void_p * n).from_buffer(array("Q", [c.data_ptr() for c in cores]))
+    ptrs = [c.data_ptr() for c in cores]
+    if n < SHORT_CHAIN:
+        bond_arr = (ctypes.c_int64 * (n + 1))(*bonds)
+        ptr_arr = (ctypes.c_void_p * n)(*ptrs)
+    else:
+        bond_arr = (ctypes.c_int64 * (n + 1)).from_buffer(array("q", bonds))
+        ptr_arr = (ctypes.c_void_p * n).from_buffer(array("Q", ptrs))
     ch = TnChain()
     ch.n = n
     ch.d = d

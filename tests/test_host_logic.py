@@ -220,3 +220,16 @@ def test_split_node_warns_at_the_sweep_limit(monkeypatch, sweeps):
         u, vh, dropped = tn.split_node(torch.ones(3, 4), [0], [1])
     assert u.shape == (3, 2) and vh.shape == (2, 4) and dropped.shape == (1,)
     assert [w.category for w in got] == ([RuntimeWarning] if sweeps < 0 else [])
+
+
+@pytest.mark.parametrize("n", [1, 2, 15, 16, 40])
+def test_chain_descriptions_short_and_long(n):
+    """Both ways of filling a chain's arrays hold the bonds and pointers."""
+    import torch
+    from paper_1905_01330_gb300 import tn
+    bonds = [1] + [2 + i % 5 for i in range(n - 1)] + [1]
+    cores = [torch.zeros(bonds[i], 3, bonds[i + 1]) for i in range(n)]
+    ch, keep = tn._chain(cores, bonds, 3)
+    assert (ch.n, ch.d) == (n, 3) and keep[2] is cores
+    assert [ch.bond[i] for i in range(n + 1)] == bonds
+    assert [ch.cores[i] for i in range(n)] == [c.data_ptr() for c in cores]
